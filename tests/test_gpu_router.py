@@ -82,3 +82,18 @@ def test_route_plan_run_end_to_end():
     ctx.check()
     ref = oracle.forward(oracle_weights(spec, W), x, None, ids_ref, w_ref)
     assert_close(b.y.float().cpu().numpy(), ref["y"])
+
+
+@pytest.mark.parametrize("E,shift", [(256, 0), (256, 1), (255, 0), (257, 0), (260, 0), (260, 3), (1024, 1), (1, 0)])
+def test_router_row_widths_and_alignment(E, shift):
+    """Rows of 16-byte aligned quads, rows that are not, and the border between the two register widths."""
+    T, k = 37, min(8, E)
+    z = np.random.default_rng([E, shift]).standard_normal((T, E), dtype=np.float32)
+    z[::3, E // 2] = -0.0                                            # -0 and +0 are equal logits
+    z[::3, E // 3] = 0.0
+    buf = torch.zeros(T * E + shift, dtype=torch.float32, device="cuda")
+    buf[shift:] = torch.from_numpy(z).cuda().reshape(-1)
+    ids, w = moe.route(buf[shift:].view(T, E), k)
+    ids_ref, w_ref = oracle.router(z, k)
+    assert np.array_equal(ids.cpu().numpy(), ids_ref)
+    np.testing.assert_allclose(w.cpu().numpy(), w_ref, rtol=2e-6, atol=1e-8)
