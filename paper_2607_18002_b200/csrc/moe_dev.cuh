@@ -20,8 +20,8 @@ constexpr int kStages = 3;           // shared-memory pipeline depth (64 KB per 
 constexpr int kCombineTokens = 16;   // tokens per combine tile ...
 constexpr int kCombineTokensSmall = 4;     // ... of an op with at most kCombineSmallBatch tokens (a decode batch): its
 constexpr int kCombineSmallBatch = 1024;   // combine is a latency chain per token, so it is spread over more units
-constexpr int kPlanChunk = 256;      // routed rows ranked by one warp in the plan kernels
-constexpr int kGroupWork = 16;       // work tiles per dependency group of the tile list
+constexpr int kPlanChunk = 1024;     // fewest routed rows a block of the plan kernels owns
+constexpr int kLagWork = 16;         // gate/up work tiles listed between an expert's gate/up tiles and its down tiles
 constexpr int kWorkRowsBf16 = 256;   // rows of a work tile: two m-tiles share each weight tile
 constexpr int kWorkRowsFp8 = 128;    // fp8: the accumulator and both partial buffers fill TMEM
 constexpr int kMaxOps = 16;
@@ -103,8 +103,7 @@ struct __align__(128) OpDev {
   __nv_bfloat16* D;      // [Rmax, H]  expert output, packed order
   MTile* mtiles;         // [max_mtiles]
   int4* tile_list;       // [max_tiles] queue entries in claim order
-  int* plan_hist;        // [n_chunks, E] per-warp histogram
-  int* plan_base;        // [n_chunks, E] per-warp base rank of each expert
+  int* plan_hist;        // [n_chunks, E] rows per plan block and expert
   PlanState* plan;
   RunState* run;
   int* g1_done;          // [max_mtiles] committed gate/up tiles per work tile

@@ -9,12 +9,11 @@
 #include "moe_dev.cuh"
 
 namespace moe {
-cudaError_t launch_plan(const OpDev* d_op, Global* g, int slot, int T, int k, int E, int NT1,
-                        int NT2, int work_rows, cudaStream_t stream);
-cudaError_t launch_plan_masked(const OpDev* d_op, Global* g, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
+cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, cudaStream_t stream);
+cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
                                cudaStream_t stream);
-cudaError_t launch_plan_pair(const OpDev* dp, const OpDev* pp, const OpDev* d, const OpDev* p, int* gather_m, int* comb_d,
-                             int* comb_p, int Rd, int Rp, int E, int NT1, int NT2, int work_rows, int carrier_rows,
+cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, const OpDev& p, int* gather, int* comb_d,
+                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows,
                              int slot_d, int slot_p, cudaStream_t stream);
 cudaError_t launch_combine(const OpDev* d_op, int T, int k, int H, cudaStream_t stream);
 cudaError_t prepare_run_kernel();
@@ -72,14 +71,14 @@ Layout make_layout(const moe_config_t* c) {
   const int comb_large = (c->max_tokens_per_op + kCombineTokens - 1) / kCombineTokens;
   const int max_comb = comb_small > comb_large ? comb_small : comb_large;
   L.max_tiles = L.max_mtiles * (L.NT1 + L.NT2) + max_comb;
-  const size_t n_chunks = ((size_t)L.max_rows + kPlanChunk - 1) / kPlanChunk;
+  const size_t n_chunks = ((size_t)L.max_rows + kPlanChunk - 1) / kPlanChunk;   // at most one histogram per chunk
 
   size_t off = 0;
   L.A_off = off;       off = align_up(off + (size_t)L.max_rows * I * 2, 1024);
   L.D_off = off;       off = align_up(off + (size_t)L.max_rows * H * 2, 1024);
   L.mtiles_off = off;  off = align_up(off + (size_t)L.max_mtiles * sizeof(MTile), 1024);
   L.tiles_off = off;   off = align_up(off + (size_t)L.max_tiles * sizeof(int4), 1024);
-  L.hist_off = off;    off = align_up(off + 2 * n_chunks * E * 4, 1024);   // histogram + base ranks
+  L.hist_off = off;    off = align_up(off + n_chunks * E * 4, 1024);
   L.plan_off = off;    off = align_up(off + sizeof(PlanState), 1024);
   L.ptiles_off = off;  off = align_up(off + (size_t)L.max_tiles * sizeof(int4), 1024);
   L.pgather_off = off; off = align_up(off + (size_t)L.max_rows * 4, 1024);
@@ -294,7 +293,6 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
   h.mtiles = reinterpret_cast<MTile*>(sb + L.mtiles_off);
   h.tile_list = reinterpret_cast<int4*>(sb + L.tiles_off);
   h.plan_hist = reinterpret_cast<int*>(sb + L.hist_off);
-  h.plan_base = h.plan_hist + (((size_t)L.max_rows + kPlanChunk - 1) / kPlanChunk) * c.n_experts;
   h.plan = reinterpret_cast<PlanState*>(sb + L.plan_off);
   h.run = reinterpret_cast<RunState*>(ctx->rs_base(slot));
   h.g1_done = reinterpret_cast<int*>(ctx->rs_base(slot) + sizeof(RunState));
@@ -339,10 +337,8 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
     ctx->uploaded[slot] = true;
   }
   const int work_rows = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
-  const cudaError_t pe = masked ? launch_plan_masked(ctx->op_dev(slot), ctx->g(), slot, c.n_experts, L.NT1, L.NT2,
-                                                     op->slab_rows, work_rows, st)
-                                : launch_plan(ctx->op_dev(slot), ctx->g(), slot, op->n_tokens, c.top_k, c.n_experts, L.NT1,
-                                              L.NT2, work_rows, st);
+  const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, st)
+                                : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, st);
   if (pe != cudaSuccess) {
     ctx->planned[slot] = false;
     return MOE_ECUDA;
@@ -508,9 +504,9 @@ int moe_plan_pair(moe_ctx_t* ctx, int slot_prefill, int slot_decode, int carrier
     ctx->host_pair[s] = *both[i];
     ctx->pair_uploaded[s] = true;
   }
-  if (launch_plan_pair(ctx->op_dev(c.max_ops + sd), ctx->op_dev(c.max_ops + sp), ctx->op_dev(sd), ctx->op_dev(sp), gather_m,
-                       reinterpret_cast<int*>(bd + L.pcomb_off), reinterpret_cast<int*>(bp + L.pcomb_off), (int)Rd, (int)Rp,
-                       c.n_experts, L.NT1, L.NT2, fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, sd, sp, st) != cudaSuccess)
+  if (launch_plan_pair(hd, hp, ctx->host_ops[sd], ctx->host_ops[sp], gather_m, reinterpret_cast<int*>(bd + L.pcomb_off),
+                       reinterpret_cast<int*>(bp + L.pcomb_off), c.n_experts, L.NT1, L.NT2,
+                       fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, sd, sp, st) != cudaSuccess)
     return MOE_ECUDA;
   if (ctx->pair_of[sp] >= 0) ctx->pair_of[ctx->pair_of[sp]] = -1;
   if (ctx->pair_of[sd] >= 0) ctx->pair_of[ctx->pair_of[sd]] = -1;

@@ -3,54 +3,21 @@
 // x_moe of Section 6.2 of the paper) and the ordered tile list the persistent kernel's
 // queues serve.
 //
-// The permutation is one stable counting-sort pass over the expert id.  No atomic decides
-// an order: every warp ranks a fixed chunk of rows, a column scan over the per-warp
-// histograms gives each warp its base rank per expert, and inside a warp rows are ranked
-// by lane order, so the result is unique and reproducible.
+// The permutation is one stable counting-sort pass over the expert id.  Every block of the rank kernel owns a
+// contiguous range of rows and knows, per expert, how many rows lie before its range; inside the block rows are
+// ranked by warp and lane order.  Atomics only count, none decides an order, so the result is unique and reproducible.
+//
+// A plan is a chain of latencies, not of bytes (8192 tokens x 8: 0.26 MB of ids), so the work is cut for few
+// launches and no serial part: the per-expert sums that every block needs are recomputed by every block instead of being
+// handed on by one, and the list is written by all blocks, one warp per expert.
 #include "moe_dev.cuh"
 
 namespace moe {
 
-constexpr int kPlanThreads = 256;
+constexpr int kPlanThreads = kPlanChunk;
 constexpr int kPlanWarps = kPlanThreads / 32;
-
-// ---------------------------------------------------------------- K1: per-warp histograms
-// one warp, one chunk of kPlanChunk routed rows; h: the warp's E counters in shared memory
-__device__ __forceinline__ void hist_chunk(const OpDev* __restrict__ op, Global* g, int slot, int R, int E,
-                                           int chunk, int* h, int lane) {
-  for (int e = lane; e < E; e += 32) h[e] = 0;
-  __syncwarp();
-  const int* ids = op->topk_ids;
-  const int base = chunk * kPlanChunk;
-  int my[kPlanChunk / 32];                    // this lane's ids of the chunk, loaded up front
-#pragma unroll
-  for (int it = 0; it < kPlanChunk / 32; ++it) {
-    const int i = base + it * 32 + lane;
-    my[it] = i < R ? ids[i] : -1;
-  }
-#pragma unroll
-  for (int it = 0; it < kPlanChunk / 32; ++it) {
-    const int i = base + it * 32 + lane;
-    int id = my[it];
-    if (i < R && (id < 0 || id >= E)) {
-      report(&g->status, MOE_EBADID, slot, i, id, 0);
-      id = -1;
-    }
-    const unsigned peers = __match_any_sync(0xffffffffu, id);
-    if (id >= 0 && (peers & ((1u << lane) - 1)) == 0) h[id] += __popc(peers);
-    __syncwarp();
-  }
-  int* out = op->plan_hist + (size_t)chunk * E;
-  if (base < R)
-    for (int e = lane; e < E; e += 32) out[e] = h[e];
-}
-
-__global__ void __launch_bounds__(kPlanThreads)
-plan_hist_kernel(const OpDev* __restrict__ op, Global* g, int slot, int R, int E) {
-  extern __shared__ int sm[];                 // [kPlanWarps][E]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  hist_chunk(op, g, slot, R, E, blockIdx.x * kPlanWarps + warp, sm + warp * E, lane);
-}
+constexpr int kPlanDirectRows = 8192;   // up to here every block counts all rows itself: no histogram launch
+constexpr int kPlanMaxBlocks = 128;     // beyond kPlanMaxBlocks x kPlanChunk rows a block owns several chunks
 
 // exclusive scan of one int per thread over a 1024-thread block
 __device__ inline int block_excl_scan(int v, int* total, int* warp_sums) {
@@ -82,79 +49,68 @@ __device__ inline int block_excl_scan(int v, int* total, int* warp_sums) {
 }
 
 // ---------------------------------------------------------------- the ordered tile list of one op
-// Shared-memory scratch of build_tile_list (one block of 1024 threads).
+// Shared-memory scratch of build_tile_list: work tiles of the experts before e.
 struct ListScratch {
   int warp_sums[33];
-  int work[kMaxExperts], grp[kMaxExperts], moff[kMaxExperts], w0[kMaxExperts];
-  int g_cnt[kMaxExperts], g_base1[kMaxExperts], g_base2[kMaxExperts];
-  int ntiles;
+  int work[kMaxExperts + 1];
 };
 
-// Writes the queue list of an op whose expert e holds rows [off[e], off[e] + cnt[e]) of the packed row space
-// (cnt / off in shared memory), and its PlanState.
+// first index i of the ascending array a[0..n) with a[i] >= v (n if none)
+__device__ __forceinline__ int lower_bound(const int* a, int n, int v) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (a[mid] >= v) hi = mid;
+    else lo = mid + 1;
+  }
+  return lo;
+}
+
+// Writes this block's share of the queue list of an op whose expert e holds rows [off[e], off[e] + cnt[e]) of the
+// packed row space (cnt / off in shared memory), and (block 0) its PlanState.  All blocks of the grid call it.
 // Work tiles (the unit the queues hand out): up to `work_rows` consecutive rows of one
 // expert, i.e. one or two adjacent m-tiles that share each weight tile they read.
-// Dependency groups: consecutive experts holding at least kGroupWork work tiles.  The list
-// is  G1(g0) G1(g1) G2(g0) G1(g2) G2(g1) ... G2(last): every down-GEMM tile comes after all
-// gate/up tiles of its group and of one more group, so by the time it is claimed the tiles
-// it depends on were claimed long before.
+// Order: the gate/up entries in expert order, and the down entries of an expert in front of the first expert whose
+// gate/up tiles start at least kLagWork work tiles behind its own, so by the time a down tile is claimed the tiles it
+// depends on were claimed long before.  Every entry's place follows from the prefix sum of the work tiles.
 __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan, const int* cnt, const int* off, int E,
                                                 int NT1, int NT2, int T, int work_rows, int x_moe, int planned,
                                                 int n_extra_gemm, int g1_kind = kGateUp) {
   __shared__ ListScratch ls;
   const int e = threadIdx.x;
-  const int we = (e < E) ? (cnt[e] + work_rows - 1) / work_rows : 0;
-  if (e < kMaxExperts) ls.work[e] = we;
+  const int we = e < E ? (cnt[e] + work_rows - 1) / work_rows : 0;
   int n_work;
   const int w0 = block_excl_scan(we, &n_work, ls.warp_sums);
-  if (e < E) ls.w0[e] = w0;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ng = 0, acc = 0;
-    for (int x = 0; x < E; ++x) {
-      const int m = ls.work[x];
-      ls.grp[x] = ng;
-      ls.moff[x] = acc;
-      acc += m;
-      if (acc >= kGroupWork || x == E - 1) {
-        if (acc > 0) { ls.g_cnt[ng] = acc; ++ng; }
-        acc = 0;
-      }
-    }
-    int pos = 0;
-    for (int gi = 0; gi < ng; ++gi) {
-      ls.g_base1[gi] = pos;
-      pos += ls.g_cnt[gi] * NT1;
-      if (gi >= 1) { ls.g_base2[gi - 1] = pos; pos += ls.g_cnt[gi - 1] * NT2; }
-    }
-    if (ng > 0) { ls.g_base2[ng - 1] = pos; pos += ls.g_cnt[ng - 1] * NT2; }
-    ls.ntiles = pos;
-  }
+  if (e < E) ls.work[e] = w0;
+  if (e == 0) ls.work[E] = n_work;
   __syncthreads();
 
   // Inside an expert: n-major over its work tiles, so an expert's entries of one GEMM are one
   // contiguous run of the list.  One warp per expert writes them (a popular expert has hundreds).
-  for (int x = threadIdx.x >> 5; x < E; x += 32) {
-    const int wx = ls.work[x];
+  const int lane = threadIdx.x & 31;
+  for (int x = (int)blockIdx.x * kPlanWarps + (int)(threadIdx.x >> 5); x < E; x += (int)gridDim.x * kPlanWarps) {
+    const int mx = ls.work[x], wx = ls.work[x + 1] - mx;
     if (wx == 0) continue;
-    const int lane = threadIdx.x & 31;
-    const int gi = ls.grp[x], cx = cnt[x], ox = off[x], mx = ls.w0[x];
-    const int b1 = ls.g_base1[gi] + ls.moff[x] * NT1, b2 = ls.g_base2[gi] + ls.moff[x] * NT2;
+    const int cx = cnt[x], ox = off[x];
+    const int before = lower_bound(ls.work + 1, E, mx - kLagWork + 1);      // experts whose down entries come first
+    const int next = min(E, lower_bound(ls.work, E + 1, mx + wx + kLagWork));
+    int4* g1 = tile_list + (size_t)mx * NT1 + (size_t)ls.work[before] * NT2;
+    int4* g2 = tile_list + (size_t)ls.work[next] * NT1 + (size_t)mx * NT2;
     for (int i = lane; i < wx * NT1; i += 32) {
       const int n = i / wx, j = i - n * wx;
-      tile_list[b1 + i] = make_entry(g1_kind, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), x);
+      g1[i] = make_entry(g1_kind, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), x);
     }
     for (int i = lane; i < wx * NT2; i += 32) {
       const int n = i / wx, j = i - n * wx;
-      tile_list[b2 + i] = make_entry(kDown, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), x);
+      g2[i] = make_entry(kDown, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), x);
     }
   }
-  const int n_gemm = ls.ntiles;
+  const int n_gemm = n_work * (NT1 + NT2);
   const int ct = combine_tile_tokens(T);
   const int n_comb = (T + ct - 1) / ct;
-  for (int c = threadIdx.x; c < n_comb; c += blockDim.x)
+  for (int c = (int)(blockIdx.x * blockDim.x + threadIdx.x); c < n_comb; c += (int)(gridDim.x * blockDim.x))
     tile_list[n_gemm + c] = make_entry(kCombine, 0, c, c * ct, min(ct, T - c * ct), 0);
-  if (threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     PlanState ps;
     ps.n_mtiles = x_moe;
     ps.n_gemm_tiles = n_gemm;
@@ -164,168 +120,156 @@ __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan,
     ps.pad[0] = ps.pad[1] = ps.pad[2] = 0;
     *plan = ps;
   }
-  __syncthreads();
   return n_gemm;
 }
 
-// ---------------------------------------------------------------- K2: scans + tile table + tile list
-// the whole block of 1024 threads
-__device__ __forceinline__ void scan_body(const OpDev* __restrict__ op, int n_chunks, int R, int E, int NT1, int NT2,
-                                          int T, int work_rows) {
-  __shared__ int warp_sums[33];
-  __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts];
-  __shared__ int s_part[1024];
-  const int e = threadIdx.x;
+// ---------------------------------------------------------------- histogram and rank
+// What the plan kernels read and write, by value: no descriptor has to be fetched first.
+struct PlanArgs {
+  const int* ids;       // [R]
+  int* counts;          // [E]
+  int* offsets;         // [E+1]
+  int* s2f;             // [R]
+  int* f2s;             // [R]
+  int* hist;            // [blocks][E] rows per block and expert
+  MTile* mtiles;
+  int4* tile_list;
+  PlanState* plan;
+  Status* status;
+  int slot, R, E, T, NT1, NT2, work_rows;
+  int own;              // rows per block: block b owns rows [b * own, (b + 1) * own)
+};
 
-  // column sums of the per-warp histograms, the device prefix sum over experts, then the base
-  // rank of every (warp chunk, expert).  Reads and writes use different arrays so that the
-  // loads of a column do not wait on the stores.
-  const int* hist = op->plan_hist;        // no __restrict__: the one-block plan wrote it earlier in the same kernel
-  int* base = op->plan_base;
-  // the 1024 threads split every expert's column into `parts` chunk ranges
-  const int parts = max(1, 1024 / E);
-  const int part = threadIdx.x / E, pe = threadIdx.x % E;
-  const int cpp = (n_chunks + parts - 1) / parts;
-  const int c0 = min(n_chunks, part * cpp), c1 = min(n_chunks, c0 + cpp);
-  int psum = 0;
-  if (part < parts) {
-#pragma unroll 32
-    for (int c = c0; c < c1; ++c) psum += hist[(size_t)c * E + pe];
-    s_part[part * E + pe] = psum;
+__global__ void __launch_bounds__(kPlanThreads) plan_hist_kernel(const __grid_constant__ PlanArgs a) {
+  __shared__ int h[kMaxExperts];
+  for (int e = threadIdx.x; e < a.E; e += kPlanThreads) h[e] = 0;
+  __syncthreads();
+  const int i0 = (int)blockIdx.x * a.own, i1 = min(a.R, i0 + a.own);
+  for (int i = i0 + (int)threadIdx.x; i < i1; i += kPlanThreads) {
+    const int id = a.ids[i];
+    if (id >= 0 && id < a.E) atomicAdd(&h[id], 1);
   }
   __syncthreads();
+  for (int e = threadIdx.x; e < a.E; e += kPlanThreads) a.hist[(size_t)blockIdx.x * a.E + e] = h[e];
+}
+
+// kDirect: no histogram was made, every block counts all rows itself (R <= kPlanDirectRows).
+template <bool kDirect>
+__global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_constant__ PlanArgs a) {
+  extern __shared__ int run[];              // [kPlanWarps][E]: next packed position of an expert's row per warp
+  __shared__ int warp_sums[33];
+  __shared__ int s_before[kMaxExperts], s_cnt[kMaxExperts], s_off[kMaxExperts];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int E = a.E, R = a.R;
+  const int i0 = min(R, (int)blockIdx.x * a.own), i1 = min(R, i0 + a.own);
+
+  for (int e = tid; e < E; e += kPlanThreads) s_before[e] = s_cnt[e] = 0;
+  for (int i = tid; i < kPlanWarps * E; i += kPlanThreads) run[i] = 0;
+  __syncthreads();
+  // rows per expert: before this block's range, and from it on
+  if (kDirect) {
+#pragma unroll 4
+    for (int i = tid; i < R; i += kPlanThreads) {
+      const int id = a.ids[i];
+      if (id >= 0 && id < E) atomicAdd(i < i0 ? &s_before[id] : &s_cnt[id], 1);
+    }
+  } else {
+    const int parts = max(1, kPlanThreads / E), part = tid / E, e = tid % E;
+    const int nb = (int)gridDim.x, per = (nb + parts - 1) / parts;
+    const int b0 = min(nb, part * per), b1 = min(nb, b0 + per);
+    int before = 0, rest = 0;
+    if (part < parts) {
+#pragma unroll 16
+      for (int b = b0; b < b1; ++b) {
+        const int v = a.hist[(size_t)b * E + e];
+        if (b < (int)blockIdx.x) before += v;
+        else rest += v;
+      }
+      if (before) atomicAdd(&s_before[e], before);
+      if (rest) atomicAdd(&s_cnt[e], rest);
+    }
+  }
+  // this block's rows: each warp counts a contiguous share of them per expert
+  const int share = a.own / kPlanWarps;
+  const int w0 = min(i1, i0 + warp * share), w1 = min(i1, w0 + share);
+  int* mine = run + warp * E;
+  const unsigned lower = (1u << lane) - 1u;
+  for (int base = w0; base < w1; base += 32) {
+    const int i = base + lane;
+    int id = i < w1 ? a.ids[i] : -1;
+    if (i < w1 && (id < 0 || id >= E)) {
+      report(a.status, MOE_EBADID, a.slot, i, id, 0);
+      id = -1;
+    }
+    const unsigned peers = __match_any_sync(0xffffffffu, id);
+    if (id >= 0 && (peers & lower) == 0) mine[id] += __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+
   int cnt = 0;
-  if (e < E)
-    for (int p = 0; p < parts; ++p) cnt += s_part[p * E + e];
+  if (tid < E) cnt = s_cnt[tid] + s_before[tid];
   int total;
   const int off = block_excl_scan(cnt, &total, warp_sums);       // device prefix sum over experts
-  if (e < E) {
-    op->counts[e] = cnt;
-    op->offsets[e] = off;
-    s_cnt[e] = cnt;
-    s_off[e] = off;
+  if (tid < E) {
+    s_cnt[tid] = cnt;
+    s_off[tid] = off;
+    int pos = off + s_before[tid];          // rows of the expert: earlier blocks, then the warps of this one
+#pragma unroll 8
+    for (int w = 0; w < kPlanWarps; ++w) {
+      const int v = run[w * E + tid];
+      run[w * E + tid] = pos;
+      pos += v;
+    }
+    if (blockIdx.x == 0) {
+      a.counts[tid] = cnt;
+      a.offsets[tid] = off;
+      if (tid == 0) a.offsets[E] = total;
+    }
   }
-  if (e == 0) op->offsets[E] = total;
+  __syncthreads();
+  // stable positions
+  for (int base = w0; base < w1; base += 32) {
+    const int i = base + lane;
+    int id = i < w1 ? a.ids[i] : -1;
+    if (id < 0 || id >= E) id = -1;         // reported above
+    const unsigned peers = __match_any_sync(0xffffffffu, id);
+    int p = -1;
+    if (id >= 0) p = mine[id] + __popc(peers & lower);
+    __syncwarp();
+    if (id >= 0 && (peers & lower) == 0) mine[id] += __popc(peers);
+    __syncwarp();
+    if (i < w1) {
+      a.f2s[i] = p;                         // -1: a rejected id, the row has no packed position
+      if (p >= 0) a.s2f[p] = i;
+    }
+  }
   // rows with a rejected expert id take no packed position: the tail of the permutation that no row
   // will claim is marked, so that nothing downstream mistakes stale memory for an index
-  for (int p = total + (int)threadIdx.x; p < R; p += (int)blockDim.x) op->sorted_to_flat[p] = -1;
-  __syncthreads();
-  if (part < parts) {
-    int run = s_off[pe];
-    for (int p = 0; p < part; ++p) run += s_part[p * E + pe];
-#pragma unroll 32
-    for (int c = c0; c < c1; ++c) {
-      const int v = hist[(size_t)c * E + pe];
-      base[(size_t)c * E + pe] = run;
-      run += v;
-    }
-  }
+  for (int p = total + (int)(blockIdx.x * kPlanThreads) + tid; p < R; p += (int)gridDim.x * kPlanThreads) a.s2f[p] = -1;
 
   // m-tiles: ceil(m_e / M_t) per expert with rows (the footprint x_moe)
-  const int me = (e < E) ? (cnt + kTileM - 1) / kTileM : 0;
+  const int me = (cnt + kTileM - 1) / kTileM;
   int x_moe;
   const int m0 = block_excl_scan(me, &x_moe, warp_sums);
-  if (e < E) {
-    for (int j = 0; j < me; ++j) {
-      MTile t;
-      t.expert = e;
-      t.row0 = off + j * kTileM;
-      t.rows = min(kTileM, cnt - j * kTileM);
-      t.pad = 0;
-      op->mtiles[m0 + j] = t;
-    }
-  }
-  __syncthreads();
-
-  build_tile_list(op->tile_list, op->plan, s_cnt, s_off, E, NT1, NT2, T, work_rows, x_moe, total == R ? 1 : 0, 0);
-}
-
-__global__ void __launch_bounds__(1024)
-plan_scan_kernel(const OpDev* __restrict__ op, int n_chunks, int R, int E, int NT1, int NT2,
-                 int T, int work_rows) {
-  scan_body(op, n_chunks, R, E, NT1, NT2, T, work_rows);
-}
-
-// ---------------------------------------------------------------- K3: stable scatter
-// one warp, one chunk; run: the warp's E running ranks in shared memory
-__device__ __forceinline__ void scatter_chunk(const OpDev* __restrict__ op, int R, int E, int chunk, int* run, int lane) {
-  const int base = chunk * kPlanChunk;
-  if (base >= R) return;
-  const int* src = op->plan_base + (size_t)chunk * E;
-  for (int e = lane; e < E; e += 32) run[e] = src[e];
-  __syncwarp();
-  const int* ids = op->topk_ids;
-  int* s2f = op->sorted_to_flat;
-  int* f2s = op->flat_to_sorted;
-  int my[kPlanChunk / 32];
-#pragma unroll
-  for (int it = 0; it < kPlanChunk / 32; ++it) {
-    const int i = base + it * 32 + lane;
-    my[it] = i < R ? ids[i] : -1;
-  }
-#pragma unroll
-  for (int it = 0; it < kPlanChunk / 32; ++it) {
-    const int i = base + it * 32 + lane;
-    int id = my[it];
-    if (id < 0 || id >= E) id = -1;         // reported by the histogram pass
-    const unsigned peers = __match_any_sync(0xffffffffu, id);
-    const unsigned before = peers & ((1u << lane) - 1);
-    int p = -1;
-    if (id >= 0) p = run[id] + __popc(before);
-    __syncwarp();
-    if (id >= 0 && before == 0) run[id] += __popc(peers);
-    __syncwarp();
-    if (p >= 0 && p < R) {
-      s2f[p] = i;
-      f2s[i] = p;
-    } else if (i < R) {
-      f2s[i] = -1;                          // a rejected id: the row has no packed position
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kPlanThreads)
-plan_scatter_kernel(const OpDev* __restrict__ op, int R, int E) {
-  extern __shared__ int sm[];                 // [kPlanWarps][E] running rank per expert
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  scatter_chunk(op, R, E, blockIdx.x * kPlanWarps + warp, sm + warp * E, lane);
-}
-
-// ---------------------------------------------------------------- small ops: the three passes in one block
-// An op of at most kSmallChunks chunks (a decode batch) is planned by ONE block of 32 warps: the
-// histogram scratch written by the first pass is read back by the same block, so two launches and
-// their gaps go away (they are about half of a small plan's time).
-constexpr int kSmallChunks = 32;
-constexpr int kSmallMaxExperts = 256;
-
-__global__ void __launch_bounds__(1024)
-plan_small_kernel(const OpDev* __restrict__ op, Global* g, int slot, int n_chunks, int R, int E, int NT1, int NT2,
-                  int T, int work_rows) {
-  extern __shared__ int sm[];                 // [32 warps][E]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp < n_chunks) hist_chunk(op, g, slot, R, E, warp, sm + warp * E, lane);
-  __threadfence_block();
-  __syncthreads();
-  scan_body(op, n_chunks, R, E, NT1, NT2, T, work_rows);
-  __threadfence_block();
-  __syncthreads();
-  if (warp < n_chunks) scatter_chunk(op, R, E, warp, sm + warp * E, lane);
+  if (blockIdx.x == 0)
+    for (int j = 0; j < me; ++j) a.mtiles[m0 + j] = MTile{tid, off + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
+  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, E, a.NT1, a.NT2, a.T, a.work_rows, x_moe, total == R ? 1 : 0, 0);
 }
 
 // ---------------------------------------------------------------- masked layout
 // The activations already sit in per-expert slabs of slab_rows rows; counts[e] (an input here) says how many
 // rows of slab e are valid.  Nothing is permuted: the plan is the exclusive prefix sum for `offsets`, the
 // m-tile table (first row of a tile = e * slab_rows + 128 j) and the queue list over the slabs' valid rows.
-__global__ void __launch_bounds__(1024)
-plan_masked_kernel(const OpDev* __restrict__ op, Global* g, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows) {
+__global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_constant__ PlanArgs a, int slab_rows) {
   __shared__ int warp_sums[33];
   __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts];
-  const int e = threadIdx.x;
+  const int e = threadIdx.x, E = a.E;
   int cnt = 0;
   if (e < E) {
-    cnt = op->counts[e];
+    cnt = a.counts[e];
     if (cnt < 0 || cnt > slab_rows) {        // a count the slab cannot hold: reported, the slab is left out
-      report(&g->status, MOE_EBOUNDS, slot, e, cnt, 4);
+      if (blockIdx.x == 0) report(a.status, MOE_EBOUNDS, a.slot, e, cnt, 4);
       cnt = 0;
     }
     s_cnt[e] = cnt;
@@ -333,29 +277,17 @@ plan_masked_kernel(const OpDev* __restrict__ op, Global* g, int slot, int E, int
   }
   int total;
   const int off = block_excl_scan(cnt, &total, warp_sums);
-  if (e < E) op->offsets[e] = off;
-  if (e == 0) op->offsets[E] = total;
-  const int me = (e < E) ? (cnt + kTileM - 1) / kTileM : 0;
+  if (blockIdx.x == 0) {
+    if (e < E) a.offsets[e] = off;
+    if (e == 0) a.offsets[E] = total;
+  }
+  const int me = (cnt + kTileM - 1) / kTileM;
   int x_moe;
   const int m0 = block_excl_scan(me, &x_moe, warp_sums);
-  if (e < E) {
-    for (int j = 0; j < me; ++j) {
-      MTile t;
-      t.expert = e;
-      t.row0 = e * slab_rows + j * kTileM;
-      t.rows = min(kTileM, cnt - j * kTileM);
-      t.pad = 0;
-      op->mtiles[m0 + j] = t;
-    }
-  }
-  __syncthreads();
-  build_tile_list(op->tile_list, op->plan, s_cnt, s_off, E, NT1, NT2, 0, work_rows, x_moe, 1, 0, kGateUpDirect);
-}
-
-cudaError_t launch_plan_masked(const OpDev* d_op, Global* g, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
-                               cudaStream_t stream) {
-  plan_masked_kernel<<<1, 1024, 0, stream>>>(d_op, g, slot, E, NT1, NT2, slab_rows, work_rows);
-  return cudaGetLastError();
+  if (blockIdx.x == 0)
+    for (int j = 0; j < me; ++j)
+      a.mtiles[m0 + j] = MTile{e, e * slab_rows + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
+  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, E, a.NT1, a.NT2, 0, a.work_rows, x_moe, 1, 0, kGateUpDirect);
 }
 
 // ---------------------------------------------------------------- the paired form of a decode + prefill op
@@ -366,92 +298,120 @@ cudaError_t launch_plan_masked(const OpDev* d_op, Global* g, int slot, int E, in
 // rows' last tile of `carrier_rows` rows ("carrier" tiles: claimed with decode priority, they stream a weight
 // tile once for rows of both ops); the prefill list takes the rest.  Nothing about a row's arithmetic depends on the
 // tile it sits in, so the outputs are those of the unpaired ops, bit for bit.
-//   dp / pp: the paired descriptors (their PlanStates and lists are written here), d / p: the plain ones,
-//   whose counts and offsets the two moe_plan calls have written earlier on the stream.
-__global__ void __launch_bounds__(1024)
-plan_pair_kernel(const OpDev* dp, const OpDev* pp, const OpDev* d, const OpDev* p, int E, int NT1, int NT2,
-                 int work_rows, int carrier_rows) {
+struct PairSide {
+  const int* ids;             // the op's plain plan, as its moe_plan call left it earlier on the stream
+  const int* counts;
+  const int* offsets;
+  const int* f2s;
+  const PlanState* plain;
+  int4* tile_list;            // the paired form's list and state, written here
+  PlanState* plan;
+  int* comb;                  // flat routed index -> row of the shared space
+  int R, T, slot;
+};
+struct PairArgs {
+  PairSide d, p;
+  int* gather;                // row of the shared space -> flat routed index, tagged with its slot
+  int E, NT1, NT2, work_rows, carrier_rows;
+};
+
+// One launch: every block scans the experts and writes its share of both lists, then moves its share of the rows
+// into the shared row space.
+__global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_constant__ PairArgs a) {
   __shared__ int cnt_d[kMaxExperts], off_d[kMaxExperts], cnt_p[kMaxExperts], off_p[kMaxExperts];
-  const int e = threadIdx.x;
+  __shared__ int base_d[kMaxExperts], base_p[kMaxExperts];   // what a row's packed position is shifted by
+  const int e = threadIdx.x, E = a.E;
   if (e < E) {
-    const int cd = d->counts[e], cp = p->counts[e];
-    const int moff = d->offsets[e] + p->offsets[e];
+    const int cd = a.d.counts[e], cp = a.p.counts[e];
+    const int od = a.d.offsets[e], op = a.p.offsets[e];
+    const int moff = od + op;
     // the carrier takes the ragged tail of the prefill rows (what is left over after the prefill op's full work
     // tiles) when that tail fits beside the decode rows: a prefill tile less to run.  A tail that does not fit
     // stays where it is -- moving part of it would make the carrier heavier and save nothing.
-    const int room = cd > 0 ? (cd + carrier_rows - 1) / carrier_rows * carrier_rows - cd : 0;
-    const int tail = cp % max(work_rows, carrier_rows);
+    const int room = cd > 0 ? (cd + a.carrier_rows - 1) / a.carrier_rows * a.carrier_rows - cd : 0;
+    const int tail = cp % max(a.work_rows, a.carrier_rows);
     const int take = tail <= room ? tail : 0;
     cnt_p[e] = cp - take;
     off_p[e] = moff;
     cnt_d[e] = cd + take;
     off_d[e] = moff + cp - take;
+    base_p[e] = od;                                          // the decode rows of the experts before
+    base_d[e] = op + cp;                                     // ... and the expert's own prefill rows
   }
   __syncthreads();
-  const int ok = (d->plan->planned && p->plan->planned) ? 1 : 0;
+  const int ok = (a.d.plain->planned && a.p.plain->planned) ? 1 : 0;
   // a carrier taller than the kernel's work tile (e4m3: 128 rows) is cut into work tiles that follow one another
-  const int n_dec = build_tile_list(dp->tile_list, dp->plan, cnt_d, off_d, E, NT1, NT2, d->n_tokens,
-                                    min(carrier_rows, work_rows), d->plan->n_mtiles, ok, 0);
+  const int n_dec = build_tile_list(a.d.tile_list, a.d.plan, cnt_d, off_d, E, a.NT1, a.NT2, a.d.T,
+                                    min(a.carrier_rows, a.work_rows), a.d.plain->n_mtiles, ok, 0);
+  __syncthreads();
   // every GEMM entry of the decode list may carry prefill rows: the prefill op is complete when they are too
-  build_tile_list(pp->tile_list, pp->plan, cnt_p, off_p, E, NT1, NT2, p->n_tokens, work_rows, p->plan->n_mtiles, ok,
+  build_tile_list(a.p.tile_list, a.p.plan, cnt_p, off_p, E, a.NT1, a.NT2, a.p.T, a.work_rows, a.p.plain->n_mtiles, ok,
                   n_dec);
-}
-
-// the shared row space's permutation: for each op, flat routed index -> packed row, and packed row -> flat
-// index tagged with the slot the row belongs to
-__global__ void __launch_bounds__(256)
-plan_pair_scatter_kernel(const OpDev* d, const OpDev* p, int* gather_m, int* comb_d, int* comb_p, int Rd, int Rp, int E,
-                         int slot_d, int slot_p) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < Rd) {
-    const int e = d->topk_ids[i], ps = d->flat_to_sorted[i];
+  // the shared row space's permutation
+  for (int i = (int)(blockIdx.x * kPlanThreads + threadIdx.x); i < a.d.R + a.p.R; i += (int)gridDim.x * kPlanThreads) {
+    const bool dec = i < a.d.R;
+    const PairSide& s = dec ? a.d : a.p;
+    const int j = dec ? i : i - a.d.R;
+    const int x = s.ids[j], ps = s.f2s[j];
     int m = -1;
-    if (e >= 0 && e < E && ps >= 0) {
-      m = ps + p->offsets[e + 1];               // behind the expert's prefill rows
-      gather_m[m] = i | (slot_d << kRowSlotShift);
+    if (x >= 0 && x < E && ps >= 0) {
+      m = ps + (dec ? base_d[x] : base_p[x]);
+      a.gather[m] = j | (s.slot << kRowSlotShift);
     }
-    comb_d[i] = m;
-  } else if (i < Rd + Rp) {
-    const int j = i - Rd;
-    const int e = p->topk_ids[j], ps = p->flat_to_sorted[j];
-    int m = -1;
-    if (e >= 0 && e < E && ps >= 0) {
-      m = ps + d->offsets[e];                   // shifted by the decode rows of the experts before
-      gather_m[m] = j | (slot_p << kRowSlotShift);
-    }
-    comb_p[j] = m;
+    s.comb[j] = m;
   }
 }
 
-cudaError_t launch_plan_pair(const OpDev* dp, const OpDev* pp, const OpDev* d, const OpDev* p, int* gather_m, int* comb_d,
-                             int* comb_p, int Rd, int Rp, int E, int NT1, int NT2, int work_rows, int carrier_rows,
+// ---------------------------------------------------------------- launches
+// blocks that write a list: a warp per expert
+static int list_blocks(int E) { return (E + kPlanWarps - 1) / kPlanWarps; }
+
+cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
+                               cudaStream_t stream) {
+  PlanArgs a{};
+  a.counts = h.counts; a.offsets = h.offsets; a.mtiles = h.mtiles; a.tile_list = h.tile_list; a.plan = h.plan;
+  a.status = h.status;
+  a.slot = slot; a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows;
+  plan_masked_kernel<<<list_blocks(E), kPlanThreads, 0, stream>>>(a, slab_rows);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, const OpDev& p, int* gather, int* comb_d,
+                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows,
                              int slot_d, int slot_p, cudaStream_t stream) {
-  plan_pair_kernel<<<1, 1024, 0, stream>>>(dp, pp, d, p, E, NT1, NT2, work_rows, carrier_rows);
-  const int n = Rd + Rp;
-  if (n > 0)
-    plan_pair_scatter_kernel<<<(n + 255) / 256, 256, 0, stream>>>(d, p, gather_m, comb_d, comb_p, Rd, Rp, E, slot_d, slot_p);
+  PairArgs a{};
+  a.d = PairSide{d.topk_ids, d.counts, d.offsets, d.flat_to_sorted, d.plan, hd.tile_list, hd.plan, comb_d, d.n_rows, d.n_tokens, slot_d};
+  a.p = PairSide{p.topk_ids, p.counts, p.offsets, p.flat_to_sorted, p.plan, hp.tile_list, hp.plan, comb_p, p.n_rows, p.n_tokens, slot_p};
+  a.gather = gather;
+  a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows; a.carrier_rows = carrier_rows;
+  const int blocks = max(list_blocks(E), min(kPlanMaxBlocks, (d.n_rows + p.n_rows + kPlanThreads - 1) / kPlanThreads));
+  plan_pair_kernel<<<blocks, kPlanThreads, 0, stream>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t prepare_plan_kernels() {
-  return cudaFuncSetAttribute(plan_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kSmallChunks * kSmallMaxExperts * (int)sizeof(int));
+  const int most = kPlanWarps * kMaxExperts * (int)sizeof(int);
+  const cudaError_t e = cudaFuncSetAttribute(plan_rank_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(plan_rank_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
-cudaError_t launch_plan(const OpDev* d_op, Global* g, int slot, int T, int k, int E, int NT1,
-                        int NT2, int work_rows, cudaStream_t stream) {
-  const int R = T * k;
-  const int n_chunks = (R + kPlanChunk - 1) / kPlanChunk;
-  const int blocks = (n_chunks + kPlanWarps - 1) / kPlanWarps;
+// h: the op's descriptor as the host holds it
+cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, cudaStream_t stream) {
+  PlanArgs a{};
+  a.ids = h.topk_ids; a.counts = h.counts; a.offsets = h.offsets; a.s2f = h.sorted_to_flat; a.f2s = h.flat_to_sorted;
+  a.hist = h.plan_hist; a.mtiles = h.mtiles; a.tile_list = h.tile_list; a.plan = h.plan; a.status = h.status;
+  a.slot = slot; a.R = h.n_rows; a.E = E; a.T = h.n_tokens; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows;
   const size_t smem = (size_t)kPlanWarps * E * sizeof(int);
-  if (n_chunks <= kSmallChunks && E <= kSmallMaxExperts) {
-    plan_small_kernel<<<1, 1024, (size_t)kSmallChunks * E * sizeof(int), stream>>>(d_op, g, slot, n_chunks, R, E, NT1, NT2, T,
-                                                                                 work_rows);
+  if (a.R <= kPlanDirectRows) {
+    const int blocks = list_blocks(E);
+    a.own = ((a.R + blocks - 1) / blocks + kPlanThreads - 1) / kPlanThreads * kPlanThreads;
+    plan_rank_kernel<true><<<blocks, kPlanThreads, smem, stream>>>(a);
     return cudaGetLastError();
   }
-  if (blocks > 0) plan_hist_kernel<<<blocks, kPlanThreads, smem, stream>>>(d_op, g, slot, R, E);
-  plan_scan_kernel<<<1, 1024, 0, stream>>>(d_op, n_chunks, R, E, NT1, NT2, T, work_rows);
-  if (blocks > 0) plan_scatter_kernel<<<blocks, kPlanThreads, smem, stream>>>(d_op, R, E);
+  a.own = kPlanThreads * (int)(((long long)a.R + kPlanThreads * kPlanMaxBlocks - 1) / (kPlanThreads * kPlanMaxBlocks));
+  const int blocks = (a.R + a.own - 1) / a.own;
+  plan_hist_kernel<<<blocks, kPlanThreads, 0, stream>>>(a);
+  plan_rank_kernel<false><<<blocks, kPlanThreads, smem, stream>>>(a);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,32 @@
+"""The plan at the sizes where its split over blocks and warps changes: around the largest op that one launch plans, rows
+per block of one and of several thousand, one to 1024 experts, routings that leave most experts empty.  Integer outputs:
+bit-exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_18002_b200 as moe
+from workloads import synth
+
+from gpu_util import bind_ops, check_plan, check_tiles, make_ctx, n_combine_tiles, weights_to
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,E,k", [(1, 1024, 1), (31, 33, 1), (1023, 256, 8), (1024, 256, 8), (1025, 256, 8), (8193, 8, 1),
+                                   (2049, 1000, 4), (131072, 16, 1), (131073, 5, 1), (40001, 40, 5)])
+def test_plan_and_queue_list(T, E, k):
+    spec = synth.Spec("sizes", synth.Shape(E, k, 256, 128), ((synth.PREFILL, T),), "uniform", None, 1.0, -1.0, 5)
+    Wd = weights_to(synth.make_weights(spec))
+    ctx = make_ctx(spec)
+    rng = np.random.default_rng([T, E, k])
+    # a skewed draw with repeats (ids of a token need not differ for the plan), so that many experts stay empty
+    ids = np.minimum(rng.zipf(1.3, size=(T, k)) - 1, rng.integers(0, E, size=(T, k))).astype(np.int32)
+    op = synth.Op(synth.PREFILL, torch.zeros(T, 256, dtype=torch.bfloat16), ids, np.full(ids.shape, 1.0 / k, np.float32))
+    b = bind_ops(ctx, [op], Wd)[0]
+    ctx.plan(0, b)
+    ctx.check()
+    counts = check_plan(b, op, E)
+    check_tiles(ctx, 0, counts)
+    rows = 256 if ctx.ctas_per_tile == 2 else moe.MOE_TILE_M        # bf16 work tiles on the default grid
+    assert ctx.footprint(0)[1] == int((-(-counts // rows)).sum()) * 2 + n_combine_tiles(T)
