@@ -73,7 +73,8 @@ struct __align__(128) OpDev {
   CUtensorMap tm_w2;    // [E*H, I]    box {64, 128} down weights
   CUtensorMap tm_a128;  // [Rmax, I]   box {64, 128}
   CUtensorMap tm_a256;  // [Rmax, I]   box {64, 256}
-  CUtensorMap tm_w1h;   // [E*2I, H]   box {64, 64}  gate/up weights, half-height box (CTA-pair kernel)
+  CUtensorMap tm_p1;    // CTA-pair kernel: gate/up weights as [E][I/8][2][8][H], box of 8 x (8 gate + 8 up) rows x 64
+  CUtensorMap tm_p2;    // CTA-pair kernel: down weights as [E][H/16][2][8][I], box of 128 consecutive rows x 64
   CUtensorMap tm_x8;    // masked layout only: x as [E*slab_rows, H], boxes of 8 / 32 / 128 / 256 rows
   CUtensorMap tm_x32;
   CUtensorMap tm_x128;

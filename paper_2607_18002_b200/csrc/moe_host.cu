@@ -150,6 +150,21 @@ int make_map(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t rows, size
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ECUDA;
 }
 
+// The weights of one GEMM for the CTA-pair kernel, seen as [E][blocks][2][8][cols]: a box is 8 blocks of 2 x 8 rows x 64
+// columns, i.e. 128 rows in one copy.  half_rows: rows between the two halves of a block, blk_rows: between blocks.
+int make_map_pair(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t cols, size_t blocks, size_t half_rows, size_t blk_rows) {
+  const size_t E = ctx->cfg.n_experts, pitch = cols * 2;
+  cuuint64_t dims[5] = {(cuuint64_t)cols, 8, 2, (cuuint64_t)blocks, (cuuint64_t)E};
+  cuuint64_t strides[4] = {(cuuint64_t)pitch, (cuuint64_t)(half_rows * pitch), (cuuint64_t)(blk_rows * pitch),
+                           (cuuint64_t)(blocks * 16 * pitch)};
+  cuuint32_t box[5] = {(cuuint32_t)kBlockK, 8, 2, 8, 1};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  CUresult r = ctx->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? MOE_OK : MOE_ECUDA;
+}
+
 // a stream-ordered 4-byte write: the value travels in the launch, not through host memory
 __global__ void set_word_kernel(int* p, int v) { *reinterpret_cast<volatile int*>(p) = v; }
 
@@ -317,9 +332,14 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
       if (!rc) rc = make_map(ctx, &h.tm_a32, h.A, (size_t)L.max_rows, (size_t)c.inter, 32);
       if (!rc) rc = make_map(ctx, &h.tm_a128, h.A, (size_t)L.max_rows, (size_t)c.inter, 128);
       if (!rc) rc = make_map(ctx, &h.tm_a256, h.A, (size_t)L.max_rows, (size_t)c.inter, 256);
-      if (!rc) rc = make_map(ctx, &h.tm_w1, op->w_gate_up, (size_t)c.n_experts * 2 * c.inter, (size_t)c.hidden, 128);
-      if (!rc) rc = make_map(ctx, &h.tm_w1h, op->w_gate_up, (size_t)c.n_experts * 2 * c.inter, (size_t)c.hidden, 64);
-      if (!rc) rc = make_map(ctx, &h.tm_w2, op->w_down, (size_t)c.n_experts * c.hidden, (size_t)c.inter, 128);
+      if (ctx->pair_kernel) {
+        const size_t H = c.hidden, I = c.inter;
+        if (!rc) rc = make_map_pair(ctx, &h.tm_p1, op->w_gate_up, H, I / 8, I, 8);   // 8 gate rows, the 8 matching up rows, ...
+        if (!rc) rc = make_map_pair(ctx, &h.tm_p2, op->w_down, I, H / 16, 8, 16);
+      } else {
+        if (!rc) rc = make_map(ctx, &h.tm_w1, op->w_gate_up, (size_t)c.n_experts * 2 * c.inter, (size_t)c.hidden, 128);
+        if (!rc) rc = make_map(ctx, &h.tm_w2, op->w_down, (size_t)c.n_experts * c.hidden, (size_t)c.inter, 128);
+      }
       if (masked) {
         const size_t xr = (size_t)c.n_experts * op->slab_rows;
         if (!rc) rc = make_map(ctx, &h.tm_x8, op->x, xr, (size_t)c.hidden, 8);

@@ -137,6 +137,24 @@ __device__ __forceinline__ void tc_ld16(unsigned taddr, unsigned (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+// 16 TMEM lanes x 32 columns in the fragment layout of an m16n8 accumulator: for column group j (8 columns) thread i
+// holds row i / 4, columns 8 j + 2 (i % 4) and + 1 in r[4 j], r[4 j + 1], and the same columns of row i / 4 + 8 in r[4 j + 2],
+// r[4 j + 3]
+__device__ __forceinline__ void tc_ld_frag(unsigned taddr, unsigned (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// four 8x8 matrices of 16-bit elements, stored transposed: thread i gives the address of a 16-byte row of matrix i / 8
+__device__ __forceinline__ void st_matrix4_trans(unsigned saddr, unsigned r0, unsigned r1, unsigned r2, unsigned r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared::cta.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+               : "memory");
+}
 __device__ __forceinline__ void tc_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -311,34 +329,37 @@ __device__ __forceinline__ void mbar_arrive_n_elect(void* bar, unsigned n) {
 }
 
 // All loads and barrier arrivals of one k-block by one CTA of a pair, as ONE instruction group under a
-// single election: expect_tx on the leader's stage barrier, up to two weight boxes, up to two
-// activation boxes, the stand-in arrivals (tiles without a gather) and the go-ahead for the gather warps.
-// Flags select what is issued; everything is warp-uniform.
+// single election: expect_tx on the leader's stage barrier, the box of 128 weight rows, up to three
+// activation boxes (a_rows rows apart), the stand-in arrivals (tiles without a gather) and the go-ahead for the
+// gather warps.  Flags select what is issued; everything is warp-uniform.
 __device__ __forceinline__ void pair_issue_kblock(unsigned bar, unsigned tx, unsigned standin_bar, unsigned standin_n,
-                                                  unsigned sB, const CUtensorMap* tmw, int x, int wy0, int wy1, unsigned has_w1,
-                                                  unsigned sA, const CUtensorMap* tma, int ay, unsigned a_boxes,
+                                                  unsigned sW, const CUtensorMap* tmw, int x, int wblk, int expert,
+                                                  unsigned sX, const CUtensorMap* tma, int ay, unsigned a_boxes, unsigned a_rows,
                                                   unsigned go_bar, unsigned has_go) {
   asm volatile(
-      "{\n\t.reg .pred e, pw1, pa1, pa2, pgo, pst;\n\t.reg .b32 r, sB1, sA1, ay1;\n\t"
+      "{\n\t.reg .pred e, pa1, pa2, pa3, pgo, pst;\n\t.reg .b32 r, st, z, sA1, ay1, sA2, ay2;\n\t"
       "elect.sync r|e, 0xffffffff;\n\t"
-      "setp.ne.and.b32 pw1, %9, 0, e;\n\t"
-      "setp.ge.and.u32 pa1, %13, 1, e;\n\t"
-      "setp.ge.and.u32 pa2, %13, 2, e;\n\t"
+      "setp.ge.and.u32 pa1, %12, 1, e;\n\t"
+      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"
+      "setp.ge.and.u32 pa3, %12, 3, e;\n\t"
       "setp.ne.and.b32 pgo, %15, 0, e;\n\t"
       "setp.ne.and.b32 pst, %3, 0, e;\n\t"
-      "add.u32 sB1, %4, 8192;\n\t"
-      "add.u32 sA1, %10, 4096;\n\t"
-      "add.s32 ay1, %12, 32;\n\t"
+      "mov.b32 z, 0;\n\t"
+      "shl.b32 st, %13, 7;\n\t"
+      "add.u32 sA1, %9, st;\n\t"
+      "add.s32 ay1, %11, %13;\n\t"
+      "add.u32 sA2, sA1, st;\n\t"
+      "add.s32 ay2, ay1, %13;\n\t"
       "@e mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;\n\t"
       "@pst mbarrier.arrive.shared::cta.b64 _, [%2], %3;\n\t"
-      "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%4], [%5, {%6, %7}], [%0];\n\t"
-      "@pw1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sB1], [%5, {%6, %8}], [%0];\n\t"
-      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%10], [%11, {%6, %12}], [%0];\n\t"
-      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%11, {%6, ay1}], [%0];\n\t"
+      "@e cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%4], [%5, {%6, z, z, %7, %8}], [%0];\n\t"
+      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%9], [%10, {%6, %11}], [%0];\n\t"
+      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%10, {%6, ay1}], [%0];\n\t"
+      "@pa3 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA2], [%10, {%6, ay2}], [%0];\n\t"
       "@pgo mbarrier.arrive.shared::cta.b64 _, [%14];\n\t}"
       ::"r"(bar), "r"(tx), "r"(standin_bar), "r"(standin_n),
-        "r"(sB), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wy0), "r"(wy1), "r"(has_w1),
-        "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes),
+        "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert),
+        "r"(sX), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "r"(a_rows),
         "r"(go_bar), "r"(has_go)
       : "memory");
 }

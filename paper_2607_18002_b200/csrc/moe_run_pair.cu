@@ -3,15 +3,14 @@
 // Same scheduling as the single-CTA kernel (two queues, budget word, claim at tile
 // boundaries: Sections 4.2 and 6.4), but the unit that claims and runs a tile is a cluster of
 // two CTAs on neighbouring SMs, and the MMAs are tcgen05.mma.cta_group::2:
-//   - a tile of up to 256 rows runs as ONE M = 256 instruction per k-step: each CTA holds 128
-//     of its rows (activations) and 128 of the 256 weight rows of the tile in its own shared
-//     memory, the tensor cores of both SMs read both halves of the weight tile.  Per SM that
-//     is half the weight bytes through L2 and shared memory for the same flops;
-//   - a tile of up to 128 rows runs as M = 128 (64 rows per CTA): the accumulator of a CTA
-//     then holds its 64 rows twice, lanes 0..63 against the pair leader's weight rows and
-//     lanes 64..127 against the other CTA's;
+//   - the WEIGHT rows are the M = 256 rows of the instruction (128 per CTA) and the tile's token rows its N columns,
+//     N = rows rounded up to 16 (half of them in each CTA's shared memory).  A tile costs tensor time and energy for
+//     the rows it has: with the tokens as M every tile of up to 128 rows paid for 128 of them, and the multipliers' power
+//     alone held a 128-token decode launch at 1.15 GHz (1350 us a pass against 1160 us; a tile there has four rows);
+//   - gate/up tiles take 64 features per CTA, the weight rows interleaved 8 gate / 8 up by one 5-D box, so that an
+//     accumulator fragment holds both factors of a SwiGLU output in one thread; down tiles take 128 features per CTA;
 //   - a stage is 32 KB (16 KB activations + 16 KB weights), six stages deep, and a tile uses
-//     256 of the 512 TMEM columns, so the epilogue of one tile overlaps the MMAs of the next.
+//     up to 256 of the 512 TMEM columns, so the epilogue of one tile overlaps the MMAs of the next.
 // Roles per CTA (16 warps): leader only -- warp 0 scheduler (claims, waits for dependencies,
 // publishes tile descriptors to both CTAs), warp 1 MMA issuer, warp 2 committer; both CTAs --
 // warp 3 producer (TMA loads of its own half, read from the descriptor ring), warps 4-7 gather,
@@ -35,10 +34,10 @@ constexpr int kBBytes = 128 * kRowBytes;                 // this CTA's 128 weigh
 constexpr int kSB = kABytes + kBBytes;
 constexpr int kAccCols = 256;
 constexpr int kFullCount = 2 + kGatherThreads + 1;
-// instruction descriptors: D fp32, A/B bf16, K-major, N = 256, M = 256 / 128 over the pair
-constexpr unsigned kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17);
-constexpr unsigned kIdesc256 = kIdescBase | ((256u >> 4) << 24);
-constexpr unsigned kIdesc128 = kIdescBase | ((128u >> 4) << 24);
+// instruction descriptor: D fp32, A/B bf16, K-major, M = 256 over the pair, N = the tile's columns
+constexpr unsigned kIdescM256 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4) << 24);
+// accumulator columns of a tile (16 is the instruction's step), half of them from each CTA's shared memory
+__device__ __forceinline__ int tile_cols(int rows) { return (rows + 15) & ~15; }
 
 struct SharedCtl {
   alignas(16) TileInfo info[kRing];
@@ -127,48 +126,34 @@ __device__ __forceinline__ void arrive_at_leader(void* bar, bool leader) {
 struct LoadPlan {
   const CUtensorMap* tmw;
   const CUtensorMap* tma;
-  int wy0, wy1;       // weight rows of the one or two boxes (wy1 < 0: one box)
+  int wblk, expert;   // place of the 128 weight rows (see OpDev)
   int ay, a_boxes;    // first activation row, number of boxes (0: none or gathered)
   int a_box_rows;
   unsigned tx;
   bool g1;
 };
 
-__device__ __forceinline__ LoadPlan make_plan(const RunArgs& a, const OpDev* op, const TileInfo& ti, int rank) {
+__device__ __forceinline__ LoadPlan make_plan(const OpDev* op, const TileInfo& ti, int rank) {
   LoadPlan p;
-  const bool pairT = ti.rows > kTileM;
-  const int rpc = pairT ? 128 : 64;
+  const int rpc = tile_cols(ti.rows) / 2;    // rows per CTA
   p.g1 = ti.kind == kGateUp;                 // activation rows come from the gather warps
   const bool w1 = ti.kind != kDown;          // gate/up weights
-  p.wy1 = -1;
+  p.tmw = w1 ? &op->tm_p1 : &op->tm_p2;
+  p.wblk = w1 ? (ti.n * kTileN1 + 64 * rank) / 8 : (ti.n * kTileN2 + 128 * rank) / 16;
+  p.expert = ti.expert;
   p.a_boxes = 0;
   p.a_box_rows = 0;
   p.ay = ti.row0 + rank * rpc;
   p.tma = &op->tm_a8;
   unsigned a_bytes = 0;
-  if (w1) {
-    const int base = ti.expert * 2 * a.I + ti.n * kTileN1;
-    if (pairT) {                 // leader: the 128 gate rows, other CTA: the 128 up rows
-      p.tmw = &op->tm_w1;
-      p.wy0 = base + (rank ? a.I : 0);
-    } else {                     // each CTA: 64 gate rows then the matching 64 up rows
-      p.tmw = &op->tm_w1h;
-      p.wy0 = base + 64 * rank;
-      p.wy1 = base + a.I + 64 * rank;
-    }
-  } else {
-    p.tmw = &op->tm_w2;
-    p.wy0 = ti.expert * a.H + ti.n * kTileN2 + 128 * rank;
-  }
   if (!p.g1) {
     // consecutive rows: of the packed intermediate (down tile) or of x itself (masked-layout gate/up tile)
     const bool fromx = w1;
     const int mine = min(ti.rows - rank * rpc, rpc);
     if (mine > 0) {
-      if (mine <= 8) { p.tma = fromx ? &op->tm_x8 : &op->tm_a8; p.a_boxes = 1; p.a_box_rows = 8; }
-      else if (mine <= 32) { p.tma = fromx ? &op->tm_x32 : &op->tm_a32; p.a_boxes = 1; p.a_box_rows = 32; }
-      else if (pairT) { p.tma = fromx ? &op->tm_x128 : &op->tm_a128; p.a_boxes = 1; p.a_box_rows = 128; }
-      else { p.tma = fromx ? &op->tm_x32 : &op->tm_a32; p.a_boxes = 2; p.a_box_rows = 32; }
+      if (mine <= 16) { p.tma = fromx ? &op->tm_x8 : &op->tm_a8; p.a_boxes = (mine + 7) / 8; p.a_box_rows = 8; }
+      else if (mine <= 96) { p.tma = fromx ? &op->tm_x32 : &op->tm_a32; p.a_boxes = (mine + 31) / 32; p.a_box_rows = 32; }
+      else { p.tma = fromx ? &op->tm_x128 : &op->tm_a128; p.a_boxes = 1; p.a_box_rows = 128; }
       a_bytes = (unsigned)(p.a_boxes * p.a_box_rows * kRowBytes);
     }
   }
@@ -180,16 +165,18 @@ __device__ __forceinline__ LoadPlan make_plan(const RunArgs& a, const OpDev* op,
 // elected lane issues each instruction (the stage is known to be free)
 __device__ __forceinline__ void issue_kblock(SharedCtl* sc, unsigned stages_addr, const LoadPlan& p, int kb,
                                              unsigned stage, bool leader, unsigned full0_addr) {
-  const unsigned sA = stages_addr + stage * (unsigned)kSB;
-  const unsigned sB = sA + (unsigned)kABytes;
+  const unsigned sX = stages_addr + stage * (unsigned)kSB;
   const unsigned bar = full0_addr + stage * 8u;            // the leader's full[stage]
-  // second weight box 64 rows (8 KB) on, second activation box 32 rows (4 KB) and 32 rows on
-  static_assert(64 * kRowBytes == 8192 && 32 * kRowBytes == 4096, "offsets used by pair_issue_kblock");
   pair_issue_kblock(bar, p.tx, smem_u32(&sc->full[stage]),
                     (leader && !p.g1) ? (unsigned)kGatherThreads + 1u : 0u,   // nobody gathers for this tile
-                    sB, p.tmw, kb * kBlockK, p.wy0, p.wy1, p.wy1 >= 0 ? 1u : 0u,
-                    sA, p.tma, p.ay, (unsigned)p.a_boxes,
+                    sX + (unsigned)kABytes, p.tmw, kb * kBlockK, p.wblk, p.expert,
+                    sX, p.tma, p.ay, (unsigned)p.a_boxes, (unsigned)p.a_box_rows,
                     smem_u32(&sc->goA[stage]), p.g1 ? 1u : 0u);
+}
+
+__device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const unsigned*>(&v);
 }
 
 // the scheduler hands a tile to the roles of both CTAs
@@ -319,7 +306,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       }
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (ti.kind == kCombine) continue;
-      const LoadPlan lp = make_plan(args, &args.ops[ti.slot], ti, rank);
+      const LoadPlan lp = make_plan(&args.ops[ti.slot], ti, rank);
       bool fail = false;
       for (int kb = 0; kb < ti.kblocks; ++kb) {
         if (!wwait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
@@ -348,7 +335,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (!wwait(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
         tc_fence_after();
         const unsigned d = __shfl_sync(0xffffffffu, tmem, 0) + b * (unsigned)kAccCols;
-        const unsigned idesc = rows > kTileM ? kIdesc256 : kIdesc128;
+        const unsigned idesc = kIdescM256 | ((unsigned)tile_cols(rows) >> 3) << 17;
         const bool g1 = kind == kGateUp;
         bool fail = false;
         bool ready = false;                           // the current stage was seen full by the look-ahead test
@@ -357,11 +344,11 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           if (!ready && !wwait(c, &sc->full[stage], par, 8)) { fail = true; break; }
           if (g1) fence_async_proxy_smem();            // this CTA's cp.async-written rows -> tensor core reads
           const unsigned sA = sbase + stage * (unsigned)kSB;
-          const unsigned long long ad = umma_desc(sA, kRowBytes), bd = umma_desc(sA + kABytes, kRowBytes);
+          const unsigned long long wd = umma_desc(sA + kABytes, kRowBytes), xd = umma_desc(sA, kRowBytes);
           const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
           // four MMAs (+32 bytes along K per step: the descriptor's address field counts 16 bytes), the
           // commit that frees the stage in both CTAs, and the test of the next stage's barrier
-          ready = pair_mma_kblock(d, ad, bd, idesc, kb ? 1u : 0u, empty0 + stage * 8u, full0 + nstage * 8u, npar);
+          ready = pair_mma_kblock(d, wd, xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u, full0 + nstage * 8u, npar);
           ready = __all_sync(0xffffffffu, ready) && kb + 1 < kblocks;
           stage = nstage;
           par = npar;
@@ -435,7 +422,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const unsigned char* X = static_cast<const unsigned char*>(op->x) + chunk * 16;
       const unsigned char* Xp = static_cast<const unsigned char*>(pop->x) + chunk * 16;
       const size_t pitch = (size_t)args.H * 2;
-      const int rpc = rows > kTileM ? 128 : 64;
+      const int rpc = tile_cols(rows) / 2;
       const int first = rank * rpc;                       // this CTA's first row of the tile
       int tok[kPasses];
       const int n_rows = op->n_rows, n_rows_p = pop->n_rows;
@@ -496,16 +483,16 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     }
   } else if (warp >= 8) {
     // ============================================================ epilogue (8 warps per CTA)
-    // Warp w reads TMEM lanes 32 (w % 4) .. +31.  M = 256 tiles: lane = one of this CTA's 128
-    // rows, 256 columns.  M = 128 tiles: lanes 0..63 and 64..127 both hold this CTA's 64
-    // rows, against the first / second 128 weight rows of the tile (128 columns).
+    // Warp w reads TMEM lanes 32 (w % 4) .. +31 (weight rows: 2 x (8 gate + 8 up), or 32 down features) and one half of the
+    // tile's columns (token rows), 32 tokens per pass.  Fragment loads and transposed 8x8 stores turn a pass into
+    // token-major rows of 32 (gate/up) or 64 bytes in the warp's scratch, which leave as 16-byte stores.
     const int q = warp & 3;
-    const int half = (warp - 8) >> 2;             // the two warps of a quadrant split the columns
+    const int half = (warp - 8) >> 2;             // the two warps of a quadrant split the tokens
     const int etid = threadIdx.x - 256;
     int islot = 0;
     unsigned iph = 0, gcount = 0;
     unsigned char* scratch = sc->epi_scratch[warp - 8];
-    const int srow = lane >> 2, schunk = lane & 3;
+    const unsigned scratch_addr = smem_u32(scratch);
     while (true) {
       if (!wait_info(c, &sc->ifull[islot], iph, 9, leader)) break;
       const TileInfo ti = sc->info[islot];
@@ -522,64 +509,87 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (!ok) break;
         ++gcount;
         tc_fence_after();
-        const bool pairT = ti.rows > kTileM;
         const bool g1 = ti.kind != kDown;                     // gate/up tile: SwiGLU, output to A
-        const int rpc = pairT ? 128 : 64;
-        const int lrow0 = pairT ? q * 32 : (q & 1) * 32;     // first of this warp's rows within the CTA's rows
-        const int cg = pairT ? 0 : (q >> 1);                  // which 128 weight rows (M = 128 tiles)
-        const int ncols = pairT ? (g1 ? 128 : 256) : (g1 ? 64 : 128);   // output columns held per lane
-        const int upoff = pairT ? 128 : 64;                   // column distance gate -> up
-        const int passes = ncols / 64;                        // 32-column passes per warp
-        const int trow0 = rank * rpc + lrow0;                 // tile row of lane 0
-        const int rows_here = min(32, ti.rows - trow0);
-        const size_t pitch = (size_t)(g1 ? args.I : args.H) * 2;
-        if (rows_here > 0) {
-          const unsigned taddr = tmem + (unsigned)(b * kAccCols) + ((unsigned)(q * 32) << 16);
+        const int cols = tile_cols(ti.rows) / 2;              // this warp's columns
+        const int live = min(cols, ti.rows - half * cols);    // ... that hold token rows
+        const int passes = (live + 31) / 32;
+        if (passes > 0) {
+          const unsigned taddr = tmem + (unsigned)(b * kAccCols + half * cols) + ((unsigned)(q * 32) << 16);
+          const size_t pitch = (size_t)(g1 ? args.I : args.H) * 2;
           unsigned char* out = reinterpret_cast<unsigned char*>(g1 ? (void*)op->A : (void*)op->D) +
-                               (size_t)(ti.row0 + trow0) * pitch +
-                               ((size_t)ti.n * (g1 ? kTileN1 : kTileN2) + (size_t)cg * ncols) * 2;
-          unsigned g[32], u[32];
-          tc_ld32(taddr + (half * passes) * 32, g);
-          if (g1) tc_ld32(taddr + upoff + (half * passes) * 32, u);
+                               (size_t)(ti.row0 + half * cols) * pitch +
+                               (size_t)(g1 ? ti.n * kTileN1 + rank * 64 + q * 16 : ti.n * kTileN2 + rank * 128 + q * 32) * 2;
+          unsigned lo[16], hi[16];                            // lanes 0..15 and 16..31 of the quadrant
+          tc_ld_frag(taddr, lo);
+          tc_ld_frag(taddr + (16u << 16), hi);
 #pragma unroll 1
           for (int p = 0; p < passes; ++p) {
-            const int pass = half * passes + p;
-            uint4 o[4];
-            __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(o);
             tc_wait_ld();
+            const bool last = p + 1 == passes;
+            if (last) {                                       // all of it is in registers: the accumulator may be overwritten
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);
+            }
+            unsigned o[16];
             if (g1) {
 #pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                const float a0 = silu_mul(__uint_as_float(g[2 * i]), __uint_as_float(u[2 * i]));
-                const float a1 = silu_mul(__uint_as_float(g[2 * i + 1]), __uint_as_float(u[2 * i + 1]));
-                oh[i] = __floats2bfloat162_rn(a0, a1);
+              for (int j = 0; j < 4; ++j) {
+                o[j] = pack_bf16(silu_mul(__uint_as_float(lo[4 * j]), __uint_as_float(lo[4 * j + 2])),
+                                 silu_mul(__uint_as_float(lo[4 * j + 1]), __uint_as_float(lo[4 * j + 3])));
+                o[4 + j] = pack_bf16(silu_mul(__uint_as_float(hi[4 * j]), __uint_as_float(hi[4 * j + 2])),
+                                     silu_mul(__uint_as_float(hi[4 * j + 1]), __uint_as_float(hi[4 * j + 3])));
               }
             } else {
 #pragma unroll
-              for (int i = 0; i < 16; ++i)
-                oh[i] = __floats2bfloat162_rn(__uint_as_float(g[2 * i]), __uint_as_float(g[2 * i + 1]));
-            }
-            if (p + 1 < passes) {
-              tc_ld32(taddr + (pass + 1) * 32, g);
-              if (g1) tc_ld32(taddr + upoff + (pass + 1) * 32, u);
-            }
-            __syncwarp();                                          // scratch free again
+              for (int j = 0; j < 4; ++j) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)     // row `lane`, 16-byte chunk j (XOR keeps banks apart)
-              *reinterpret_cast<uint4*>(scratch + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = o[j];
+                for (int r = 0; r < 2; ++r) {
+                  o[4 * r + j] = pack_bf16(__uint_as_float(lo[4 * j + 2 * r]), __uint_as_float(lo[4 * j + 2 * r + 1]));
+                  o[8 + 4 * r + j] = pack_bf16(__uint_as_float(hi[4 * j + 2 * r]), __uint_as_float(hi[4 * j + 2 * r + 1]));
+                }
+              }
+            }
+            if (!last) {
+              tc_ld_frag(taddr + (unsigned)((p + 1) * 32), lo);
+              tc_ld_frag(taddr + (unsigned)((p + 1) * 32) + (16u << 16), hi);
+            }
+            __syncwarp();                                     // scratch free again
+            // matrix i / 8 of a store is token group i / 8, its row i % 8 is token `lane` of the pass
+            if (g1) {
+#pragma unroll
+              for (int cch = 0; cch < 2; ++cch)
+                st_matrix4_trans(scratch_addr + lane * 32 + cch * 16, o[4 * cch], o[4 * cch + 1], o[4 * cch + 2], o[4 * cch + 3]);
+            } else {
+#pragma unroll
+              for (int cch = 0; cch < 4; ++cch)               // XOR keeps the banks of eight rows apart
+                st_matrix4_trans(scratch_addr + lane * 64 + ((cch ^ ((lane >> 1) & 3)) << 4), o[4 * cch], o[4 * cch + 1],
+                                 o[4 * cch + 2], o[4 * cch + 3]);
+            }
             __syncwarp();
+            unsigned char* dst = out + (size_t)(p * 32) * pitch;
+            const int left = live - p * 32;
+            if (g1) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int r = 8 * j + srow;
-              const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 64 + ((schunk ^ ((r >> 1) & 3)) << 4));
-              if (r < rows_here)
-                *reinterpret_cast<uint4*>(out + (size_t)r * pitch + pass * 64 + schunk * 16) = v4;
+              for (int j = 0; j < 2; ++j) {
+                const int r = 16 * j + (lane >> 1), cch = lane & 1;
+                const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 32 + cch * 16);
+                if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + cch * 16) = v4;
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const int r = 8 * j + (lane >> 2), cch = lane & 3;
+                const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 64 + ((cch ^ ((r >> 1) & 3)) << 4));
+                if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + cch * 16) = v4;
+              }
             }
           }
+        } else {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);   // accumulator may be overwritten
       }
       __syncwarp();
       if (lane == 0) {
