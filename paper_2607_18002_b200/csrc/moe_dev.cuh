@@ -56,7 +56,7 @@ struct PlanState {
   int pad[3];
 };
 
-// Zeroed by moe_run before every launch.
+// Part of the run state, see RunHead.
 struct RunState {
   int gemm_done;      // committed GEMM tiles
   int tiles_done;     // committed tiles of any kind
@@ -106,8 +106,8 @@ struct __align__(128) OpDev {
   int4* tile_list;       // [max_tiles] queue entries in claim order
   int* plan_hist;        // [n_chunks, E] rows per plan block and expert
   PlanState* plan;
-  RunState* run;
-  int* g1_done;          // [max_mtiles] committed gate/up tiles per work tile
+  RunState* run;         // in the first half of the run state
+  int* g1_done;          // [max_mtiles] committed gate/up tiles per work tile (first half)
   Status* status;        // the context's device status block
   // Which list of routed rows the run kernels walk.  A plain op: its own permutation (the plan's public
   // outputs).  The paired form of a decode + prefill op that share their weights (moe_plan_pair): one row
@@ -133,11 +133,15 @@ struct Status {   // first error wins (atomicCAS on code)
 struct Global {
   Status status;
   int budget;             // decode SM budget q (Section 6.4)
-  int pad[7];
+  unsigned launches;      // launches of the run kernels so far: half `launches & 1` of the run state is the next one's
+  unsigned started;       // claiming units of the current launch that have read `launches`
+  int pad[5];
 };
 
-// Start of the region moe_run zeroes before every launch; the per-slot RunState blocks and
-// g1_done arrays follow it.
+// The run state exists twice.  A launch works on one half, which is zero when it starts, and zeroes the other for the
+// next one; the unit that is last to read `launches` advances it.  That keeps a memset (with its gaps 6 us of a 70 us decode pass)
+// off the stream.
+// Start of a half; the per-slot RunState blocks and g1_done arrays follow it.
 struct RunHead {
   unsigned heads[2];      // next ticket of the decode / prefill queue
   unsigned log_count;
@@ -154,12 +158,39 @@ struct RunArgs {
   int E, k, H, I;
   int dtype, kb_elems;    // MOE_DTYPE_*; K elements per pipeline stage (64 bf16 / 128 e4m3)
   long long wait_ns;
+  unsigned run_bytes;     // size of one half of the run state
   int n_slots;            // slots of the context; descriptor d >= n_slots is the paired form of slot d - n_slots
   signed char desc[kMaxOps];   // slot -> the descriptor that stands for it in this launch
   int static_kind;        // -1: persistent launch served from the queues.  >= 0: a plain launch, claiming unit u
                           // of the grid runs queue entry u of slots[0] and ends
   int slots[kMaxOps];     // descriptor indices of the launch's ops, in the order given
+  const PlanState* plan[kMaxOps];   // of slots[i]; with the two below all that the queue tables are built from
+  signed char cls[kMaxOps];
+  signed char free_op[kMaxOps];     // 1: the op has no ready word and no predecessor
 };
+
+// ------------------------------------------------------------------ launches that overlap the tail of the one before
+// All kernels of the library are launched so that their blocks may become resident while the previous kernel of the stream
+// still runs.  Each calls grid_dep_wait before it touches global memory, which returns when that kernel is complete and its writes
+// are visible, and then lets the next one in.
+__device__ __forceinline__ void grid_dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... Params, class... Args>
+inline cudaError_t launch_after(void (*kernel)(Params...), int blocks, int threads, size_t smem, cudaStream_t stream, Args&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
 
 __device__ __forceinline__ int slot_of(const RunArgs* a, int desc) { return desc >= a->n_slots ? desc - a->n_slots : desc; }
 

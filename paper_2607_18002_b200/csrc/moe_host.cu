@@ -30,11 +30,11 @@ namespace {
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Layout {
-  size_t global_off, ops_off, runzero_off, runzero_bytes, log_off, slots_off, slot_stride;
+  size_t global_off, ops_off, run_off, run_bytes, log_off, slots_off, slot_stride;
   // inside a slot
   size_t A_off, D_off, mtiles_off, tiles_off, hist_off, plan_off;
   size_t ptiles_off, pgather_off, pcomb_off, pplan_off;   // paired form: queue list, shared-space permutation, plan state
-  // inside the run-zero region (after RunHead)
+  // inside a half of the run state (after RunHead)
   size_t rs_stride;      // RunState + g1_done[max_mtiles], per slot
   size_t total;
   int max_rows, max_mtiles, max_tiles, NT1, NT2;
@@ -89,10 +89,10 @@ Layout make_layout(const moe_config_t* c) {
   size_t g = 0;
   L.global_off = g;    g = align_up(g + sizeof(Global), 1024);
   L.ops_off = g;       g = align_up(g + sizeof(OpDev) * 2 * c->max_ops, 1024);   // plain and paired descriptors
-  L.runzero_off = g;
+  L.run_off = g;
   L.rs_stride = align_up(sizeof(RunState) + (size_t)L.max_mtiles * 4, 16);
-  L.runzero_bytes = align_up(sizeof(RunHead) + L.rs_stride * c->max_ops, 1024);
-  g += L.runzero_bytes;
+  L.run_bytes = align_up(sizeof(RunHead) + L.rs_stride * c->max_ops, 1024);
+  g += 2 * L.run_bytes;
   L.log_off = g;       g = align_up(g + (size_t)c->tile_log_entries * sizeof(moe_tile_rec_t), 1024);
   L.slots_off = g;
   L.total = g + L.slot_stride * c->max_ops;
@@ -123,10 +123,10 @@ struct moe_ctx {
   int pair_of[kMaxOps];         // slot paired with this one by moe_plan_pair since both were last planned, or -1
   bool ran_paired[kMaxOps];     // the slot's last moe_run used its paired form (moe_combine follows it)
   Global* g() const { return reinterpret_cast<Global*>(ws + L.global_off); }
-  RunHead* rh() const { return reinterpret_cast<RunHead*>(ws + L.runzero_off); }
+  RunHead* rh() const { return reinterpret_cast<RunHead*>(ws + L.run_off); }
   unsigned char* slot_base(int s) const { return ws + L.slots_off + L.slot_stride * s; }
   OpDev* op_dev(int s) const { return reinterpret_cast<OpDev*>(ws + L.ops_off) + s; }
-  unsigned char* rs_base(int s) const { return ws + L.runzero_off + sizeof(RunHead) + L.rs_stride * s; }
+  unsigned char* rs_base(int s) const { return ws + L.run_off + sizeof(RunHead) + L.rs_stride * s; }
 };
 
 namespace {
@@ -166,10 +166,14 @@ int make_map_pair(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t cols,
 }
 
 // a stream-ordered 4-byte write: the value travels in the launch, not through host memory
-__global__ void set_word_kernel(int* p, int v) { *reinterpret_cast<volatile int*>(p) = v; }
+__global__ void set_word_kernel(int* p, int v) {
+  grid_dep_wait();
+  *reinterpret_cast<volatile int*>(p) = v;
+}
 
 // The op descriptor travels as a kernel parameter (no pageable-memory copy on the stream).
 __global__ void write_op_kernel(const __grid_constant__ OpDev src, OpDev* dst) {
+  grid_dep_wait();
   const int n = (int)(sizeof(OpDev) / sizeof(int));
   const int* s = reinterpret_cast<const int*>(&src);
   int* d = reinterpret_cast<int*>(dst);
@@ -350,8 +354,7 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
       if (rc) return rc;
     }
     ctx->planned[slot] = false;
-    write_op_kernel<<<1, 128, 0, st>>>(h, ctx->op_dev(slot));
-    if (cudaGetLastError() != cudaSuccess) { ctx->uploaded[slot] = false; return MOE_ECUDA; }
+    if (launch_after(write_op_kernel, 1, 128, 0, st, h, ctx->op_dev(slot)) != cudaSuccess) { ctx->uploaded[slot] = false; return MOE_ECUDA; }
     ctx->host_ops[slot] = h;
     ctx->ops[slot] = *op;             // what the device copy of the slot now describes
     ctx->uploaded[slot] = true;
@@ -410,8 +413,14 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   a.kb_elems = c.dtype == MOE_DTYPE_FP8_E4M3 ? 128 : kBlockK;
   a.wait_ns = (long long)c.wait_limit_us * 1000;
   a.static_kind = -1;
+  a.run_bytes = (unsigned)ctx->L.run_bytes;
+  for (int i = 0; i < n_ops; ++i) {
+    const OpDev& h = ctx->ran_paired[slots[i]] ? ctx->host_pair[slots[i]] : ctx->host_ops[slots[i]];
+    a.plan[i] = h.plan;
+    a.cls[i] = (signed char)h.cls;
+    a.free_op[i] = h.ready == nullptr && h.after_op < 0 ? 1 : 0;
+  }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(ctx->rh(), 0, ctx->L.runzero_bytes, st) != cudaSuccess) return MOE_ECUDA;
   if (ctx->poison) {
     for (int i = 0; i < n_ops; ++i) {
       unsigned char* sb = ctx->slot_base(slots[i]);
@@ -455,8 +464,11 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream) {
   a.n_slots = c.max_ops;
   for (int s = 0; s < kMaxOps; ++s) a.desc[s] = (signed char)s;
   ctx->ran_paired[slot] = false;
-  if (cudaMemsetAsync(ctx->rh(), 0, ctx->L.runzero_bytes, st) != cudaSuccess) return MOE_ECUDA;
   a.static_kind = 0;
+  a.run_bytes = (unsigned)ctx->L.run_bytes;
+  a.plan[0] = ctx->host_ops[slot].plan;
+  a.cls[0] = (signed char)ctx->host_ops[slot].cls;
+  a.free_op[0] = 1;
   if (ps.n_gemm_tiles > 0 && launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, st) != cudaSuccess) return MOE_ECUDA;
   if (ctx->ops[slot].layout == MOE_LAYOUT_GATHERED &&
       launch_combine(ctx->op_dev(slot), ctx->ops[slot].n_tokens, c.top_k, c.hidden, st) != cudaSuccess)
@@ -519,8 +531,7 @@ int moe_plan_pair(moe_ctx_t* ctx, int slot_prefill, int slot_decode, int carrier
   for (int i = 0; i < 2; ++i) {
     const int s = which[i];
     if (ctx->pair_uploaded[s] && memcmp(&ctx->host_pair[s], both[i], sizeof(OpDev)) == 0) continue;
-    write_op_kernel<<<1, 128, 0, st>>>(*both[i], ctx->op_dev(c.max_ops + s));
-    if (cudaGetLastError() != cudaSuccess) { ctx->pair_uploaded[s] = false; return MOE_ECUDA; }
+    if (launch_after(write_op_kernel, 1, 128, 0, st, *both[i], ctx->op_dev(c.max_ops + s)) != cudaSuccess) { ctx->pair_uploaded[s] = false; return MOE_ECUDA; }
     ctx->host_pair[s] = *both[i];
     ctx->pair_uploaded[s] = true;
   }
@@ -537,13 +548,14 @@ int moe_plan_pair(moe_ctx_t* ctx, int slot_prefill, int slot_decode, int carrier
 
 int moe_set_budget(moe_ctx_t* ctx, int decode_sms, void* stream) {
   if (!ctx || decode_sms < 0) return MOE_EINVAL;
-  set_word_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(&ctx->g()->budget, decode_sms);
-  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ECUDA;
+  return launch_after(set_word_kernel, 1, 1, 0, static_cast<cudaStream_t>(stream), &ctx->g()->budget, decode_sms) == cudaSuccess
+             ? MOE_OK : MOE_ECUDA;
 }
 
 namespace {
 // q' = min(q_max, ceil_c(q * x_moe / x_star)) from the slot's planned footprint (Section 6.4)
 __global__ void scaled_budget_kernel(int* budget, const PlanState* plan, int q, double x_star, int q_max, int c) {
+  grid_dep_wait();
   const double want = ceil((double)q * (double)plan->n_mtiles / x_star);
   long long v = want > 2147483000.0 ? 2147483000ll : (long long)want;
   v = (v + c - 1) / c * c;
@@ -555,9 +567,8 @@ int moe_set_budget_scaled(moe_ctx_t* ctx, int slot, int q, double x_moe_star, in
   if (!ctx || slot < 0 || slot >= ctx->cfg.max_ops || q < 0 || q_max < 0 || !(x_moe_star > 0.0)) return MOE_EINVAL;
   if (!ctx->planned[slot]) return MOE_ENOTPLANNED;
   const PlanState* ps = reinterpret_cast<const PlanState*>(ctx->slot_base(slot) + ctx->L.plan_off);
-  scaled_budget_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(&ctx->g()->budget, ps, q, x_moe_star, q_max,
-                                                                      ctx->pair_kernel ? 2 : 1);
-  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ECUDA;
+  return launch_after(scaled_budget_kernel, 1, 1, 0, static_cast<cudaStream_t>(stream), &ctx->g()->budget, ps, q, x_moe_star, q_max,
+                      ctx->pair_kernel ? 2 : 1) == cudaSuccess ? MOE_OK : MOE_ECUDA;
 }
 
 int moe_get_budget(moe_ctx_t* ctx, int32_t* out) {
@@ -606,8 +617,12 @@ int moe_read_tile_table(moe_ctx_t* ctx, int slot, int32_t* host_out, int max_til
 
 int moe_read_tile_log(moe_ctx_t* ctx, moe_tile_rec_t* host_out, int max_records, int* n) {
   if (!ctx || !host_out || !n || max_records < 0) return MOE_EINVAL;
+  Global g;
   RunHead rh;
-  if (cudaMemcpy(&rh, ctx->rh(), sizeof(rh), cudaMemcpyDeviceToHost) != cudaSuccess) return MOE_ECUDA;
+  if (cudaMemcpy(&g, ctx->g(), sizeof(g), cudaMemcpyDeviceToHost) != cudaSuccess) return MOE_ECUDA;
+  const size_t half = (g.launches & 1) ? 0 : ctx->L.run_bytes;            // the one the last launch worked on
+  if (cudaMemcpy(&rh, reinterpret_cast<unsigned char*>(ctx->rh()) + half, sizeof(rh), cudaMemcpyDeviceToHost) != cudaSuccess)
+    return MOE_ECUDA;
   int cnt = (int)rh.log_count;
   if (cnt > ctx->cfg.tile_log_entries) cnt = ctx->cfg.tile_log_entries;
   if (cnt > max_records) cnt = max_records;

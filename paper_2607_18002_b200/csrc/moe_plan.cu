@@ -143,6 +143,7 @@ struct PlanArgs {
 __global__ void __launch_bounds__(kPlanThreads) plan_hist_kernel(const __grid_constant__ PlanArgs a) {
   __shared__ int h[kMaxExperts];
   for (int e = threadIdx.x; e < a.E; e += kPlanThreads) h[e] = 0;
+  grid_dep_wait();
   __syncthreads();
   const int i0 = (int)blockIdx.x * a.own, i1 = min(a.R, i0 + a.own);
   for (int i = i0 + (int)threadIdx.x; i < i1; i += kPlanThreads) {
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
 
   for (int e = tid; e < E; e += kPlanThreads) s_before[e] = s_cnt[e] = 0;
   for (int i = tid; i < kPlanWarps * E; i += kPlanThreads) run[i] = 0;
+  grid_dep_wait();
   __syncthreads();
   // rows per expert: before this block's range, and from it on
   if (kDirect) {
@@ -266,6 +268,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_
   __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts];
   const int e = threadIdx.x, E = a.E;
   int cnt = 0;
+  grid_dep_wait();
   if (e < E) {
     cnt = a.counts[e];
     if (cnt < 0 || cnt > slab_rows) {        // a count the slab cannot hold: reported, the slab is left out
@@ -321,6 +324,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_co
   __shared__ int cnt_d[kMaxExperts], off_d[kMaxExperts], cnt_p[kMaxExperts], off_p[kMaxExperts];
   __shared__ int base_d[kMaxExperts], base_p[kMaxExperts];   // what a row's packed position is shifted by
   const int e = threadIdx.x, E = a.E;
+  grid_dep_wait();
   if (e < E) {
     const int cd = a.d.counts[e], cp = a.p.counts[e];
     const int od = a.d.offsets[e], op = a.p.offsets[e];
@@ -372,8 +376,7 @@ cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2
   a.counts = h.counts; a.offsets = h.offsets; a.mtiles = h.mtiles; a.tile_list = h.tile_list; a.plan = h.plan;
   a.status = h.status;
   a.slot = slot; a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows;
-  plan_masked_kernel<<<list_blocks(E), kPlanThreads, 0, stream>>>(a, slab_rows);
-  return cudaGetLastError();
+  return launch_after(plan_masked_kernel, list_blocks(E), kPlanThreads, 0, stream, a, slab_rows);
 }
 
 cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, const OpDev& p, int* gather, int* comb_d,
@@ -385,8 +388,7 @@ cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, c
   a.gather = gather;
   a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows; a.carrier_rows = carrier_rows;
   const int blocks = max(list_blocks(E), min(kPlanMaxBlocks, (d.n_rows + p.n_rows + kPlanThreads - 1) / kPlanThreads));
-  plan_pair_kernel<<<blocks, kPlanThreads, 0, stream>>>(a);
-  return cudaGetLastError();
+  return launch_after(plan_pair_kernel, blocks, kPlanThreads, 0, stream, a);
 }
 
 cudaError_t prepare_plan_kernels() {
@@ -405,14 +407,12 @@ cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int w
   if (a.R <= kPlanDirectRows) {
     const int blocks = list_blocks(E);
     a.own = ((a.R + blocks - 1) / blocks + kPlanThreads - 1) / kPlanThreads * kPlanThreads;
-    plan_rank_kernel<true><<<blocks, kPlanThreads, smem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_after(plan_rank_kernel<true>, blocks, kPlanThreads, smem, stream, a);
   }
   a.own = kPlanThreads * (int)(((long long)a.R + kPlanThreads * kPlanMaxBlocks - 1) / (kPlanThreads * kPlanMaxBlocks));
   const int blocks = (a.R + a.own - 1) / a.own;
-  plan_hist_kernel<<<blocks, kPlanThreads, 0, stream>>>(a);
-  plan_rank_kernel<false><<<blocks, kPlanThreads, smem, stream>>>(a);
-  return cudaGetLastError();
+  const cudaError_t e = launch_after(plan_hist_kernel, blocks, kPlanThreads, 0, stream, a);
+  return e != cudaSuccess ? e : launch_after(plan_rank_kernel<false>, blocks, kPlanThreads, smem, stream, a);
 }
 
 }  // namespace moe

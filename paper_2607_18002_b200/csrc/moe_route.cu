@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(const float* __
                                                                  int* __restrict__ ids, float* __restrict__ w) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * kRouteWarps + warp;
+  grid_dep_wait();
   if (t >= T) return;
   const float* z = logits + (size_t)t * E;
   unsigned key[kPer];                      // expert of key i: see id_of
@@ -94,6 +95,6 @@ extern "C" int moe_route(const float* logits, int32_t n_tokens, int32_t n_expert
   const bool small = n_experts <= 256;
   auto* kernel = small ? (vec ? route_kernel<8, true> : route_kernel<8, false>)
                        : (vec ? route_kernel<32, true> : route_kernel<32, false>);
-  kernel<<<blocks, kRouteWarps * 32, 0, static_cast<cudaStream_t>(stream)>>>(logits, n_tokens, n_experts, top_k, topk_ids, topk_w);
-  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ECUDA;
+  return launch_after(kernel, blocks, kRouteWarps * 32, 0, static_cast<cudaStream_t>(stream), logits, n_tokens, n_experts, top_k,
+                      topk_ids, topk_w) == cudaSuccess ? MOE_OK : MOE_ECUDA;
 }

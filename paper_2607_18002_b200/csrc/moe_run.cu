@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   SharedCtl* sc = reinterpret_cast<SharedCtl*>(stages + (size_t)kNS * kSB);
   static_assert(kNS * kSB == 3 * (kABytes + kBBytes), "ring size");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  Ctx c{&args, &args.g->status};
+  Ctx c{&args, &args.g->status, 0u};
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kNS; ++s) {
@@ -254,8 +254,6 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       mbar_init(&sc->iempty[s], 2 + kGatherThreads / 32);
       mbar_init(&sc->done[s], 256);
     }
-    build_queues(&args, &sc->qt);
-    if (blockIdx.x == 0) finish_empty_ops(&args, -1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_proxy();
   }
@@ -266,10 +264,21 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  grid_dep_wait();             // everything above overlaps the kernel before this one
+  if (warp == 0) {
+    build_queues(&args, &sc->qt, lane);
+    if (lane == 0) sc->qt.run_off = begin_unit(&args, (int)gridDim.x);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const unsigned tmem = sc->tmem_base;
+  c.run_off = sc->qt.run_off;
+  if (blockIdx.x == 0 && warp == 3) {
+    clear_next_run(&args, rh, c.run_off, lane);
+    if (lane == 0) finish_empty_ops(c, -1);
+  }
+  rh = reinterpret_cast<RunHead*>(reinterpret_cast<char*>(rh) + c.run_off);
   // The fp8 epilogue keeps 128 fp32 accumulators per thread: the two epilogue warpgroups take
   // registers from the two others (64 + 192 = 2 x 128 per thread pair).  Each role changes its
   // allowance at the top of its own branch, so the compiler can budget the branch by it.
@@ -303,8 +312,8 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         int ok = 1;
         if (lane == 0) {
           // a claimed tile only ever waits on tiles that were claimed before it
-          if (ti.kind == kDown) ok = wait_counter(c, &op->g1_done[ti.m], args.I / kTileN1, 3);
-          if (ti.kind == kCombine) ok = wait_counter(c, &op->run->gemm_done, op_gemm_tiles(op), 4);
+          if (ti.kind == kDown) ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
+          if (ti.kind == kCombine) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op), 4);
           if (!ok) ti.kind = kEnd;
           fence_async_proxy();
           sc->info[islot] = ti;
@@ -348,12 +357,12 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
             // takes no waiting: free ring slot, op ready, dependencies already met.
             const OpDev* nop = &args.ops[nx.slot];
             bool can = __all_sync(0xffffffffu, mbar_try(&sc->iempty[islot], iph ^ 1u));
-            if (can && nx_need_ready) can = __shfl_sync(0xffffffffu, op_ready(&args, nop) ? 1 : 0, 0) != 0;   // lane 0's look
+            if (can && nx_need_ready) can = __shfl_sync(0xffffffffu, op_ready(c, nop) ? 1 : 0, 0) != 0;   // lane 0's look
             if (can) {
               int met = 1;
               if (lane == 0) {
-                if (nx.kind == kDown) met = ld_acquire(&nop->g1_done[nx.m]) >= args.I / kTileN1;
-                if (nx.kind == kCombine) met = ld_acquire(&nop->run->gemm_done) >= op_gemm_tiles(nop);
+                if (nx.kind == kDown) met = ld_acquire(&g1_done_of(c, nop)[nx.m]) >= args.I / kTileN1;
+                if (nx.kind == kCombine) met = ld_acquire(&run_of(c, nop)->gemm_done) >= op_gemm_tiles(nop);
                 if (met) {
                   fence_async_proxy();
                   sc->info[islot] = nx;
@@ -697,9 +706,8 @@ cudaError_t prepare_run_kernel() {
 }
 
 cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
-  if (args.dtype == MOE_DTYPE_FP8_E4M3) moe_apk_kernel<true><<<n_ctas, kThreads, kSmemBytes, stream>>>(args, rh);
-  else moe_apk_kernel<false><<<n_ctas, kThreads, kSmemBytes, stream>>>(args, rh);
-  return cudaGetLastError();
+  return launch_after(args.dtype == MOE_DTYPE_FP8_E4M3 ? moe_apk_kernel<true> : moe_apk_kernel<false>, n_ctas, kThreads, kSmemBytes,
+                      stream, args, rh);
 }
 
 }  // namespace moe

@@ -202,7 +202,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const bool leader = rank == 0;
-  Ctx c{&args, &args.g->status};
+  Ctx c{&args, &args.g->status, 0u};
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kNS; ++s) {
@@ -223,8 +223,6 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       mbar_init(&sc->done[s], 16);
       mbar_init(&sc->taken[s], 1);
     }
-    if (leader) build_queues(&args, &sc->qt);
-    if (blockIdx.x == 0) finish_empty_ops(&args, -1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_proxy();
   }
@@ -235,11 +233,24 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  grid_dep_wait();             // everything above overlaps the kernel before this one
+  if (warp == 0 && leader) {
+    build_queues(&args, &sc->qt, lane);
+    if (lane == 0) sc->qt.run_off = begin_unit(&args, (int)(gridDim.x >> 1));
+  }
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();          // the other CTA's barriers exist before anything arrives on them
   tc_fence_after();
   const unsigned tmem = sc->tmem_base;
+  if (leader) {                // the second CTA has no business with the run state
+    c.run_off = sc->qt.run_off;
+    if (blockIdx.x == 0 && warp == 2) {
+      clear_next_run(&args, rh, c.run_off, lane);
+      if (lane == 0) finish_empty_ops(c, -1);
+    }
+    rh = reinterpret_cast<RunHead*>(reinterpret_cast<char*>(rh) + c.run_off);
+  }
 
   if (warp == 0 && leader) {
     // ============================================================ scheduler (leader)
@@ -264,8 +275,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (ti.kind != kEnd && need_ready && !wait_op_ready(c, lane, ti)) ti.kind = kEnd;
       int ok = 1;
       if (lane == 0) {
-        if (ti.kind == kDown) ok = wait_counter(c, &op->g1_done[ti.m], args.I / kTileN1, 3);
-        if (ti.kind == kCombine) ok = wait_counter(c, &op->run->gemm_done, op_gemm_tiles(op), 4);
+        if (ti.kind == kDown) ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
+        if (ti.kind == kCombine) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op), 4);
         if (!ok) ti.kind = kEnd;
         publish(sc, islot, ti);
       }
@@ -620,8 +631,7 @@ cudaError_t prepare_pair_kernel() {
 
 // n_ctas: the persistent grid, or 2 x the number of queue entries for a plain launch
 cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
-  pairk::moe_apk_pair_kernel<<<n_ctas, pairk::kThreads, pairk::kSmemBytes, stream>>>(args, rh);
-  return cudaGetLastError();
+  return launch_after(pairk::moe_apk_pair_kernel, n_ctas, pairk::kThreads, pairk::kSmemBytes, stream, args, rh);
 }
 
 }  // namespace moe

@@ -18,6 +18,7 @@ struct TileInfo {
 
 // per-class queue tables of one launch (built once per CTA in shared memory)
 struct QueueTables {
+  unsigned run_off;                // of this launch
   int n_cls[2];
   int cls_slot[2][kMaxOps];
   int cls_free[2][kMaxOps];        // 1: the op has no ready word and no predecessor
@@ -28,7 +29,14 @@ struct QueueTables {
 struct Ctx {
   const RunArgs* a;
   Status* st;
+  unsigned run_off;              // 0 or run_bytes: the half of the run state this launch works on
 };
+__device__ __forceinline__ RunState* run_of(const Ctx& c, const OpDev* op) {
+  return reinterpret_cast<RunState*>(reinterpret_cast<char*>(op->run) + c.run_off);
+}
+__device__ __forceinline__ int* g1_done_of(const Ctx& c, const OpDev* op) {
+  return reinterpret_cast<int*>(reinterpret_cast<char*>(op->g1_done) + c.run_off);
+}
 
 __device__ __forceinline__ bool aborted(const Ctx& c) { return ld_volatile(&c.st->abort) != 0; }
 
@@ -109,24 +117,26 @@ __device__ __forceinline__ int op_gemm_tiles(const OpDev* op) { return op->plan-
 
 // An op without tiles (no tokens, or a plan that was rejected) never commits anything: it counts as
 // finished as soon as its own predecessor has, and its ready word is not consulted.
-__device__ inline bool op_finished(const RunArgs* a, int slot) {
+__device__ inline bool op_finished(const Ctx& c, int slot) {
+  const RunArgs* a = c.a;
   for (int hop = 0; slot >= 0 && hop <= kMaxOps; ++hop) {
     const OpDev* op = &a->ops[a->desc[slot]];
-    if (op_total_tiles(op, a->fuse_combine) > 0) return ld_acquire(&op->run->done) != 0;
+    if (op_total_tiles(op, a->fuse_combine) > 0) return ld_acquire(&run_of(c, op)->done) != 0;
     slot = op->after_op;
   }
   return true;
 }
 
-__device__ inline bool op_ready(const RunArgs* a, const OpDev* op) {
+__device__ inline bool op_ready(const Ctx& c, const OpDev* op) {
   if (op->ready != nullptr && ld_acquire_sys(op->ready) == 0) return false;
-  return op_finished(a, op->after_op);
+  return op_finished(c, op->after_op);
 }
 
 // Marks as done every tile-less op of the run whose chain of predecessors ends at `finished`
 // (-1: at no op at all) through tile-less ops only.  One thread; called at kernel start and when an
 // op's last tile commits.
-__device__ inline void finish_empty_ops(const RunArgs* a, int finished) {
+__device__ inline void finish_empty_ops(const Ctx& c, int finished) {
+  const RunArgs* a = c.a;
   for (int i = 0; i < a->n_ops; ++i) {
     OpDev* op = &a->ops[a->slots[i]];
     if (op_total_tiles(op, a->fuse_combine) > 0) continue;
@@ -134,7 +144,7 @@ __device__ inline void finish_empty_ops(const RunArgs* a, int finished) {
     for (int hop = 0; dep >= 0 && hop <= kMaxOps && op_total_tiles(&a->ops[a->desc[dep]], a->fuse_combine) == 0; ++hop)
       dep = a->ops[dep].after_op;
     if (dep != finished) continue;
-    atomicExch(&op->run->done, 1);
+    atomicExch(&run_of(c, op)->done, 1);
     if (op->done != nullptr) st_release_sys(op->done, 1u);
     if (op->notify != nullptr) st_release_sys(op->notify, 1u);
   }
@@ -146,8 +156,9 @@ __device__ inline void finish_empty_ops(const RunArgs* a, int finished) {
 // the price is that a ticket can land just past an op boundary, in an op that is not ready
 // yet -- the caller then waits for it (bounded), holding only tickets whose predecessors in
 // the queue are all claimed already.
-__device__ inline int try_claim(const RunArgs* a, QueueTables* sc, RunHead* rh, int cls, unsigned h,
+__device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int cls, unsigned h,
                                 int lane, TileInfo& ti, bool& need_ready) {
+  const RunArgs* a = c.a;
   const int n = sc->n_cls[cls];
   if (n == 0) return 0;
   const unsigned total = sc->cum[cls][n];
@@ -162,11 +173,11 @@ __device__ inline int try_claim(const RunArgs* a, QueueTables* sc, RunHead* rh, 
   // sleep, and words such as an op's done flag or the GEMM counter change between one lane's load and the next's.
   int takeable = 1;
   if (lane == 0) {
-    if (!sc->cls_free[cls][i] && !op_ready(a, op)) takeable = 0;
+    if (!sc->cls_free[cls][i] && !op_ready(c, op)) takeable = 0;
     // The head stands at the op's combine entries while GEMM entries they depend on are still running
     // (other units hold them; for a paired prefill op, the decode list's carrier tiles): nothing to take here
     // yet -- the caller turns to the other class instead of holding a combine ticket it cannot run.
-    else if (base >= (unsigned)op->plan->n_gemm_tiles && ld_acquire(&op->run->gemm_done) < op_gemm_tiles(op)) takeable = 0;
+    else if (base >= (unsigned)op->plan->n_gemm_tiles && ld_acquire(&run_of(c, op)->gemm_done) < op_gemm_tiles(op)) takeable = 0;
   }
   if (__shfl_sync(0xffffffffu, takeable, 0) == 0) return -1;
   // the 32 entries from the head on are fetched while the fetch-add is in flight
@@ -234,9 +245,9 @@ __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int
   if (ab != 0) return 0;
   const int first = ((int)blockIdx.x < q) ? MOE_CLASS_DECODE : MOE_CLASS_PREFILL;
   need_ready = false;
-  const int r1 = try_claim(a, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready);
+  const int r1 = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready);
   int r2 = 0;
-  if (r1 != 1) r2 = try_claim(a, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready);
+  if (r1 != 1) r2 = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready);
   if (r1 == 1 || r2 == 1) {
     ti.t_claim = gtime_ns();
     return 1;
@@ -252,7 +263,7 @@ __device__ inline bool wait_op_ready(const Ctx& c, int lane, const TileInfo& ti)
   while (true) {
     int r = 0;                                   // 1: ready, -1: give up
     if (lane == 0) {
-      if (op_ready(a, &a->ops[ti.slot])) r = 1;
+      if (op_ready(c, &a->ops[ti.slot])) r = 1;
       else if (aborted(c)) r = -1;
       else if ((long long)(gtime_ns() - w0) > a->wait_ns) {
         report(c.st, MOE_ETIMEOUT, 11, (int)blockIdx.x, slot_of(a, ti.slot), ti.tile);
@@ -314,15 +325,17 @@ __device__ inline void claim_next(const Ctx& c, QueueTables* sc, RunHead* rh, in
 }
 
 // one committed entry counted for `op` (descriptor `desc`): counters, notify word, completion
-__device__ inline void count_commit(const RunArgs* a, OpDev* op, int desc, bool gemm) {
-  if (gemm) atomicAdd(&op->run->gemm_done, 1);
-  const int done = atomicAdd(&op->run->tiles_done, 1) + 1;
+__device__ inline void count_commit(const Ctx& c, OpDev* op, int desc, bool gemm) {
+  const RunArgs* a = c.a;
+  RunState* run = run_of(c, op);
+  if (gemm) atomicAdd(&run->gemm_done, 1);
+  const int done = atomicAdd(&run->tiles_done, 1) + 1;
   if (op->notify != nullptr && done == op->notify_after) st_release_sys(op->notify, 1u);
   if (done == op_total_tiles(op, a->fuse_combine)) {
     __threadfence();
-    atomicExch(&op->run->done, 1);
+    atomicExch(&run->done, 1);
     if (op->done != nullptr) st_release_sys(op->done, 1u);
-    finish_empty_ops(a, slot_of(a, desc));
+    finish_empty_ops(c, slot_of(a, desc));
   }
 }
 
@@ -334,10 +347,10 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
   __threadfence();
   fence_async_proxy();
   const unsigned long long t_commit = a->log_cap > 0 ? gtime_ns() : 0ull;   // before it is published
-  if (ti.kind == kGateUp || ti.kind == kGateUpDirect) atomicAdd(&op->g1_done[ti.m], 1);
-  count_commit(a, op, ti.slot, ti.kind != kCombine);
+  if (ti.kind == kGateUp || ti.kind == kGateUpDirect) atomicAdd(&g1_done_of(c, op)[ti.m], 1);
+  count_commit(c, op, ti.slot, ti.kind != kCombine);
   // a GEMM entry of a paired decode op carries rows of the prefill op too: it counts for both
-  if (op->paired && op->cls == MOE_CLASS_DECODE && ti.kind != kCombine) count_commit(a, &a->ops[op->partner], op->partner, true);
+  if (op->paired && op->cls == MOE_CLASS_DECODE && ti.kind != kCombine) count_commit(c, &a->ops[op->partner], op->partner, true);
   if (a->log_cap > 0) {
     const unsigned idx = atomicAdd(&rh->log_count, 1u);
     if (idx < (unsigned)a->log_cap) {
@@ -357,18 +370,44 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
   }
 }
 
-__device__ inline void build_queues(const RunArgs* a, QueueTables* sc) {
-  sc->n_cls[0] = sc->n_cls[1] = 0;
-  sc->cum[0][0] = sc->cum[1][0] = 0;
-  for (int i = 0; i < a->n_ops; ++i) {
-    const int slot = a->slots[i];
-    const OpDev* op = &a->ops[slot];
-    const int cls = op->cls;
-    const int j = sc->n_cls[cls]++;
-    sc->cls_slot[cls][j] = slot;
-    sc->cls_free[cls][j] = (op->ready == nullptr && op->after_op < 0) ? 1 : 0;
-    sc->cum[cls][j + 1] = sc->cum[cls][j] + (unsigned)op_queue_entries(op, a->fuse_combine);
+// The per-class queue tables, built by one warp: lane i reads the plan of op i, so that the loads of all ops overlap.
+__device__ inline void build_queues(const RunArgs* a, QueueTables* sc, int lane) {
+  int entries = 0, cls = 0;
+  if (lane < a->n_ops) {
+    const PlanState ps = *a->plan[lane];
+    cls = a->cls[lane];
+    entries = ps.planned == 0 ? 0 : ps.n_gemm_tiles + (a->fuse_combine ? ps.n_comb_tiles : 0);
   }
+  if (lane == 0) {
+    sc->n_cls[0] = sc->n_cls[1] = 0;
+    sc->cum[0][0] = sc->cum[1][0] = 0;
+  }
+  for (int i = 0; i < a->n_ops; ++i) {
+    const int ei = __shfl_sync(0xffffffffu, entries, i), ci = __shfl_sync(0xffffffffu, cls, i);
+    if (lane == 0) {
+      const int j = sc->n_cls[ci]++;
+      sc->cls_slot[ci][j] = a->slots[i];
+      sc->cls_free[ci][j] = a->free_op[i];
+      sc->cum[ci][j + 1] = sc->cum[ci][j] + (unsigned)ei;
+    }
+  }
+}
+
+// Start of a claiming unit, one thread: which half of the run state is this launch's.  The last of the grid's `units` units to
+// ask passes the state on to the next launch.
+__device__ inline unsigned begin_unit(const RunArgs* a, int units) {
+  const unsigned off = (ld_volatile(reinterpret_cast<const int*>(&a->g->launches)) & 1) ? a->run_bytes : 0u;
+  __threadfence();
+  if (atomicAdd(&a->g->started, 1u) == (unsigned)units - 1u) {
+    a->g->started = 0;
+    atomicAdd(&a->g->launches, 1u);
+  }
+  return off;
+}
+// One warp of the grid: zeroes the other half, which the launch before this one left behind.
+__device__ inline void clear_next_run(const RunArgs* a, RunHead* first_half, unsigned run_off, int lane) {
+  int4* p = reinterpret_cast<int4*>(reinterpret_cast<char*>(first_half) + (run_off ? 0u : a->run_bytes));
+  for (unsigned i = lane; i < a->run_bytes / 16; i += 32) p[i] = make_int4(0, 0, 0, 0);
 }
 
 // silu(g) * u through the hardware tanh approximation (one special-function op per element;

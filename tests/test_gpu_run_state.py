@@ -1,0 +1,51 @@
+"""Launches hand the run state on from one to the next: each works on one half of it and clears the other.  Whatever a launch did
+-- all slots, one slot, a wait that ran out, a plain launch -- the next one starts from zero, also without a host synchronisation."""
+import pytest
+import torch
+
+import paper_2607_18002_b200 as moe
+from workloads import synth
+
+from gpu_util import bind_ops, make_ctx, weights_to
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,n_ctas", [("bf16", 0), ("bf16", 3), ("fp8", 0)], ids=["pairs", "single", "fp8"])
+def test_every_kind_of_launch_leaves_a_clean_state(dtype, n_ctas):
+    spec = synth.Spec("state", synth.Shape(8, 2, 512, 256, dtype), ((synth.PREFILL, 300), (synth.DECODE, 37)), "zipf", 1.0, 1.0, -1.0, 71)
+    W = weights_to(synth.make_weights(spec))
+    ctx = make_ctx(spec, n_ctas=n_ctas, wait_limit_us=20000, tile_log_entries=1 << 12)
+    bound = bind_ops(ctx, synth.make_ops(spec), W)
+    for s, b in enumerate(bound):
+        ctx.plan(s, b)
+    n = [ctx.footprint(s)[1] for s in range(2)]
+    ctx.run([0, 1], fuse_combine=True)
+    ctx.check()
+    want = [b.y.clone() for b in bound]
+    assert len(ctx.tile_log()) == sum(n)
+    word = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for step in ("both", "one", "late", "both", "both", "one"):
+        for b in bound:
+            b.y.zero_()
+        if step == "late":                       # a ready word that nothing sets: the wait runs out, tiles stay unserved
+            bound[1].c.ready = word.data_ptr()
+            ctx.plan(1, bound[1])
+            ctx.run([0, 1], fuse_combine=True)
+            torch.cuda.synchronize()
+            assert ctx.status()[0] == moe.MOE_ETIMEOUT
+            bound[1].c.ready = None
+            ctx.plan(1, bound[1])
+            continue
+        slots = [0, 1] if step == "both" else [0]
+        for _ in range(3):                       # back to back, nothing waits in between
+            ctx.run(slots, fuse_combine=True)
+        ctx.check()
+        assert len(ctx.tile_log()) == sum(n[s] for s in slots)
+        for s in slots:
+            assert torch.equal(bound[s].y, want[s]), (step, s)
+    if ctx.ctas_per_tile == 2 and dtype == "bf16":
+        ctx.run_plain(0)
+        ctx.run([0, 1], fuse_combine=True)
+        ctx.check()
+        assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
