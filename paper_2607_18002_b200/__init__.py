@@ -122,6 +122,10 @@ def _check(rc: int, where: str) -> None:
 
 
 # ------------------------------------------------------------------ the C entry points
+# The argument types declared in lib() turn ints into pointers; the calls of a layer's step (plan, run, route, budget) hand
+# them over as they are, because every object made here shows in a step of a small batch.
+
+_slot_arrays = {}                  # number of ops -> ctypes array type
 
 def moe_workspace_bytes(cfg: moe_config_t) -> int:
     out = C.c_size_t()
@@ -141,18 +145,25 @@ def moe_destroy(ctx: int) -> None:
 
 
 def moe_plan(ctx: int, slot: int, op: moe_op_t, stream: int) -> None:
-    _check(lib().moe_plan(C.c_void_p(ctx), slot, C.byref(op), C.c_void_p(stream)), "moe_plan")
+    rc = (_lib or lib()).moe_plan(ctx, slot, C.byref(op), stream)
+    if rc:
+        raise MoeError(rc, "moe_plan")
 
 
 def moe_run(ctx: int, slots: Sequence[int], fuse_combine: bool, stream: int) -> None:
-    arr = (C.c_int32 * len(slots))(*slots)
-    _check(lib().moe_run(C.c_void_p(ctx), arr, len(slots), int(bool(fuse_combine)),
-                         C.c_void_p(stream)), "moe_run")
+    n = len(slots)
+    array = _slot_arrays.get(n)
+    if array is None:
+        array = _slot_arrays[n] = C.c_int32 * n
+    rc = (_lib or lib()).moe_run(ctx, array(*slots), n, 1 if fuse_combine else 0, stream)
+    if rc:
+        raise MoeError(rc, "moe_run")
 
 
 def moe_plan_pair(ctx: int, slot_prefill: int, slot_decode: int, carrier_rows: int, stream: int) -> None:
-    _check(lib().moe_plan_pair(C.c_void_p(ctx), slot_prefill, slot_decode, carrier_rows, C.c_void_p(stream)),
-           "moe_plan_pair")
+    rc = (_lib or lib()).moe_plan_pair(ctx, slot_prefill, slot_decode, carrier_rows, stream)
+    if rc:
+        raise MoeError(rc, "moe_plan_pair")
 
 
 def moe_run_plain(ctx: int, slot: int, stream: int) -> None:
@@ -164,8 +175,9 @@ def moe_combine(ctx: int, slot: int, stream: int) -> None:
 
 
 def moe_set_budget(ctx: int, decode_sms: int, stream: int) -> None:
-    _check(lib().moe_set_budget(C.c_void_p(ctx), int(decode_sms), C.c_void_p(stream)),
-           "moe_set_budget")
+    rc = (_lib or lib()).moe_set_budget(ctx, int(decode_sms), stream)
+    if rc:
+        raise MoeError(rc, "moe_set_budget")
 
 
 def moe_set_budget_scaled(ctx: int, slot: int, q: int, x_moe_star: float, q_max: int, stream: int) -> None:
@@ -221,8 +233,9 @@ def moe_plan_static(topk_ids_ptr: int, n_tokens: int, top_k: int, n_experts: int
 
 def moe_route(logits_ptr: int, n_tokens: int, n_experts: int, top_k: int, ids_ptr: int, w_ptr: int,
               stream: int) -> None:
-    _check(lib().moe_route(C.c_void_p(logits_ptr), int(n_tokens), int(n_experts), int(top_k),
-                           C.c_void_p(ids_ptr), C.c_void_p(w_ptr), C.c_void_p(stream)), "moe_route")
+    rc = (_lib or lib()).moe_route(logits_ptr, n_tokens, n_experts, top_k, ids_ptr, w_ptr, stream)
+    if rc:
+        raise MoeError(rc, "moe_route")
 
 
 def route(logits, top_k: int, stream=None):
@@ -256,14 +269,13 @@ class BoundOp:
     """A moe_op_t plus the tensors it points to (kept alive) and its plan outputs."""
 
     def __init__(self, c_op: moe_op_t, keep: dict):
+        self.__dict__.update(keep)       # plain attributes: op.y, op.topk_ids, ...
         self.c = c_op
-        self.t = keep
 
-    def __getattr__(self, name):
-        try:
-            return self.__dict__["t"][name]
-        except KeyError:
-            raise AttributeError(name)
+    @property
+    def t(self) -> dict:
+        """All of them by name."""
+        return self.__dict__
 
 
 def bind_op(cls: int, x, topk_ids, topk_w, w_gate_up, w_down, top_k: int, n_experts: int,
@@ -307,6 +319,9 @@ def bind_masked_op(cls: int, x_slabs, counts, w_gate_up, w_down, x_scale=None, s
     return BoundOp(c_op, keep)
 
 
+_get_device = _raw_stream = None   # torch's own, set by the first Context
+
+
 class Context:
     """Owns the device workspace (a torch uint8 tensor) and the library context."""
 
@@ -317,6 +332,8 @@ class Context:
         import torch
         if not torch.cuda.is_available():
             raise RuntimeError("no CUDA device: this library has no CPU path")
+        global _get_device, _raw_stream
+        _get_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
         lib()
         self.cfg = moe_config_t(n_experts, top_k, hidden, inter, dtype, max_tokens_per_op,
                                 max_ops, wait_limit_us, tile_log_entries, n_ctas)
@@ -339,9 +356,10 @@ class Context:
 
     @staticmethod
     def _stream(stream) -> int:
-        import torch
-        s = torch.cuda.current_stream() if stream is None else stream
-        return int(s.cuda_stream)
+        if stream is not None:
+            return int(stream.cuda_stream)
+        # the handle of the current stream of the current device, without a Stream object around it
+        return _raw_stream(_get_device())
 
     def bind(self, cls, x, topk_ids, topk_w, w_gate_up, w_down, **kw) -> BoundOp:
         return bind_op(cls, x, topk_ids, topk_w, w_gate_up, w_down, self.cfg.top_k,
