@@ -33,8 +33,14 @@ __device__ __forceinline__ void combine_add4(float (&acc)[8], const uint4 (&d)[4
 
 __device__ __forceinline__ int f2s_entry(const OpDev* op, int i) { return op->comb_index[i]; }
 
-__device__ __noinline__ inline void combine_tokens(const OpDev* op, int t0, int t1, int k, int H, int tid,
-                                                   int nthr) {
+// ready: called by every thread once, after the permutation entries and router weights of its first token have been read and before any
+// expert output is; false gives up.  (The combine tiles of the persistent kernel wait there for the op's last GEMM tiles, with
+// those loads already behind them.)
+struct CombineNow {
+  __device__ __forceinline__ bool operator()() const { return true; }
+};
+template <class Ready>
+__device__ __noinline__ bool combine_tokens(const OpDev* op, int t0, int t1, int k, int H, int tid, int nthr, Ready ready) {
   const unsigned n_rows = (unsigned)op->space_rows;    // rows of the packed space D lives in
   // every permutation entry of these tokens is checked once, ahead of the loops that use them
   for (int i = t0 * k + tid; i < t1 * k; i += nthr)
@@ -49,24 +55,28 @@ __device__ __noinline__ inline void combine_tokens(const OpDev* op, int t0, int 
     int L = 16;
     while (2 * L * (t1 - t0) <= nthr && vec_per_row % (2 * L) == 0) L *= 2;
     const int tpp = nthr / L;                 // tokens per pass
-    const int sub = tid % L, trow = tid / L;
-    if (trow >= tpp) return;
+    const int sub = tid % L, trow = tid / L;      // nthr is a multiple of L: every thread has a group
     const int nslice = vec_per_row / L;
-    for (int t = t0 + trow; t < t1; t += tpp) {
-      // row offsets in 16-byte units (moe_create rejects shapes whose D buffer exceeds 2^32 units)
-      unsigned off[8];
-      float wj[8];
+    // row offsets in 16-byte units (moe_create rejects shapes whose D buffer exceeds 2^32 units)
+    unsigned off[8];
+    float wj[8];
+    const auto read_slots = [&](int t) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         off[i] = 0u;
         wj[i] = 0.f;
-        if (i < k) {
+        if (i < k && t < t1) {
           const unsigned p = (unsigned)f2s[(size_t)t * k + i];
           const bool ok = p < n_rows;                      // reported by the check above; adds nothing
           off[i] = ok ? p * (unsigned)vec_per_row : 0u;
           wj[i] = ok ? w[(size_t)t * k + i] : 0.f;
         }
       }
+    };
+    read_slots(t0 + trow);
+    if (!ready()) return false;
+    for (int t = t0 + trow; t < t1; t += tpp) {
+      if (t > t0 + trow) read_slots(t);
       const uint4* src = D + sub;
       uint4* dst = y + (size_t)t * vec_per_row + sub;
       const int na = k < 4 ? k : 4, nb = k - na;          // slots in the two buffers
@@ -100,8 +110,9 @@ __device__ __noinline__ inline void combine_tokens(const OpDev* op, int t0, int 
         dst += L;
       }
     }
-    return;
+    return true;
   }
+  if (!ready()) return false;
   for (int idx = tid; idx < total; idx += nthr) {
     const int t = t0 + idx / vec_per_row, v = idx % vec_per_row;
     float acc[8];
@@ -142,6 +153,7 @@ __device__ __noinline__ inline void combine_tokens(const OpDev* op, int t0, int 
     for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(acc[2 * i], acc[2 * i + 1]);
     y[(size_t)t * vec_per_row + v] = o;
   }
+  return true;
 }
 
 }  // namespace moe

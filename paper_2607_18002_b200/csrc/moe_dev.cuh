@@ -23,6 +23,8 @@ constexpr int kCombineSmallBatch = 1024;   // combine is a latency chain per tok
 constexpr int kPlanChunk = 1024;     // fewest routed rows a block of the plan kernels owns
 constexpr int kLagWork = 16;         // gate/up work tiles listed between an expert's gate/up tiles and its down tiles
 constexpr int kWorkRowsBf16 = 256;   // rows of a work tile: two m-tiles share each weight tile
+constexpr int kWorkRowsMid = 128;    // bf16 on CTA pairs: ops whose experts get at most so many rows (unless a token names an expert
+constexpr int kWorkRowsSmall = 32;   // twice) leave shared memory for a deeper pipeline, see moe_run_pair.cu
 constexpr int kWorkRowsFp8 = 128;    // fp8: the accumulator and both partial buffers fill TMEM
 constexpr int kMaxOps = 16;
 constexpr int kMaxExperts = 1024;
@@ -133,13 +135,13 @@ struct Status {   // first error wins (atomicCAS on code)
 struct Global {
   Status status;
   int budget;             // decode SM budget q (Section 6.4)
-  unsigned launches;      // launches of the run kernels so far: half `launches & 1` of the run state is the next one's
-  unsigned started;       // claiming units of the current launch that have read `launches`
-  int pad[5];
+  unsigned turn;          // bit 31: which half of the run state the next launch works on; below: claiming units of the
+                          // current launch that have asked
+  int pad[6];
 };
 
 // The run state exists twice.  A launch works on one half, which is zero when it starts, and zeroes the other for the
-// next one; the unit that is last to read `launches` advances it.  That keeps a memset (with its gaps 6 us of a 70 us decode pass)
+// next one; the unit that is last to ask turns the halves over.  That keeps a memset (with its gaps 6 us of a 70 us decode pass)
 // off the stream.
 // Start of a half; the per-slot RunState blocks and g1_done arrays follow it.
 struct RunHead {
@@ -161,10 +163,12 @@ struct RunArgs {
   unsigned run_bytes;     // size of one half of the run state
   int n_slots;            // slots of the context; descriptor d >= n_slots is the paired form of slot d - n_slots
   signed char desc[kMaxOps];   // slot -> the descriptor that stands for it in this launch
+  int work_rows;          // rows of the largest work tile of the launch's ops
   int static_kind;        // -1: persistent launch served from the queues.  >= 0: a plain launch, claiming unit u
                           // of the grid runs queue entry u of slots[0] and ends
   int slots[kMaxOps];     // descriptor indices of the launch's ops, in the order given
-  const PlanState* plan[kMaxOps];   // of slots[i]; with the two below all that the queue tables are built from
+  const PlanState* plan[kMaxOps];   // of slots[i]; with the three below all that the queue tables are built from
+  const int4* tile_list[kMaxOps];
   signed char cls[kMaxOps];
   signed char free_op[kMaxOps];     // 1: the op has no ready word and no predecessor
 };

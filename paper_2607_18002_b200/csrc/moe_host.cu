@@ -121,6 +121,7 @@ struct moe_ctx {
   OpDev host_pair[kMaxOps];     // what the device copy of each slot's paired descriptor holds
   bool pair_uploaded[kMaxOps];
   int pair_of[kMaxOps];         // slot paired with this one by moe_plan_pair since both were last planned, or -1
+  int work_rows[kMaxOps];       // rows of a work tile of the slot's plan
   bool ran_paired[kMaxOps];     // the slot's last moe_run used its paired form (moe_combine follows it)
   Global* g() const { return reinterpret_cast<Global*>(ws + L.global_off); }
   RunHead* rh() const { return reinterpret_cast<RunHead*>(ws + L.run_off); }
@@ -359,7 +360,12 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
     ctx->ops[slot] = *op;             // what the device copy of the slot now describes
     ctx->uploaded[slot] = true;
   }
-  const int work_rows = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
+  int work_rows = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
+  if (ctx->pair_kernel) {          // an expert gets at most one row per token or slab row
+    const int most = masked ? op->slab_rows : op->n_tokens;
+    work_rows = most <= kWorkRowsSmall ? kWorkRowsSmall : most <= kWorkRowsMid ? kWorkRowsMid : kWorkRowsBf16;
+  }
+  ctx->work_rows[slot] = work_rows;
   const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, st)
                                 : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, st);
   if (pe != cudaSuccess) {
@@ -417,8 +423,11 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   for (int i = 0; i < n_ops; ++i) {
     const OpDev& h = ctx->ran_paired[slots[i]] ? ctx->host_pair[slots[i]] : ctx->host_ops[slots[i]];
     a.plan[i] = h.plan;
+    a.tile_list[i] = h.tile_list;
     a.cls[i] = (signed char)h.cls;
     a.free_op[i] = h.ready == nullptr && h.after_op < 0 ? 1 : 0;
+    const int rows = ctx->ran_paired[slots[i]] ? kWorkRowsBf16 : ctx->work_rows[slots[i]];
+    a.work_rows = rows > a.work_rows ? rows : a.work_rows;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (ctx->poison) {
@@ -467,8 +476,10 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream) {
   a.static_kind = 0;
   a.run_bytes = (unsigned)ctx->L.run_bytes;
   a.plan[0] = ctx->host_ops[slot].plan;
+  a.tile_list[0] = ctx->host_ops[slot].tile_list;
   a.cls[0] = (signed char)ctx->host_ops[slot].cls;
   a.free_op[0] = 1;
+  a.work_rows = ctx->work_rows[slot];
   if (ps.n_gemm_tiles > 0 && launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, st) != cudaSuccess) return MOE_ECUDA;
   if (ctx->ops[slot].layout == MOE_LAYOUT_GATHERED &&
       launch_combine(ctx->op_dev(slot), ctx->ops[slot].n_tokens, c.top_k, c.hidden, st) != cudaSuccess)
@@ -620,7 +631,7 @@ int moe_read_tile_log(moe_ctx_t* ctx, moe_tile_rec_t* host_out, int max_records,
   Global g;
   RunHead rh;
   if (cudaMemcpy(&g, ctx->g(), sizeof(g), cudaMemcpyDeviceToHost) != cudaSuccess) return MOE_ECUDA;
-  const size_t half = (g.launches & 1) ? 0 : ctx->L.run_bytes;            // the one the last launch worked on
+  const size_t half = (g.turn >> 31) ? 0 : ctx->L.run_bytes;            // the one the last launch worked on
   if (cudaMemcpy(&rh, reinterpret_cast<unsigned char*>(ctx->rh()) + half, sizeof(rh), cudaMemcpyDeviceToHost) != cudaSuccess)
     return MOE_ECUDA;
   int cnt = (int)rh.log_count;

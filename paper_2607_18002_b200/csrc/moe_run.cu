@@ -265,10 +265,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   grid_dep_wait();             // everything above overlaps the kernel before this one
-  if (warp == 0) {
-    build_queues(&args, &sc->qt, lane);
-    if (lane == 0) sc->qt.run_off = begin_unit(&args, (int)gridDim.x);
-  }
+  if (warp == 0) begin_unit(&args, &sc->qt, (int)gridDim.x, lane);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -301,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
     ti.t_claim = 0;
     nx = ti;
-    claim_next(c, &sc->qt, rh, lane, ti, ti_need_ready);
+    claim_next<false>(c, &sc->qt, rh, lane, ti, ti_need_ready);
     while (true) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);      // the claim loops exit warp-uniformly
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
@@ -351,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
           }
           if (++stage == kNS) { stage = 0; ph ^= 1u; }
           if (kb == claim_at)              // claim ahead (never blocks here)
-            have_nx = claim_once(c, &sc->qt, rh, lane, nx, nx_need_ready) == 1;
+            have_nx = claim_once<false>(c, &sc->qt, rh, lane, nx, nx_need_ready) == 1;
           if (have_nx && !nx_published && kb > claim_at && kb >= ti.kblocks - kPublishLead) {
             // Hand the next tile to the other warps before this one's last loads go out, if that
             // takes no waiting: free ring slot, op ready, dependencies already met.
@@ -386,7 +383,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         ti_published = nx_published;
         have_nx = nx_published = false;
       } else {
-        claim_next(c, &sc->qt, rh, lane, ti, ti_need_ready);
+        claim_next<false>(c, &sc->qt, rh, lane, ti, ti_need_ready);
       }
     }
   } else if (warp == 1) {
@@ -604,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       OpDev* op = &args.ops[ti.slot];
       bool ok = true;
       if (ti.kind == kCombine) {
-        combine_tokens(op, ti.row0, ti.row0 + ti.rows, args.k, args.H, etid, 256);
+        combine_tokens(op, ti.row0, ti.row0 + ti.rows, args.k, args.H, etid, 256, CombineNow{});
       } else if (kFp8) {
         ok = epilogue_fp8(c, sc, op, ti, tmem, warp, lane, eph, xph);
       } else {

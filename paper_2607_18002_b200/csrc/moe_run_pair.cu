@@ -9,8 +9,11 @@
 //     alone held a 128-token decode launch at 1.15 GHz (1350 us a pass against 1160 us; a tile there has four rows);
 //   - gate/up tiles take 64 features per CTA, the weight rows interleaved 8 gate / 8 up by one 5-D box, so that an
 //     accumulator fragment holds both factors of a SwiGLU output in one thread; down tiles take 128 features per CTA;
-//   - a stage is 32 KB (16 KB activations + 16 KB weights), six stages deep, and a tile uses
-//     up to 256 of the 512 TMEM columns, so the epilogue of one tile overlaps the MMAs of the next.
+//   - a stage is 16 KB of weights and room for this CTA's half of the tile's rows: six stages for tiles of up to 256 rows, eight
+//     for 128, eleven for 32 (the launch's ops decide).  Where few units have work the rate of a unit is its bytes in
+//     flight over the load latency (one token, 96 tiles on 74 units: 80 -> 73 us a pass with eleven stages for six), and where all
+//     have, more bytes in flight keep HBM busier (128 tokens on 252 experts: 1085 -> 1040 us with eight);
+//   - a tile uses up to 256 of the 512 TMEM columns, so the epilogue of one tile overlaps the MMAs of the next.
 // Roles per CTA (16 warps): leader only -- warp 0 scheduler (claims, waits for dependencies,
 // publishes tile descriptors to both CTAs), warp 1 MMA issuer, warp 2 committer; both CTAs --
 // warp 3 producer (TMA loads of its own half, read from the descriptor ring), warps 4-7 gather,
@@ -28,10 +31,15 @@ namespace pairk {
 
 constexpr int kThreads = 512;
 constexpr int kGatherThreads = 128;
-constexpr int kNS = 6;                                   // pipeline stages
-constexpr int kABytes = 128 * kRowBytes;                 // up to 128 activation rows of this CTA
-constexpr int kBBytes = 128 * kRowBytes;                 // this CTA's 128 weight rows
-constexpr int kSB = kABytes + kBBytes;
+constexpr int kBBytes = 128 * kRowBytes;                 // this CTA's 128 weight rows of a stage
+// the pipeline for work tiles of up to kTileRows rows
+template <int kTileRows>
+struct Ring {
+  static constexpr int kRows = kTileRows / 2;            // activation rows of this CTA
+  static constexpr int kABytes = kRows * kRowBytes;
+  static constexpr int kSB = kABytes + kBBytes;
+  static constexpr int kNS = kTileRows == 256 ? 6 : kTileRows == 128 ? 8 : 11;
+};
 constexpr int kAccCols = 256;
 constexpr int kFullCount = 2 + kGatherThreads + 1;
 // instruction descriptor: D fp32, A/B bf16, K-major, M = 256 over the pair, N = the tile's columns
@@ -39,16 +47,17 @@ constexpr unsigned kIdescM256 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4
 // accumulator columns of a tile (16 is the instruction's step), half of them from each CTA's shared memory
 __device__ __forceinline__ int tile_cols(int rows) { return (rows + 15) & ~15; }
 
+template <int kTileRows>
 struct SharedCtl {
   alignas(16) TileInfo info[kRing];
   // leader's: everything the MMAs of a stage read is in place.  kFullCount arrivals: one expect_tx
   // per producer (TMA bytes of both CTAs), one per gather thread of the leader (completion of its
   // cp.async copies) and one from the other CTA's relay warp (that CTA's gathered rows are in
   // place); on tiles without a gather the leader's producer arrives in their place
-  unsigned long long full[kNS];
-  unsigned long long fullA[kNS];     // second CTA: completion of its own gather threads' copies
-  unsigned long long goA[kNS];       // producer -> gather warps: the stage may be overwritten
-  unsigned long long empty[kNS];     // both (multicast commit): the stage's MMAs retired
+  unsigned long long full[Ring<kTileRows>::kNS];
+  unsigned long long fullA[Ring<kTileRows>::kNS];     // second CTA: completion of its own gather threads' copies
+  unsigned long long goA[Ring<kTileRows>::kNS];       // producer -> gather warps: the stage may be overwritten
+  unsigned long long empty[Ring<kTileRows>::kNS];     // both (multicast commit): the stage's MMAs retired
   unsigned long long tfull[2];       // both (multicast commit): accumulator complete
   unsigned long long tempty[2];      // leader's: accumulator drained by the 16 epilogue warps
   unsigned long long ifull[kRing];   // own: tile descriptor published
@@ -61,7 +70,8 @@ struct SharedCtl {
 };
 static_assert(sizeof(TileInfo) == 48, "descriptor is copied as three 16-byte words");
 
-constexpr size_t kSmemBytes = 1024 + (size_t)kNS * kSB + sizeof(SharedCtl);
+template <int kTileRows>
+constexpr size_t kSmemBytes = 1024 + (size_t)Ring<kTileRows>::kNS * Ring<kTileRows>::kSB + sizeof(SharedCtl<kTileRows>);
 
 // bounded wait that also synchronises with arrivals of the other CTA
 __device__ __noinline__ bool wait_slow(const Ctx& c, void* bar, unsigned parity, int where) {
@@ -163,13 +173,14 @@ __device__ __forceinline__ LoadPlan make_plan(const OpDev* op, const TileInfo& t
 
 // one k-block of loads, executed by the whole producer warp with warp-uniform arguments; one
 // elected lane issues each instruction (the stage is known to be free)
-__device__ __forceinline__ void issue_kblock(SharedCtl* sc, unsigned stages_addr, const LoadPlan& p, int kb,
+template <int kTileRows>
+__device__ __forceinline__ void issue_kblock(SharedCtl<kTileRows>* sc, unsigned stages_addr, const LoadPlan& p, int kb,
                                              unsigned stage, bool leader, unsigned full0_addr) {
-  const unsigned sX = stages_addr + stage * (unsigned)kSB;
+  const unsigned sX = stages_addr + stage * (unsigned)Ring<kTileRows>::kSB;
   const unsigned bar = full0_addr + stage * 8u;            // the leader's full[stage]
   pair_issue_kblock(bar, p.tx, smem_u32(&sc->full[stage]),
                     (leader && !p.g1) ? (unsigned)kGatherThreads + 1u : 0u,   // nobody gathers for this tile
-                    sX + (unsigned)kABytes, p.tmw, kb * kBlockK, p.wblk, p.expert,
+                    sX + (unsigned)Ring<kTileRows>::kABytes, p.tmw, kb * kBlockK, p.wblk, p.expert,
                     sX, p.tma, p.ay, (unsigned)p.a_boxes, (unsigned)p.a_box_rows,
                     smem_u32(&sc->goA[stage]), p.g1 ? 1u : 0u);
 }
@@ -179,8 +190,21 @@ __device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const unsigned*>(&v);
 }
 
+// The epilogue warps' wait inside a combine tile: one thread of the CTA looks at the op's counter, the others meet it at a barrier.
+struct CombineWhenDone {
+  const Ctx* c;
+  const OpDev* op;
+  bool look;
+  __device__ __forceinline__ bool operator()() const {
+    if (look) wait_counter(*c, &run_of(*c, op)->gemm_done, op_gemm_tiles(op), 4);
+    named_barrier(1, 256);
+    return !aborted(*c);
+  }
+};
+
 // the scheduler hands a tile to the roles of both CTAs
-__device__ __forceinline__ void publish(SharedCtl* sc, int islot, const TileInfo& ti) {
+template <int kTileRows>
+__device__ __forceinline__ void publish(SharedCtl<kTileRows>* sc, int islot, const TileInfo& ti) {
   fence_async_proxy();
   sc->info[islot] = ti;
   const unsigned ra = map_to_cta(&sc->info[islot], 1);      // same layout as TileInfo
@@ -193,12 +217,14 @@ __device__ __forceinline__ void publish(SharedCtl* sc, int islot, const TileInfo
   mbar_arrive(&sc->ifull[islot]);
 }
 
+template <int kTileRows>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
+  constexpr int kNS = Ring<kTileRows>::kNS, kSB = Ring<kTileRows>::kSB, kABytes = Ring<kTileRows>::kABytes;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* stages = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  SharedCtl* sc = reinterpret_cast<SharedCtl*>(stages + (size_t)kNS * kSB);
+  SharedCtl<kTileRows>* sc = reinterpret_cast<SharedCtl<kTileRows>*>(stages + (size_t)kNS * kSB);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const bool leader = rank == 0;
@@ -234,16 +260,17 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   grid_dep_wait();             // everything above overlaps the kernel before this one
-  if (warp == 0 && leader) {
-    build_queues(&args, &sc->qt, lane);
-    if (lane == 0) sc->qt.run_off = begin_unit(&args, (int)(gridDim.x >> 1));
-  }
+  if (warp == 0 && leader) begin_unit(&args, &sc->qt, (int)(gridDim.x >> 1), lane);
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();          // the other CTA's barriers exist before anything arrives on them
   tc_fence_after();
   const unsigned tmem = sc->tmem_base;
-  if (leader) {                // the second CTA has no business with the run state
+  if (!leader) {               // the second CTA's epilogue looks at the run state too
+    unsigned off;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(off) : "r"(map_to_cta(&sc->qt.run_off, 0)) : "memory");
+    c.run_off = off;
+  } else {
     c.run_off = sc->qt.run_off;
     if (blockIdx.x == 0 && warp == 2) {
       clear_next_run(&args, rh, c.run_off, lane);
@@ -267,7 +294,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     ti.t_claim = 0;
     const bool plain = args.static_kind >= 0;             // plain launch: this pair runs one given entry
     if (plain) claim_static(&args, (int)(blockIdx.x >> 1), ti);
-    else claim_next(c, &sc->qt, rh, lane, ti, need_ready);
+    else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready);
     while (true) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
@@ -276,7 +303,6 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       int ok = 1;
       if (lane == 0) {
         if (ti.kind == kDown) ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
-        if (ti.kind == kCombine) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op), 4);
         if (!ok) ti.kind = kEnd;
         publish(sc, islot, ti);
       }
@@ -286,10 +312,16 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       // now, the weight stream has usually pushed it out since the plan wrote it.
       if (ti.kind == kGateUp && lane * 32 < ti.rows) prefetch_l2(op->gather_list + ti.row0 + lane * 32);
       if (ti.kind == kEnd || !ok) break;
+      // A combine tile is handed over at once: its epilogue warps read row indices and router weights and then wait for the op's
+      // GEMM tiles themselves.  The next claim waits with them, so that a unit holds one such tile at most.
+      if (ti.kind == kCombine) {
+        if (lane == 0) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op), 4);
+        if (__shfl_sync(0xffffffffu, ok, 0) == 0) break;
+      }
       if (!wwait(c, &sc->taken[islot], iph, 26)) break;
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (plain) ti.kind = kEnd;
-      else claim_next(c, &sc->qt, rh, lane, ti, need_ready);
+      else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready);
     }
   } else if (warp == 3) {
     // ============================================================ producer (both CTAs)
@@ -410,7 +442,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     const int gt = threadIdx.x - 128;
     constexpr int kCpr = kRowBytes / 16;                  // 16-byte chunks per row slice
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // 16 rows per cp.async round
-    constexpr int kPasses = 128 / kRowsPerPass;
+    constexpr int kPasses = Ring<kTileRows>::kRows / kRowsPerPass;
     const int chunk = gt % kCpr, rbase = gt / kCpr;
     int islot = 0;
     unsigned iph = 0, kiter = 0, gmask = 0;
@@ -512,8 +544,9 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       bool ok = true;
       if (ti.kind == kCombine) {
         const int mid = ti.row0 + (ti.rows + 1) / 2;
-        if (leader) combine_tokens(op, ti.row0, mid, args.k, args.H, etid, 256);
-        else combine_tokens(op, mid, ti.row0 + ti.rows, args.k, args.H, etid, 256);
+        const CombineWhenDone ready{&c, op, warp == 8 && lane == 0};
+        ok = combine_tokens(op, leader ? ti.row0 : mid, leader ? mid : ti.row0 + ti.rows, args.k, args.H, etid, 256, ready);
+        if (!ok) break;
       } else {
         const int b = (int)(gcount & 1u);
         ok = wwait(c, &sc->tfull[b], (gcount >> 1) & 1u, 10);
@@ -602,11 +635,10 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);
         }
       }
+      // The warp's stores, before the tile is published: the arrival releases them (across the pair: at cluster scope), the
+      // committer's fence is cumulative over what it acquires here
       __syncwarp();
-      if (lane == 0) {
-        __threadfence();                          // the warp's stores, before the tile is published
-        arrive_at_leader(&sc->done[islot], leader);
-      }
+      if (lane == 0) arrive_at_leader(&sc->done[islot], leader);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
   }
@@ -624,14 +656,26 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
 
 }  // namespace pairk
 
+template <int kTileRows>
+static cudaError_t prepare_one() {
+  return cudaFuncSetAttribute(pairk::moe_apk_pair_kernel<kTileRows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)pairk::kSmemBytes<kTileRows>);
+}
 cudaError_t prepare_pair_kernel() {
-  return cudaFuncSetAttribute(pairk::moe_apk_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)pairk::kSmemBytes);
+  cudaError_t e = prepare_one<kWorkRowsBf16>();
+  if (e == cudaSuccess) e = prepare_one<kWorkRowsMid>();
+  return e == cudaSuccess ? prepare_one<kWorkRowsSmall>() : e;
 }
 
 // n_ctas: the persistent grid, or 2 x the number of queue entries for a plain launch
+template <int kTileRows>
+static cudaError_t launch_one(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
+  return launch_after(pairk::moe_apk_pair_kernel<kTileRows>, n_ctas, pairk::kThreads, pairk::kSmemBytes<kTileRows>, stream, args, rh);
+}
 cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
-  return launch_after(pairk::moe_apk_pair_kernel, n_ctas, pairk::kThreads, pairk::kSmemBytes, stream, args, rh);
+  return args.work_rows <= kWorkRowsSmall ? launch_one<kWorkRowsSmall>(args, rh, n_ctas, stream)
+         : args.work_rows <= kWorkRowsMid ? launch_one<kWorkRowsMid>(args, rh, n_ctas, stream)
+                                          : launch_one<kWorkRowsBf16>(args, rh, n_ctas, stream);
 }
 
 }  // namespace moe

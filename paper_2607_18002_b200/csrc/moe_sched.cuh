@@ -22,6 +22,9 @@ struct QueueTables {
   int n_cls[2];
   int cls_slot[2][kMaxOps];
   int cls_free[2][kMaxOps];        // 1: the op has no ready word and no predecessor
+  unsigned n_gemm[2][kMaxOps];     // GEMM entries of the op's list; the combine entries follow them
+  int all_gemm[2][kMaxOps];        // GEMM entries that must have committed before its combine may run
+  const int4* list[2][kMaxOps];
   unsigned cum[2][kMaxOps + 1];
 };
 
@@ -156,8 +159,9 @@ __device__ inline void finish_empty_ops(const Ctx& c, int finished) {
 // the price is that a ticket can land just past an op boundary, in an op that is not ready
 // yet -- the caller then waits for it (bounded), holding only tickets whose predecessors in
 // the queue are all claimed already.
+// early_combine: also take a combine entry whose GEMM entries are still running.
 __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int cls, unsigned h,
-                                int lane, TileInfo& ti, bool& need_ready) {
+                                int lane, TileInfo& ti, bool& need_ready, bool early_combine = false) {
   const RunArgs* a = c.a;
   const int n = sc->n_cls[cls];
   if (n == 0) return 0;
@@ -177,15 +181,15 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
     // The head stands at the op's combine entries while GEMM entries they depend on are still running
     // (other units hold them; for a paired prefill op, the decode list's carrier tiles): nothing to take here
     // yet -- the caller turns to the other class instead of holding a combine ticket it cannot run.
-    else if (base >= (unsigned)op->plan->n_gemm_tiles && ld_acquire(&run_of(c, op)->gemm_done) < op_gemm_tiles(op)) takeable = 0;
+    else if (!early_combine && base >= sc->n_gemm[cls][i] && ld_acquire(&run_of(c, op)->gemm_done) < sc->all_gemm[cls][i]) takeable = 0;
   }
   if (__shfl_sync(0xffffffffu, takeable, 0) == 0) return -1;
   // the 32 entries from the head on are fetched while the fetch-add is in flight
   const unsigned n_op = sc->cum[cls][i + 1] - sc->cum[cls][i];
   int4 e = make_int4(0, 0, 0, 0);
-  if (base + lane < n_op) e = op->tile_list[base + lane];
   unsigned t = 0;
   if (lane == 0) t = atomicAdd(&rh->heads[cls], 1u);
+  if (base + lane < n_op) e = sc->list[cls][i][base + lane];
   t = __shfl_sync(0xffffffffu, t, 0);
   if (t >= total) return 0;
   need_ready = false;
@@ -207,7 +211,7 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
   got.y = __shfl_sync(0xffffffffu, e.y, hit ? d : 0);
   got.z = __shfl_sync(0xffffffffu, e.z, hit ? d : 0);
   got.w = __shfl_sync(0xffffffffu, e.w, hit ? d : 0);
-  if (!hit) got = op->tile_list[local];
+  if (!hit) got = sc->list[cls][i][local];
   ti.kind = entry_kind(got);
   ti.n = entry_n(got);
   ti.m = entry_m(got);
@@ -225,6 +229,10 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
 // queues exhausted, -1 = something exists but is not ready yet.  The abort word, the budget
 // word and both queue heads are loaded together (one round trip), then at most one
 // fetch-add per class.
+// kEarlyCombine: a unit that finds nothing to run in either class takes a combine entry that has to wait for GEMM entries running
+// elsewhere, so that the wait for the last of them starts with the entry in hand (the caller must then not hold up
+// anything else with it).
+template <bool kEarlyCombine>
 __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int lane, TileInfo& ti,
                                  bool& need_ready) {
   const RunArgs* a = c.a;
@@ -245,9 +253,13 @@ __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int
   if (ab != 0) return 0;
   const int first = ((int)blockIdx.x < q) ? MOE_CLASS_DECODE : MOE_CLASS_PREFILL;
   need_ready = false;
-  const int r1 = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready);
+  int r1 = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready);
   int r2 = 0;
   if (r1 != 1) r2 = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready);
+  if (kEarlyCombine && r1 != 1 && r2 != 1) {
+    if (r1 == -1) r1 = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready, true);
+    if (r1 != 1 && r2 == -1) r2 = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready, true);
+  }
   if (r1 == 1 || r2 == 1) {
     ti.t_claim = gtime_ns();
     return 1;
@@ -300,11 +312,12 @@ __device__ inline void claim_static(const RunArgs* a, int unit, TileInfo& ti) {
 
 // Blocking form: waits (bounded) while an op exists that is not ready.  Returns with
 // ti.kind == kEnd when nothing is left (or the run was aborted).
+template <bool kEarlyCombine>
 __device__ inline void claim_next(const Ctx& c, QueueTables* sc, RunHead* rh, int lane, TileInfo& ti,
                                   bool& need_ready) {
   unsigned long long t0 = 0;
   for (unsigned it = 0;; ++it) {
-    const int r = claim_once(c, sc, rh, lane, ti, need_ready);
+    const int r = claim_once<kEarlyCombine>(c, sc, rh, lane, ti, need_ready);
     if (r == 1) return;
     if (r == 0) break;
     __nanosleep(256);                         // an op exists but is not ready yet
@@ -370,39 +383,41 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
   }
 }
 
-// The per-class queue tables, built by one warp: lane i reads the plan of op i, so that the loads of all ops overlap.
-__device__ inline void build_queues(const RunArgs* a, QueueTables* sc, int lane) {
-  int entries = 0, cls = 0;
+// Start of a claiming unit, one warp: which half of the run state is this launch's, and the per-class queue tables.  Lane i reads
+// the plan of op i, so that the loads of all ops overlap each other and the atomic.  The last of the grid's `units` units to ask
+// turns the halves over for the next launch.
+__device__ inline void begin_unit(const RunArgs* a, QueueTables* sc, int units, int lane) {
+  unsigned turn = 0;
+  if (lane == 0) turn = atomicAdd(&a->g->turn, 1u);
+  PlanState ps{};
+  int cls = 0;
   if (lane < a->n_ops) {
-    const PlanState ps = *a->plan[lane];
+    ps = *a->plan[lane];
     cls = a->cls[lane];
-    entries = ps.planned == 0 ? 0 : ps.n_gemm_tiles + (a->fuse_combine ? ps.n_comb_tiles : 0);
   }
+  const int entries = ps.planned == 0 ? 0 : ps.n_gemm_tiles + (a->fuse_combine ? ps.n_comb_tiles : 0);
+  const int all_gemm = ps.n_gemm_tiles + ps.n_extra_gemm;
   if (lane == 0) {
     sc->n_cls[0] = sc->n_cls[1] = 0;
     sc->cum[0][0] = sc->cum[1][0] = 0;
   }
   for (int i = 0; i < a->n_ops; ++i) {
     const int ei = __shfl_sync(0xffffffffu, entries, i), ci = __shfl_sync(0xffffffffu, cls, i);
+    const int gi = __shfl_sync(0xffffffffu, ps.n_gemm_tiles, i), ai = __shfl_sync(0xffffffffu, all_gemm, i);
     if (lane == 0) {
       const int j = sc->n_cls[ci]++;
       sc->cls_slot[ci][j] = a->slots[i];
       sc->cls_free[ci][j] = a->free_op[i];
       sc->cum[ci][j + 1] = sc->cum[ci][j] + (unsigned)ei;
+      sc->n_gemm[ci][j] = (unsigned)gi;
+      sc->all_gemm[ci][j] = ai;
+      sc->list[ci][j] = a->tile_list[i];
     }
   }
-}
-
-// Start of a claiming unit, one thread: which half of the run state is this launch's.  The last of the grid's `units` units to
-// ask passes the state on to the next launch.
-__device__ inline unsigned begin_unit(const RunArgs* a, int units) {
-  const unsigned off = (ld_volatile(reinterpret_cast<const int*>(&a->g->launches)) & 1) ? a->run_bytes : 0u;
-  __threadfence();
-  if (atomicAdd(&a->g->started, 1u) == (unsigned)units - 1u) {
-    a->g->started = 0;
-    atomicAdd(&a->g->launches, 1u);
+  if (lane == 0) {
+    sc->run_off = (turn >> 31) ? a->run_bytes : 0u;
+    if ((turn & 0x7fffffffu) == (unsigned)units - 1u) atomicExch(&a->g->turn, ~turn & 0x80000000u);
   }
-  return off;
 }
 // One warp of the grid: zeroes the other half, which the launch before this one left behind.
 __device__ inline void clear_next_run(const RunArgs* a, RunHead* first_half, unsigned run_off, int lane) {

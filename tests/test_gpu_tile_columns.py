@@ -49,3 +49,48 @@ def test_every_tile_shape_matches_oracle(layout):
     untouched = np.ones(E * slab, dtype=bool)
     untouched[flat] = False
     assert np.all(y[untouched] == 0.0)
+
+
+@pytest.mark.parametrize("T", [1, 15, 31, 32, 33, 64, 127, 128, 129])
+def test_small_ops_on_their_deeper_pipelines(T):
+    """Ops of up to 32 and up to 128 tokens run with smaller work tiles and more stages.  Tokens may name an expert several times, so
+    an expert can still get more rows than the op has tokens: its rows are then cut into several work tiles."""
+    E, k, H, I = 6, 4, 512, 256
+    spec = synth.Spec("deep", synth.Shape(E, k, H, I), ((synth.DECODE, T),), "uniform", None, 1.0, -1.0, 62)
+    W = synth.make_weights(spec)
+    rng = np.random.default_rng(T)
+    ids = rng.integers(0, E, size=(T, k)).astype(np.int32)
+    ids[: T // 2] = 5                                                # half of the tokens name one expert k times
+    x, _ = synth.make_x(spec, T, 0, 0)
+    op = synth.Op(synth.DECODE, x, ids, rng.random((T, k), dtype=np.float32))
+    ctx = make_ctx(spec)
+    b = bind_ops(ctx, [op], weights_to(W))[0]
+    for fuse in (True, False):
+        b.y.fill_(7.0)
+        ctx.plan(0, b)
+        ctx.run([0], fuse_combine=fuse)
+        if not fuse:
+            ctx.combine(0)
+        ctx.check()
+        assert_close(b.y.float().cpu().numpy(), oracle.forward(oracle_weights(spec, W), x, None, ids, op.w)["y"])
+
+
+@pytest.mark.parametrize("slab", [8, 32, 33, 128, 129])
+def test_masked_slabs_on_the_deeper_pipelines(slab):
+    E, H, I = 6, 512, 256
+    counts = np.array([0, 1, slab // 2, slab - 1, slab, slab], dtype=np.int32)
+    spec = synth.Spec("deepm", synth.Shape(E, 1, H, I), ((synth.DECODE, 1),), "uniform", None, 1.0, -1.0, 63)
+    W = synth.make_weights(spec)
+    x, _ = synth.make_x(spec, E * slab, 0, 0)
+    Wd = weights_to(W)
+    ctx = make_ctx(spec, max_tokens=E * slab)
+    b = moe.bind_masked_op(moe.MOE_CLASS_DECODE, x.view(E, slab, H).cuda(), torch.from_numpy(counts).cuda(), Wd.w_gate_up, Wd.w_down)
+    ctx.plan(0, b)
+    ctx.run([0], fuse_combine=True)
+    ctx.check()
+    rows_e = np.repeat(np.arange(E), counts).astype(np.int32)
+    flat = rows_e * slab + np.concatenate([np.arange(c) for c in counts]).astype(np.int32)
+    y = b.y.float().cpu().numpy().reshape(E * slab, H)
+    assert_close(y[flat], oracle.ffn_rows(oracle_weights(spec, W), x, None, flat, rows_e))
+    y[flat] = 0.0
+    assert np.all(y == 0.0)
