@@ -62,8 +62,12 @@ struct SharedCtl {
 constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + sizeof(SharedCtl);
 
 // ------------------------------------------------------------------ FP8 (e4m3, fp32 block scales)
-// instruction descriptor: D fp32, A/B e4m3, both K-major, M = 128, N = 256
+// instruction descriptors: D fp32, A/B e4m3, both K-major, M = 128 or (tiles of up to 64 rows) 64, N = 256.  With M = 64 the
+// accumulator's rows lie 16 to a TMEM lane quadrant; the instruction takes as long, but half of the multipliers rest: under the
+// 1000 W cap a 48-token decode launch went from 1535 us at 1.16 GHz to 1356 us at 1.42 GHz (2000 prefill tokens: 2511 -> 2342 us).
 constexpr unsigned kIdescF8 = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr unsigned kIdescF8M64 = (1u << 4) | ((256u >> 3) << 17) | ((64u >> 4) << 24);
+__device__ __forceinline__ int quadrant_rows(int rows) { return rows <= 64 ? 16 : 32; }
 
 // One e4m3 tile on the epilogue warps.  Thread = (accumulator row, 64-column slice of each
 // 128-column half); its 128 fp32 accumulators stay in registers (the epilogue warps raise
@@ -76,8 +80,9 @@ __device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl* sc, OpDev*
                                              unsigned& xph) {
   const RunArgs& a = *c.a;
   const int q = warp & 3, ch = (warp - 8) >> 2;
-  const int row = q * 32 + lane;
-  const bool valid = row < ti.rows;
+  const int per_q = quadrant_rows(ti.rows);
+  const int row = q * per_q + lane;
+  const bool valid = lane < per_q && row < ti.rows;
   const bool g1 = ti.kind != kDown;
   const int HB = a.H / 128, IB = a.I / 128;
   const unsigned lane_addr = tmem + ((unsigned)(q * 32) << 16);
@@ -108,7 +113,7 @@ __device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl* sc, OpDev*
     sw0 = op->s_down + ((size_t)ti.expert * HB + 2 * ti.n) * IB;
     sw1 = sw0 + IB;
   }
-  if (q * 32 >= ti.rows) {
+  if (q * per_q >= ti.rows) {
     // No row of the tile lies in this warp's TMEM lane quadrant (both warps of a quadrant see
     // the same q): nothing to read, scale or store.  The warp still takes part in every partial
     // buffer hand-off, so that the barrier counts and phases stay those of a full tile.
@@ -404,6 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         // so every k-block (= one scale block) is multiplied into a FRESH partial buffer, one
         // per 128-column half of the weight tile (each half has a single weight scale), and the
         // epilogue warps scale-and-add it into the fp32 accumulator columns of TMEM.
+        const unsigned idesc8 = rows <= 64 ? kIdescF8M64 : kIdescF8;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->full[stage], ph, 8))) { fail = true; break; }
           if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->fullA[stage], ph, 12))) { fail = true; break; }
@@ -418,7 +424,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
               const unsigned long long ad = umma_desc(sA, kRowBytes);
               const unsigned long long bd = umma_desc(sA + kBOff, kRowBytes);
               // four MMAs of 32 e4m3 elements (32 bytes) each, partial full, stage empty
-              f8_mma_kblock(tmem + (unsigned)(pb * 256), ad, bd, kIdescF8, smem_u32(&sc->pfull[pb]),
+              f8_mma_kblock(tmem + (unsigned)(pb * 256), ad, bd, idesc8, smem_u32(&sc->pfull[pb]),
                             smem_u32(&sc->empty[stage]));
             }
           }
