@@ -16,7 +16,6 @@ constexpr int kTileN1 = 128;         // SwiGLU output columns per gate/up tile (
 constexpr int kTileN2 = 256;         // output columns per down-GEMM tile
 constexpr int kBlockK = 64;          // K elements per pipeline stage (one 128-byte swizzle row of bf16)
 constexpr int kRowBytes = kBlockK * 2;
-constexpr int kStages = 3;           // shared-memory pipeline depth (64 KB per stage)
 constexpr int kCombineTokens = 16;   // tokens per combine tile ...
 constexpr int kCombineTokensSmall = 4;     // ... of an op with at most kCombineSmallBatch tokens (a decode batch): its
 constexpr int kCombineSmallBatch = 1024;   // combine is a latency chain per token, so it is spread over more units
@@ -26,6 +25,7 @@ constexpr int kWorkRowsBf16 = 256;   // rows of a work tile: two m-tiles share e
 constexpr int kWorkRowsMid = 128;    // bf16 on CTA pairs: ops whose experts get at most so many rows (unless a token names an expert
 constexpr int kWorkRowsSmall = 32;   // twice) leave shared memory for a deeper pipeline, see moe_run_pair.cu
 constexpr int kWorkRowsFp8 = 128;    // fp8: the accumulator and both partial buffers fill TMEM
+constexpr int kWorkRowsFp8Small = 64;   // fp8 ops of up to so many tokens: see the small tiles in moe_run.cu
 constexpr int kMaxOps = 16;
 constexpr int kMaxExperts = 1024;
 
@@ -75,8 +75,9 @@ struct __align__(128) OpDev {
   CUtensorMap tm_w2;    // [E*H, I]    box {64, 128} down weights
   CUtensorMap tm_a128;  // [Rmax, I]   box {64, 128}
   CUtensorMap tm_a256;  // [Rmax, I]   box {64, 256}
-  CUtensorMap tm_p1;    // CTA-pair kernel: gate/up weights as [E][I/8][2][8][H], box of 8 x (8 gate + 8 up) rows x 64
-  CUtensorMap tm_p2;    // CTA-pair kernel: down weights as [E][H/16][2][8][I], box of 128 consecutive rows x 64
+  CUtensorMap tm_p1;    // weights as the M operand: gate/up, box of 128 rows x 128 bytes: 64 gate rows and the matching up rows in
+                        // groups of eight (bf16: [E][I/8][gate, up][8][H]; e4m3: [4][2 E I][gate, up][8 every other][H])
+  CUtensorMap tm_p2;    // ... down, as [E][H/16][2][8][I], box of 128 consecutive rows x 128 bytes
   CUtensorMap tm_x8;    // masked layout only: x as [E*slab_rows, H], boxes of 8 / 32 / 128 / 256 rows
   CUtensorMap tm_x32;
   CUtensorMap tm_x128;

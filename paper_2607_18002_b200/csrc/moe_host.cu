@@ -151,18 +151,24 @@ int make_map(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t rows, size
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ECUDA;
 }
 
-// The weights of one GEMM for the CTA-pair kernel, seen as [E][blocks][2][8][cols]: a box is 8 blocks of 2 x 8 rows x 64
-// columns, i.e. 128 rows in one copy.  half_rows: rows between the two halves of a block, blk_rows: between blocks.
-int make_map_pair(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t cols, size_t blocks, size_t half_rows, size_t blk_rows) {
-  const size_t E = ctx->cfg.n_experts, pitch = cols * 2;
-  cuuint64_t dims[5] = {(cuuint64_t)cols, 8, 2, (cuuint64_t)blocks, (cuuint64_t)E};
-  cuuint64_t strides[4] = {(cuuint64_t)pitch, (cuuint64_t)(half_rows * pitch), (cuuint64_t)(blk_rows * pitch),
-                           (cuuint64_t)(blocks * 16 * pitch)};
-  cuuint32_t box[5] = {(cuuint32_t)kBlockK, 8, 2, 8, 1};
-  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  CUresult r = ctx->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+// The weights of one GEMM as the M operand: a 5-D view whose box is 128 rows x 128 bytes in one copy.
+// rows: what one step of dimensions 1..4 moves by, in weight rows.
+int make_map_m(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t cols, const size_t (&size)[4], const size_t (&rows)[4],
+                  const cuuint32_t (&boxes)[4]) {
+  const bool fp8 = ctx->cfg.dtype == MOE_DTYPE_FP8_E4M3;
+  const size_t el = fp8 ? 1 : 2;
+  cuuint64_t dims[5], strides[4];
+  cuuint32_t box[5], estr[5] = {1, 1, 1, 1, 1};
+  dims[0] = cols;
+  box[0] = (cuuint32_t)(kRowBytes / el);
+  for (int i = 0; i < 4; ++i) {
+    dims[i + 1] = size[i];
+    strides[i] = rows[i] * cols * el;
+    box[i + 1] = boxes[i];
+  }
+  CUresult r = ctx->encode(out, fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base),
+                           dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ECUDA;
 }
 
@@ -337,13 +343,17 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
       if (!rc) rc = make_map(ctx, &h.tm_a32, h.A, (size_t)L.max_rows, (size_t)c.inter, 32);
       if (!rc) rc = make_map(ctx, &h.tm_a128, h.A, (size_t)L.max_rows, (size_t)c.inter, 128);
       if (!rc) rc = make_map(ctx, &h.tm_a256, h.A, (size_t)L.max_rows, (size_t)c.inter, 256);
-      if (ctx->pair_kernel) {
-        const size_t H = c.hidden, I = c.inter;
-        if (!rc) rc = make_map_pair(ctx, &h.tm_p1, op->w_gate_up, H, I / 8, I, 8);   // 8 gate rows, the 8 matching up rows, ...
-        if (!rc) rc = make_map_pair(ctx, &h.tm_p2, op->w_down, I, H / 16, 8, 16);
-      } else {
-        if (!rc) rc = make_map(ctx, &h.tm_w1, op->w_gate_up, (size_t)c.n_experts * 2 * c.inter, (size_t)c.hidden, 128);
-        if (!rc) rc = make_map(ctx, &h.tm_w2, op->w_down, (size_t)c.n_experts * c.hidden, (size_t)c.inter, 128);
+      const size_t E = c.n_experts, H = c.hidden, I = c.inter;
+      const bool fp8 = c.dtype == MOE_DTYPE_FP8_E4M3;
+      if (!rc && ctx->pair_kernel)                 // 8 gate rows, the 8 matching up rows, the next 8 gate rows, ...
+        rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, I / 8, E}, {1, I, 8, 2 * I}, {8, 2, 8, 1});
+      if (!rc && fp8)                              // ... of 16 rows: 8 even gate, 8 even up, 8 odd gate, 8 odd up rows
+        rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, 2 * E * I, 4}, {2, I, 1, 16}, {8, 2, 2, 4});
+      if (!rc && (ctx->pair_kernel || fp8))
+        rc = make_map_m(ctx, &h.tm_p2, op->w_down, I, {8, 2, H / 16, E}, {1, 8, 16, H}, {8, 2, 8, 1});
+      if (!ctx->pair_kernel) {
+        if (!rc) rc = make_map(ctx, &h.tm_w1, op->w_gate_up, E * 2 * I, H, 128);
+        if (!rc) rc = make_map(ctx, &h.tm_w2, op->w_down, E * H, I, 128);
       }
       if (masked) {
         const size_t xr = (size_t)c.n_experts * op->slab_rows;
@@ -361,8 +371,10 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
     ctx->uploaded[slot] = true;
   }
   int work_rows = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
-  if (ctx->pair_kernel) {          // an expert gets at most one row per token or slab row
-    const int most = masked ? op->slab_rows : op->n_tokens;
+  const int most = masked ? op->slab_rows : op->n_tokens;       // rows an expert gets unless a token names it twice
+  if (c.dtype == MOE_DTYPE_FP8_E4M3) {
+    if (most <= kWorkRowsFp8Small) work_rows = kWorkRowsFp8Small;
+  } else if (ctx->pair_kernel) {
     work_rows = most <= kWorkRowsSmall ? kWorkRowsSmall : most <= kWorkRowsMid ? kWorkRowsMid : kWorkRowsBf16;
   }
   ctx->work_rows[slot] = work_rows;
@@ -426,7 +438,8 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     a.tile_list[i] = h.tile_list;
     a.cls[i] = (signed char)h.cls;
     a.free_op[i] = h.ready == nullptr && h.after_op < 0 ? 1 : 0;
-    const int rows = ctx->ran_paired[slots[i]] ? kWorkRowsBf16 : ctx->work_rows[slots[i]];
+    const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
+    const int rows = ctx->ran_paired[slots[i]] ? full : ctx->work_rows[slots[i]];
     a.work_rows = rows > a.work_rows ? rows : a.work_rows;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -144,6 +144,15 @@ __device__ __forceinline__ void tc_ld_frag(unsigned taddr, unsigned (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+// 16 TMEM lanes x 16 columns: thread i holds column 4 j + i % 4 of row i / 4 in r[2 j] and of row i / 4 + 8 in r[2 j + 1] (twice
+// the rate of the layout above)
+__device__ __forceinline__ void tc_ld_pairs(unsigned taddr, unsigned (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x128b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+}
 // four 8x8 matrices of 16-bit elements, stored transposed: thread i gives the address of a 16-byte row of matrix i / 8
 __device__ __forceinline__ void st_matrix4_trans(unsigned saddr, unsigned r0, unsigned r1, unsigned r2, unsigned r3) {
   asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared::cta.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
@@ -157,6 +166,9 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 }
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+__device__ __forceinline__ void cp_async_4(unsigned dst_smem, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_smem), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_16(unsigned dst_smem, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
@@ -389,6 +401,55 @@ __device__ __forceinline__ bool pair_mma_kblock(unsigned d_tmem, unsigned long l
       : "memory");
   return ready != 0;
 }
+// two fp32 lanes per instruction, each rounded like the scalar operation
+__device__ __forceinline__ unsigned long long f32x2(float lo, float hi) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ float2 f32x2_parts(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {
+  unsigned long long v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+  return v;
+}
+// One e4m3 k-block of a small tile: both halves of the weight tile as M = 128 operands against the same few token rows, into
+// the columns from d and from d + half on; the commit that frees the stage and (end_of_group) the one that hands the group of partials over.
+__device__ __forceinline__ void f8_small_kblock(unsigned d_tmem, unsigned long long w0desc, unsigned long long w1desc,
+                                                unsigned long long xdesc, unsigned idesc, unsigned half, unsigned pfull_bar, unsigned end_of_group,
+                                                unsigned empty_bar) {
+  asm volatile(
+      "{\n\t.reg .pred e, p0, p1, pg;\n\t.reg .b32 r, d1;\n\t.reg .b64 x1, x2, x3, a1, a2, a3, b1, b2, b3;\n\t"
+      "elect.sync r|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p0, 0, 0;\n\t"
+      "setp.eq.b32 p1, 0, 0;\n\t"
+      "setp.ne.and.b32 pg, %6, 0, e;\n\t"
+      "add.u32 d1, %0, %8;\n\t"
+      "add.u64 x1, %3, 2;\n\tadd.u64 x2, %3, 4;\n\tadd.u64 x3, %3, 6;\n\t"
+      "add.u64 a1, %1, 2;\n\tadd.u64 a2, %1, 4;\n\tadd.u64 a3, %1, 6;\n\t"
+      "add.u64 b1, %2, 2;\n\tadd.u64 b2, %2, 4;\n\tadd.u64 b3, %2, 6;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %3, %4, p0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a1, x1, %4, p1;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a2, x2, %4, p1;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a3, x3, %4, p1;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], %2, %3, %4, p0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b1, x1, %4, p1;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b2, x2, %4, p1;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b3, x3, %4, p1;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n\t"
+      "@pg tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}"
+      ::"r"(d_tmem), "l"(w0desc), "l"(w1desc), "l"(xdesc), "r"(idesc), "r"(pfull_bar), "r"(end_of_group), "r"(empty_bar), "r"(half)
+      : "memory");
+}
 // One e4m3 k-block (128 elements = four 32-element MMAs) into a fresh partial buffer, then the two
 // commits (partial full, stage empty), as one group.  Whole warp, warp-uniform operands; one elected
 // lane issues: instructions issued from a divergent single-lane branch cost about 100 clocks each.
@@ -426,6 +487,28 @@ __device__ __forceinline__ void single_issue_kblock(unsigned bar, unsigned tx, u
       "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%5, %10}], [%0];\n\t}"
       ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wy0),
         "r"(wy1), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(has_a)
+      : "memory");
+}
+// ... with the two halves of the weight tile as boxes of a 5-D map (coordinates 1 and 2 zero), and up to two activation
+// boxes of 32 rows
+__device__ __forceinline__ void single_issue_kblock_5d(unsigned bar, unsigned tx, unsigned sB0, unsigned sB1,
+                                                       const CUtensorMap* tmw, int x, int c3_0, int c3_1, int c4, unsigned sA,
+                                                       const CUtensorMap* tma, int ay, unsigned a_boxes) {
+  asm volatile(
+      "{\n\t.reg .pred e, pa, pa2;\n\t.reg .b32 r, z, sA1, ay1;\n\t"
+      "elect.sync r|e, 0xffffffff;\n\t"
+      "mov.b32 z, 0;\n\t"
+      "setp.ge.and.u32 pa, %12, 1, e;\n\t"
+      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"
+      "add.u32 sA1, %9, 4096;\n\t"
+      "add.s32 ay1, %11, 32;\n\t"
+      "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%4, {%5, z, z, %6, %8}], [%0];\n\t"
+      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%3], [%4, {%5, z, z, %7, %8}], [%0];\n\t"
+      "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%9], [%10, {%5, %11}], [%0];\n\t"
+      "@pa2 cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [sA1], [%10, {%5, ay1}], [%0];\n\t}"
+      ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(c3_0), "r"(c3_1),
+        "r"(c4), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes)
       : "memory");
 }
 }  // namespace moe

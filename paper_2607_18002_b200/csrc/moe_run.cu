@@ -33,25 +33,37 @@
 #include "moe_sched.cuh"
 #include <cuda_fp8.h>
 #include <climits>
+#include <type_traits>
 
 namespace moe {
 
 constexpr int kGatherThreads = 128;                     // 4 gather warps
 constexpr int kThreads = 512;                           // 16 warps, see the role list above
 constexpr int kAHalfBytes = kTileM * kRowBytes;        // 128 activation rows of one k-block
-constexpr int kABytes = 2 * kAHalfBytes;               // up to 256 activation rows per stage
 constexpr int kBHalfBytes = 128 * kRowBytes;           // 128 weight rows of one k-block
 constexpr int kBBytes = 2 * kBHalfBytes;               // 256 weight rows per stage
-constexpr int kStageBytes = kABytes + kBBytes;
-constexpr int kMaxStages = 4;                          // fp8: four 48 KB stages, bf16: three 64 KB stages
+constexpr int kMaxStages = 5;                          // bf16: three 64 KB stages, fp8: four of 48 KB or (small tiles) five of 40 KB
+// registers per thread of the control, gather and epilogue warpgroups (control + gather + 2 x epilogue = 4 x 128)
+constexpr int kRegsControl = 64, kRegsGather = 64, kRegsEpilogue = 192;
+constexpr int kRegsControlSmall = 96, kRegsGatherSmall = 96, kRegsEpilogueSmall = 160;
+// what a launch's tiles need: bf16, e4m3, or e4m3 with small tiles only
+enum Mode : int { kBf16 = 0, kF8 = 1, kF8Small = 2 };
 constexpr int kAccCols = 256;                          // TMEM columns per accumulator
 
+struct F8Big {
+  float amax_x[2][4][32];                          // amax exchange between the two warps of a quadrant
+};
+struct F8Small {
+  alignas(16) unsigned char scale[16][256];        // ring of token scales, one slot per k-block
+  float amax[8][64];                               // per warp and token
+};
+template <int kMode>
 struct SharedCtl {
   unsigned long long full[kMaxStages], fullA[kMaxStages], empty[kMaxStages];
   unsigned long long tfull[2], tempty[2];
   unsigned long long pfull[2], pempty[2];          // fp8: per-k-block partial products, two 256-column buffers
   unsigned long long xbar[4];                      // fp8: amax exchange between the two warps of a quadrant
-  float amax_x[2][4][32];
+  std::conditional_t<kMode == kF8Small, F8Small, F8Big> f8;
   unsigned long long ifull[kRing], iempty[kRing], done[kRing];
   TileInfo info[kRing];
   unsigned tmem_base;
@@ -59,7 +71,16 @@ struct SharedCtl {
   QueueTables qt;
 };
 
-constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + sizeof(SharedCtl);
+template <int kMode>
+struct Ring {
+  static constexpr int kARows = kMode == kBf16 ? 256 : kMode == kF8 ? 128 : kWorkRowsFp8Small;
+  static constexpr int kBOff = kARows * kRowBytes;       // activations first, then the 256 weight rows
+  static constexpr int kSB = kBOff + kBBytes;
+  static constexpr int kNS = kMode == kBf16 ? 3 : kMode == kF8 ? 4 : 5;
+};
+template <int kMode>
+constexpr size_t kSmemBytes = 1024 + (size_t)Ring<kMode>::kNS * Ring<kMode>::kSB + sizeof(SharedCtl<kMode>);
+static_assert(kSmemBytes<kBf16> <= 227 * 1024 && kSmemBytes<kF8> <= 227 * 1024 && kSmemBytes<kF8Small> <= 227 * 1024, "one SM");
 
 // ------------------------------------------------------------------ FP8 (e4m3, fp32 block scales)
 // instruction descriptors: D fp32, A/B e4m3, both K-major, M = 128 or (tiles of up to 64 rows) 64, N = 256.  With M = 64 the
@@ -69,13 +90,176 @@ constexpr unsigned kIdescF8 = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 
 constexpr unsigned kIdescF8M64 = (1u << 4) | ((256u >> 3) << 17) | ((64u >> 4) << 24);
 __device__ __forceinline__ int quadrant_rows(int rows) { return rows <= 64 ? 16 : 32; }
 
+// Small tiles (a launch whose ops have up to 64 tokens each; tiles of up to 64 rows) run with the weight rows as the M operand,
+// twice 128 of them, and the token rows as the N columns: tensor energy for the rows there are, and all eight epilogue warps share
+// the work that a 16-row tile otherwise leaves to the two of one TMEM quadrant (a chain of 1050 clocks per k-block).  The hand-off costs
+// hundreds of clocks whatever it carries, so four (tiles of more than 32 rows: two) k-blocks share one: half of TMEM holds their
+// partials.  The token scales of every k-block are copied by the gather warps into a ring: what the epilogue has not read when
+// a k-block's are written is two groups and the five k-blocks in the stages, of the ring's sixteen.
+// Measured under the power cap (48 tokens, 200 experts of 256): 1245 -> 1108 us a pass at 1.58 -> 1.72 GHz, and
+// 8..10 % on 1 to 64 tokens over 8 to 256 experts.  Beyond 64 rows the scale of every column makes
+// the epilogue longer than that of the tokens-as-M form, and a kernel that holds both forms spills.
+constexpr unsigned kIdescF8M128 = (1u << 4) | ((128u >> 4) << 24);
+__device__ __forceinline__ int small_cols(int rows) { return (rows + 15) & ~15; }
+// columns set aside per k-block and weight half
+__device__ __forceinline__ int small_slot(int rows) { return rows <= 32 ? 32 : 64; }
+// Place of a token among the scales of a k-block: in blocks of 16, ordered so that the four that one thread's fragment
+// needs lie together.
+__device__ __forceinline__ int scale_index(int tok) { return (tok & ~15) | ((tok & 3) << 2) | ((tok >> 2) & 3); }
+
+// One small e4m3 tile on an epilogue warp: weight half r = (warp - 8) / 4, TMEM lanes 32 q .. +31 (gate/up: 16 features, 8 even
+// gate / 8 even up / 8 odd gate / 8 odd up rows; down: 32 features).  A fragment of 16 tokens holds, per token 4 j + lane % 4, rows
+// lane / 4 and lane / 4 + 8 -- the gate and the up value of a feature, or two features -- as one register pair, of lanes 0..15 and of lanes
+// 16..31.  kSlot: columns set aside per k-block and weight half; kseq: k-blocks so far.
+template <int kSlot>
+__device__ __forceinline__ bool epilogue_fp8_small(const Ctx& c, SharedCtl<kF8Small>* sc, OpDev* op, const TileInfo& ti, unsigned tmem,
+                                                   int warp, int lane, unsigned& eph, unsigned& kseq) {
+  constexpr int kGroup = 128 / kSlot, kChunks = kSlot / 16;
+  const RunArgs& a = *c.a;
+  const int q = warp & 3, half = (warp - 8) >> 2;
+  const bool g1 = ti.kind != kDown;
+  const int cols = small_cols(ti.rows);
+  const int HB = a.H / 128, IB = a.I / 128;
+  // weight scales: one per k-block and 128 rows of the matrix
+  const float *sw0, *sw1;
+  if (g1) {
+    sw0 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + ti.n) * HB;
+    sw1 = sw0 + (size_t)IB * HB;
+  } else {
+    sw0 = sw1 = op->s_down + ((size_t)ti.expert * HB + 2 * ti.n + half) * IB;
+  }
+  unsigned long long acc[kChunks][4][2];
+#pragma unroll
+  for (int i = 0; i < kChunks * 8; ++i) acc[i >> 3][(i >> 1) & 3][i & 1] = 0ull;
+  float nw0 = sw0[0], nw1 = sw1[0];                 // the next k-block's weight scales
+  unsigned lo[2][8], hi[2][8];                      // fragments of a chunk; those of the next travel while it is added in
+  unsigned pb = 0;
+  for (int kb0 = 0; kb0 < ti.kblocks; kb0 += kGroup, pb ^= 1u) {
+    const int n = min(kGroup, ti.kblocks - kb0);
+    if (!__all_sync(0xffffffffu, mbar_wait_inline(c, &sc->pfull[pb], (eph >> pb) & 1u, 19))) return false;
+    eph ^= 1u << pb;
+    tc_fence_after();
+    unsigned taddr = tmem + pb * 256u + (unsigned)(half * kSlot) + ((unsigned)(q * 32) << 16);
+    tc_ld_pairs(taddr, lo[0]);
+    tc_ld_pairs(taddr + (16u << 16), hi[0]);
+#pragma unroll 1
+    for (int g = 0; g < n; ++g) {
+      const unsigned long long w = f32x2(nw0, nw1);
+      if (kb0 + g + 1 < ti.kblocks) { nw0 = sw0[kb0 + g + 1]; nw1 = sw1[kb0 + g + 1]; }
+      const float* xs = reinterpret_cast<const float*>(sc->f8.scale[kseq++ & 15u]) + 4 * (lane & 3);
+      float4 nx = *reinterpret_cast<const float4*>(xs);
+#pragma unroll
+      for (int ch = 0; ch < kChunks; ++ch) {
+        if (ch * 16 >= cols) break;
+        const float4 x = nx;
+        tc_wait_ld();
+        const bool more = ch + 1 < kChunks && (ch + 1) * 16 < cols;
+        if (more) {
+          tc_ld_pairs(taddr + (unsigned)((ch + 1) * 16), lo[(ch + 1) & 1]);
+          tc_ld_pairs(taddr + (unsigned)((ch + 1) * 16) + (16u << 16), hi[(ch + 1) & 1]);
+          nx = *reinterpret_cast<const float4*>(xs + (ch + 1) * 16);
+        }
+        const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const unsigned long long sw = mul_f32x2(f32x2(xv[j], xv[j]), w);
+          acc[ch][j][0] = fma_f32x2(f32x2(__uint_as_float(lo[ch & 1][2 * j]), __uint_as_float(lo[ch & 1][2 * j + 1])), sw, acc[ch][j][0]);
+          acc[ch][j][1] = fma_f32x2(f32x2(__uint_as_float(hi[ch & 1][2 * j]), __uint_as_float(hi[ch & 1][2 * j + 1])), sw, acc[ch][j][1]);
+        }
+      }
+      taddr += 2u * kSlot;
+      if (g + 1 < n) {
+        tc_ld_pairs(taddr, lo[0]);
+        tc_ld_pairs(taddr + (16u << 16), hi[0]);
+      }
+    }
+    tc_fence_before();
+    __syncwarp();                                   // every lane's TMEM and scale loads have completed
+    if (lane == 0) mbar_arrive(&sc->pempty[pb]);
+  }
+  unsigned char* scratch = sc->epi_scratch[warp - 8];
+  const unsigned scratch_addr = smem_u32(scratch);
+  // stored row lane % 8 of matrix lane / 8 (8 tokens) is this token: the matrix' columns 2 i, 2 i + 1 are tokens i, i + 4
+  const int row = (lane & ~7) + 4 * (lane & 1) + ((lane & 7) >> 1);
+  if (!g1) {
+    unsigned char* out = reinterpret_cast<unsigned char*>(op->D) + (size_t)ti.row0 * a.H * 2 +
+                         (size_t)(ti.n * kTileN2 + half * 128 + q * 32) * 2;
+#pragma unroll
+    for (int p = 0; p < kChunks / 2; ++p) {
+      if (p * 32 >= ti.rows) break;
+      unsigned o[16];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {                 // matrix j: tokens 8 j .. + 7 of the pass
+        const int ch = 2 * p + (j >> 1), k = 2 * (j & 1);
+        const float2 e0 = f32x2_parts(acc[ch][k][0]), e1 = f32x2_parts(acc[ch][k + 1][0]);
+        const float2 f0 = f32x2_parts(acc[ch][k][1]), f1 = f32x2_parts(acc[ch][k + 1][1]);
+        o[j] = pack_bf16(e0.x, e1.x);
+        o[4 + j] = pack_bf16(e0.y, e1.y);
+        o[8 + j] = pack_bf16(f0.x, f1.x);
+        o[12 + j] = pack_bf16(f0.y, f1.y);
+      }
+      store_features32(scratch, scratch_addr, o, row, out + (size_t)(p * 32) * a.H * 2, (size_t)a.H * 2, ti.rows - p * 32, lane);
+    }
+    return true;
+  }
+  // SwiGLU; per token the largest of this warp's 16 features, then of the tile's 128
+  float* mine = sc->f8.amax[warp - 8];
+#pragma unroll
+  for (int ch = 0; ch < kChunks; ++ch) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 e = f32x2_parts(acc[ch][j][0]), d = f32x2_parts(acc[ch][j][1]);
+      const float v0 = __fdividef(e.x, 1.0f + __expf(-e.x)) * e.y, v1 = __fdividef(d.x, 1.0f + __expf(-d.x)) * d.y;
+      acc[ch][j][0] = f32x2(v0, v1);                // the even and the odd feature
+      float m = fmaxf(fabsf(v0), fabsf(v1));
+#pragma unroll
+      for (int s = 4; s < 32; s <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, s));
+      if (lane < 4) mine[ch * 16 + 4 * j + lane] = m;
+    }
+  }
+  named_barrier(1, 256);                            // the eight warps
+  float inv[kSlot / 32];                            // of tokens lane, lane + 32
+#pragma unroll
+  for (int p = 0; p < kSlot / 32; ++p) {
+    const int tok = 32 * p + lane;
+    float amax = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) amax = fmaxf(amax, sc->f8.amax[w][tok]);
+    inv[p] = amax > 0.f ? 448.0f / amax : 0.0f;
+    if (warp == 8 && tok < ti.rows) op->a_scale[(size_t)(ti.row0 + tok) * IB + ti.n] = amax > 0.f ? amax / 448.0f : 1.0f;
+  }
+  named_barrier(1, 256);                            // read by all: the next tile may write
+  unsigned char* out = reinterpret_cast<unsigned char*>(op->A) + (size_t)ti.row0 * a.I + (size_t)(ti.n * kTileN1 + half * 64 + q * 16);
+#pragma unroll
+  for (int p = 0; p < kSlot / 32; ++p) {
+    unsigned o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      o[j] = 0u;
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {                 // 16-bit elements: the two neighbouring features of a token
+        const int g = 2 * (j & 1) + s;
+        const float2 v = f32x2_parts(acc[2 * p + (j >> 1)][g][0]);
+        const float k = __shfl_sync(0xffffffffu, inv[p], 16 * (j >> 1) + 4 * g + (lane & 3));
+        o[j] |= (unsigned)__nv_cvt_float2_to_fp8x2(make_float2(v.x * k, v.y * k), __NV_SATFINITE, __NV_E4M3) << (16 * s);
+      }
+    }
+    __syncwarp();
+    st_matrix4_trans(scratch_addr + row * 16, o[0], o[1], o[2], o[3]);
+    __syncwarp();
+    const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + lane * 16);
+    if (32 * p + lane < ti.rows) *reinterpret_cast<uint4*>(out + (size_t)(32 * p + lane) * a.I) = v4;
+  }
+  return true;
+}
+
 // One e4m3 tile on the epilogue warps.  Thread = (accumulator row, 64-column slice of each
 // 128-column half); its 128 fp32 accumulators stay in registers (the epilogue warps raise
 // their register allowance for this).  Per k-block and half: partial * (activation scale of
 // the row and k-block * weight scale of the half and k-block) is added in.  Then gate/up
 // tiles apply SwiGLU and re-quantise the 128 outputs of the row to e4m3 with one fp32 scale
 // (amax / 448) -- the one quantisation on the path -- and down tiles store bf16.
-__device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl* sc, OpDev* op, const TileInfo& ti,
+__device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl<kF8>* sc, OpDev* op, const TileInfo& ti,
                                              unsigned tmem, int warp, int lane, unsigned& eph,
                                              unsigned& xph) {
   const RunArgs& a = *c.a;
@@ -167,11 +351,11 @@ __device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl* sc, OpDev*
       amax = fmaxf(amax, fabsf(v));
     }
     // the row's 128 outputs live in two threads (ch = 0, 1): exchange the partial maxima
-    sc->amax_x[ch][q][lane] = amax;
+    sc->f8.amax_x[ch][q][lane] = amax;
     mbar_arrive(&sc->xbar[q]);
     if (!__all_sync(0xffffffffu, mbar_wait_inline(c, &sc->xbar[q], xph, 20))) return false;
     xph ^= 1u;
-    amax = fmaxf(amax, sc->amax_x[ch ^ 1][q][lane]);
+    amax = fmaxf(amax, sc->f8.amax_x[ch ^ 1][q][lane]);
     const float scale = amax > 0.f ? amax / 448.0f : 1.0f;
     const float inv = amax > 0.f ? 448.0f / amax : 0.0f;
     if (valid) {
@@ -209,6 +393,14 @@ __device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl* sc, OpDev*
   return true;
 }
 
+// a warpgroup's registers per thread, of the launch's 128
+template <int kMode, int kRegs, int kRegsSmall>
+__device__ __forceinline__ void take_registers() {
+  constexpr int n = kMode == kF8 ? kRegs : kMode == kF8Small ? kRegsSmall : 128;
+  if constexpr (n < 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(n));
+  else if constexpr (n > 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(n));
+}
+
 // ------------------------------------------------------------------ the persistent kernel
 // which accumulator(s) a tile uses: a tile of up to 128 rows alternates between the two, a
 // tile of up to 256 rows takes both (rows 0..127 -> accumulator 0, rows 128..255 -> 1).
@@ -221,20 +413,17 @@ struct AccUse {
   }
 };
 
-template <bool kFp8>
+template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_constant__ RunArgs args,
                                                               RunHead* rh) {
+  constexpr bool kFp8 = kMode != kBf16, kSmall = kMode == kF8Small;
   constexpr int kKb = kFp8 ? 128 : kBlockK;     // K elements per stage (128 bytes per row either way)
   constexpr int kEl = kFp8 ? 1 : 2;             // bytes per element
-  // fp8 tiles have at most 128 rows: a stage holds 128 activation rows + 256 weight rows
-  constexpr int kNS = kFp8 ? 4 : 3;
-  constexpr int kBOff = kFp8 ? kAHalfBytes : kABytes;
-  constexpr int kSB = kBOff + kBBytes;
+  constexpr int kNS = Ring<kMode>::kNS, kBOff = Ring<kMode>::kBOff, kSB = Ring<kMode>::kSB;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* stages = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  SharedCtl* sc = reinterpret_cast<SharedCtl*>(stages + (size_t)kNS * kSB);
-  static_assert(kNS * kSB == 3 * (kABytes + kBBytes), "ring size");
+  SharedCtl<kMode>* sc = reinterpret_cast<SharedCtl<kMode>*>(stages + (size_t)kNS * kSB);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   Ctx c{&args, &args.g->status, 0u};
 
@@ -284,11 +473,12 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   // The fp8 epilogue keeps 128 fp32 accumulators per thread: the two epilogue warpgroups take
   // registers from the two others (64 + 192 = 2 x 128 per thread pair).  Each role changes its
   // allowance at the top of its own branch, so the compiler can budget the branch by it.
-#define MOE_REGS_DEC() do { if constexpr (kFp8) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;"); } while (0)
-#define MOE_REGS_INC() do { if constexpr (kFp8) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;"); } while (0)
+  const auto control_regs = [] { take_registers<kMode, kRegsControl, kRegsControlSmall>(); };
+  const auto gather_regs = [] { take_registers<kMode, kRegsGather, kRegsGatherSmall>(); };
+  const auto epilogue_regs = [] { take_registers<kMode, kRegsEpilogue, kRegsEpilogueSmall>(); };
 
   if (warp == 0) {
-    MOE_REGS_DEC();
+    control_regs();
     // ============================================================ scheduler + TMA producer
     // The next tile is claimed while the current one is still being loaded (after its
     // kClaimAt-th k-block), so the claim's round trips and the first loads of the next tile
@@ -338,15 +528,21 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         const CUtensorMap* tmw = g1 ? &op->tm_w1 : &op->tm_w2;
         const int wrow0 = g1 ? ti.expert * 2 * args.I + ti.n * kTileN1 : ti.expert * args.H + ti.n * kTileN2;
         const int wrow1 = g1 ? wrow0 + args.I : wrow0 + 128;
-        const int box = ti.rows <= 8 ? 8 : (ti.rows <= 32 ? 32 : (ti.rows <= 128 ? 128 : 256));
+        const int box = ti.rows <= 8 ? 8 : (ti.rows <= 32 || kSmall ? 32 : (ti.rows <= 128 ? 128 : 256));
+        const int boxes = kSmall && ti.rows > 32 ? 2 : 1;
         const CUtensorMap* tma = fromx ? (box == 8 ? &op->tm_x8 : (box == 32 ? &op->tm_x32 : (box == 128 ? &op->tm_x128 : &op->tm_x256)))
                                        : (box == 8 ? &op->tm_a8 : (box == 32 ? &op->tm_a32 : (box == 128 ? &op->tm_a128 : &op->tm_a256)));
-        const unsigned tx = (unsigned)kBBytes + (gathered ? 0u : (unsigned)(box * kRowBytes));
+        const unsigned tx = (unsigned)kBBytes + (gathered ? 0u : (unsigned)(boxes * box * kRowBytes));
         const int claim_at = min(kClaimAt, ti.kblocks - 1);
         bool fail = false;
         for (int kb = 0; kb < ti.kblocks; ++kb) {
           if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->empty[stage], ph ^ 1u, 5))) { fail = true; break; }
-          {
+          if constexpr (kSmall) {
+            const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
+            const int c3 = g1 ? ti.expert * 2 * args.I + ti.n * kTileN1 : ti.n * kTileN2 / 16;
+            single_issue_kblock_5d(smem_u32(&sc->full[stage]), tx, sA + kBOff, sA + kBOff + kBHalfBytes, g1 ? &op->tm_p1 : &op->tm_p2,
+                                   kb * kKb, c3, c3 + (g1 ? 64 : 8), g1 ? 0 : ti.expert, sA, tma, ti.row0, gathered ? 0u : (unsigned)boxes);
+          } else {
             const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
             single_issue_kblock(smem_u32(&sc->full[stage]), tx, sA + kBOff, sA + kBOff + kBHalfBytes, tmw, kb * kKb,
                                 wrow0, wrow1, sA, tma, ti.row0, gathered ? 0u : 1u);
@@ -392,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       }
     }
   } else if (warp == 1) {
-    MOE_REGS_DEC();
+    control_regs();
     // ============================================================ MMA issuer
     int stage = 0, islot = 0;
     unsigned ph = 0, iph = 0, aph[2] = {0, 0}, pph = 0;
@@ -410,10 +606,24 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         // per 128-column half of the weight tile (each half has a single weight scale), and the
         // epilogue warps scale-and-add it into the fp32 accumulator columns of TMEM.
         const unsigned idesc8 = rows <= 64 ? kIdescF8M64 : kIdescF8;
+        const unsigned idesc_small = kIdescF8M128 | ((unsigned)small_cols(rows) >> 3) << 17;
+        const int slot = small_slot(rows), last_of_group = 128 / slot - 1;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->full[stage], ph, 8))) { fail = true; break; }
           if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->fullA[stage], ph, 12))) { fail = true; break; }
-          {
+          if constexpr (kSmall) {
+            const int g = kb & last_of_group, pb = (kb / (last_of_group + 1)) & 1;
+            if (g == 0) {
+              if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->pempty[pb], ((pph >> pb) & 1u) ^ 1u, 18))) { fail = true; break; }
+              pph ^= 1u << pb;
+            }
+            tc_fence_after();
+            fence_async_proxy_smem();
+            const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
+            f8_small_kblock(tmem + (unsigned)(pb * 256 + g * 2 * slot), umma_desc(sA + kBOff, kRowBytes),
+                            umma_desc(sA + kBOff + kBHalfBytes, kRowBytes), umma_desc(sA, kRowBytes), idesc_small, (unsigned)slot,
+                            smem_u32(&sc->pfull[pb]), g == last_of_group || kb + 1 == kblocks ? 1u : 0u, smem_u32(&sc->empty[stage]));
+          } else {
             const int pb = kb & 1;                        // partial buffer of this k-block
             if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->pempty[pb], ((pph >> pb) & 1u) ^ 1u, 18))) { fail = true; break; }
             pph ^= 1u << pb;
@@ -488,7 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
   } else if (warp >= 4 && warp < 4 + kGatherThreads / 32) {
-    MOE_REGS_DEC();
+    gather_regs();
     // ============================================================ gather warps (cp.async)
     // Rows of a gate/up tile are scattered tokens: row r of the tile is token
     // sorted_to_flat[row0 + r] / k.  Adjacent lanes copy one row slice (16 bytes each)
@@ -496,7 +706,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     const int gt = threadIdx.x - 128;
     constexpr int kCpr = kRowBytes / 16;                  // 16-byte chunks per row slice
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // rows covered by one cp.async per thread
-    constexpr int kPasses = (kFp8 ? 128 : 256) / kRowsPerPass;   // fp8 work tiles have at most 128 rows
+    constexpr int kPasses = Ring<kMode>::kARows / kRowsPerPass;
     const int chunk = gt % kCpr, rbase = gt / kCpr;       // rows rbase + kRowsPerPass * j
     int islot = 0;
     unsigned iph = 0, kiter = 0;                          // kiter: k-blocks of all GEMM tiles so far
@@ -510,7 +720,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (kind == kEnd) break;
       if (kind == kCombine) continue;
-      if (kind != kGateUp) {           // nothing to gather: hand every stage on empty-handed
+      if (kind != kGateUp && !kSmall) {   // nothing to gather: hand every stage on empty-handed
         bool failed = false;
         for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
           const int stage = (int)(kiter % kNS);
@@ -528,6 +738,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       const unsigned char* X = static_cast<const unsigned char*>(op->x) + chunk * 16;
       const unsigned char* Xp = static_cast<const unsigned char*>(pop->x) + chunk * 16;
       const size_t pitch = (size_t)args.H * kEl;
+      const int n_gather = kind == kGateUp ? rows : 0;
       int tok[kPasses];
       const int n_rows = op->n_rows, n_rows_p = pop->n_rows;
       const int own_tag = paired ? slot_of(&args, slot) : 0, partner_tag = paired ? slot_of(&args, op->partner) : 0;
@@ -535,24 +746,39 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
 #pragma unroll
       for (int j = 0; j < kPasses; ++j) {
         const int r = rbase + kRowsPerPass * j;
-        const int v = r < rows ? op->gather_list[row0 + r] : 0;
+        const int v = r < n_gather ? op->gather_list[row0 + r] : 0;
         const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
         const bool theirs = tag != own_tag;
         // an index the plan never wrote is reported below and its row is skipped
         const bool in_range = v >= 0 && (tag == own_tag || tag == partner_tag) && flat < (theirs ? n_rows_p : n_rows);
-        bad |= r < rows && !in_range;
-        tok[j] = (r < rows && in_range) ? (theirs ? ~(flat / args.k) : flat / args.k) : INT_MIN;
+        bad |= r < n_gather && !in_range;
+        tok[j] = (r < n_gather && in_range) ? (theirs ? ~(flat / args.k) : flat / args.k) : INT_MIN;
       }
       if (bad) report(c.st, MOE_EBOUNDS, slot_of(&args, slot), row0, rows, 0);
+      // a small e4m3 tile: the scale of token gt of every k-block
+      const float* sx = nullptr;
+      if (kSmall && gt < rows) {
+        if (kind == kGateUp) {
+          const int v = op->gather_list[row0 + gt];
+          const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
+          const OpDev* src = tag != own_tag && tag == partner_tag ? pop : op;
+          const bool in_range = v >= 0 && (tag == own_tag || src != op) && flat < src->n_rows;   // reported above if not
+          sx = src->x_scale + (size_t)(in_range ? flat / args.k : 0) * (args.H / 128);
+        } else {
+          sx = kind == kDown ? op->a_scale + (size_t)(row0 + gt) * (args.I / 128) : op->x_scale + (size_t)(row0 + gt) * (args.H / 128);
+        }
+      }
+      unsigned scale_at = 0;
+      if constexpr (kSmall) scale_at = smem_u32(sc->f8.scale) + (unsigned)scale_index(gt & 63) * 4u;
       bool fail = false;
       for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
         const int stage = (int)(kiter % kNS);
         if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->empty[stage], ((kiter / kNS) & 1u) ^ 1u, 14))) { fail = true; break; }
+        if (kSmall && sx) cp_async_4(scale_at + (kiter & 15u) * 256u, sx + kb);
         const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
         const unsigned char* Xk = X + (size_t)kb * kRowBytes;
         const unsigned char* Xpk = Xp + (size_t)kb * kRowBytes;
-#pragma unroll
-        for (int j = 0; j < kPasses; ++j) {
+        const auto copy_row = [&](int j) {
           const int r = rbase + kRowsPerPass * j;
           // the swizzle XORs the 16-byte chunk index with the row's position in its 8-row group
           const int sw = kRowBytes == 128 ? (r & 7) : ((r >> 1) & 3);
@@ -560,6 +786,11 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
           if (t != INT_MIN)
             cp_async_16(sA + r * kRowBytes + ((chunk ^ sw) << 4),
                         (t >= 0 ? Xk : Xpk) + (size_t)(t >= 0 ? t : ~t) * pitch);
+        };
+        copy_row(0);
+        if (!kSmall || n_gather > kRowsPerPass) {        // most small tiles need one pass
+#pragma unroll
+          for (int j = 1; j < kPasses; ++j) copy_row(j);
         }
         cp_async_arrive_noinc(&sc->fullA[stage]);
       }
@@ -567,7 +798,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     }
     cp_async_wait_all();
   } else if (warp == 2) {
-    MOE_REGS_DEC();
+    control_regs();
     // ============================================================ committer
     // Publishes a tile once all epilogue threads have arrived on the tile's barrier: the
     // barrier orders their stores before this warp's fence and release (cumulativity).
@@ -588,7 +819,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
   } else if (warp >= 8) {
-    MOE_REGS_INC();
+    epilogue_regs();
     // ============================================================ epilogue (8 warps)
     // Warp w may read TMEM lanes 32 (w % 4) .. +31, i.e. accumulator rows of that quadrant.
     // The two warps of a quadrant split the columns of every accumulator the tile used.
@@ -596,7 +827,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     const int half = (warp - 8) >> 2;             // which half of the columns
     const int etid = threadIdx.x - 256;           // 0..255
     int islot = 0;
-    unsigned iph = 0, aph[2] = {0, 0}, eph = 0, xph = 0;
+    unsigned iph = 0, aph[2] = {0, 0}, eph = 0, xph = 0, kseq = 0;
     AccUse accs;
     unsigned char* scratch = sc->epi_scratch[warp - 8];
     const int srow = lane >> 2, schunk = lane & 3;          // this lane's part of a store
@@ -608,7 +839,10 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       bool ok = true;
       if (ti.kind == kCombine) {
         combine_tokens(op, ti.row0, ti.row0 + ti.rows, args.k, args.H, etid, 256, CombineNow{});
-      } else if (kFp8) {
+      } else if constexpr (kSmall) {
+        ok = ti.rows <= 32 ? epilogue_fp8_small<32>(c, sc, op, ti, tmem, warp, lane, eph, kseq)
+                           : epilogue_fp8_small<64>(c, sc, op, ti, tmem, warp, lane, eph, kseq);
+      } else if constexpr (kFp8) {
         ok = epilogue_fp8(c, sc, op, ti, tmem, warp, lane, eph, xph);
       } else {
         bool use[2];
@@ -687,7 +921,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   }
 
   else {
-    MOE_REGS_DEC();        // warp 3: idle, but its warpgroup changes its allowance together
+    control_regs();        // warp 3: idle, but its warpgroup changes its allowance together
   }
 
   // teardown: nothing is claimed any more; let asynchronous work settle, then free TMEM
@@ -700,17 +934,24 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   }
 }
 
+template <int kMode>
+static cudaError_t prepare_mode() {
+  return cudaFuncSetAttribute(moe_apk_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes<kMode>);
+}
 cudaError_t prepare_run_kernel() {
-  cudaError_t e = cudaFuncSetAttribute(moe_apk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kSmemBytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(moe_apk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kSmemBytes);
+  cudaError_t e = prepare_mode<kBf16>();
+  if (e == cudaSuccess) e = prepare_mode<kF8>();
+  return e == cudaSuccess ? prepare_mode<kF8Small>() : e;
 }
 
+template <int kMode>
+static cudaError_t launch_mode(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
+  return launch_after(moe_apk_kernel<kMode>, n_ctas, kThreads, kSmemBytes<kMode>, stream, args, rh);
+}
 cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
-  return launch_after(args.dtype == MOE_DTYPE_FP8_E4M3 ? moe_apk_kernel<true> : moe_apk_kernel<false>, n_ctas, kThreads, kSmemBytes,
-                      stream, args, rh);
+  return args.dtype != MOE_DTYPE_FP8_E4M3            ? launch_mode<kBf16>(args, rh, n_ctas, stream)
+         : args.work_rows <= kWorkRowsFp8Small ? launch_mode<kF8Small>(args, rh, n_ctas, stream)
+                                               : launch_mode<kF8>(args, rh, n_ctas, stream);
 }
 
 }  // namespace moe

@@ -185,11 +185,6 @@ __device__ __forceinline__ void issue_kblock(SharedCtl<kTileRows>* sc, unsigned 
                     smem_u32(&sc->goA[stage]), p.g1 ? 1u : 0u);
 }
 
-__device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const unsigned*>(&v);
-}
-
 // The epilogue warps' wait inside a combine tile: one thread of the CTA looks at the op's counter, the others meet it at a barrier.
 struct CombineWhenDone {
   const Ctx* c;
@@ -598,35 +593,23 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
               tc_ld_frag(taddr + (unsigned)((p + 1) * 32), lo);
               tc_ld_frag(taddr + (unsigned)((p + 1) * 32) + (16u << 16), hi);
             }
-            __syncwarp();                                     // scratch free again
-            // matrix i / 8 of a store is token group i / 8, its row i % 8 is token `lane` of the pass
-            if (g1) {
-#pragma unroll
-              for (int cch = 0; cch < 2; ++cch)
-                st_matrix4_trans(scratch_addr + lane * 32 + cch * 16, o[4 * cch], o[4 * cch + 1], o[4 * cch + 2], o[4 * cch + 3]);
-            } else {
-#pragma unroll
-              for (int cch = 0; cch < 4; ++cch)               // XOR keeps the banks of eight rows apart
-                st_matrix4_trans(scratch_addr + lane * 64 + ((cch ^ ((lane >> 1) & 3)) << 4), o[4 * cch], o[4 * cch + 1],
-                                 o[4 * cch + 2], o[4 * cch + 3]);
-            }
-            __syncwarp();
             unsigned char* dst = out + (size_t)(p * 32) * pitch;
             const int left = live - p * 32;
             if (g1) {
+              __syncwarp();                                   // scratch free again
+              // matrix i / 8 of a store is token group i / 8, its row i % 8 is token `lane` of the pass
+#pragma unroll
+              for (int f = 0; f < 2; ++f)
+                st_matrix4_trans(scratch_addr + lane * 32 + f * 16, o[4 * f], o[4 * f + 1], o[4 * f + 2], o[4 * f + 3]);
+              __syncwarp();
 #pragma unroll
               for (int j = 0; j < 2; ++j) {
-                const int r = 16 * j + (lane >> 1), cch = lane & 1;
-                const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 32 + cch * 16);
-                if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + cch * 16) = v4;
+                const int r = 16 * j + (lane >> 1), f = lane & 1;
+                const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 32 + f * 16);
+                if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + f * 16) = v4;
               }
             } else {
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const int r = 8 * j + (lane >> 2), cch = lane & 3;
-                const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 64 + ((cch ^ ((r >> 1) & 3)) << 4));
-                if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + cch * 16) = v4;
-              }
+              store_features32(scratch, scratch_addr, o, lane, dst, pitch, left, lane);
             }
           }
         } else {

@@ -434,4 +434,26 @@ __device__ __forceinline__ float silu_mul(float g, float u) {
   return fmaf(hg, t, hg) * u;                     // g * sigmoid(g) = g/2 * (1 + tanh(g/2))
 }
 
+__device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const unsigned*>(&v);
+}
+
+// Stores 32 tokens x 32 features of bf16 through the warp's scratch: o[4 f + j] is the 8x8 matrix of feature group f and token group
+// j; stored row i % 8 of group i / 8 is token `row` (of lane i).
+__device__ __forceinline__ void store_features32(unsigned char* scratch, unsigned scratch_addr, const unsigned (&o)[16], int row,
+                                                 unsigned char* dst, size_t pitch, int left, int lane) {
+  __syncwarp();                                     // scratch free again
+#pragma unroll
+  for (int f = 0; f < 4; ++f)                       // XOR keeps the banks of eight rows apart
+    st_matrix4_trans(scratch_addr + row * 64 + ((f ^ ((row >> 1) & 3)) << 4), o[4 * f], o[4 * f + 1], o[4 * f + 2], o[4 * f + 3]);
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int r = 8 * j + (lane >> 2), f = lane & 3;
+    const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 64 + ((f ^ ((r >> 1) & 3)) << 4));
+    if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + f * 16) = v4;
+  }
+}
+
 }  // namespace moe

@@ -197,3 +197,40 @@ def test_c5_full_size_sampled():
         print(f"c5 cls={op.cls} tokens={len(toks)} rel_l2={rel:.3e} share outside the stated bound={miss:.4f}")
         assert miss <= C5_STATED_BOUND_MISS_MAX
         assert torch.isfinite(b.y.float()).all()
+
+
+@pytest.mark.parametrize("T,slab", [(t, 0) for t in (1, 15, 16, 17, 31, 32, 33, 48, 63, 64, 65)] + [(0, s) for s in (8, 33, 64, 65)])
+def test_fp8_small_launches(T, slab):
+    """Launches whose ops have up to 64 rows an expert run with the weights as the M operand; columns go in steps of 16, partials
+    are grouped by four or two k-blocks.  T tokens, a third of which name one expert four times (more rows than a tile holds), or
+    masked slabs of empty, partly filled and full experts."""
+    E, k = 6, 4 if T else 1
+    spec = synth.Spec("small8", synth.Shape(E, k, 768, 640, "fp8"), ((synth.DECODE, T or 1),), "uniform", None, 1.0, -1.0, 81)
+    W = synth.make_weights(spec)
+    Wo = oracle_weights(spec, W)
+    if T:
+        rng = np.random.default_rng(T)
+        ids = rng.integers(0, E - 1, size=(T, k)).astype(np.int32)
+        ids[: T // 3] = E - 1
+        x, xs = synth.make_x(spec, T, 0, 0)
+        w = rng.random((T, k), dtype=np.float32)
+        op = synth.Op(synth.DECODE, x, ids, (w / w.sum(axis=1, keepdims=True)).astype(np.float32), xs)
+        b = _run(spec, ops=[op], W=W)[1][0]
+        ref = oracle.forward(Wo, x, xs, ids, op.w, round_A=oracle.ROUND_E4M3_1X128)["y"]
+        y = b.y.float().cpu().numpy()
+    else:
+        counts = np.array([0, 1, slab // 2, slab - 1, slab, slab], dtype=np.int32)
+        x, xs = synth.make_x(spec, E * slab, 0, 0)
+        Wd = weights_to(W)
+        ctx = make_ctx(spec, max_tokens=E * slab)
+        b = moe.bind_masked_op(moe.MOE_CLASS_DECODE, x.view(E, slab, -1).cuda(), torch.from_numpy(counts).cuda(), Wd.w_gate_up, Wd.w_down,
+                               x_scale=xs.view(E, slab, -1).cuda(), s_gate_up=Wd.s_gate_up, s_down=Wd.s_down)
+        ctx.plan(0, b)
+        ctx.run([0], fuse_combine=True)
+        ctx.check()
+        rows_e = np.repeat(np.arange(E), counts).astype(np.int32)
+        flat = rows_e * slab + np.concatenate([np.arange(c) for c in counts]).astype(np.int32)
+        ref = np.zeros((E * slab, spec.shape.H), np.float32)        # rows past an expert's count are zero
+        ref[flat] = oracle.ffn_rows(Wo, x, xs, flat, rows_e, round_A=oracle.ROUND_E4M3_1X128)
+        y = b.y.float().cpu().numpy().reshape(E * slab, -1)
+    assert_close(y, ref, atol=ATOL8, rtol=RTOL8, rel_l2=REL_L2_8)
