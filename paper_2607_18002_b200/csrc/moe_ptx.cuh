@@ -47,6 +47,12 @@ __device__ __forceinline__ bool mbar_test(void* bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
+// L2 policy of bytes that nobody reads a second time
+__device__ __forceinline__ unsigned long long l2_evict_first() {
+  unsigned long long p;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
 __device__ __forceinline__ void tma_tile_2d(void* dst, const CUtensorMap* tm, int x, int y,
                                             void* bar) {
   asm volatile(
@@ -339,37 +345,42 @@ __device__ __forceinline__ void mbar_arrive_n_elect(void* bar, unsigned n) {
 // All loads and barrier arrivals of one k-block by one CTA of a pair, as ONE instruction group under a
 // single election: expect_tx on the leader's stage barrier, the box of 128 weight rows, up to three
 // activation boxes (a_rows rows apart), the stand-in arrivals (tiles without a gather) and the go-ahead for the
-// gather warps.  Flags select what is issued; everything is warp-uniform.
+// gather warps.  Flags select what is issued; everything is warp-uniform.  kEvictFirst: w_policy is the L2 policy of the weights.
+template <bool kEvictFirst>
 __device__ __forceinline__ void pair_issue_kblock(unsigned bar, unsigned tx, unsigned standin_bar, unsigned standin_n,
                                                   unsigned sW, const CUtensorMap* tmw, int x, int wblk, int expert,
                                                   unsigned sX, const CUtensorMap* tma, int ay, unsigned a_boxes, unsigned a_rows,
-                                                  unsigned go_bar, unsigned has_go) {
-  asm volatile(
-      "{\n\t.reg .pred e, pa1, pa2, pa3, pgo, pst;\n\t.reg .b32 r, st, z, sA1, ay1, sA2, ay2;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "setp.ge.and.u32 pa1, %12, 1, e;\n\t"
-      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"
-      "setp.ge.and.u32 pa3, %12, 3, e;\n\t"
-      "setp.ne.and.b32 pgo, %15, 0, e;\n\t"
-      "setp.ne.and.b32 pst, %3, 0, e;\n\t"
-      "mov.b32 z, 0;\n\t"
-      "shl.b32 st, %13, 7;\n\t"
-      "add.u32 sA1, %9, st;\n\t"
-      "add.s32 ay1, %11, %13;\n\t"
-      "add.u32 sA2, sA1, st;\n\t"
-      "add.s32 ay2, ay1, %13;\n\t"
-      "@e mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;\n\t"
-      "@pst mbarrier.arrive.shared::cta.b64 _, [%2], %3;\n\t"
-      "@e cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%4], [%5, {%6, z, z, %7, %8}], [%0];\n\t"
-      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%9], [%10, {%6, %11}], [%0];\n\t"
-      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%10, {%6, ay1}], [%0];\n\t"
-      "@pa3 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA2], [%10, {%6, ay2}], [%0];\n\t"
-      "@pgo mbarrier.arrive.shared::cta.b64 _, [%14];\n\t}"
-      ::"r"(bar), "r"(tx), "r"(standin_bar), "r"(standin_n),
-        "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert),
-        "r"(sX), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "r"(a_rows),
-        "r"(go_bar), "r"(has_go)
-      : "memory");
+                                                  unsigned go_bar, unsigned has_go, unsigned long long w_policy) {
+#define MOE_PAIR_KBLOCK(HINT, POLICY)                                                                                  \
+  asm volatile(                                                                                                        \
+      "{\n\t.reg .pred e, pa1, pa2, pa3, pgo, pst;\n\t.reg .b32 r, st, z, sA1, ay1, sA2, ay2;\n\t"                     \
+      "elect.sync r|e, 0xffffffff;\n\t"                                                                                \
+      "setp.ge.and.u32 pa1, %12, 1, e;\n\t"                                                                            \
+      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"                                                                            \
+      "setp.ge.and.u32 pa3, %12, 3, e;\n\t"                                                                            \
+      "setp.ne.and.b32 pgo, %15, 0, e;\n\t"                                                                            \
+      "setp.ne.and.b32 pst, %3, 0, e;\n\t"                                                                             \
+      "mov.b32 z, 0;\n\t"                                                                                              \
+      "shl.b32 st, %13, 7;\n\t"                                                                                        \
+      "add.u32 sA1, %9, st;\n\t"                                                                                       \
+      "add.s32 ay1, %11, %13;\n\t"                                                                                     \
+      "add.u32 sA2, sA1, st;\n\t"                                                                                      \
+      "add.s32 ay2, ay1, %13;\n\t"                                                                                     \
+      "@e mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;\n\t"                                              \
+      "@pst mbarrier.arrive.shared::cta.b64 _, [%2], %3;\n\t"                                                          \
+      "@e cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes" HINT " [%4], [%5, {%6, z, z, %7, %8}], [%0]" POLICY ";\n\t" \
+      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%9], [%10, {%6, %11}], [%0];\n\t" \
+      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%10, {%6, ay1}], [%0];\n\t" \
+      "@pa3 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA2], [%10, {%6, ay2}], [%0];\n\t" \
+      "@pgo mbarrier.arrive.shared::cta.b64 _, [%14];\n\t}"                                                            \
+      ::"r"(bar), "r"(tx), "r"(standin_bar), "r"(standin_n),                                                           \
+        "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert),                       \
+        "r"(sX), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "r"(a_rows),                   \
+        "r"(go_bar), "r"(has_go), "l"(w_policy)                                                                        \
+      : "memory")
+  if constexpr (kEvictFirst) MOE_PAIR_KBLOCK(".L2::cache_hint", ", %16");
+  else MOE_PAIR_KBLOCK("", "");
+#undef MOE_PAIR_KBLOCK
 }
 
 // One k-block of the pair's MMAs as ONE instruction group: the next stage's barrier is tested first and
@@ -490,10 +501,10 @@ __device__ __forceinline__ void single_issue_kblock(unsigned bar, unsigned tx, u
       : "memory");
 }
 // ... with the two halves of the weight tile as boxes of a 5-D map (coordinates 1 and 2 zero), and up to two activation
-// boxes of 32 rows
+// boxes of 32 rows; w_policy is the L2 policy of the weights
 __device__ __forceinline__ void single_issue_kblock_5d(unsigned bar, unsigned tx, unsigned sB0, unsigned sB1,
                                                        const CUtensorMap* tmw, int x, int c3_0, int c3_1, int c4, unsigned sA,
-                                                       const CUtensorMap* tma, int ay, unsigned a_boxes) {
+                                                       const CUtensorMap* tma, int ay, unsigned a_boxes, unsigned long long w_policy) {
   asm volatile(
       "{\n\t.reg .pred e, pa, pa2;\n\t.reg .b32 r, z, sA1, ay1;\n\t"
       "elect.sync r|e, 0xffffffff;\n\t"
@@ -503,12 +514,12 @@ __device__ __forceinline__ void single_issue_kblock_5d(unsigned bar, unsigned tx
       "add.u32 sA1, %9, 4096;\n\t"
       "add.s32 ay1, %11, 32;\n\t"
       "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
-      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%4, {%5, z, z, %6, %8}], [%0];\n\t"
-      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%3], [%4, {%5, z, z, %7, %8}], [%0];\n\t"
+      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%2], [%4, {%5, z, z, %6, %8}], [%0], %13;\n\t"
+      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%3], [%4, {%5, z, z, %7, %8}], [%0], %13;\n\t"
       "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%9], [%10, {%5, %11}], [%0];\n\t"
       "@pa2 cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [sA1], [%10, {%5, ay1}], [%0];\n\t}"
       ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(c3_0), "r"(c3_1),
-        "r"(c4), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes)
+        "r"(c4), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "l"(w_policy)
       : "memory");
 }
 }  // namespace moe

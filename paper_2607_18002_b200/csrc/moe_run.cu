@@ -97,8 +97,9 @@ __device__ __forceinline__ int quadrant_rows(int rows) { return rows <= 64 ? 16 
 // partials.  The token scales of every k-block are copied by the gather warps into a ring: what the epilogue has not read when
 // a k-block's are written is two groups and the five k-blocks in the stages, of the ring's sixteen.
 // Measured under the power cap (48 tokens, 200 experts of 256): 1245 -> 1108 us a pass at 1.58 -> 1.72 GHz, and
-// 8..10 % on 1 to 64 tokens over 8 to 256 experts.  Beyond 64 rows the scale of every column makes
-// the epilogue longer than that of the tokens-as-M form, and a kernel that holds both forms spills.
+// 8..10 % on 1 to 64 tokens over 8 to 256 experts.  A weight byte is read once a launch and leaves L2 first (1141 -> 1127 us).
+// Beyond 64 rows the scale of every column makes the epilogue longer than that of the tokens-as-M form, and a kernel that holds
+// both forms spills.
 constexpr unsigned kIdescF8M128 = (1u << 4) | ((128u >> 4) << 24);
 __device__ __forceinline__ int small_cols(int rows) { return (rows + 15) & ~15; }
 // columns set aside per k-block and weight half
@@ -541,7 +542,8 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
             const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
             const int c3 = g1 ? ti.expert * 2 * args.I + ti.n * kTileN1 : ti.n * kTileN2 / 16;
             single_issue_kblock_5d(smem_u32(&sc->full[stage]), tx, sA + kBOff, sA + kBOff + kBHalfBytes, g1 ? &op->tm_p1 : &op->tm_p2,
-                                   kb * kKb, c3, c3 + (g1 ? 64 : 8), g1 ? 0 : ti.expert, sA, tma, ti.row0, gathered ? 0u : (unsigned)boxes);
+                                   kb * kKb, c3, c3 + (g1 ? 64 : 8), g1 ? 0 : ti.expert, sA, tma, ti.row0, gathered ? 0u : (unsigned)boxes,
+                                   l2_evict_first());
           } else {
             const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
             single_issue_kblock(smem_u32(&sc->full[stage]), tx, sA + kBOff, sA + kBOff + kBHalfBytes, tmw, kb * kKb,
