@@ -17,85 +17,74 @@ namespace moe {
 constexpr int kPlanThreads = kPlanChunk;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr int kPlanDirectRows = 8192;   // up to here every block counts all rows itself: no histogram launch
+// experts per block of a list, a warp each: the fewer, the more SMs share the stores (1024 rows over 252 experts: 7.8 us a plan with
+// 32, 7.1 with 8)
+constexpr int kPlanListExperts = 8;
 constexpr int kPlanMaxBlocks = 128;     // beyond kPlanMaxBlocks x kPlanChunk rows a block owns several chunks
 
-// exclusive scan of one int per thread over a 1024-thread block
-__device__ inline int block_excl_scan(int v, int* total, int* warp_sums) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int inc = v;
+// One warp: out[i] = f(0) + ... + f(i - 1) for i in [0, E], in shared memory; returns the sum over all E.  The scans of a plan run side
+// by side on different warps with one barrier behind them; as block-wide scans one after the other (three barriers of 1024
+// threads each) they took a good part of a small plan.
+template <class F>
+__device__ __forceinline__ int warp_scan(int* out, int E, F f) {
+  const int lane = threadIdx.x & 31, per = (E + 31) >> 5;
+  const int e0 = min(E, lane * per), e1 = min(E, e0 + per);
+  int sum = 0;
+#pragma unroll 8
+  for (int e = e0; e < e1; ++e) sum += f(e);
+  int inc = sum;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    int n = __shfl_up_sync(0xffffffffu, inc, d);
-    if (lane >= d) inc += n;
+    const int v = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= d) inc += v;
   }
-  if (lane == 31) warp_sums[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    int s = warp_sums[lane];
-    int si = s;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      int n = __shfl_up_sync(0xffffffffu, si, d);
-      if (lane >= d) si += n;
-    }
-    warp_sums[lane] = si - s;               // exclusive warp offsets
-    if (lane == 31) warp_sums[32] = si;     // grand total
+  int pos = inc - sum;
+#pragma unroll 8
+  for (int e = e0; e < e1; ++e) {
+    out[e] = pos;
+    pos += f(e);
   }
-  __syncthreads();
-  const int res = warp_sums[warp] + inc - v;
-  *total = warp_sums[32];
-  __syncthreads();
-  return res;
+  const int total = __shfl_sync(0xffffffffu, inc, 31);
+  if (lane == 0) out[E] = total;
+  return total;
 }
+
+// tile: a power of two
+__device__ __forceinline__ int tiles_of(int rows, int tile) { return (rows + tile - 1) >> (31 - __clz(tile)); }
 
 // ---------------------------------------------------------------- the ordered tile list of one op
-// Shared-memory scratch of build_tile_list: work tiles of the experts before e.
-struct ListScratch {
-  int warp_sums[33];
-  int work[kMaxExperts + 1];
-};
-
-// first index i of the ascending array a[0..n) with a[i] >= v (n if none)
-__device__ __forceinline__ int lower_bound(const int* a, int n, int v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] >= v) hi = mid;
-    else lo = mid + 1;
-  }
-  return lo;
-}
-
 // Writes this block's share of the queue list of an op whose expert e holds rows [off[e], off[e] + cnt[e]) of the
-// packed row space (cnt / off in shared memory), and (block 0) its PlanState.  All blocks of the grid call it.
+// packed row space (cnt / off / work in shared memory; work[e]: work tiles of the experts before e), and (block 0) its
+// PlanState.  All blocks of the grid call it.
 // Work tiles (the unit the queues hand out): up to `work_rows` consecutive rows of one
 // expert, i.e. one or two adjacent m-tiles that share each weight tile they read.
 // Order: the gate/up entries in expert order, and the down entries of an expert in front of the first expert whose
 // gate/up tiles start at least kLagWork work tiles behind its own, so by the time a down tile is claimed the tiles it
 // depends on were claimed long before.  Every entry's place follows from the prefix sum of the work tiles.
-__device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan, const int* cnt, const int* off, int E,
-                                                int NT1, int NT2, int T, int work_rows, int x_moe, int planned,
+__device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan, const int* cnt, const int* off, const int* work,
+                                                int E, int NT1, int NT2, int T, int work_rows, int x_moe, int planned,
                                                 int n_extra_gemm, int g1_kind = kGateUp) {
-  __shared__ ListScratch ls;
-  const int e = threadIdx.x;
-  const int we = e < E ? (cnt[e] + work_rows - 1) / work_rows : 0;
-  int n_work;
-  const int w0 = block_excl_scan(we, &n_work, ls.warp_sums);
-  if (e < E) ls.work[e] = w0;
-  if (e == 0) ls.work[E] = n_work;
-  __syncthreads();
-
+  const int n_work = work[E];
   // Inside an expert: n-major over its work tiles, so an expert's entries of one GEMM are one
   // contiguous run of the list.  One warp per expert writes them (a popular expert has hundreds).
   const int lane = threadIdx.x & 31;
-  for (int x = (int)blockIdx.x * kPlanWarps + (int)(threadIdx.x >> 5); x < E; x += (int)gridDim.x * kPlanWarps) {
-    const int mx = ls.work[x], wx = ls.work[x + 1] - mx;
+  for (int x = (int)blockIdx.x + (int)gridDim.x * (int)(threadIdx.x >> 5); x < E; x += (int)gridDim.x * kPlanWarps) {
+    const int mx = work[x], wx = work[x + 1] - mx;
     if (wx == 0) continue;
     const int cx = cnt[x], ox = off[x];
-    const int before = lower_bound(ls.work + 1, E, mx - kLagWork + 1);      // experts whose down entries come first
-    const int next = min(E, lower_bound(ls.work, E + 1, mx + wx + kLagWork));
-    int4* g1 = tile_list + (size_t)mx * NT1 + (size_t)ls.work[before] * NT2;
-    int4* g2 = tile_list + (size_t)ls.work[next] * NT1 + (size_t)mx * NT2;
+    // Work tiles whose down entries come before expert x's gate/up entries (those of the experts that end kLagWork tiles
+    // ahead of it), and whose gate/up entries come before its down entries (up to the first expert that starts kLagWork tiles
+    // after its end): the largest work[i] <= mx - kLagWork, and the smallest work[i] >= mx + wx + kLagWork.
+    int down_before = 0, up_before = n_work;
+    for (int i = lane; i <= E; i += 32) {
+      const int v = work[i];
+      if (v <= mx - kLagWork) down_before = max(down_before, v);
+      if (v >= mx + wx + kLagWork) up_before = min(up_before, v);
+    }
+    down_before = __reduce_max_sync(0xffffffffu, down_before);
+    up_before = __reduce_min_sync(0xffffffffu, up_before);
+    int4* g1 = tile_list + (size_t)mx * NT1 + (size_t)down_before * NT2;
+    int4* g2 = tile_list + (size_t)up_before * NT1 + (size_t)mx * NT2;
     for (int i = lane; i < wx * NT1; i += 32) {
       const int n = i / wx, j = i - n * wx;
       g1[i] = make_entry(g1_kind, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), x);
@@ -158,8 +147,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_hist_kernel(const __grid_co
 template <bool kDirect>
 __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_constant__ PlanArgs a) {
   extern __shared__ int run[];              // [kPlanWarps][E]: next packed position of an expert's row per warp
-  __shared__ int warp_sums[33];
-  __shared__ int s_before[kMaxExperts], s_cnt[kMaxExperts], s_off[kMaxExperts];
+  __shared__ int s_before[kMaxExperts], s_cnt[kMaxExperts], s_off[kMaxExperts + 1], s_work[kMaxExperts + 1], s_mtile[kMaxExperts + 1];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int E = a.E, R = a.R;
   const int i0 = min(R, (int)blockIdx.x * a.own), i1 = min(R, i0 + a.own);
@@ -209,16 +197,18 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
   }
   __syncthreads();
 
-  int cnt = 0;
-  if (tid < E) cnt = s_cnt[tid] + s_before[tid];
-  int total;
-  const int off = block_excl_scan(cnt, &total, warp_sums);       // device prefix sum over experts
+  const auto rows_of = [&](int e) { return s_cnt[e] + s_before[e]; };
+  if (warp == 0) warp_scan(s_off, E, rows_of);                   // device prefix sum over experts
+  if (warp == 1) warp_scan(s_work, E, [&](int e) { return tiles_of(rows_of(e), a.work_rows); });
+  if (warp == 2) warp_scan(s_mtile, E, [&](int e) { return tiles_of(rows_of(e), kTileM); });
+  __syncthreads();
+  const int cnt = tid < E ? rows_of(tid) : 0, off = tid < E ? s_off[tid] : 0, total = s_off[E];
   if (tid < E) {
     s_cnt[tid] = cnt;
-    s_off[tid] = off;
     int pos = off + s_before[tid];          // rows of the expert: earlier blocks, then the warps of this one
+    const int warps = min(kPlanWarps, (i1 - i0 + share - 1) / share);
 #pragma unroll 8
-    for (int w = 0; w < kPlanWarps; ++w) {
+    for (int w = 0; w < warps; ++w) {
       const int v = run[w * E + tid];
       run[w * E + tid] = pos;
       pos += v;
@@ -251,12 +241,10 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
   for (int p = total + (int)(blockIdx.x * kPlanThreads) + tid; p < R; p += (int)gridDim.x * kPlanThreads) a.s2f[p] = -1;
 
   // m-tiles: ceil(m_e / M_t) per expert with rows (the footprint x_moe)
-  const int me = (cnt + kTileM - 1) / kTileM;
-  int x_moe;
-  const int m0 = block_excl_scan(me, &x_moe, warp_sums);
-  if (blockIdx.x == 0)
-    for (int j = 0; j < me; ++j) a.mtiles[m0 + j] = MTile{tid, off + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
-  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, E, a.NT1, a.NT2, a.T, a.work_rows, x_moe, total == R ? 1 : 0, 0);
+  if (blockIdx.x == 0 && tid < E)
+    for (int j = 0, m0 = s_mtile[tid], me = s_mtile[tid + 1] - m0; j < me; ++j)
+      a.mtiles[m0 + j] = MTile{tid, off + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
+  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, s_work, E, a.NT1, a.NT2, a.T, a.work_rows, s_mtile[E], total == R ? 1 : 0, 0);
 }
 
 // ---------------------------------------------------------------- masked layout
@@ -264,9 +252,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
 // rows of slab e are valid.  Nothing is permuted: the plan is the exclusive prefix sum for `offsets`, the
 // m-tile table (first row of a tile = e * slab_rows + 128 j) and the queue list over the slabs' valid rows.
 __global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_constant__ PlanArgs a, int slab_rows) {
-  __shared__ int warp_sums[33];
-  __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts];
-  const int e = threadIdx.x, E = a.E;
+  __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts], s_pos[kMaxExperts + 1], s_work[kMaxExperts + 1], s_mtile[kMaxExperts + 1];
+  const int e = threadIdx.x, warp = e >> 5, E = a.E;
   int cnt = 0;
   grid_dep_wait();
   if (e < E) {
@@ -278,19 +265,18 @@ __global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_
     s_cnt[e] = cnt;
     s_off[e] = e * slab_rows;
   }
-  int total;
-  const int off = block_excl_scan(cnt, &total, warp_sums);
+  __syncthreads();
+  if (warp == 0) warp_scan(s_pos, E, [&](int x) { return s_cnt[x]; });
+  if (warp == 1) warp_scan(s_work, E, [&](int x) { return tiles_of(s_cnt[x], a.work_rows); });
+  if (warp == 2) warp_scan(s_mtile, E, [&](int x) { return tiles_of(s_cnt[x], kTileM); });
+  __syncthreads();
   if (blockIdx.x == 0) {
-    if (e < E) a.offsets[e] = off;
-    if (e == 0) a.offsets[E] = total;
+    for (int i = e; i <= E; i += kPlanThreads) a.offsets[i] = s_pos[i];
+    if (e < E)
+      for (int j = 0, m0 = s_mtile[e], me = s_mtile[e + 1] - m0; j < me; ++j)
+        a.mtiles[m0 + j] = MTile{e, e * slab_rows + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
   }
-  const int me = (cnt + kTileM - 1) / kTileM;
-  int x_moe;
-  const int m0 = block_excl_scan(me, &x_moe, warp_sums);
-  if (blockIdx.x == 0)
-    for (int j = 0; j < me; ++j)
-      a.mtiles[m0 + j] = MTile{e, e * slab_rows + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
-  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, E, a.NT1, a.NT2, 0, a.work_rows, x_moe, 1, 0, kGateUpDirect);
+  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, s_work, E, a.NT1, a.NT2, 0, a.work_rows, s_mtile[E], 1, 0, kGateUpDirect);
 }
 
 // ---------------------------------------------------------------- the paired form of a decode + prefill op
@@ -323,6 +309,7 @@ struct PairArgs {
 __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_constant__ PairArgs a) {
   __shared__ int cnt_d[kMaxExperts], off_d[kMaxExperts], cnt_p[kMaxExperts], off_p[kMaxExperts];
   __shared__ int base_d[kMaxExperts], base_p[kMaxExperts];   // what a row's packed position is shifted by
+  __shared__ int work_d[kMaxExperts + 1], work_p[kMaxExperts + 1];
   const int e = threadIdx.x, E = a.E;
   grid_dep_wait();
   if (e < E) {
@@ -345,11 +332,14 @@ __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_co
   __syncthreads();
   const int ok = (a.d.plain->planned && a.p.plain->planned) ? 1 : 0;
   // a carrier taller than the kernel's work tile (e4m3: 128 rows) is cut into work tiles that follow one another
-  const int n_dec = build_tile_list(a.d.tile_list, a.d.plan, cnt_d, off_d, E, a.NT1, a.NT2, a.d.T,
-                                    min(a.carrier_rows, a.work_rows), a.d.plain->n_mtiles, ok, 0);
+  const int rows_d = min(a.carrier_rows, a.work_rows);
+  if (e < 32) warp_scan(work_d, E, [&](int x) { return tiles_of(cnt_d[x], rows_d); });
+  else if (e < 64) warp_scan(work_p, E, [&](int x) { return tiles_of(cnt_p[x], a.work_rows); });
   __syncthreads();
+  const int n_dec = build_tile_list(a.d.tile_list, a.d.plan, cnt_d, off_d, work_d, E, a.NT1, a.NT2, a.d.T, rows_d,
+                                    a.d.plain->n_mtiles, ok, 0);
   // every GEMM entry of the decode list may carry prefill rows: the prefill op is complete when they are too
-  build_tile_list(a.p.tile_list, a.p.plan, cnt_p, off_p, E, a.NT1, a.NT2, a.p.T, a.work_rows, a.p.plain->n_mtiles, ok,
+  build_tile_list(a.p.tile_list, a.p.plan, cnt_p, off_p, work_p, E, a.NT1, a.NT2, a.p.T, a.work_rows, a.p.plain->n_mtiles, ok,
                   n_dec);
   // the shared row space's permutation
   for (int i = (int)(blockIdx.x * kPlanThreads + threadIdx.x); i < a.d.R + a.p.R; i += (int)gridDim.x * kPlanThreads) {
@@ -367,8 +357,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_co
 }
 
 // ---------------------------------------------------------------- launches
-// blocks that write a list: a warp per expert
-static int list_blocks(int E) { return (E + kPlanWarps - 1) / kPlanWarps; }
+// blocks that write a list
+static int list_blocks(int E) { return (E + kPlanListExperts - 1) / kPlanListExperts; }
 
 cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
                                cudaStream_t stream) {
