@@ -272,6 +272,18 @@ __device__ __forceinline__ bool mbar_try_cluster(void* bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
+// non-blocking test that also synchronises with arrivals of the other CTA
+__device__ __forceinline__ bool mbar_test_cluster(void* bar, unsigned parity) {
+  unsigned ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void st_cluster_v4(unsigned cluster_addr, uint4 v) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
@@ -381,6 +393,27 @@ __device__ __forceinline__ void pair_issue_kblock(unsigned bar, unsigned tx, uns
   if constexpr (kEvictFirst) MOE_PAIR_KBLOCK(".L2::cache_hint", ", %16");
   else MOE_PAIR_KBLOCK("", "");
 #undef MOE_PAIR_KBLOCK
+}
+
+// The activation boxes alone, for a k-block whose weights and expect_tx went out before
+__device__ __forceinline__ void pair_issue_rows(unsigned bar, int x, unsigned sX, const CUtensorMap* tma, int ay, unsigned a_boxes,
+                                                unsigned a_rows) {
+  asm volatile(
+      "{\n\t.reg .pred e, pa1, pa2, pa3;\n\t.reg .b32 r, st, sA1, ay1, sA2, ay2;\n\t"
+      "elect.sync r|e, 0xffffffff;\n\t"
+      "setp.ge.and.u32 pa1, %5, 1, e;\n\t"
+      "setp.ge.and.u32 pa2, %5, 2, e;\n\t"
+      "setp.ge.and.u32 pa3, %5, 3, e;\n\t"
+      "shl.b32 st, %6, 7;\n\t"
+      "add.u32 sA1, %2, st;\n\t"
+      "add.s32 ay1, %4, %6;\n\t"
+      "add.u32 sA2, sA1, st;\n\t"
+      "add.s32 ay2, ay1, %6;\n\t"
+      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%2], [%3, {%1, %4}], [%0];\n\t"
+      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%3, {%1, ay1}], [%0];\n\t"
+      "@pa3 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA2], [%3, {%1, ay2}], [%0];\n\t}"
+      ::"r"(bar), "r"(x), "r"(sX), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "r"(a_rows)
+      : "memory");
 }
 
 // One k-block of the pair's MMAs as ONE instruction group: the next stage's barrier is tested first and

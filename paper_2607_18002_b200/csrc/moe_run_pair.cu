@@ -64,6 +64,7 @@ struct SharedCtl {
   unsigned long long iempty[kRing];  // leader's: ring slot released by the roles of both CTAs
   unsigned long long done[kRing];    // leader's: the 16 epilogue warps have stored the tile
   unsigned long long taken[kRing];   // leader's: its producer has started on the tile
+  unsigned long long rows_in[kRing]; // own: the rows that the tile reads are in place (down tiles: its gate/up tiles are committed)
   unsigned tmem_base;
   alignas(16) unsigned char epi_scratch[8][2048];
   QueueTables qt;
@@ -124,6 +125,13 @@ __device__ __noinline__ bool info_wait_one(const Ctx& c, void* bar, unsigned par
 }
 __device__ __forceinline__ bool wait_info(const Ctx& c, void* bar, unsigned parity, int where, bool leader) {
   return __all_sync(0xffffffffu, info_wait_one(c, bar, parity, where, leader));
+}
+
+// whether the scheduler has seen the rows of the tile in ring slot `islot` in place
+template <int kTileRows>
+__device__ __forceinline__ bool rows_in_place(SharedCtl<kTileRows>* sc, int islot, unsigned parity, bool leader) {
+  const bool in = leader ? mbar_test(&sc->rows_in[islot], parity) : mbar_test_cluster(&sc->rows_in[islot], parity);
+  return __all_sync(0xffffffffu, in);
 }
 
 // arrival on a barrier that lives in the leader's shared memory
@@ -247,6 +255,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       mbar_init(&sc->iempty[s], 13);
       mbar_init(&sc->done[s], 16);
       mbar_init(&sc->taken[s], 1);
+      mbar_init(&sc->rows_in[s], 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_proxy();
@@ -299,14 +308,21 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
       if (!wwait(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
       if (ti.kind != kEnd && need_ready && !wait_op_ready(c, lane, ti)) ti.kind = kEnd;
+      // A down tile is handed over at once: the producers fill the free stages with its weights and add the rows when its gate/up
+      // tiles are committed (one token: 67.6 -> 67.0 us a pass, 128 tokens on 8 experts: 80.3 -> 79.1).
       int ok = 1;
       if (lane == 0) {
-        if (ti.kind == kDown) ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
-        if (!ok) ti.kind = kEnd;
         publish(sc, islot, ti);
+        if (ti.kind == kDown) {
+          ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
+          fence_async_proxy();
+        }
+        if (ok) {
+          mbar_arrive_cluster(map_to_cta(&sc->rows_in[islot], 1));
+          mbar_arrive(&sc->rows_in[islot]);
+        }
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
-      ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       // The gather warps will read the tile's row list (4 bytes per row) first thing: pull it into L2
       // now, the weight stream has usually pushed it out since the plan wrote it.
       if (ti.kind == kGateUp && lane * 32 < ti.rows) prefetch_l2(op->gather_list + ti.row0 + lane * 32);
@@ -342,15 +358,37 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       ti.kblocks = __shfl_sync(0xffffffffu, sc->info[islot].kblocks, 0);
       ti.expert = __shfl_sync(0xffffffffu, sc->info[islot].expert, 0);
       if (ti.kind == kEnd) break;
-      if (lane == 0) {
-        arrive_at_leader(&sc->iempty[islot], leader);
-        if (leader) mbar_arrive(&sc->taken[islot]);
-      }
+      const int tslot = islot;
+      const unsigned tph = iph;
+      if (leader && lane == 0) mbar_arrive(&sc->taken[tslot]);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (ti.kind == kCombine) continue;
-      const LoadPlan lp = make_plan(&args.ops[ti.slot], ti, rank);
+      if (ti.kind == kCombine) {
+        if (lane == 0) arrive_at_leader(&sc->iempty[tslot], leader);
+        continue;
+      }
+      LoadPlan lp = make_plan(&args.ops[ti.slot], ti, rank);
       bool fail = false;
-      for (int kb = 0; kb < ti.kblocks; ++kb) {
+      int kb = 0;
+      if (ti.kind == kDown && !rows_in_place(sc, tslot, tph, leader)) {
+        const unsigned boxes = (unsigned)lp.a_boxes, stage0 = stage;
+        lp.a_boxes = 0;
+        bool in = false;
+        do {
+          if (!wwait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
+          issue_kblock(sc, stages_addr, lp, kb, stage, leader, full0_addr);
+          if (++stage == kNS) { stage = 0; par ^= 1u; }
+          in = rows_in_place(sc, tslot, tph, leader);
+        } while (++kb < min(ti.kblocks, kNS) && !in);
+        if (fail || !wait_info(c, &sc->rows_in[tslot], tph, 27, leader)) break;
+        for (int j = 0, s = (int)stage0; j < kb; ++j) {
+          pair_issue_rows(full0_addr + s * 8u, j * kBlockK, stages_addr + s * (unsigned)kSB, lp.tma, lp.ay, boxes,
+                          (unsigned)lp.a_box_rows);
+          if (++s == kNS) s = 0;
+        }
+        lp.a_boxes = (int)boxes;
+      }
+      if (lane == 0) arrive_at_leader(&sc->iempty[tslot], leader);   // the ring slot's barriers are not looked at any more
+      for (; kb < ti.kblocks; ++kb) {
         if (!wwait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
         issue_kblock(sc, stages_addr, lp, kb, stage, leader, full0_addr);
         if (++stage == kNS) { stage = 0; par ^= 1u; }

@@ -94,3 +94,24 @@ def test_masked_slabs_on_the_deeper_pipelines(slab):
     assert_close(y[flat], oracle.ffn_rows(oracle_weights(spec, W), x, None, flat, rows_e))
     y[flat] = 0.0
     assert np.all(y == 0.0)
+
+
+@pytest.mark.parametrize("T,I", [(t, i) for t in (1, 24, 90, 180, 250) for i in (128, 768, 1536)])
+def test_down_tiles_that_wait_for_their_rows(T, I):
+    """Few tiles on many units: every down tile is handed over before its gate/up tiles are done, and its weights wait in the
+    stages -- fewer k-blocks than the pipeline has stages, and more -- for activation rows of one to three boxes."""
+    E, H = 2, 256
+    spec = synth.Spec("wait", synth.Shape(E, 1, H, I), ((synth.DECODE, T),), "uniform", None, 1.0, -1.0, 64)
+    W = synth.make_weights(spec)
+    ids = (np.arange(T) == 0).astype(np.int32).reshape(-1, 1)        # expert 1 has one row, expert 0 the others
+    x, _ = synth.make_x(spec, T, 0, 0)
+    op = synth.Op(synth.DECODE, x, ids, np.ones(ids.shape, np.float32))
+    ctx = make_ctx(spec)
+    b = bind_ops(ctx, [op], weights_to(W))[0]
+    ref = oracle.forward(oracle_weights(spec, W), x, None, ids, op.w)["y"]
+    for _ in range(3):
+        b.y.fill_(7.0)
+        ctx.plan(0, b)
+        ctx.run([0], fuse_combine=True)
+        ctx.check()
+        assert_close(b.y.float().cpu().numpy(), ref)
