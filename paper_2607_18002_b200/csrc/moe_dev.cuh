@@ -60,7 +60,7 @@ struct PlanState {
 
 // Part of the run state, see RunHead.
 struct RunState {
-  int gemm_done;      // committed GEMM tiles
+  int gemm_done;      // committed GEMM tiles (CTA pairs: times the warps that store one)
   int tiles_done;     // committed tiles of any kind
   int done;           // 1 when the op has fully finished
   int pad;
@@ -110,7 +110,7 @@ struct __align__(128) OpDev {
   int* plan_hist;        // [n_chunks, E] rows per plan block and expert
   PlanState* plan;
   RunState* run;         // in the first half of the run state
-  int* g1_done;          // [max_mtiles] committed gate/up tiles per work tile (first half)
+  int* g1_done;          // [max_mtiles] committed gate/up tiles per work tile, counted like gemm_done (first half)
   Status* status;        // the context's device status block
   // Which list of routed rows the run kernels walk.  A plain op: its own permutation (the plan's public
   // outputs).  The paired form of a decode + prefill op that share their weights (moe_plan_pair): one row
@@ -159,7 +159,8 @@ struct RunArgs {
   int n_ops;
   int fuse_combine;
   int E, k, H, I;
-  int dtype, kb_elems;    // MOE_DTYPE_*; K elements per pipeline stage (64 bf16 / 128 e4m3)
+  int dtype;              // MOE_DTYPE_*
+  int kb_gate_up, kb_down;   // k-blocks (pipeline stages: 64 elements of K in bf16, 128 in e4m3) of a gate/up and a down tile
   long long wait_ns;
   unsigned run_bytes;     // size of one half of the run state
   int n_slots;            // slots of the context; descriptor d >= n_slots is the paired form of slot d - n_slots

@@ -428,7 +428,9 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   a.fuse_combine = fuse_combine ? 1 : 0;
   a.E = c.n_experts; a.k = c.top_k; a.H = c.hidden; a.I = c.inter;
   a.dtype = c.dtype;
-  a.kb_elems = c.dtype == MOE_DTYPE_FP8_E4M3 ? 128 : kBlockK;
+  const int kb_elems = c.dtype == MOE_DTYPE_FP8_E4M3 ? 128 : kBlockK;
+  a.kb_gate_up = c.hidden / kb_elems;
+  a.kb_down = c.inter / kb_elems;
   a.wait_ns = (long long)c.wait_limit_us * 1000;
   a.static_kind = -1;
   a.run_bytes = (unsigned)ctx->L.run_bytes;
@@ -481,7 +483,8 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream) {
   a.fuse_combine = 0;
   a.E = c.n_experts; a.k = c.top_k; a.H = c.hidden; a.I = c.inter;
   a.dtype = c.dtype;
-  a.kb_elems = kBlockK;
+  a.kb_gate_up = c.hidden / kBlockK;
+  a.kb_down = c.inter / kBlockK;
   a.wait_ns = (long long)c.wait_limit_us * 1000;
   a.n_slots = c.max_ops;
   for (int s = 0; s < kMaxOps; ++s) a.desc[s] = (signed char)s;

@@ -47,6 +47,8 @@ __device__ __forceinline__ bool mbar_test(void* bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
+// orders what this thread wrote or saw before what it writes after, for all of the device
+__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // L2 policy of bytes that nobody reads a second time
 __device__ __forceinline__ unsigned long long l2_evict_first() {
   unsigned long long p;

@@ -460,12 +460,13 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   grid_dep_wait();             // everything above overlaps the kernel before this one
-  if (warp == 0) begin_unit(&args, &sc->qt, (int)gridDim.x, lane);
+  if (warp == 0) begin_unit(&args, &sc->qt, rh, lane, 1);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const unsigned tmem = sc->tmem_base;
   c.run_off = sc->qt.run_off;
+  if (warp == 3 && lane == 0) end_turn(&args, take_turn(&args), (int)gridDim.x);
   if (blockIdx.x == 0 && warp == 3) {
     clear_next_run(&args, rh, c.run_off, lane);
     if (lane == 0) finish_empty_ops(c, -1);
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       if (kind == kEnd) break;
       if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->done[islot], iph, 17))) break;
       if (lane == 0) {
-        commit_tile(c, rh, ti);
+        commit_tile<true>(c, rh, ti);
         mbar_arrive(&sc->iempty[islot]);
       }
       __syncwarp();

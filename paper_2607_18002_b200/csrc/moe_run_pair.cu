@@ -41,6 +41,10 @@ struct Ring {
   static constexpr int kNS = kTileRows == 256 ? 6 : kTileRows == 128 ? 8 : 11;
 };
 constexpr int kAccCols = 256;
+// Warps that store a tile, in both CTAs.  Each counts the tile in the words that down and combine tiles wait for as soon as its own
+// part is out: one token takes 63.9 us a pass where 65.9 with one thread that counts for all of them after they have met.  (In the
+// e4m3 kernel the same costs registers that its epilogue needs, 4 % at 2000 tokens: there the committer counts.)
+constexpr int kStoreWarps = 16;
 constexpr int kFullCount = 2 + kGatherThreads + 1;
 // instruction descriptor: D fp32, A/B bf16, K-major, M = 256 over the pair, N = the tile's columns
 constexpr unsigned kIdescM256 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4) << 24);
@@ -65,6 +69,7 @@ struct SharedCtl {
   unsigned long long done[kRing];    // leader's: the 16 epilogue warps have stored the tile
   unsigned long long taken[kRing];   // leader's: its producer has started on the tile
   unsigned long long rows_in[kRing]; // own: the rows that the tile reads are in place (down tiles: its gate/up tiles are committed)
+  unsigned long long began;          // leader's: the queue tables and qt.run_off are in place
   unsigned tmem_base;
   alignas(16) unsigned char epi_scratch[8][2048];
   QueueTables qt;
@@ -203,7 +208,7 @@ struct CombineWhenDone {
   const OpDev* op;
   bool look;
   __device__ __forceinline__ bool operator()() const {
-    if (look) wait_counter(*c, &run_of(*c, op)->gemm_done, op_gemm_tiles(op), 4);
+    if (look) wait_counter(*c, &run_of(*c, op)->gemm_done, op_gemm_tiles(op) * kStoreWarps, 4);
     named_barrier(1, 256);
     return !aborted(*c);
   }
@@ -257,6 +262,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       mbar_init(&sc->taken[s], 1);
       mbar_init(&sc->rows_in[s], 1);
     }
+    mbar_init(&sc->began, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_proxy();
   }
@@ -267,25 +273,20 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  grid_dep_wait();             // everything above overlaps the kernel before this one
-  if (warp == 0 && leader) begin_unit(&args, &sc->qt, (int)(gridDim.x >> 1), lane);
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();          // the other CTA's barriers exist before anything arrives on them
   tc_fence_after();
   const unsigned tmem = sc->tmem_base;
-  if (!leader) {               // the second CTA's epilogue looks at the run state too
-    unsigned off;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(off) : "r"(map_to_cta(&sc->qt.run_off, 0)) : "memory");
-    c.run_off = off;
-  } else {
+  touch_params(args);
+  grid_dep_wait();             // everything above overlaps the kernel before this one
+  // From here to the first loads of a tile everything is latency: tables, first claim, hand-over.  So no barrier of the CTA stands in
+  // between, only the scheduler's own two round trips (4300 + 3900 clocks to a claim before, 2750 + 3500 now).
+  // The half of the run state is known to the scheduler first; the roles that need it read it behind a barrier.
+  const auto set_run_off = [&] {
     c.run_off = sc->qt.run_off;
-    if (blockIdx.x == 0 && warp == 2) {
-      clear_next_run(&args, rh, c.run_off, lane);
-      if (lane == 0) finish_empty_ops(c, -1);
-    }
     rh = reinterpret_cast<RunHead*>(reinterpret_cast<char*>(rh) + c.run_off);
-  }
+  };
 
   if (warp == 0 && leader) {
     // ============================================================ scheduler (leader)
@@ -300,9 +301,14 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     ti.kind = kEnd;
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
     ti.t_claim = 0;
+    const ClaimWords seen = begin_unit(&args, &sc->qt, rh, lane, kStoreWarps);
+    set_run_off();
+    if (lane == 0) mbar_arrive(&sc->began);
     const bool plain = args.static_kind >= 0;             // plain launch: this pair runs one given entry
     if (plain) claim_static(&args, (int)(blockIdx.x >> 1), ti);
-    else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready);
+    else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready, &seen);
+    unsigned ticket = 0;
+    if (lane == 0) ticket = take_turn(&args);
     while (true) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
@@ -314,7 +320,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (lane == 0) {
         publish(sc, islot, ti);
         if (ti.kind == kDown) {
-          ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
+          ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1 * kStoreWarps, 3);
           fence_async_proxy();
         }
         if (ok) {
@@ -330,7 +336,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       // A combine tile is handed over at once: its epilogue warps read row indices and router weights and then wait for the op's
       // GEMM tiles themselves.  The next claim waits with them, so that a unit holds one such tile at most.
       if (ti.kind == kCombine) {
-        if (lane == 0) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op), 4);
+        if (lane == 0) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op) * kStoreWarps, 4);
         if (__shfl_sync(0xffffffffu, ok, 0) == 0) break;
       }
       if (!wwait(c, &sc->taken[islot], iph, 26)) break;
@@ -338,6 +344,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (plain) ti.kind = kEnd;
       else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready);
     }
+    if (lane == 0) end_turn(&args, ticket, (int)(gridDim.x >> 1));
   } else if (warp == 3) {
     // ============================================================ producer (both CTAs)
     // Reads tiles from the ring and issues this CTA's loads, one stage per k-block.  The whole
@@ -547,6 +554,11 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // ============================================================ committer (leader)
     int islot = 0;
     unsigned iph = 0;
+    if (wwait(c, &sc->began, 0u, 28)) {
+      if (blockIdx.x == 0) clear_next_run(&args, rh, sc->qt.run_off, lane);
+      set_run_off();
+      if (blockIdx.x == 0 && lane == 0) finish_empty_ops(c, -1);
+    }
     while (true) {
       if (!wait_info(c, &sc->ifull[islot], iph, 16, leader)) break;
       TileInfo ti;
@@ -555,7 +567,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (kind == kEnd) break;
       if (!wwait_cluster(c, &sc->done[islot], iph, 17)) break;
       if (lane == 0) {
-        commit_tile(c, rh, ti);
+        commit_tile<false>(c, rh, ti);
         mbar_arrive(&sc->iempty[islot]);
       }
       __syncwarp();
@@ -571,6 +583,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     const int etid = threadIdx.x - 256;
     int islot = 0;
     unsigned iph = 0, gcount = 0;
+    bool first = true;
     unsigned char* scratch = sc->epi_scratch[warp - 8];
     const unsigned scratch_addr = smem_u32(scratch);
     while (true) {
@@ -578,6 +591,16 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const TileInfo ti = sc->info[islot];
       if (ti.kind == kEnd) break;
       OpDev* op = &args.ops[ti.slot];
+      if (first) {
+        first = false;
+        if (leader) {
+          c.run_off = sc->qt.run_off;
+        } else {
+          unsigned off;
+          asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(off) : "r"(map_to_cta(&sc->qt.run_off, 0)) : "memory");
+          c.run_off = off;
+        }
+      }
       bool ok = true;
       if (ti.kind == kCombine) {
         const int mid = ti.row0 + (ti.rows + 1) / 2;
@@ -591,6 +614,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         ++gcount;
         tc_fence_after();
         const bool g1 = ti.kind != kDown;                     // gate/up tile: SwiGLU, output to A
+        const StoredWords words = stored_words(c, op, ti);
         const int cols = tile_cols(ti.rows) / 2;              // this warp's columns
         const int live = min(cols, ti.rows - half * cols);    // ... that hold token rows
         const int passes = (live + 31) / 32;
@@ -659,6 +683,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           __syncwarp();
           if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);
         }
+        __syncwarp();
+        if (lane == 0) count_stored(words);
       }
       // The warp's stores, before the tile is published: the arrival releases them (across the pair: at cluster scope), the
       // committer's fence is cumulative over what it acquires here

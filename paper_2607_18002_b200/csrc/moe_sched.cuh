@@ -16,6 +16,11 @@ struct TileInfo {
   unsigned long long t_claim;
 };
 
+// what a unit reads before it claims
+struct ClaimWords {
+  unsigned abort, budget, head[2];
+};
+
 // per-class queue tables of one launch (built once per CTA in shared memory)
 struct QueueTables {
   unsigned run_off;                // of this launch
@@ -23,7 +28,7 @@ struct QueueTables {
   int cls_slot[2][kMaxOps];
   int cls_free[2][kMaxOps];        // 1: the op has no ready word and no predecessor
   unsigned n_gemm[2][kMaxOps];     // GEMM entries of the op's list; the combine entries follow them
-  int all_gemm[2][kMaxOps];        // GEMM entries that must have committed before its combine may run
+  int all_gemm[2][kMaxOps];        // gemm_done when its combine may run
   const int4* list[2][kMaxOps];
   unsigned cum[2][kMaxOps + 1];
 };
@@ -221,7 +226,7 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
   ti.slot = slot;
   ti.tile = (int)local;
   ti.cls = cls;
-  ti.kblocks = ti.kind == kCombine ? 0 : (ti.kind == kDown ? a->I : a->H) / a->kb_elems;
+  ti.kblocks = ti.kind == kCombine ? 0 : ti.kind == kDown ? a->kb_down : a->kb_gate_up;
   return 1;
 }
 
@@ -232,39 +237,51 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
 // kEarlyCombine: a unit that finds nothing to run in either class takes a combine entry that has to wait for GEMM entries running
 // elsewhere, so that the wait for the last of them starts with the entry in hand (the caller must then not hold up
 // anything else with it).
+// seen: the words as the unit's start read them (its first claim); they only tell where to look, the fetch-add decides.
 template <bool kEarlyCombine>
 __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int lane, TileInfo& ti,
-                                 bool& need_ready) {
+                                 bool& need_ready, const ClaimWords* seen = nullptr) {
   const RunArgs* a = c.a;
-  // one lane reads the words and the warp takes ITS values: the budget word, the abort word and the heads
-  // change while the kernel runs, and the lanes do not load them at the same instant
-  int ab = 0, q = 0;
-  unsigned h0 = 0, h1 = 0;
-  if (lane == 0) {
-    ab = ld_volatile(&c.st->abort);
-    q = ld_volatile(&a->g->budget);
-    h0 = *reinterpret_cast<volatile unsigned*>(&rh->heads[0]);
-    h1 = *reinterpret_cast<volatile unsigned*>(&rh->heads[1]);
+  ClaimWords w{};
+  if (seen) {
+    w = *seen;
+  } else {
+    // one lane reads the words and the warp takes ITS values: the budget word, the abort word and the heads
+    // change while the kernel runs, and the lanes do not load them at the same instant
+    if (lane == 0) {
+      w.abort = (unsigned)ld_volatile(&c.st->abort);
+      w.budget = (unsigned)ld_volatile(&a->g->budget);
+      w.head[0] = *reinterpret_cast<volatile unsigned*>(&rh->heads[0]);
+      w.head[1] = *reinterpret_cast<volatile unsigned*>(&rh->heads[1]);
+    }
+    w.abort = __shfl_sync(0xffffffffu, w.abort, 0);
+    w.budget = __shfl_sync(0xffffffffu, w.budget, 0);
+    w.head[0] = __shfl_sync(0xffffffffu, w.head[0], 0);
+    w.head[1] = __shfl_sync(0xffffffffu, w.head[1], 0);
   }
-  ab = __shfl_sync(0xffffffffu, ab, 0);
-  q = __shfl_sync(0xffffffffu, q, 0);
-  h0 = __shfl_sync(0xffffffffu, h0, 0);
-  h1 = __shfl_sync(0xffffffffu, h1, 0);
-  if (ab != 0) return 0;
-  const int first = ((int)blockIdx.x < q) ? MOE_CLASS_DECODE : MOE_CLASS_PREFILL;
+  if (w.abort != 0) return 0;
+  const unsigned h0 = w.head[0], h1 = w.head[1];
+  const int first = ((int)blockIdx.x < (int)w.budget) ? MOE_CLASS_DECODE : MOE_CLASS_PREFILL;
   need_ready = false;
-  int r1 = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready);
-  int r2 = 0;
-  if (r1 != 1) r2 = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready);
-  if (kEarlyCombine && r1 != 1 && r2 != 1) {
-    if (r1 == -1) r1 = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready, true);
-    if (r1 != 1 && r2 == -1) r2 = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready, true);
+  int none[2] = {0, 0};                          // in the order tried: 0 nothing left, -1 not yet
+  if constexpr (kEarlyCombine) {
+    // one body for all attempts: a unit's first claim waits for these instructions to be fetched
+#pragma unroll 1
+    for (int p = 0; p < 4; ++p) {
+      if (p >= 2 && none[p & 1] == 0) continue;
+      const int cls = (p & 1) ? 1 - first : first;
+      none[p & 1] = try_claim(c, sc, rh, cls, cls == 0 ? h0 : h1, lane, ti, need_ready, p >= 2);
+      if (none[p & 1] == 1) break;
+    }
+  } else {                                       // (in a loop this kernel's scheduler spills)
+    none[0] = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready);
+    if (none[0] != 1) none[1] = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready);
   }
-  if (r1 == 1 || r2 == 1) {
-    ti.t_claim = gtime_ns();
+  if (none[0] == 1 || none[1] == 1) {
+    if (a->log_cap > 0) ti.t_claim = gtime_ns();
     return 1;
   }
-  return (r1 == 0 && r2 == 0) ? 0 : -1;
+  return (none[0] | none[1]) == 0 ? 0 : -1;
 }
 
 // A ticket that landed in an op that is not ready yet: wait for it (bounded).  Whole warp; lane 0 looks and
@@ -306,18 +323,19 @@ __device__ inline void claim_static(const RunArgs* a, int unit, TileInfo& ti) {
   ti.slot = slot;
   ti.tile = unit;
   ti.cls = op->cls;
-  ti.kblocks = (ti.kind == kDown ? a->I : a->H) / a->kb_elems;
-  ti.t_claim = gtime_ns();
+  ti.kblocks = ti.kind == kDown ? a->kb_down : a->kb_gate_up;
+  if (a->log_cap > 0) ti.t_claim = gtime_ns();
 }
 
 // Blocking form: waits (bounded) while an op exists that is not ready.  Returns with
 // ti.kind == kEnd when nothing is left (or the run was aborted).
 template <bool kEarlyCombine>
 __device__ inline void claim_next(const Ctx& c, QueueTables* sc, RunHead* rh, int lane, TileInfo& ti,
-                                  bool& need_ready) {
+                                  bool& need_ready, const ClaimWords* seen = nullptr) {
   unsigned long long t0 = 0;
   for (unsigned it = 0;; ++it) {
-    const int r = claim_once<kEarlyCombine>(c, sc, rh, lane, ti, need_ready);
+    const int r = claim_once<kEarlyCombine>(c, sc, rh, lane, ti, need_ready, seen);
+    seen = nullptr;
     if (r == 1) return;
     if (r == 0) break;
     __nanosleep(256);                         // an op exists but is not ready yet
@@ -337,11 +355,33 @@ __device__ inline void claim_next(const Ctx& c, QueueTables* sc, RunHead* rh, in
   ti.kind = kEnd;
 }
 
-// one committed entry counted for `op` (descriptor `desc`): counters, notify word, completion
-__device__ inline void count_commit(const Ctx& c, OpDev* op, int desc, bool gemm) {
+// The words that down and combine tiles wait for, for a tile of `op` (of a combine tile: not counted).  A GEMM entry of a paired
+// decode op carries rows of the prefill op too: it counts for both.
+struct StoredWords {
+  int* rows;           // gate/up tiles: g1_done of the work tile
+  int* op;             // gemm_done
+  int* partner;        // ... of the other op
+};
+__device__ __forceinline__ StoredWords stored_words(const Ctx& c, const OpDev* op, const TileInfo& ti) {
+  StoredWords w;
+  w.rows = ti.kind != kDown ? &g1_done_of(c, op)[ti.m] : nullptr;
+  w.op = &run_of(c, op)->gemm_done;
+  w.partner = op->paired && ti.cls == MOE_CLASS_DECODE ? &run_of(c, &c.a->ops[op->partner])->gemm_done : nullptr;
+  return w;
+}
+// By one lane of each warp that stores a tile, after a __syncwarp behind its last store, or by one thread for all of them.
+__device__ __forceinline__ void count_stored(const StoredWords& w) {
+  fence_acq_rel_gpu();
+  fence_async_proxy();
+  if (w.rows) atomicAdd(w.rows, 1);
+  atomicAdd(w.op, 1);
+  if (w.partner) atomicAdd(w.partner, 1);
+}
+
+// one committed entry counted for `op` (descriptor `desc`): notify word, completion
+__device__ inline void count_commit(const Ctx& c, OpDev* op, int desc) {
   const RunArgs* a = c.a;
   RunState* run = run_of(c, op);
-  if (gemm) atomicAdd(&run->gemm_done, 1);
   const int done = atomicAdd(&run->tiles_done, 1) + 1;
   if (op->notify != nullptr && done == op->notify_after) st_release_sys(op->notify, 1u);
   if (done == op_total_tiles(op, a->fuse_combine)) {
@@ -352,18 +392,17 @@ __device__ inline void count_commit(const Ctx& c, OpDev* op, int desc, bool gemm
   }
 }
 
-// Publishing a finished tile: dependency counter, op completion, done word, log.
-// Called by one thread after all writers of the tile have fenced and synchronised.
+// Publishing a finished tile: op completion, done word, log, and unless the storing warps have done so (kCounts false) the words that
+// other tiles wait for.  Called by one thread after all writers of the tile have fenced and synchronised.
+template <bool kCounts>
 __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti) {
   const RunArgs* a = c.a;
   OpDev* op = &a->ops[ti.slot];
-  __threadfence();
-  fence_async_proxy();
   const unsigned long long t_commit = a->log_cap > 0 ? gtime_ns() : 0ull;   // before it is published
-  if (ti.kind == kGateUp || ti.kind == kGateUpDirect) atomicAdd(&g1_done_of(c, op)[ti.m], 1);
-  count_commit(c, op, ti.slot, ti.kind != kCombine);
-  // a GEMM entry of a paired decode op carries rows of the prefill op too: it counts for both
-  if (op->paired && op->cls == MOE_CLASS_DECODE && ti.kind != kCombine) count_commit(c, &a->ops[op->partner], op->partner, true);
+  if (kCounts && ti.kind != kCombine) count_stored(stored_words(c, op, ti));
+  else fence_acq_rel_gpu();
+  count_commit(c, op, ti.slot);
+  if (op->paired && op->cls == MOE_CLASS_DECODE && ti.kind != kCombine) count_commit(c, &a->ops[op->partner], op->partner);
   if (a->log_cap > 0) {
     const unsigned idx = atomicAdd(&rh->log_count, 1u);
     if (idx < (unsigned)a->log_cap) {
@@ -383,12 +422,22 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
   }
 }
 
-// Start of a claiming unit, one warp: which half of the run state is this launch's, and the per-class queue tables.  Lane i reads
-// the plan of op i, so that the loads of all ops overlap each other and the atomic.  The last of the grid's `units` units to ask
-// turns the halves over for the next launch.
-__device__ inline void begin_unit(const RunArgs* a, QueueTables* sc, int units, int lane) {
-  unsigned turn = 0;
-  if (lane == 0) turn = atomicAdd(&a->g->turn, 1u);
+// Start of a claiming unit, one warp: which half of the run state is this launch's, the per-class queue tables, and the words of the
+// unit's first claim (heads: of both halves, the half is only known when they arrive).  All of it is one round trip: lane i reads
+// the plan of op i, the last lanes a word each.  The unit asks for the half with a plain load; the fetch-add that counts it
+// (take_turn) comes later, so that no claim waits behind those of all other units.
+// per_tile: what a committed GEMM entry adds to gemm_done.
+__device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const RunHead* first_half, int lane, int per_tile) {
+  constexpr int kW = 25;
+  static_assert(kMaxOps <= kW, "a lane per op, and one per word");
+  const RunHead* second = reinterpret_cast<const RunHead*>(reinterpret_cast<const char*>(first_half) + a->run_bytes);
+  unsigned word = 0;
+  if (lane >= kW) {
+    const void* p = lane == kW ? (const void*)&a->g->turn : lane == kW + 1 ? (const void*)&a->g->status.abort
+                  : lane == kW + 2 ? (const void*)&a->g->budget
+                  : (const void*)&(lane < kW + 5 ? first_half : second)->heads[(lane - kW - 3) & 1];
+    word = *reinterpret_cast<const volatile unsigned*>(p);
+  }
   PlanState ps{};
   int cls = 0;
   if (lane < a->n_ops) {
@@ -396,7 +445,7 @@ __device__ inline void begin_unit(const RunArgs* a, QueueTables* sc, int units, 
     cls = a->cls[lane];
   }
   const int entries = ps.planned == 0 ? 0 : ps.n_gemm_tiles + (a->fuse_combine ? ps.n_comb_tiles : 0);
-  const int all_gemm = ps.n_gemm_tiles + ps.n_extra_gemm;
+  const int all_gemm = (ps.n_gemm_tiles + ps.n_extra_gemm) * per_tile;
   if (lane == 0) {
     sc->n_cls[0] = sc->n_cls[1] = 0;
     sc->cum[0][0] = sc->cum[1][0] = 0;
@@ -414,10 +463,28 @@ __device__ inline void begin_unit(const RunArgs* a, QueueTables* sc, int units, 
       sc->list[ci][j] = a->tile_list[i];
     }
   }
-  if (lane == 0) {
-    sc->run_off = (turn >> 31) ? a->run_bytes : 0u;
-    if ((turn & 0x7fffffffu) == (unsigned)units - 1u) atomicExch(&a->g->turn, ~turn & 0x80000000u);
-  }
+  const unsigned turn = __shfl_sync(0xffffffffu, word, kW);
+  const bool odd = (turn >> 31) != 0;
+  if (lane == 0) sc->run_off = odd ? a->run_bytes : 0u;
+  __syncwarp();
+  ClaimWords w;
+  w.abort = __shfl_sync(0xffffffffu, word, kW + 1);
+  w.budget = __shfl_sync(0xffffffffu, word, kW + 2);
+  w.head[0] = __shfl_sync(0xffffffffu, word, odd ? kW + 5 : kW + 3);
+  w.head[1] = __shfl_sync(0xffffffffu, word, odd ? kW + 6 : kW + 4);
+  return w;
+}
+// One lane, once a launch and after begin_unit: counts the unit.  The last of the grid's `units` units turns the halves over for the
+// next launch (end_turn).
+__device__ inline unsigned take_turn(const RunArgs* a) { return atomicAdd(&a->g->turn, 1u); }
+__device__ inline void end_turn(const RunArgs* a, unsigned ticket, int units) {
+  if ((ticket & 0x7fffffffu) == (unsigned)units - 1u) atomicExch(&a->g->turn, ~ticket & 0x80000000u);
+}
+// The launch parameters into the constant cache, while the kernel before still runs.
+__device__ __forceinline__ void touch_params(const RunArgs& a) {
+  const int* p = reinterpret_cast<const int*>(&a);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(RunArgs) / 4); i += 16) asm volatile("" ::"r"(p[i]));
 }
 // One warp of the grid: zeroes the other half, which the launch before this one left behind.
 __device__ inline void clear_next_run(const RunArgs* a, RunHead* first_half, unsigned run_off, int lane) {
