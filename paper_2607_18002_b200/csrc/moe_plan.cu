@@ -17,21 +17,26 @@ namespace moe {
 constexpr int kPlanThreads = kPlanChunk;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr int kPlanDirectRows = 8192;   // up to here every block counts all rows itself: no histogram launch
-// experts per block of a list, a warp each: the fewer, the more SMs share the stores (1024 rows over 252 experts: 7.8 us a plan with
-// 32, 7.1 with 8)
+// experts per block of a list, a warp each: the fewer, the more SMs share the stores (1024 rows over 252 experts: 0.7 us less a
+// plan with 8 than with 32)
 constexpr int kPlanListExperts = 8;
 constexpr int kPlanMaxBlocks = 128;     // beyond kPlanMaxBlocks x kPlanChunk rows a block owns several chunks
 
-// One warp: out[i] = f(0) + ... + f(i - 1) for i in [0, E], in shared memory; returns the sum over all E.  The scans of a plan run side
-// by side on different warps with one barrier behind them; as block-wide scans one after the other (three barriers of 1024
-// threads each) they took a good part of a small plan.
+// One warp: out[e] = f(rows[0]) + ... + f(rows[e - 1]) for e in [0, E], in shared memory.  Both arrays hold kScan entries, rows[e] is 0
+// from E on and f(0) = 0: a lane's experts are neighbours and come four at a time.  The scans of a plan run side by side on different
+// warps with one barrier behind them (8 rows over 256 experts: 5.2 us a plan with block-wide scans of three barriers each, one
+// after the other; 4.1 us).
+constexpr int kScan = kMaxExperts + 4;
 template <class F>
-__device__ __forceinline__ int warp_scan(int* out, int E, F f) {
-  const int lane = threadIdx.x & 31, per = (E + 31) >> 5;
-  const int e0 = min(E, lane * per), e1 = min(E, e0 + per);
+__device__ __forceinline__ void warp_scan(int* out, const int* rows, int E, F f) {
+  const int lane = threadIdx.x & 31, quads = ((E + 31) / 32 + 3) / 4;           // a lane has 4 * quads experts
+  const int4* in = reinterpret_cast<const int4*>(rows) + lane * quads;
   int sum = 0;
-#pragma unroll 8
-  for (int e = e0; e < e1; ++e) sum += f(e);
+#pragma unroll 2
+  for (int i = 0; i < quads; ++i) {
+    const int4 v = in[i];
+    sum += f(v.x) + f(v.y) + f(v.z) + f(v.w);
+  }
   int inc = sum;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -39,14 +44,18 @@ __device__ __forceinline__ int warp_scan(int* out, int E, F f) {
     if (lane >= d) inc += v;
   }
   int pos = inc - sum;
-#pragma unroll 8
-  for (int e = e0; e < e1; ++e) {
-    out[e] = pos;
-    pos += f(e);
+#pragma unroll 2
+  for (int i = 0; i < quads; ++i) {
+    const int4 v = in[i];
+    int4 o;
+    o.x = pos;
+    o.y = o.x + f(v.x);
+    o.z = o.y + f(v.y);
+    o.w = o.z + f(v.z);
+    pos = o.w + f(v.w);
+    reinterpret_cast<int4*>(out)[lane * quads + i] = o;
   }
-  const int total = __shfl_sync(0xffffffffu, inc, 31);
-  if (lane == 0) out[E] = total;
-  return total;
+  if (lane == 31) out[128 * quads] = inc;           // (E where E fills the lanes)
 }
 
 // tile: a power of two
@@ -86,11 +95,11 @@ __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan,
     int4* g1 = tile_list + (size_t)mx * NT1 + (size_t)down_before * NT2;
     int4* g2 = tile_list + (size_t)up_before * NT1 + (size_t)mx * NT2;
     for (int i = lane; i < wx * NT1; i += 32) {
-      const int n = i / wx, j = i - n * wx;
+      const int n = wx == 1 ? i : i / wx, j = i - n * wx;
       g1[i] = make_entry(g1_kind, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), x);
     }
     for (int i = lane; i < wx * NT2; i += 32) {
-      const int n = i / wx, j = i - n * wx;
+      const int n = wx == 1 ? i : i / wx, j = i - n * wx;
       g2[i] = make_entry(kDown, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), x);
     }
   }
@@ -143,68 +152,74 @@ __global__ void __launch_bounds__(kPlanThreads) plan_hist_kernel(const __grid_co
   for (int e = threadIdx.x; e < a.E; e += kPlanThreads) a.hist[(size_t)blockIdx.x * a.E + e] = h[e];
 }
 
-// kDirect: no histogram was made, every block counts all rows itself (R <= kPlanDirectRows).
+// kDirect: no histogram was made, every block counts all rows itself (R <= kPlanDirectRows).  A warp's first 32 ids and their peers
+// stay in registers from the count to the ranking (8 rows over 256 experts: 4.25 -> 3.70 us a plan, 1024 rows: 7.3 -> 5.8).
 template <bool kDirect>
 __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_constant__ PlanArgs a) {
   extern __shared__ int run[];              // [kPlanWarps][E]: next packed position of an expert's row per warp
-  __shared__ int s_before[kMaxExperts], s_cnt[kMaxExperts], s_off[kMaxExperts + 1], s_work[kMaxExperts + 1], s_mtile[kMaxExperts + 1];
+  __shared__ alignas(16) int s_cnt[kScan], s_off[kScan], s_work[kScan], s_mtile[kScan];
+  __shared__ int s_before[kMaxExperts];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int E = a.E, R = a.R;
   const int i0 = min(R, (int)blockIdx.x * a.own), i1 = min(R, i0 + a.own);
 
-  for (int e = tid; e < E; e += kPlanThreads) s_before[e] = s_cnt[e] = 0;
+  const int share = a.own / kPlanWarps;
+  const int w0 = min(i1, i0 + warp * share), w1 = min(i1, w0 + share);
+  for (int e = tid; e < kMaxExperts; e += kPlanThreads) s_before[e] = s_cnt[e] = 0;
   for (int i = tid; i < kPlanWarps * E; i += kPlanThreads) run[i] = 0;
   grid_dep_wait();
+  const int first_id = w0 + lane < w1 ? a.ids[w0 + lane] : -1;   // of this warp's share; read while the counts are
   __syncthreads();
-  // rows per expert: before this block's range, and from it on
+  // rows per expert: all of them, and those before this block's range
   if (kDirect) {
 #pragma unroll 4
     for (int i = tid; i < R; i += kPlanThreads) {
       const int id = a.ids[i];
-      if (id >= 0 && id < E) atomicAdd(i < i0 ? &s_before[id] : &s_cnt[id], 1);
+      if (id >= 0 && id < E) {
+        atomicAdd(&s_cnt[id], 1);
+        if (i < i0) atomicAdd(&s_before[id], 1);
+      }
     }
   } else {
     const int parts = max(1, kPlanThreads / E), part = tid / E, e = tid % E;
     const int nb = (int)gridDim.x, per = (nb + parts - 1) / parts;
     const int b0 = min(nb, part * per), b1 = min(nb, b0 + per);
-    int before = 0, rest = 0;
+    int before = 0, all = 0;
     if (part < parts) {
 #pragma unroll 16
       for (int b = b0; b < b1; ++b) {
         const int v = a.hist[(size_t)b * E + e];
         if (b < (int)blockIdx.x) before += v;
-        else rest += v;
+        all += v;
       }
       if (before) atomicAdd(&s_before[e], before);
-      if (rest) atomicAdd(&s_cnt[e], rest);
+      if (all) atomicAdd(&s_cnt[e], all);
     }
   }
   // this block's rows: each warp counts a contiguous share of them per expert
-  const int share = a.own / kPlanWarps;
-  const int w0 = min(i1, i0 + warp * share), w1 = min(i1, w0 + share);
   int* mine = run + warp * E;
   const unsigned lower = (1u << lane) - 1u;
+  unsigned first_peers = 0;
   for (int base = w0; base < w1; base += 32) {
     const int i = base + lane;
-    int id = i < w1 ? a.ids[i] : -1;
+    int id = base == w0 ? first_id : i < w1 ? a.ids[i] : -1;
     if (i < w1 && (id < 0 || id >= E)) {
       report(a.status, MOE_EBADID, a.slot, i, id, 0);
       id = -1;
     }
     const unsigned peers = __match_any_sync(0xffffffffu, id);
+    if (base == w0) first_peers = peers;
     if (id >= 0 && (peers & lower) == 0) mine[id] += __popc(peers);
     __syncwarp();
   }
   __syncthreads();
 
-  const auto rows_of = [&](int e) { return s_cnt[e] + s_before[e]; };
-  if (warp == 0) warp_scan(s_off, E, rows_of);                   // device prefix sum over experts
-  if (warp == 1) warp_scan(s_work, E, [&](int e) { return tiles_of(rows_of(e), a.work_rows); });
-  if (warp == 2) warp_scan(s_mtile, E, [&](int e) { return tiles_of(rows_of(e), kTileM); });
+  if (warp == 0) warp_scan(s_off, s_cnt, E, [](int rows) { return rows; });      // device prefix sum over experts
+  if (warp == 1) warp_scan(s_work, s_cnt, E, [&](int rows) { return tiles_of(rows, a.work_rows); });
+  if (warp == 2) warp_scan(s_mtile, s_cnt, E, [](int rows) { return tiles_of(rows, kTileM); });
   __syncthreads();
-  const int cnt = tid < E ? rows_of(tid) : 0, off = tid < E ? s_off[tid] : 0, total = s_off[E];
+  const int cnt = tid < E ? s_cnt[tid] : 0, off = tid < E ? s_off[tid] : 0, total = s_off[E];
   if (tid < E) {
-    s_cnt[tid] = cnt;
     int pos = off + s_before[tid];          // rows of the expert: earlier blocks, then the warps of this one
     const int warps = min(kPlanWarps, (i1 - i0 + share - 1) / share);
 #pragma unroll 8
@@ -223,9 +238,9 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
   // stable positions
   for (int base = w0; base < w1; base += 32) {
     const int i = base + lane;
-    int id = i < w1 ? a.ids[i] : -1;
+    int id = base == w0 ? first_id : i < w1 ? a.ids[i] : -1;
     if (id < 0 || id >= E) id = -1;         // reported above
-    const unsigned peers = __match_any_sync(0xffffffffu, id);
+    const unsigned peers = base == w0 ? first_peers : __match_any_sync(0xffffffffu, id);
     int p = -1;
     if (id >= 0) p = mine[id] + __popc(peers & lower);
     __syncwarp();
@@ -252,7 +267,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
 // rows of slab e are valid.  Nothing is permuted: the plan is the exclusive prefix sum for `offsets`, the
 // m-tile table (first row of a tile = e * slab_rows + 128 j) and the queue list over the slabs' valid rows.
 __global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_constant__ PlanArgs a, int slab_rows) {
-  __shared__ int s_cnt[kMaxExperts], s_off[kMaxExperts], s_pos[kMaxExperts + 1], s_work[kMaxExperts + 1], s_mtile[kMaxExperts + 1];
+  __shared__ alignas(16) int s_cnt[kScan], s_pos[kScan], s_work[kScan], s_mtile[kScan];
+  __shared__ int s_off[kMaxExperts];
   const int e = threadIdx.x, warp = e >> 5, E = a.E;
   int cnt = 0;
   grid_dep_wait();
@@ -262,13 +278,13 @@ __global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_
       if (blockIdx.x == 0) report(a.status, MOE_EBOUNDS, a.slot, e, cnt, 4);
       cnt = 0;
     }
-    s_cnt[e] = cnt;
     s_off[e] = e * slab_rows;
   }
+  s_cnt[e] = cnt;                            // 0 from E on
   __syncthreads();
-  if (warp == 0) warp_scan(s_pos, E, [&](int x) { return s_cnt[x]; });
-  if (warp == 1) warp_scan(s_work, E, [&](int x) { return tiles_of(s_cnt[x], a.work_rows); });
-  if (warp == 2) warp_scan(s_mtile, E, [&](int x) { return tiles_of(s_cnt[x], kTileM); });
+  if (warp == 0) warp_scan(s_pos, s_cnt, E, [](int rows) { return rows; });
+  if (warp == 1) warp_scan(s_work, s_cnt, E, [&](int rows) { return tiles_of(rows, a.work_rows); });
+  if (warp == 2) warp_scan(s_mtile, s_cnt, E, [](int rows) { return tiles_of(rows, kTileM); });
   __syncthreads();
   if (blockIdx.x == 0) {
     for (int i = e; i <= E; i += kPlanThreads) a.offsets[i] = s_pos[i];
@@ -307,9 +323,9 @@ struct PairArgs {
 // One launch: every block scans the experts and writes its share of both lists, then moves its share of the rows
 // into the shared row space.
 __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_constant__ PairArgs a) {
-  __shared__ int cnt_d[kMaxExperts], off_d[kMaxExperts], cnt_p[kMaxExperts], off_p[kMaxExperts];
+  __shared__ alignas(16) int cnt_d[kScan], cnt_p[kScan], work_d[kScan], work_p[kScan];
+  __shared__ int off_d[kMaxExperts], off_p[kMaxExperts];
   __shared__ int base_d[kMaxExperts], base_p[kMaxExperts];   // what a row's packed position is shifted by
-  __shared__ int work_d[kMaxExperts + 1], work_p[kMaxExperts + 1];
   const int e = threadIdx.x, E = a.E;
   grid_dep_wait();
   if (e < E) {
@@ -328,13 +344,15 @@ __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_co
     off_d[e] = moff + cp - take;
     base_p[e] = od;                                          // the decode rows of the experts before
     base_d[e] = op + cp;                                     // ... and the expert's own prefill rows
+  } else {
+    cnt_p[e] = cnt_d[e] = 0;
   }
   __syncthreads();
   const int ok = (a.d.plain->planned && a.p.plain->planned) ? 1 : 0;
   // a carrier taller than the kernel's work tile (e4m3: 128 rows) is cut into work tiles that follow one another
   const int rows_d = min(a.carrier_rows, a.work_rows);
-  if (e < 32) warp_scan(work_d, E, [&](int x) { return tiles_of(cnt_d[x], rows_d); });
-  else if (e < 64) warp_scan(work_p, E, [&](int x) { return tiles_of(cnt_p[x], a.work_rows); });
+  if (e < 32) warp_scan(work_d, cnt_d, E, [&](int rows) { return tiles_of(rows, rows_d); });
+  else if (e < 64) warp_scan(work_p, cnt_p, E, [&](int rows) { return tiles_of(rows, a.work_rows); });
   __syncthreads();
   const int n_dec = build_tile_list(a.d.tile_list, a.d.plan, cnt_d, off_d, work_d, E, a.NT1, a.NT2, a.d.T, rows_d,
                                     a.d.plain->n_mtiles, ok, 0);
