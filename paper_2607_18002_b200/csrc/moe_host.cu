@@ -62,7 +62,12 @@ Layout make_layout(const moe_config_t* c) {
   Layout L{};
   const size_t E = c->n_experts, H = c->hidden, I = c->inter;
   L.max_rows = c->max_tokens_per_op * c->top_k;
-  L.max_mtiles = (L.max_rows + kTileM - 1) / kTileM + c->n_experts;
+  // Work tiles of an op: at most one partly filled tile per expert besides the full ones.  An op of few tokens is cut into lower tiles,
+  // and where its tokens name an expert more than once it has more of them than m-tiles.
+  const int low = c->dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8Small : kWorkRowsSmall;
+  const int low_rows = (c->max_tokens_per_op < low ? c->max_tokens_per_op : low) * c->top_k;
+  const int full_tiles = (L.max_rows + kTileM - 1) / kTileM, low_tiles = (low_rows + low - 1) / low;
+  L.max_mtiles = (full_tiles > low_tiles ? full_tiles : low_tiles) + c->n_experts;
   L.NT1 = (int)(I / kTileN1);
   L.NT2 = (int)(H / kTileN2);
   // combine entries of the largest op: small batches use smaller combine tiles

@@ -5,10 +5,12 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2607_18002_b200 as moe
 from workloads import synth
 
-from gpu_util import bind_ops, check_plan, check_tiles, make_ctx, n_combine_tiles, weights_to
+from gpu_util import (ATOL, ATOL8, REL_L2, REL_L2_8, RTOL, RTOL8, assert_close, bind_ops, check_plan, check_tiles, make_ctx,
+                      n_combine_tiles, oracle_weights, weights_to)
 
 pytestmark = pytest.mark.gpu
 
@@ -30,3 +32,32 @@ def test_plan_and_queue_list(T, E, k):
     check_tiles(ctx, 0, counts)
     rows = 256 if ctx.ctas_per_tile == 2 else moe.MOE_TILE_M        # bf16 work tiles on the default grid
     assert ctx.footprint(0)[1] == int((-(-counts // rows)).sum()) * 2 + n_combine_tiles(T)
+
+
+@pytest.mark.parametrize("dtype,T", [("bf16", 32), ("fp8", 64)])
+def test_more_low_tiles_than_mtiles(dtype, T):
+    """An op of few tokens is cut into lower tiles.  When its tokens name one expert with every slot it has more of them than m-tiles
+    plus experts: list and dependency counters of a context of just that size hold them, the neighbouring slot stays intact."""
+    E = k = 8
+    spec = synth.Spec("low", synth.Shape(E, k, 256, 128, dtype), ((synth.DECODE, T), (synth.PREFILL, T)), "uniform", None, 1.0, -1.0, 7)
+    W = synth.make_weights(spec)
+    ids = np.zeros((T, k), np.int32)
+    ids[np.arange(7), k - 1] = np.arange(1, 8)                      # the other experts get a row each
+    ctx = make_ctx(spec)
+    ops = []
+    for i, (cls, _) in enumerate(spec.ops):
+        x, xs = synth.make_x(spec, T, 0, i)
+        ops.append(synth.Op(cls, x, ids, np.full(ids.shape, 1.0 / k, np.float32), xs))
+    bound = bind_ops(ctx, ops, weights_to(W))
+    for s, b in enumerate(bound):
+        ctx.plan(s, b)
+    ctx.run([0, 1], fuse_combine=True)
+    ctx.check()
+    rows = 32 if dtype == "bf16" and ctx.ctas_per_tile == 2 else 64 if dtype == "fp8" else 128
+    tol = dict(atol=ATOL, rtol=RTOL, rel_l2=REL_L2) if dtype == "bf16" else dict(atol=ATOL8, rtol=RTOL8, rel_l2=REL_L2_8)
+    for s, (b, op) in enumerate(zip(bound, ops)):
+        counts = check_plan(b, op, E)
+        assert ctx.footprint(s)[1] == int((-(-counts // rows)).sum()) * 2 + n_combine_tiles(T)
+        ref = oracle.forward(oracle_weights(spec, W), op.x, op.x_scale, op.ids, op.w,
+                             round_A=oracle.ROUND_NONE if dtype == "bf16" else oracle.ROUND_E4M3_1X128)["y"]
+        assert_close(b.y.float().cpu().numpy(), ref, **tol)
