@@ -152,6 +152,20 @@ __device__ __forceinline__ void tc_ld_frag(unsigned taddr, unsigned (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+// 16 lanes x 64 columns: register pair (4 j + 2 r, + 1) is row lane / 4 + 8 r, columns 8 j + 2 (lane % 4) and the next
+__device__ __forceinline__ void tc_ld_frag64(unsigned taddr, unsigned (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+}
 // 16 TMEM lanes x 16 columns: thread i holds column 4 j + i % 4 of row i / 4 in r[2 j] and of row i / 4 + 8 in r[2 j + 1] (twice
 // the rate of the layout above)
 __device__ __forceinline__ void tc_ld_pairs(unsigned taddr, unsigned (&r)[8]) {

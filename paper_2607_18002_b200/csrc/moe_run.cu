@@ -51,7 +51,7 @@ enum Mode : int { kBf16 = 0, kF8 = 1, kF8Small = 2 };
 constexpr int kAccCols = 256;                          // TMEM columns per accumulator
 
 struct F8Big {
-  float amax_x[2][4][32];                          // amax exchange between the two warps of a quadrant
+  float amax_x[2][2][4][32];                       // amax exchange between the two warps of a quadrant, tiles alternate
 };
 struct F8Small {
   alignas(16) unsigned char scale[16][256];        // ring of token scales, one slot per k-block
@@ -254,6 +254,155 @@ __device__ __forceinline__ bool epilogue_fp8_small(const Ctx& c, SharedCtl<kF8Sm
   return true;
 }
 
+// The activation scales of one row of a tile: its own op's, or (paired form) its partner's when the row is tagged so.
+__device__ __forceinline__ const float* row_scales(const Ctx& c, const OpDev* op, const TileInfo& ti, int row, bool valid) {
+  const RunArgs& a = *c.a;
+  if (ti.kind == kDown) return op->a_scale + (size_t)(ti.row0 + (valid ? row : 0)) * (a.I / 128);
+  if (ti.kind == kGateUpDirect) return op->x_scale + (size_t)(ti.row0 + (valid ? row : 0)) * (a.H / 128);   // masked layout
+  int tok = 0;
+  const OpDev* src = op;
+  if (valid) {
+    const int v = op->gather_list[ti.row0 + row];
+    const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
+    const int own_tag = op->paired ? slot_of(&a, ti.slot) : 0;
+    if (op->paired && tag != own_tag && tag == slot_of(&a, op->partner)) src = &a.ops[op->partner];
+    if (v >= 0 && (tag == own_tag || src != op) && flat < src->n_rows) tok = flat / a.k;
+    else { src = op; report(c.st, MOE_EBOUNDS, slot_of(&a, ti.slot), ti.row0 + row, v, 1); }
+  }
+  return src->x_scale + (size_t)tok * (a.H / 128);
+}
+
+// The weight scales of a tile, one per k-block and 128 rows of the matrix.
+__device__ __forceinline__ void weight_scales(const RunArgs& a, const OpDev* op, const TileInfo& ti, const float*& sw0, const float*& sw1) {
+  const int HB = a.H / 128, IB = a.I / 128;
+  if (ti.kind != kDown) {
+    sw0 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + ti.n) * HB;
+    sw1 = sw0 + (size_t)IB * HB;
+  } else {
+    sw0 = op->s_down + ((size_t)ti.expert * HB + 2 * ti.n) * IB;
+    sw1 = sw0 + IB;
+  }
+}
+
+// One e4m3 tile of up to 64 rows on the epilogue warps.  With M = 64 only 16 lanes of a TMEM quadrant hold rows, so a fragment load
+// spreads 16 rows x 64 columns over the whole warp: row lane / 4 and the row eight below, columns 8 j + 2 (lane % 4) and the next as
+// register pairs.  That is half of the registers and a quarter of the multiply-add instructions that a thread per row needs, and a
+// k-block's two loads are in flight together; the partial buffer is handed back before they are multiplied in.  2000 tokens over 256
+// experts: 2128 -> 2090 us a pass, 4096 + 512 paired: 3184 -> 3152.  (The same packed adds and early hand-back in the form of a thread per
+// row, whose registers hold one chunk at a time, gave nothing: 3152 -> 3160.)
+__device__ __forceinline__ bool epilogue_fp8_m64(const Ctx& c, SharedCtl<kF8>* sc, OpDev* op, const TileInfo& ti, unsigned tmem, int warp,
+                                                 int lane, unsigned& eph, unsigned& xph) {
+  const RunArgs& a = *c.a;
+  const int q = warp & 3, ch = (warp - 8) >> 2;
+  const bool g1 = ti.kind != kDown;
+  const int IB = a.I / 128;
+  const int r0 = q * 16 + (lane >> 2);              // and r0 + 8
+  const float* sx0 = row_scales(c, op, ti, r0, r0 < ti.rows);
+  const float* sx1 = row_scales(c, op, ti, r0 + 8, r0 + 8 < ti.rows);
+  const float *sw0, *sw1;
+  weight_scales(a, op, ti, sw0, sw1);
+  unsigned long long acc[2][8][2];                  // [128-column half][8-column group][row]
+#pragma unroll
+  for (int i = 0; i < 32; ++i) acc[i >> 4][(i >> 1) & 7][i & 1] = 0ull;
+  float nx0 = sx0[0], nx1 = sx1[0], nw0 = sw0[0], nw1 = sw1[0];      // of the next k-block
+  const unsigned lane_addr = tmem + ((unsigned)(q * 32) << 16) + (unsigned)(ch * 64);
+  for (int kb = 0; kb < ti.kblocks; ++kb) {
+    const float s[2][2] = {{nx0 * nw0, nx1 * nw0}, {nx0 * nw1, nx1 * nw1}};
+    if (kb + 1 < ti.kblocks) { nx0 = sx0[kb + 1]; nx1 = sx1[kb + 1]; nw0 = sw0[kb + 1]; nw1 = sw1[kb + 1]; }
+    const int pb = kb & 1;
+    if (!__all_sync(0xffffffffu, mbar_wait_inline(c, &sc->pfull[pb], (eph >> pb) & 1u, 19))) return false;
+    eph ^= 1u << pb;
+    tc_fence_after();
+    unsigned p[2][32];
+    tc_ld_frag64(lane_addr + (unsigned)(pb * 256), p[0]);
+    tc_ld_frag64(lane_addr + (unsigned)(pb * 256 + 128), p[1]);
+    tc_wait_ld();
+    tc_fence_before();
+    __syncwarp();                                   // every lane's TMEM loads have completed
+    if (lane == 0) mbar_arrive(&sc->pempty[pb]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          acc[h][j][r] = fma_f32x2(f32x2(__uint_as_float(p[h][4 * j + 2 * r]), __uint_as_float(p[h][4 * j + 2 * r + 1])),
+                                   f32x2(s[h][r], s[h][r]), acc[h][j][r]);
+  }
+  // rows leave through the warp's scratch, 16 bytes a lane; the 16-byte chunks of a row are rotated by XOR to keep banks apart
+  unsigned char* scratch = sc->epi_scratch[warp - 8];
+  const int fr = lane >> 2, fc = lane & 3;
+  if (g1) {
+    float amax[2] = {0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float2 g = f32x2_parts(acc[0][j][r]), u = f32x2_parts(acc[1][j][r]);
+        const float v0 = __fdividef(g.x, 1.0f + __expf(-g.x)) * u.x, v1 = __fdividef(g.y, 1.0f + __expf(-g.y)) * u.y;
+        acc[0][j][r] = f32x2(v0, v1);
+        amax[r] = fmaxf(amax[r], fmaxf(fabsf(v0), fabsf(v1)));
+      }
+    float* mine = sc->f8.amax_x[xph & 1u][ch][q];
+    const float* other = sc->f8.amax_x[xph & 1u][ch ^ 1][q];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      amax[r] = fmaxf(amax[r], __shfl_xor_sync(0xffffffffu, amax[r], 1));
+      amax[r] = fmaxf(amax[r], __shfl_xor_sync(0xffffffffu, amax[r], 2));
+      if (fc == 0) mine[fr + 8 * r] = amax[r];
+    }
+    mbar_arrive(&sc->xbar[q]);
+    if (!__all_sync(0xffffffffu, mbar_wait_inline(c, &sc->xbar[q], xph, 20))) return false;
+    xph ^= 1u;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const float m = fmaxf(amax[r], other[fr + 8 * r]);
+      const float inv = m > 0.f ? 448.0f / m : 0.0f;
+      const int row = fr + 8 * r;
+      if (ch == 0 && fc == 0 && q * 16 + row < ti.rows)
+        op->a_scale[(size_t)(ti.row0 + q * 16 + row) * IB + ti.n] = m > 0.f ? m / 448.0f : 1.0f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float2 v = f32x2_parts(acc[0][j][r]);
+        *reinterpret_cast<unsigned short*>(scratch + row * 64 + (((j >> 1) ^ ((row >> 1) & 3)) << 4) + (j & 1) * 8 + fc * 2) =
+            (unsigned short)__nv_cvt_float2_to_fp8x2(make_float2(v.x * inv, v.y * inv), __NV_SATFINITE, __NV_E4M3);
+      }
+    }
+    __syncwarp();
+    unsigned char* out = reinterpret_cast<unsigned char*>(op->A) + (size_t)(ti.row0 + q * 16) * a.I + (size_t)(ti.n * kTileN1 + ch * 64);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int row = 8 * i + fr;
+      const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + row * 64 + ((fc ^ ((row >> 1) & 3)) << 4));
+      if (q * 16 + row < ti.rows) *reinterpret_cast<uint4*>(out + (size_t)row * a.I + fc * 16) = v4;
+    }
+    __syncwarp();                                   // scratch free again
+    return true;
+  }
+  unsigned char* out = reinterpret_cast<unsigned char*>(op->D) + ((size_t)(ti.row0 + q * 16) * a.H + (size_t)ti.n * kTileN2 + ch * 64) * 2;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int row = fr + 8 * r;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float2 v = f32x2_parts(acc[h][j][r]);
+        *reinterpret_cast<unsigned*>(scratch + row * 128 + ((j ^ (row & 7)) << 4) + fc * 4) = pack_bf16(v.x, v.y);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int row = 4 * i + (lane >> 3), f = lane & 7;
+      const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + row * 128 + ((f ^ (row & 7)) << 4));
+      if (q * 16 + row < ti.rows) *reinterpret_cast<uint4*>(out + ((size_t)row * a.H + h * 128) * 2 + f * 16) = v4;
+    }
+    __syncwarp();
+  }
+  return true;
+}
+
 // One e4m3 tile on the epilogue warps.  Thread = (accumulator row, 64-column slice of each
 // 128-column half); its 128 fp32 accumulators stay in registers (the epilogue warps raise
 // their register allowance for this).  Per k-block and half: partial * (activation scale of
@@ -266,38 +415,11 @@ __device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl<kF8>* sc, O
   const RunArgs& a = *c.a;
   const int q = warp & 3, ch = (warp - 8) >> 2;
   const int per_q = quadrant_rows(ti.rows);
-  const int row = q * per_q + lane;
-  const bool valid = lane < per_q && row < ti.rows;
+  const int row = q * 32 + lane;
+  const bool valid = row < ti.rows;
   const bool g1 = ti.kind != kDown;
-  const int HB = a.H / 128, IB = a.I / 128;
+  const int IB = a.I / 128;
   const unsigned lane_addr = tmem + ((unsigned)(q * 32) << 16);
-  // scale streams of this row / tile
-  const float* sx;
-  const float *sw0, *sw1;
-  if (ti.kind == kGateUpDirect) {       // masked layout: the row's scales sit at the row's own index
-    sx = op->x_scale + (size_t)(ti.row0 + (valid ? row : 0)) * HB;
-    sw0 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + ti.n) * HB;
-    sw1 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + IB + ti.n) * HB;
-  } else if (g1) {
-    // the row's activation scales: its own op's, or (paired form) the partner's when the row is tagged so
-    int tok = 0;
-    const OpDev* src = op;
-    if (valid) {
-      const int v = op->gather_list[ti.row0 + row];
-      const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
-      const int own_tag = op->paired ? slot_of(&a, ti.slot) : 0;
-      if (op->paired && tag != own_tag && tag == slot_of(&a, op->partner)) src = &a.ops[op->partner];
-      if (v >= 0 && (tag == own_tag || src != op) && flat < src->n_rows) tok = flat / a.k;
-      else { src = op; report(c.st, MOE_EBOUNDS, slot_of(&a, ti.slot), ti.row0 + row, v, 1); }
-    }
-    sx = src->x_scale + (size_t)tok * HB;
-    sw0 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + ti.n) * HB;
-    sw1 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + IB + ti.n) * HB;
-  } else {
-    sx = op->a_scale + (size_t)(ti.row0 + (valid ? row : 0)) * IB;
-    sw0 = op->s_down + ((size_t)ti.expert * HB + 2 * ti.n) * IB;
-    sw1 = sw0 + IB;
-  }
   if (q * per_q >= ti.rows) {
     // No row of the tile lies in this warp's TMEM lane quadrant (both warps of a quadrant see
     // the same q): nothing to read, scale or store.  The warp still takes part in every partial
@@ -310,6 +432,10 @@ __device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl<kF8>* sc, O
     }
     return true;
   }
+  if (ti.rows <= 64) return epilogue_fp8_m64(c, sc, op, ti, tmem, warp, lane, eph, xph);
+  const float* sx = row_scales(c, op, ti, row, valid);
+  const float *sw0, *sw1;
+  weight_scales(a, op, ti, sw0, sw1);
   float acc[128];                                 // [half][64]
 #pragma unroll
   for (int i = 0; i < 128; ++i) acc[i] = 0.f;
@@ -352,11 +478,11 @@ __device__ __forceinline__ bool epilogue_fp8(const Ctx& c, SharedCtl<kF8>* sc, O
       amax = fmaxf(amax, fabsf(v));
     }
     // the row's 128 outputs live in two threads (ch = 0, 1): exchange the partial maxima
-    sc->f8.amax_x[ch][q][lane] = amax;
+    sc->f8.amax_x[xph & 1u][ch][q][lane] = amax;
     mbar_arrive(&sc->xbar[q]);
     if (!__all_sync(0xffffffffu, mbar_wait_inline(c, &sc->xbar[q], xph, 20))) return false;
+    amax = fmaxf(amax, sc->f8.amax_x[xph & 1u][ch ^ 1][q][lane]);
     xph ^= 1u;
-    amax = fmaxf(amax, sc->f8.amax_x[ch ^ 1][q][lane]);
     const float scale = amax > 0.f ? amax / 448.0f : 1.0f;
     const float inv = amax > 0.f ? 448.0f / amax : 0.0f;
     if (valid) {

@@ -234,3 +234,26 @@ def test_fp8_small_launches(T, slab):
         ref[flat] = oracle.ffn_rows(Wo, x, xs, flat, rows_e, round_A=oracle.ROUND_E4M3_1X128)
         y = b.y.float().cpu().numpy().reshape(E * slab, -1)
     assert_close(y, ref, atol=ATOL8, rtol=RTOL8, rel_l2=REL_L2_8)
+
+
+@pytest.mark.parametrize("H,I", [(256, 128), (768, 640)])
+def test_fp8_tile_rows_of_large_launches(H, I):
+    """Launches of larger ops: tiles of up to 64 rows lie 16 to a TMEM quadrant and are read as fragments, others have a thread per row.
+    One expert for every edge of either form, as one op and with a second op of the other class beside it; the smallest shape has two
+    k-blocks a gate/up tile and one a down tile."""
+    counts = np.array([1, 8, 15, 16, 17, 32, 33, 49, 63, 64, 65, 96, 127, 128, 129, 0, 193], dtype=np.int32)
+    E, T = len(counts), int(counts.sum())
+    spec = synth.Spec("rows8", synth.Shape(E, 1, H, I, "fp8"), ((synth.PREFILL, T),), "uniform", None, 1.0, -1.0, 83)
+    W = synth.make_weights(spec)
+    Wo = oracle_weights(spec, W)
+    rng = np.random.default_rng(H)
+    ops = []
+    for n, cls in enumerate((synth.PREFILL, synth.DECODE)):
+        ids = rng.permutation(np.repeat(np.arange(E), np.roll(counts, n))).astype(np.int32).reshape(T, 1)
+        x, xs = synth.make_x(spec, T, 0, n)
+        ops.append(synth.Op(cls, x, ids, rng.uniform(0.5, 1.0, size=(T, 1)).astype(np.float32), xs))
+    for launch in (ops[:1], ops):
+        bound = _run(spec, ops=launch, W=W)[1]
+        for b, op in zip(bound, launch):
+            ref = oracle.forward(Wo, op.x, op.x_scale, op.ids, op.w, round_A=oracle.ROUND_E4M3_1X128)["y"]
+            assert_close(b.y.float().cpu().numpy(), ref, atol=ATOL8, rtol=RTOL8, rel_l2=REL_L2_8)
