@@ -17,7 +17,7 @@ cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, c
                              int slot_d, int slot_p, cudaStream_t stream);
 cudaError_t launch_combine(const OpDev* d_op, int T, int k, int H, cudaStream_t stream);
 cudaError_t prepare_run_kernel();
-cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream);
+cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, bool weights_once, cudaStream_t stream);
 cudaError_t prepare_pair_kernel();
 cudaError_t prepare_plan_kernels();
 cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream);
@@ -439,6 +439,7 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   a.wait_ns = (long long)c.wait_limit_us * 1000;
   a.static_kind = -1;
   a.run_bytes = (unsigned)ctx->L.run_bytes;
+  bool weights_once = true;
   for (int i = 0; i < n_ops; ++i) {
     const OpDev& h = ctx->ran_paired[slots[i]] ? ctx->host_pair[slots[i]] : ctx->host_ops[slots[i]];
     a.plan[i] = h.plan;
@@ -448,6 +449,8 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
     const int rows = ctx->ran_paired[slots[i]] ? full : ctx->work_rows[slots[i]];
     a.work_rows = rows > a.work_rows ? rows : a.work_rows;
+    const moe_op_t& op = ctx->ops[slots[i]];
+    if (ctx->ran_paired[slots[i]] || (op.layout == MOE_LAYOUT_MASKED ? op.slab_rows : op.n_tokens) > rows) weights_once = false;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (ctx->poison) {
@@ -459,7 +462,7 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     }
   }
   const cudaError_t le = ctx->pair_kernel ? launch_pair(a, ctx->rh(), ctx->n_ctas, st)
-                                          : launch_run(a, ctx->rh(), ctx->n_ctas, st);
+                                          : launch_run(a, ctx->rh(), ctx->n_ctas, weights_once, st);
   if (le != cudaSuccess) return MOE_ECUDA;
   return MOE_OK;
 }

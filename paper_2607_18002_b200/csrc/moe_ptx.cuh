@@ -534,20 +534,36 @@ __device__ __forceinline__ void f8_mma_kblock(unsigned d_tmem, unsigned long lon
 // The loads of one k-block of the single-CTA kernel as ONE group: expect_tx, the two halves of the
 // weight tile and (down tiles) the box of packed intermediate rows.  Whole warp, warp-uniform
 // operands; one elected lane issues.
+// kOnce: the weights are marked to leave L2 first.
+template <bool kOnce>
 __device__ __forceinline__ void single_issue_kblock(unsigned bar, unsigned tx, unsigned sB0, unsigned sB1,
                                                     const CUtensorMap* tmw, int x, int wy0, int wy1, unsigned sA,
                                                     const CUtensorMap* tma, int ay, unsigned has_a) {
-  asm volatile(
-      "{\n\t.reg .pred e, pa;\n\t.reg .b32 r;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "setp.ne.and.b32 pa, %11, 0, e;\n\t"
-      "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
-      "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%4, {%5, %6}], [%0];\n\t"
-      "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%3], [%4, {%5, %7}], [%0];\n\t"
-      "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%5, %10}], [%0];\n\t}"
-      ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wy0),
-        "r"(wy1), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(has_a)
-      : "memory");
+  if constexpr (kOnce) {
+    asm volatile(
+        "{\n\t.reg .pred e, pa;\n\t.reg .b32 r;\n\t"
+        "elect.sync r|e, 0xffffffff;\n\t"
+        "setp.ne.and.b32 pa, %11, 0, e;\n\t"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%2], [%4, {%5, %6}], [%0], %12;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%3], [%4, {%5, %7}], [%0], %12;\n\t"
+        "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%5, %10}], [%0];\n\t}"
+        ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wy0),
+          "r"(wy1), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(has_a), "l"(l2_evict_first())
+        : "memory");
+  } else {
+    asm volatile(
+        "{\n\t.reg .pred e, pa;\n\t.reg .b32 r;\n\t"
+        "elect.sync r|e, 0xffffffff;\n\t"
+        "setp.ne.and.b32 pa, %11, 0, e;\n\t"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%4, {%5, %6}], [%0];\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%3], [%4, {%5, %7}], [%0];\n\t"
+        "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%5, %10}], [%0];\n\t}"
+        ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wy0),
+          "r"(wy1), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(has_a)
+        : "memory");
+  }
 }
 // ... with the two halves of the weight tile as boxes of a 5-D map (coordinates 1 and 2 zero), and up to two activation
 // boxes of 32 rows; w_policy is the L2 policy of the weights

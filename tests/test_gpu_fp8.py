@@ -199,7 +199,7 @@ def test_c5_full_size_sampled():
         assert torch.isfinite(b.y.float()).all()
 
 
-@pytest.mark.parametrize("T,slab", [(t, 0) for t in (1, 15, 16, 17, 31, 32, 33, 48, 63, 64, 65)] + [(0, s) for s in (8, 33, 64, 65)])
+@pytest.mark.parametrize("T,slab", [(t, 0) for t in (1, 15, 16, 17, 31, 32, 33, 48, 63, 64, 65, 128, 129)] + [(0, s) for s in (8, 33, 64, 65)])
 def test_fp8_small_launches(T, slab):
     """Launches whose ops have up to 64 rows an expert run with the weights as the M operand; columns go in steps of 16, partials
     are grouped by four or two k-blocks.  T tokens, a third of which name one expert four times (more rows than a tile holds), or
