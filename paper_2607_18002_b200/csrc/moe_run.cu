@@ -55,14 +55,14 @@ struct F8Big {
 };
 struct F8Small {
   alignas(16) unsigned char scale[16][256];        // ring of token scales, one slot per k-block
-  float amax[8][64];                               // per warp and token
+  float amax[2][8][64];                            // per warp and token, gate/up tiles alternate
 };
 template <int kMode>
 struct SharedCtl {
   unsigned long long full[kMaxStages], fullA[kMaxStages], empty[kMaxStages];
   unsigned long long tfull[2], tempty[2];
   unsigned long long pfull[2], pempty[2];          // fp8: per-k-block partial products, two 256-column buffers
-  unsigned long long xbar[4];                      // fp8: amax exchange between the two warps of a quadrant
+  unsigned long long xbar[4];                      // fp8: amax exchange between the two warps of a quadrant (small tiles: [0], all eight)
   std::conditional_t<kMode == kF8Small, F8Small, F8Big> f8;
   unsigned long long ifull[kRing], iempty[kRing], done[kRing];
   TileInfo info[kRing];
@@ -114,7 +114,7 @@ __device__ __forceinline__ int scale_index(int tok) { return (tok & ~15) | ((tok
 // 16..31.  kSlot: columns set aside per k-block and weight half; kseq: k-blocks so far.
 template <int kSlot>
 __device__ __forceinline__ bool epilogue_fp8_small(const Ctx& c, SharedCtl<kF8Small>* sc, OpDev* op, const TileInfo& ti, unsigned tmem,
-                                                   int warp, int lane, unsigned& eph, unsigned& kseq) {
+                                                   int warp, int lane, unsigned& eph, unsigned& xph, unsigned& kseq) {
   constexpr int kGroup = 128 / kSlot, kChunks = kSlot / 16;
   const RunArgs& a = *c.a;
   const int q = warp & 3, half = (warp - 8) >> 2;
@@ -204,7 +204,7 @@ __device__ __forceinline__ bool epilogue_fp8_small(const Ctx& c, SharedCtl<kF8Sm
     return true;
   }
   // SwiGLU; per token the largest of this warp's 16 features, then of the tile's 128
-  float* mine = sc->f8.amax[warp - 8];
+  float* mine = sc->f8.amax[xph & 1u][warp - 8];
 #pragma unroll
   for (int ch = 0; ch < kChunks; ++ch) {
 #pragma unroll
@@ -218,18 +218,23 @@ __device__ __forceinline__ bool epilogue_fp8_small(const Ctx& c, SharedCtl<kF8Sm
       if (lane < 4) mine[ch * 16 + 4 * j + lane] = m;
     }
   }
-  named_barrier(1, 256);                            // the eight warps
+  // The eight warps meet here.  Like every wait it is bounded: a warp may have left because the launch was aborted.  One meeting a
+  // tile is enough: a warp writes this half of amax again two tiles on, past the meeting that all come to after reading it.
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&sc->xbar[0]);
+  if (!__all_sync(0xffffffffu, mbar_wait_inline(c, &sc->xbar[0], xph & 1u, 20))) return false;
+  const float(&all)[8][64] = sc->f8.amax[xph & 1u];
+  xph ^= 1u;
   float inv[kSlot / 32];                            // of tokens lane, lane + 32
 #pragma unroll
   for (int p = 0; p < kSlot / 32; ++p) {
     const int tok = 32 * p + lane;
     float amax = 0.f;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) amax = fmaxf(amax, sc->f8.amax[w][tok]);
+    for (int w = 0; w < 8; ++w) amax = fmaxf(amax, all[w][tok]);
     inv[p] = amax > 0.f ? 448.0f / amax : 0.0f;
     if (warp == 8 && tok < ti.rows) op->a_scale[(size_t)(ti.row0 + tok) * IB + ti.n] = amax > 0.f ? amax / 448.0f : 1.0f;
   }
-  named_barrier(1, 256);                            // read by all: the next tile may write
   unsigned char* out = reinterpret_cast<unsigned char*>(op->A) + (size_t)ti.row0 * a.I + (size_t)(ti.n * kTileN1 + half * 64 + q * 16);
 #pragma unroll
   for (int p = 0; p < kSlot / 32; ++p) {
@@ -571,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       mbar_init(&sc->pfull[s], 1);
       mbar_init(&sc->pempty[s], 8);
     }
-    for (int s = 0; s < 4; ++s) mbar_init(&sc->xbar[s], 64);
+    for (int s = 0; s < 4; ++s) mbar_init(&sc->xbar[s], kSmall ? 8 : 64);
     // a ring slot is released by the MMA warp, the committer and each gather warp
     for (int s = 0; s < kRing; ++s) {
       mbar_init(&sc->ifull[s], 1);
@@ -972,8 +977,8 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       if (ti.kind == kCombine) {
         combine_tokens(op, ti.row0, ti.row0 + ti.rows, args.k, args.H, etid, 256, CombineNow{});
       } else if constexpr (kSmall) {
-        ok = ti.rows <= 32 ? epilogue_fp8_small<32>(c, sc, op, ti, tmem, warp, lane, eph, kseq)
-                           : epilogue_fp8_small<64>(c, sc, op, ti, tmem, warp, lane, eph, kseq);
+        ok = ti.rows <= 32 ? epilogue_fp8_small<32>(c, sc, op, ti, tmem, warp, lane, eph, xph, kseq)
+                           : epilogue_fp8_small<64>(c, sc, op, ti, tmem, warp, lane, eph, xph, kseq);
       } else if constexpr (kFp8) {
         ok = epilogue_fp8(c, sc, op, ti, tmem, warp, lane, eph, xph);
       } else {

@@ -49,3 +49,37 @@ def test_every_kind_of_launch_leaves_a_clean_state(dtype, n_ctas):
         ctx.run([0, 1], fuse_combine=True)
         ctx.check()
         assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
+
+
+@pytest.mark.parametrize("dtype,T", [("fp8", 20), ("fp8", 48)])
+def test_small_launches_end_when_they_are_aborted(dtype, T):
+    """An index out of range met in the middle of a launch and a ready word that nothing sets both stop it: every role leaves, also the
+    epilogue warps that wait for one another, the error is reported, and the launches behind it are right again."""
+    spec = synth.Spec("abort", synth.Shape(16, 4, 1024, 512, dtype), ((synth.PREFILL, T), (synth.DECODE, T)), "uniform", None, 1.0, -1.0, 73)
+    W = weights_to(synth.make_weights(spec))
+    ctx = make_ctx(spec, wait_limit_us=2000)
+    bound = bind_ops(ctx, synth.make_ops(spec), W)
+
+    def launch():
+        ctx.run([0, 1], fuse_combine=True)
+        torch.cuda.synchronize()
+        return ctx.status()[0]
+
+    for s, b in enumerate(bound):
+        ctx.plan(s, b)
+    assert launch() == moe.MOE_OK
+    want = [b.y.clone() for b in bound]
+    word = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(3):
+        bound[0].sorted_to_flat[3] = 1 << 28
+        assert launch() == moe.MOE_EBOUNDS
+        ctx.plan(0, bound[0])
+        bound[1].c.ready = word.data_ptr()
+        ctx.plan(1, bound[1])
+        assert launch() == moe.MOE_ETIMEOUT
+        bound[1].c.ready = None
+        ctx.plan(1, bound[1])
+        for b in bound:
+            b.y.zero_()
+        assert launch() == moe.MOE_OK
+        assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
