@@ -70,6 +70,7 @@ struct SharedCtl {
   unsigned long long taken[kRing];   // leader's: its producer has started on the tile
   unsigned long long rows_in[kRing]; // own: the rows that the tile reads are in place (down tiles: its gate/up tiles are committed)
   unsigned long long began;          // leader's: the queue tables and qt.run_off are in place
+  unsigned combine_ready;            // own: combine tiles so far whose op's expert outputs were seen in place
   unsigned tmem_base;
   alignas(16) unsigned char epi_scratch[8][2048];
   QueueTables qt;
@@ -202,15 +203,30 @@ __device__ __forceinline__ void issue_kblock(SharedCtl<kTileRows>* sc, unsigned 
                     smem_u32(&sc->goA[stage]), p.g1 ? 1u : 0u, l2_evict_first());
 }
 
-// The epilogue warps' wait inside a combine tile: one thread of the CTA looks at the op's counter, the others meet it at a barrier.
+// The epilogue warps' wait inside a combine tile: one lane of the CTA looks at the op's counter and counts the tile (its `turn`-th) in
+// shared memory, where a lane of every warp looks.  Bounded like every wait: any of the warps may have left because the launch was
+// aborted.  (With all lanes looking, or on an mbarrier, one token takes 65.4 us a pass where it takes 63.6 this way.)
 struct CombineWhenDone {
   const Ctx* c;
   const OpDev* op;
+  unsigned* ready;
+  unsigned turn;
   bool look;
   __device__ __forceinline__ bool operator()() const {
-    if (look) wait_counter(*c, &run_of(*c, op)->gemm_done, op_gemm_tiles(op) * kStoreWarps, 4);
-    named_barrier(1, 256);
-    return !aborted(*c);
+    if (look && wait_counter(*c, &run_of(*c, op)->gemm_done, op_gemm_tiles(op) * kStoreWarps, 4)) st_release_cta(ready, turn);
+    __syncwarp();
+    const bool first = (threadIdx.x & 31) == 0;
+    unsigned long long t0 = 0;
+    for (unsigned it = 1;; ++it) {
+      int state = 0;                                 // 1: in place, -1: give up
+      if (first) {
+        if (ld_acquire_cta(ready) >= turn) state = 1;
+        else if ((it & 63u) == 0 && !still_waiting(*c, t0, 29)) state = -1;
+      }
+      state = __shfl_sync(0xffffffffu, state, 0);
+      if (state != 0) return state > 0;
+      __nanosleep(20);
+    }
   }
 };
 
@@ -263,6 +279,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       mbar_init(&sc->rows_in[s], 1);
     }
     mbar_init(&sc->began, 1);
+    sc->combine_ready = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_proxy();
   }
@@ -582,7 +599,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     const int half = (warp - 8) >> 2;             // the two warps of a quadrant split the tokens
     const int etid = threadIdx.x - 256;
     int islot = 0;
-    unsigned iph = 0, gcount = 0;
+    unsigned iph = 0, gcount = 0, combines = 0;
     bool first = true;
     unsigned char* scratch = sc->epi_scratch[warp - 8];
     const unsigned scratch_addr = smem_u32(scratch);
@@ -604,7 +621,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       bool ok = true;
       if (ti.kind == kCombine) {
         const int mid = ti.row0 + (ti.rows + 1) / 2;
-        const CombineWhenDone ready{&c, op, warp == 8 && lane == 0};
+        const CombineWhenDone ready{&c, op, &sc->combine_ready, ++combines, warp == 8 && lane == 0};
         ok = combine_tokens(op, leader ? ti.row0 : mid, leader ? mid : ti.row0 + ti.rows, args.k, args.H, etid, 256, ready);
         if (!ok) break;
       } else {

@@ -51,8 +51,8 @@ def test_every_kind_of_launch_leaves_a_clean_state(dtype, n_ctas):
         assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
 
 
-@pytest.mark.parametrize("dtype,T", [("fp8", 20), ("fp8", 48)])
-def test_small_launches_end_when_they_are_aborted(dtype, T):
+@pytest.mark.parametrize("dtype,T", [("fp8", 20), ("fp8", 48), ("bf16", 20), ("bf16", 100), ("bf16", 600)])
+def test_launches_end_when_they_are_aborted(dtype, T):
     """An index out of range met in the middle of a launch and a ready word that nothing sets both stop it: every role leaves, also the
     epilogue warps that wait for one another, the error is reported, and the launches behind it are right again."""
     spec = synth.Spec("abort", synth.Shape(16, 4, 1024, 512, dtype), ((synth.PREFILL, T), (synth.DECODE, T)), "uniform", None, 1.0, -1.0, 73)
