@@ -173,6 +173,7 @@ struct RunArgs {
   const int4* tile_list[kMaxOps];
   signed char cls[kMaxOps];
   signed char free_op[kMaxOps];     // 1: the op has no ready word and no predecessor
+  signed char carrier[kMaxOps];     // paired prefill op: which of the launch's decode ops carries rows of it (0: the first), else -1
 };
 
 // ------------------------------------------------------------------ launches that overlap the tail of the one before

@@ -446,6 +446,11 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     a.tile_list[i] = h.tile_list;
     a.cls[i] = (signed char)h.cls;
     a.free_op[i] = h.ready == nullptr && h.after_op < 0 ? 1 : 0;
+    a.carrier[i] = -1;
+    if (ctx->ran_paired[slots[i]] && h.cls == MOE_CLASS_PREFILL) {
+      a.carrier[i] = 0;
+      for (int j = 0; slots[j] != ctx->pair_of[slots[i]]; ++j) a.carrier[i] += ctx->ops[slots[j]].cls == MOE_CLASS_DECODE ? 1 : 0;
+    }
     const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
     const int rows = ctx->ran_paired[slots[i]] ? full : ctx->work_rows[slots[i]];
     a.work_rows = rows > a.work_rows ? rows : a.work_rows;
@@ -503,6 +508,7 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream) {
   a.tile_list[0] = ctx->host_ops[slot].tile_list;
   a.cls[0] = (signed char)ctx->host_ops[slot].cls;
   a.free_op[0] = 1;
+  a.carrier[0] = -1;
   a.work_rows = ctx->work_rows[slot];
   if (ps.n_gemm_tiles > 0 && launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, st) != cudaSuccess) return MOE_ECUDA;
   if (ctx->ops[slot].layout == MOE_LAYOUT_GATHERED &&

@@ -31,6 +31,7 @@ struct QueueTables {
   int all_gemm[2][kMaxOps];        // gemm_done when its combine may run
   const int4* list[2][kMaxOps];
   unsigned cum[2][kMaxOps + 1];
+  int carrier[2][kMaxOps];         // paired prefill op: the decode op (its place in that class) whose GEMM entries carry its rows, else -1
 };
 
 // ------------------------------------------------------------------ bounded waits
@@ -169,14 +170,21 @@ __device__ inline void finish_empty_ops(const Ctx& c, int finished) {
   }
 }
 
+// whether the decode queue's head has passed the GEMM entries of its op `j` (-1: there are none to pass)
+__device__ __forceinline__ bool carriers_claimed(const QueueTables* sc, int j, unsigned decode_head) {
+  return j < 0 || decode_head >= sc->cum[MOE_CLASS_DECODE][j] + sc->n_gemm[MOE_CLASS_DECODE][j];
+}
+
 // Claim by the whole producer warp.  1: claimed (ti filled), 0: queue exhausted, -1: the op
 // at the head of the queue is not ready.  The head is only peeked before the fetch-add, so no
 // CTA can be starved by others (a compare-and-swap loop starves the SMs far from the counter);
 // the price is that a ticket can land just past an op boundary, in an op that is not ready
 // yet -- the caller then waits for it (bounded), holding only tickets whose predecessors in
 // the queue are all claimed already.
-// early_combine: also take a combine entry whose GEMM entries are still running.
-__device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int cls, unsigned h,
+// early_combine: also take a combine entry whose GEMM entries are still running -- all of them must have been claimed, or every unit
+// could end up holding such an entry with none left for what they wait for.  The op's own are (the head stands behind them); those of
+// the decode list that carry rows of a paired prefill op are once the head of the decode queue, other_head, has passed them.
+__device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int cls, unsigned h, unsigned other_head,
                                 int lane, TileInfo& ti, bool& need_ready, bool early_combine = false) {
   const RunArgs* a = c.a;
   const int n = sc->n_cls[cls];
@@ -196,8 +204,10 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
     if (!sc->cls_free[cls][i] && !op_ready(c, op)) takeable = 0;
     // The head stands at the op's combine entries while GEMM entries they depend on are still running
     // (other units hold them; for a paired prefill op, the decode list's carrier tiles): nothing to take here
-    // yet -- the caller turns to the other class instead of holding a combine ticket it cannot run.
-    else if (!early_combine && base >= sc->n_gemm[cls][i] && ld_acquire(&run_of(c, op)->gemm_done) < sc->all_gemm[cls][i]) takeable = 0;
+    // yet -- the caller turns to the other class first.
+    else if (base >= sc->n_gemm[cls][i] && !(early_combine && carriers_claimed(sc, sc->carrier[cls][i], other_head)) &&
+             ld_acquire(&run_of(c, op)->gemm_done) < sc->all_gemm[cls][i])
+      takeable = 0;
   }
   if (__shfl_sync(0xffffffffu, takeable, 0) == 0) return -1;
   // the 32 entries from the head on are fetched while the fetch-add is in flight
@@ -246,8 +256,7 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
 // word and both queue heads are loaded together (one round trip), then at most one
 // fetch-add per class.
 // kEarlyCombine: a unit that finds nothing to run in either class takes a combine entry that has to wait for GEMM entries running
-// elsewhere, so that the wait for the last of them starts with the entry in hand (the caller must then not hold up
-// anything else with it).
+// elsewhere (see try_claim), so that the wait for the last of them starts with the entry in hand.  It claims nothing more meanwhile.
 // seen: the words as the unit's start read them (its first claim); they only tell where to look, the fetch-add decides.
 template <bool kEarlyCombine>
 __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int lane, TileInfo& ti,
@@ -281,12 +290,12 @@ __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int
     for (int p = 0; p < 4; ++p) {
       if (p >= 2 && none[p & 1] == 0) continue;
       const int cls = (p & 1) ? 1 - first : first;
-      none[p & 1] = try_claim(c, sc, rh, cls, cls == 0 ? h0 : h1, lane, ti, need_ready, p >= 2);
+      none[p & 1] = try_claim(c, sc, rh, cls, cls == 0 ? h0 : h1, cls == 0 ? h1 : h0, lane, ti, need_ready, p >= 2);
       if (none[p & 1] == 1) break;
     }
   } else {                                       // (in a loop this kernel's scheduler spills)
-    none[0] = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, lane, ti, need_ready);
-    if (none[0] != 1) none[1] = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, lane, ti, need_ready);
+    none[0] = try_claim(c, sc, rh, first, first == 0 ? h0 : h1, 0u, lane, ti, need_ready);
+    if (none[0] != 1) none[1] = try_claim(c, sc, rh, 1 - first, first == 0 ? h1 : h0, 0u, lane, ti, need_ready);
   }
   if (none[0] == 1 || none[1] == 1) {
     if (a->log_cap > 0) ti.t_claim = gtime_ns();
@@ -472,6 +481,7 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
       sc->n_gemm[ci][j] = (unsigned)gi;
       sc->all_gemm[ci][j] = ai;
       sc->list[ci][j] = a->tile_list[i];
+      sc->carrier[ci][j] = a->carrier[i];
     }
   }
   const unsigned turn = __shfl_sync(0xffffffffu, word, kW);

@@ -175,6 +175,56 @@ def test_paired_ops_with_done_words_and_a_successor():
         assert_close(b.y.float().cpu().numpy(), oracle.forward(OW, op.x, None, op.ids, op.w)["y"])
 
 
+@pytest.mark.parametrize("T,after_op", [(600, False), (1600, False), (600, True)])
+def test_a_decode_op_that_becomes_ready_when_its_prefill_partner_waits_for_it(T, after_op):
+    """The decode op of a pair becomes ready only after all GEMM tiles of the prefill op's own list have committed -- by its own ready word,
+    or as the successor of an op whose ready word it is.  Every unit is idle then, the prefill op's combine entries (more of them than units)
+    wait for the rows that decode tiles carry, and the units still have to serve those.  Outputs equal the both-ready launch."""
+    import time
+    shape = synth.Shape(16, 4, 512, 256)
+    spec = synth.Spec("lateready", shape, ((synth.PREFILL, T), (synth.DECODE, 70), (synth.DECODE, 9)), "zipf", 0.8, 1.0, -1.0, 28)
+    W = weights_to(synth.make_weights(spec))
+    ops = synth.make_ops(spec)
+    ctx = make_ctx(spec, max_tokens=T + 70, max_ops=3, wait_limit_us=300000)
+    words = torch.zeros(2, dtype=torch.int32).pin_memory()        # [0] ready (host -> device), [1] notify (device -> host)
+    host = words.numpy()
+    cp, cd = (np.bincount(o.ids.reshape(-1), minlength=shape.E) for o in ops[:2])
+    tail = cp % 256                                               # what the carriers of 256 rows take, where it fits
+    take = np.where((cd > 0) & (tail <= -cd % 256), tail, 0)
+    assert take.sum() > 0
+    own = int((-(-(cp - take) // 256)).sum()) * (shape.I // 128 + shape.H // 256)
+    bound = bind_ops(ctx, ops, W)
+    b0 = bind_ops(ctx, ops[:1], W, notify=words[1:2], notify_after=own)[0]
+    b1 = bind_ops(ctx, ops[1:2], W, **(dict(after_op=2) if after_op else dict(ready=words[0:1])))[0]
+    b2 = bind_ops(ctx, ops[2:], W, **(dict(ready=words[0:1]) if after_op else {}))[0]
+
+    def plan(bs):
+        for s, b in enumerate(bs):
+            ctx.plan(s, b)
+        ctx.plan_pair(0, 1, 256)
+        torch.cuda.synchronize()
+
+    plan(bound)
+    ctx.run([0, 2, 1], fuse_combine=True)
+    ctx.check()
+    want = [b.y.clone() for b in bound]
+    for budget in (0, 148):
+        ctx.set_budget(budget)
+        plan((b0, b1, b2))
+        host[:] = 0
+        ctx.run([0, 2, 1], fuse_combine=True)
+        t0 = time.perf_counter()
+        while host[1] == 0 and time.perf_counter() - t0 < 0.2:
+            pass
+        assert host[1] == 1
+        time.sleep(0.005)                                         # the units look around meanwhile
+        host[0] = 1
+        ctx.check()
+        for b, y in zip((b0, b1, b2), want):
+            assert torch.equal(b.y, y)
+            b.y.zero_()
+
+
 @pytest.mark.parametrize("shape", [synth.Shape(8, 2, 512, 256, "fp8"), synth.Shape(16, 4, 768, 384, "fp8")], ids=["h512", "h768"])
 def test_paired_fp8_equals_unpaired_and_mirrored_oracle(shape):
     spec = synth.Spec("fp8p", shape, ((synth.PREFILL, 300), (synth.DECODE, 37)), "softmax_topk", None, 1.0, -1.0, 35)
