@@ -45,6 +45,7 @@ constexpr int kAccCols = 256;
 // part is out: one token takes 63.9 us a pass where 65.9 with one thread that counts for all of them after they have met.  (In the
 // e4m3 kernel the same costs registers that its epilogue needs, 4 % at 2000 tokens: there the committer counts.)
 constexpr int kStoreWarps = 16;
+constexpr long long kBeginLimitNs = 1000000000;         // for two round trips of the scheduler
 constexpr int kFullCount = 2 + kGatherThreads + 1;
 // instruction descriptor: D fp32, A/B bf16, K-major, M = 256 over the pair, N = the tile's columns
 constexpr unsigned kIdescM256 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4) << 24);
@@ -571,7 +572,13 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // ============================================================ committer (leader)
     int islot = 0;
     unsigned iph = 0;
-    if (wwait(c, &sc->began, 0u, 28)) {
+    // The scheduler's arrival comes whatever the state of the launch, and the other half has to be cleared in any case (this launch turns
+    // the halves over): neither the abort word, which may be set from before, nor a short wait limit ends this wait.
+    unsigned long long t0 = 0;
+    bool begun = true;
+    for (unsigned it = 1; begun && !__all_sync(0xffffffffu, mbar_try(&sc->began, 0u)); ++it)
+      if ((it & 63u) == 0) begun = __all_sync(0xffffffffu, in_time(c, t0, kBeginLimitNs, 28));
+    if (begun) {
       if (blockIdx.x == 0) clear_next_run(&args, rh, sc->qt.run_off, lane);
       set_run_off();
       if (blockIdx.x == 0 && lane == 0) finish_empty_ops(c, -1);

@@ -49,17 +49,19 @@ __device__ __forceinline__ int* g1_done_of(const Ctx& c, const OpDev* op) {
 
 __device__ __forceinline__ bool aborted(const Ctx& c) { return ld_volatile(&c.st->abort) != 0; }
 
-// One look of a wait at the abort word and the clock (t0: 0 at the wait's start): false when it has to give up.
+// One look of a wait at the clock (t0: 0 at the wait's start), or at the abort word and the clock: false when it has to give up.
 // where: a small code telling which wait gave up (reported in detail[0])
-__device__ __noinline__ inline bool still_waiting(const Ctx& c, unsigned long long& t0, int where) {
-  if (aborted(c)) return false;
+__device__ __noinline__ inline bool in_time(const Ctx& c, unsigned long long& t0, long long limit_ns, int where) {
   const unsigned long long now = gtime_ns();
   if (t0 == 0) t0 = now;
-  else if ((long long)(now - t0) > c.a->wait_ns) {
+  else if ((long long)(now - t0) > limit_ns) {
     report(c.st, MOE_ETIMEOUT, where, (int)blockIdx.x, (int)threadIdx.x, 0);
     return false;
   }
   return true;
+}
+__device__ __forceinline__ bool still_waiting(const Ctx& c, unsigned long long& t0, int where) {
+  return !aborted(c) && in_time(c, t0, c.a->wait_ns, where);
 }
 __device__ __noinline__ inline bool mbar_wait_slow(const Ctx& c, void* bar, unsigned parity, int where) {
   unsigned long long t0 = 0;

@@ -83,3 +83,32 @@ def test_launches_end_when_they_are_aborted(dtype, T):
             b.y.zero_()
         assert launch() == moe.MOE_OK
         assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
+
+
+@pytest.mark.parametrize("dtype,n_ctas", [("bf16", 0), ("bf16", 3), ("fp8", 0)], ids=["pairs", "single", "fp8"])
+@pytest.mark.parametrize("launches", [1, 2], ids=["one_half", "other_half"])
+def test_a_launch_behind_a_rejected_plan_leaves_a_clean_state(dtype, n_ctas, launches):
+    """A plan with an expert id out of range sets the abort word before the launch behind it begins.  That launch does nothing, but it
+    too has to clear the half of the run state that the next one works on; both halves have been used by then."""
+    spec = synth.Spec("rejected", synth.Shape(8, 2, 512, 256, dtype), ((synth.DECODE, 37),), "uniform", None, 1.0, -1.0, 77)
+    ctx = make_ctx(spec, n_ctas=n_ctas, tile_log_entries=1 << 12)
+    b = bind_ops(ctx, synth.make_ops(spec), weights_to(synth.make_weights(spec)))[0]
+    ctx.plan(0, b)
+    for _ in range(1 + launches):                     # both halves, and either parity for what follows
+        ctx.run([0], fuse_combine=True)
+    ctx.check()
+    want, n, good = b.y.clone(), len(ctx.tile_log()), b.topk_ids.clone()
+    for _ in range(2):
+        b.topk_ids[5, 1] = 99
+        ctx.plan(0, b)
+        ctx.run([0], fuse_combine=True)
+        torch.cuda.synchronize()
+        assert ctx.status()[0] == moe.MOE_EBADID
+        assert len(ctx.tile_log()) == 0
+        b.topk_ids.copy_(good)
+        ctx.plan(0, b)
+        for _ in range(2):
+            b.y.zero_()
+            ctx.run([0], fuse_combine=True)
+            ctx.check()
+            assert len(ctx.tile_log()) == n and torch.equal(b.y, want)
