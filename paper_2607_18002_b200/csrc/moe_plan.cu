@@ -414,7 +414,7 @@ cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int w
   const size_t smem = (size_t)kPlanWarps * E * sizeof(int);
   if (a.R <= kPlanDirectRows) {
     const int blocks = list_blocks(E);
-    a.own = ((a.R + blocks - 1) / blocks + kPlanThreads - 1) / kPlanThreads * kPlanThreads;
+    a.own = max(1, ((a.R + blocks - 1) / blocks + kPlanThreads - 1) / kPlanThreads) * kPlanThreads;   // (an op without tokens too)
     return launch_after(plan_rank_kernel<true>, blocks, kPlanThreads, smem, stream, a);
   }
   a.own = kPlanThreads * (int)(((long long)a.R + kPlanThreads * kPlanMaxBlocks - 1) / (kPlanThreads * kPlanMaxBlocks));

@@ -61,3 +61,21 @@ def test_more_low_tiles_than_mtiles(dtype, T):
         ref = oracle.forward(oracle_weights(spec, W), op.x, op.x_scale, op.ids, op.w,
                              round_A=oracle.ROUND_NONE if dtype == "bf16" else oracle.ROUND_E4M3_1X128)["y"]
         assert_close(b.y.float().cpu().numpy(), ref, **tol)
+
+
+@pytest.mark.parametrize("E", [1, 8, 33, 256, 1024])
+def test_an_op_without_tokens(E):
+    """Its blocks own no rows: zero counts and offsets, no tiles, nothing written to the permutation, whatever the slot held before."""
+    spec = synth.Spec("empty", synth.Shape(E, 1, 256, 128), ((synth.DECODE, 40), (synth.DECODE, 0)), "uniform", None, 1.0, -1.0, 9)
+    ctx = make_ctx(spec, max_ops=1)
+    full, empty = bind_ops(ctx, synth.make_ops(spec), weights_to(synth.make_weights(spec)))
+    for _ in range(2):
+        ctx.plan(0, full)
+        for t in (empty.counts, empty.offsets, empty.sorted_to_flat, empty.flat_to_sorted):
+            t.fill_(77)
+        ctx.plan(0, empty)
+        ctx.run([0], fuse_combine=True)
+        ctx.check()
+        assert ctx.footprint(0) == (0, 0)
+        assert not empty.counts.any() and not empty.offsets.any()
+        assert empty.sorted_to_flat.tolist() == [77] and empty.flat_to_sorted.tolist() == [77]
