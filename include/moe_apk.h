@@ -18,6 +18,9 @@
  *   - `stream` is a cudaStream_t passed as void*.  Calls only enqueue work; none of
  *     them synchronises the host except moe_status and moe_read_tile_log.
  *   - Row-major everywhere.  bf16 = 2-byte bfloat16, e4m3 = 1-byte OCP E4M3FN.
+ *   - Everything but moe_run_plain and the calls that read back can be captured in a CUDA graph.  A
+ *     captured moe_plan / moe_plan_pair binds its op again on every replay; a moe_run captured
+ *     without the plans of its slots runs what they are planned for when it is replayed.
  *   - Return value: 0 on success, a negative MOE_E* code otherwise.  Errors that only
  *     the device can see (an expert id out of range, a wait that ran out) are recorded
  *     in a device status word and read back with moe_status after a stream sync; a

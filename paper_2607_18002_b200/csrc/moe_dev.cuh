@@ -55,7 +55,9 @@ struct PlanState {
   int n_comb_tiles;   // queue entries of kind combine (follow the GEMM entries)
   int planned;        // 1 after a moe_plan that accepted every expert id, else 0
   int n_extra_gemm;   // paired prefill op: GEMM entries of the decode op's list that carry rows of this op
-  int pad[3];
+  int work_rows;      // most rows of a GEMM entry
+  int cls;            // of the op that was planned
+  int free_op;        // 1: it has no ready word and no predecessor
 };
 
 // Part of the run state, see RunHead.
@@ -169,11 +171,10 @@ struct RunArgs {
   int static_kind;        // -1: persistent launch served from the queues.  >= 0: a plain launch, claiming unit u
                           // of the grid runs queue entry u of slots[0] and ends
   int slots[kMaxOps];     // descriptor indices of the launch's ops, in the order given
-  const PlanState* plan[kMaxOps];   // of slots[i]; with the three below all that the queue tables are built from
+  const PlanState* plan[kMaxOps];   // of slots[i], as tile_list: where a slot keeps them.  What depends on the op that is bound to a slot
+                                    // is read there and in its descriptor: a captured launch may be replayed on another op
   const int4* tile_list[kMaxOps];
-  signed char cls[kMaxOps];
-  signed char free_op[kMaxOps];     // 1: the op has no ready word and no predecessor
-  signed char carrier[kMaxOps];     // paired prefill op: which of the launch's decode ops carries rows of it (0: the first), else -1
+  signed char carrier[kMaxOps];     // paired prefill op: its decode op's place in `slots` (that op's tiles carry rows of it), else -1
 };
 
 // ------------------------------------------------------------------ launches that overlap the tail of the one before

@@ -109,6 +109,28 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// When the device has a descriptor, and when it has to be sent again.  A plan in a stream capture always brings its descriptor along,
+// so that a replay runs the op that was captured, whatever the slot has been bound to since; and a slot that has been in a capture
+// may have been rebound by a replay, which the host does not see.
+struct Upload {
+  bool sent;                    // the host's copy is what the last upload carries
+  bool captured;                // one of the uploads was captured
+  unsigned long long capture;   // where the last upload is: a capture, 0: none
+  bool there(unsigned long long cap) const { return sent && (cap ? capture == cap : !captured); }
+  void now(unsigned long long cap) { sent = true; captured |= cap != 0; capture = cap; }
+};
+
+// the capture that is under way on a stream, 0: none
+unsigned long long capture_of(cudaStream_t stream) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(stream, &status, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return status == cudaStreamCaptureStatusActive ? id | 1ull << 63 : 0;
+}
+
 }  // namespace
 
 struct moe_ctx {
@@ -122,11 +144,11 @@ struct moe_ctx {
   moe_op_t ops[kMaxOps];
   bool planned[kMaxOps];
   OpDev host_ops[kMaxOps];      // what the device copy of each slot holds (tensor maps included)
-  bool uploaded[kMaxOps];
   OpDev host_pair[kMaxOps];     // what the device copy of each slot's paired descriptor holds
-  bool pair_uploaded[kMaxOps];
+  Upload up[kMaxOps], pair_up[kMaxOps];
   int pair_of[kMaxOps];         // slot paired with this one by moe_plan_pair since both were last planned, or -1
   int work_rows[kMaxOps];       // rows of a work tile of the slot's plan
+  unsigned long long plan_capture[kMaxOps];   // the stream capture that plan was issued in, 0: none
   bool ran_paired[kMaxOps];     // the slot's last moe_run used its paired form (moe_combine follows it)
   Global* g() const { return reinterpret_cast<Global*>(ws + L.global_off); }
   RunHead* rh() const { return reinterpret_cast<RunHead*>(ws + L.run_off); }
@@ -256,15 +278,28 @@ int moe_create(const moe_config_t* cfg, void* dev_workspace, size_t bytes, moe_c
   ctx->poison = poison && poison[0] == '1';
   ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
   memset(ctx->planned, 0, sizeof(ctx->planned));
-  memset(ctx->uploaded, 0, sizeof(ctx->uploaded));
+  memset(ctx->up, 0, sizeof(ctx->up));
+  memset(ctx->pair_up, 0, sizeof(ctx->pair_up));
+  memset(ctx->plan_capture, 0, sizeof(ctx->plan_capture));
   memset(ctx->ran_paired, 0, sizeof(ctx->ran_paired));
-  memset(ctx->pair_uploaded, 0, sizeof(ctx->pair_uploaded));
   for (int s = 0; s < kMaxOps; ++s) ctx->pair_of[s] = -1;
   // zero the control blocks (status, budget, run state, plan states)
   cudaError_t e = cudaMemset(ctx->ws, 0, L.slots_off);
   for (int s = 0; s < cfg->max_ops && e == cudaSuccess; ++s) {
     e = cudaMemset(ctx->slot_base(s) + L.plan_off, 0, sizeof(PlanState));
     if (e == cudaSuccess) e = cudaMemset(ctx->slot_base(s) + L.pplan_off, 0, sizeof(PlanState));
+  }
+  // A plan that was captured and not replayed yet counts as issued: a launch on its slot has to find a descriptor, of an op without tiles.
+  for (int d = 0; d < 2 * cfg->max_ops && e == cudaSuccess; ++d) {
+    const int s = d % cfg->max_ops;
+    OpDev h;
+    memset(&h, 0, sizeof(h));
+    h.after_op = h.partner = -1;
+    h.plan = reinterpret_cast<PlanState*>(ctx->slot_base(s) + (d < cfg->max_ops ? L.plan_off : L.pplan_off));
+    h.run = reinterpret_cast<RunState*>(ctx->rs_base(s));
+    h.g1_done = reinterpret_cast<int*>(ctx->rs_base(s) + sizeof(RunState));
+    h.status = &ctx->g()->status;
+    e = cudaMemcpy(ctx->op_dev(d), &h, sizeof(h), cudaMemcpyHostToDevice);
   }
   if (e != cudaSuccess) { delete ctx; return MOE_ECUDA; }
   *out = ctx;
@@ -339,11 +374,14 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
   ctx->ran_paired[slot] = false;
   // Re-planning a slot with the same buffers (the usual serving loop) reuses the descriptors
   // already on the device: encoding seven tensor maps and uploading them is host time.
-  const bool same = ctx->uploaded[slot] && memcmp(&ctx->ops[slot], op, sizeof(moe_op_t)) == 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (!same) {
+  const unsigned long long cap = capture_of(st);
+  const bool same = ctx->up[slot].sent && memcmp(&ctx->ops[slot], op, sizeof(moe_op_t)) == 0;
+  if (!same || !ctx->up[slot].there(cap)) {
     int rc = MOE_OK;
-    if (op->n_tokens > 0 || masked) {
+    if (same) {
+      h = ctx->host_ops[slot];
+    } else if (op->n_tokens > 0 || masked) {
       rc = make_map(ctx, &h.tm_a8, h.A, (size_t)L.max_rows, (size_t)c.inter, 8);
       if (!rc) rc = make_map(ctx, &h.tm_a32, h.A, (size_t)L.max_rows, (size_t)c.inter, 32);
       if (!rc) rc = make_map(ctx, &h.tm_a128, h.A, (size_t)L.max_rows, (size_t)c.inter, 128);
@@ -370,10 +408,10 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
       if (rc) return rc;
     }
     ctx->planned[slot] = false;
-    if (launch_after(write_op_kernel, 1, 128, 0, st, h, ctx->op_dev(slot)) != cudaSuccess) { ctx->uploaded[slot] = false; return MOE_ECUDA; }
+    if (launch_after(write_op_kernel, 1, 128, 0, st, h, ctx->op_dev(slot)) != cudaSuccess) { ctx->up[slot].sent = false; return MOE_ECUDA; }
     ctx->host_ops[slot] = h;
     ctx->ops[slot] = *op;             // what the device copy of the slot now describes
-    ctx->uploaded[slot] = true;
+    ctx->up[slot].now(cap);
   }
   int work_rows = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
   const int most = masked ? op->slab_rows : op->n_tokens;       // rows an expert gets unless a token names it twice
@@ -383,6 +421,7 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
     work_rows = most <= kWorkRowsSmall ? kWorkRowsSmall : most <= kWorkRowsMid ? kWorkRowsMid : kWorkRowsBf16;
   }
   ctx->work_rows[slot] = work_rows;
+  ctx->plan_capture[slot] = cap;
   const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, st)
                                 : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, st);
   if (pe != cudaSuccess) {
@@ -439,25 +478,26 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   a.wait_ns = (long long)c.wait_limit_us * 1000;
   a.static_kind = -1;
   a.run_bytes = (unsigned)ctx->L.run_bytes;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const unsigned long long cap = capture_of(st);
+  const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
   bool weights_once = true;
   for (int i = 0; i < n_ops; ++i) {
     const OpDev& h = ctx->ran_paired[slots[i]] ? ctx->host_pair[slots[i]] : ctx->host_ops[slots[i]];
     a.plan[i] = h.plan;
     a.tile_list[i] = h.tile_list;
-    a.cls[i] = (signed char)h.cls;
-    a.free_op[i] = h.ready == nullptr && h.after_op < 0 ? 1 : 0;
     a.carrier[i] = -1;
-    if (ctx->ran_paired[slots[i]] && h.cls == MOE_CLASS_PREFILL) {
-      a.carrier[i] = 0;
-      for (int j = 0; slots[j] != ctx->pair_of[slots[i]]; ++j) a.carrier[i] += ctx->ops[slots[j]].cls == MOE_CLASS_DECODE ? 1 : 0;
-    }
-    const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
-    const int rows = ctx->ran_paired[slots[i]] ? full : ctx->work_rows[slots[i]];
+    if (ctx->ran_paired[slots[i]] && h.cls == MOE_CLASS_PREFILL)
+      for (int j = 0; j < n_ops; ++j)
+        if (slots[j] == ctx->pair_of[slots[i]]) a.carrier[i] = (signed char)j;
+    // The kernels for small ops have room for small work tiles only.  Plan and launch captured together are replayed together; a launch
+    // captured by itself runs whatever the slot has been planned for by then.
+    const bool any_plan = ctx->ran_paired[slots[i]] || ctx->plan_capture[slots[i]] != cap;
+    const int rows = any_plan ? full : ctx->work_rows[slots[i]];
     a.work_rows = rows > a.work_rows ? rows : a.work_rows;
     const moe_op_t& op = ctx->ops[slots[i]];
-    if (ctx->ran_paired[slots[i]] || (op.layout == MOE_LAYOUT_MASKED ? op.slab_rows : op.n_tokens) > rows) weights_once = false;
+    if (any_plan || (op.layout == MOE_LAYOUT_MASKED ? op.slab_rows : op.n_tokens) > rows) weights_once = false;
   }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (ctx->poison) {
     for (int i = 0; i < n_ops; ++i) {
       unsigned char* sb = ctx->slot_base(slots[i]);
@@ -506,10 +546,8 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream) {
   a.run_bytes = (unsigned)ctx->L.run_bytes;
   a.plan[0] = ctx->host_ops[slot].plan;
   a.tile_list[0] = ctx->host_ops[slot].tile_list;
-  a.cls[0] = (signed char)ctx->host_ops[slot].cls;
-  a.free_op[0] = 1;
   a.carrier[0] = -1;
-  a.work_rows = ctx->work_rows[slot];
+  a.work_rows = ps.work_rows;
   if (ps.n_gemm_tiles > 0 && launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, st) != cudaSuccess) return MOE_ECUDA;
   if (ctx->ops[slot].layout == MOE_LAYOUT_GATHERED &&
       launch_combine(ctx->op_dev(slot), ctx->ops[slot].n_tokens, c.top_k, c.hidden, st) != cudaSuccess)
@@ -567,14 +605,15 @@ int moe_plan_pair(moe_ctx_t* ctx, int slot_prefill, int slot_decode, int carrier
     h->partner = c.max_ops + (i == 0 ? sd : sp);
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const unsigned long long cap = capture_of(st);
   // the usual loop pairs the same two ops on the same buffers again and again: upload only what changed
   const int which[2] = {sp, sd};
   for (int i = 0; i < 2; ++i) {
     const int s = which[i];
-    if (ctx->pair_uploaded[s] && memcmp(&ctx->host_pair[s], both[i], sizeof(OpDev)) == 0) continue;
-    if (launch_after(write_op_kernel, 1, 128, 0, st, *both[i], ctx->op_dev(c.max_ops + s)) != cudaSuccess) { ctx->pair_uploaded[s] = false; return MOE_ECUDA; }
+    if (ctx->pair_up[s].there(cap) && memcmp(&ctx->host_pair[s], both[i], sizeof(OpDev)) == 0) continue;
+    if (launch_after(write_op_kernel, 1, 128, 0, st, *both[i], ctx->op_dev(c.max_ops + s)) != cudaSuccess) { ctx->pair_up[s].sent = false; return MOE_ECUDA; }
     ctx->host_pair[s] = *both[i];
-    ctx->pair_uploaded[s] = true;
+    ctx->pair_up[s].now(cap);
   }
   if (launch_plan_pair(hd, hp, ctx->host_ops[sd], ctx->host_ops[sp], gather_m, reinterpret_cast<int*>(bd + L.pcomb_off),
                        reinterpret_cast<int*>(bp + L.pcomb_off), c.n_experts, L.NT1, L.NT2,

@@ -61,6 +61,12 @@ __device__ __forceinline__ void warp_scan(int* out, const int* rows, int E, F f)
 // tile: a power of two
 __device__ __forceinline__ int tiles_of(int rows, int tile) { return (rows + tile - 1) >> (31 - __clz(tile)); }
 
+// what a launch needs to know of the op before it looks at its descriptor
+struct OpKind {
+  int cls, free_op;
+};
+static OpKind kind_of(const OpDev& h) { return OpKind{h.cls, h.ready == nullptr && h.after_op < 0 ? 1 : 0}; }
+
 // ---------------------------------------------------------------- the ordered tile list of one op
 // Writes this block's share of the queue list of an op whose expert e holds rows [off[e], off[e] + cnt[e]) of the
 // packed row space (cnt / off / work in shared memory; work[e]: work tiles of the experts before e), and (block 0) its
@@ -70,7 +76,7 @@ __device__ __forceinline__ int tiles_of(int rows, int tile) { return (rows + til
 // Order: the gate/up entries in expert order, and the down entries of an expert in front of the first expert whose
 // gate/up tiles start at least kLagWork work tiles behind its own, so by the time a down tile is claimed the tiles it
 // depends on were claimed long before.  Every entry's place follows from the prefix sum of the work tiles.
-__device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan, const int* cnt, const int* off, const int* work,
+__device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan, OpKind op, const int* cnt, const int* off, const int* work,
                                                 int E, int NT1, int NT2, int T, int work_rows, int x_moe, int planned,
                                                 int n_extra_gemm, int g1_kind = kGateUp) {
   const int n_work = work[E];
@@ -115,7 +121,9 @@ __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan,
     ps.n_comb_tiles = n_comb;
     ps.planned = planned;                   // a plan with a rejected id leaves the slot without tiles to run
     ps.n_extra_gemm = n_extra_gemm;
-    ps.pad[0] = ps.pad[1] = ps.pad[2] = 0;
+    ps.work_rows = work_rows;
+    ps.cls = op.cls;
+    ps.free_op = op.free_op;
     *plan = ps;
   }
   return n_gemm;
@@ -134,6 +142,7 @@ struct PlanArgs {
   int4* tile_list;
   PlanState* plan;
   Status* status;
+  OpKind op;
   int slot, R, E, T, NT1, NT2, work_rows;
   int own;              // rows per block: block b owns rows [b * own, (b + 1) * own)
 };
@@ -259,7 +268,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
   if (blockIdx.x == 0 && tid < E)
     for (int j = 0, m0 = s_mtile[tid], me = s_mtile[tid + 1] - m0; j < me; ++j)
       a.mtiles[m0 + j] = MTile{tid, off + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
-  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, s_work, E, a.NT1, a.NT2, a.T, a.work_rows, s_mtile[E], total == R ? 1 : 0, 0);
+  build_tile_list(a.tile_list, a.plan, a.op, s_cnt, s_off, s_work, E, a.NT1, a.NT2, a.T, a.work_rows, s_mtile[E], total == R ? 1 : 0, 0);
 }
 
 // ---------------------------------------------------------------- masked layout
@@ -292,7 +301,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_
       for (int j = 0, m0 = s_mtile[e], me = s_mtile[e + 1] - m0; j < me; ++j)
         a.mtiles[m0 + j] = MTile{e, e * slab_rows + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
   }
-  build_tile_list(a.tile_list, a.plan, s_cnt, s_off, s_work, E, a.NT1, a.NT2, 0, a.work_rows, s_mtile[E], 1, 0, kGateUpDirect);
+  build_tile_list(a.tile_list, a.plan, a.op, s_cnt, s_off, s_work, E, a.NT1, a.NT2, 0, a.work_rows, s_mtile[E], 1, 0, kGateUpDirect);
 }
 
 // ---------------------------------------------------------------- the paired form of a decode + prefill op
@@ -313,6 +322,7 @@ struct PairSide {
   PlanState* plan;
   int* comb;                  // flat routed index -> row of the shared space
   int R, T, slot;
+  OpKind op;
 };
 struct PairArgs {
   PairSide d, p;
@@ -354,10 +364,10 @@ __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_co
   if (e < 32) warp_scan(work_d, cnt_d, E, [&](int rows) { return tiles_of(rows, rows_d); });
   else if (e < 64) warp_scan(work_p, cnt_p, E, [&](int rows) { return tiles_of(rows, a.work_rows); });
   __syncthreads();
-  const int n_dec = build_tile_list(a.d.tile_list, a.d.plan, cnt_d, off_d, work_d, E, a.NT1, a.NT2, a.d.T, rows_d,
+  const int n_dec = build_tile_list(a.d.tile_list, a.d.plan, a.d.op, cnt_d, off_d, work_d, E, a.NT1, a.NT2, a.d.T, rows_d,
                                     a.d.plain->n_mtiles, ok, 0);
   // every GEMM entry of the decode list may carry prefill rows: the prefill op is complete when they are too
-  build_tile_list(a.p.tile_list, a.p.plan, cnt_p, off_p, work_p, E, a.NT1, a.NT2, a.p.T, a.work_rows, a.p.plain->n_mtiles, ok,
+  build_tile_list(a.p.tile_list, a.p.plan, a.p.op, cnt_p, off_p, work_p, E, a.NT1, a.NT2, a.p.T, a.work_rows, a.p.plain->n_mtiles, ok,
                   n_dec);
   // the shared row space's permutation
   for (int i = (int)(blockIdx.x * kPlanThreads + threadIdx.x); i < a.d.R + a.p.R; i += (int)gridDim.x * kPlanThreads) {
@@ -383,6 +393,7 @@ cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2
   PlanArgs a{};
   a.counts = h.counts; a.offsets = h.offsets; a.mtiles = h.mtiles; a.tile_list = h.tile_list; a.plan = h.plan;
   a.status = h.status;
+  a.op = kind_of(h);
   a.slot = slot; a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows;
   return launch_after(plan_masked_kernel, list_blocks(E), kPlanThreads, 0, stream, a, slab_rows);
 }
@@ -391,8 +402,8 @@ cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, c
                              int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows,
                              int slot_d, int slot_p, cudaStream_t stream) {
   PairArgs a{};
-  a.d = PairSide{d.topk_ids, d.counts, d.offsets, d.flat_to_sorted, d.plan, hd.tile_list, hd.plan, comb_d, d.n_rows, d.n_tokens, slot_d};
-  a.p = PairSide{p.topk_ids, p.counts, p.offsets, p.flat_to_sorted, p.plan, hp.tile_list, hp.plan, comb_p, p.n_rows, p.n_tokens, slot_p};
+  a.d = PairSide{d.topk_ids, d.counts, d.offsets, d.flat_to_sorted, d.plan, hd.tile_list, hd.plan, comb_d, d.n_rows, d.n_tokens, slot_d, kind_of(d)};
+  a.p = PairSide{p.topk_ids, p.counts, p.offsets, p.flat_to_sorted, p.plan, hp.tile_list, hp.plan, comb_p, p.n_rows, p.n_tokens, slot_p, kind_of(p)};
   a.gather = gather;
   a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows; a.carrier_rows = carrier_rows;
   const int blocks = max(list_blocks(E), min(kPlanMaxBlocks, (d.n_rows + p.n_rows + kPlanThreads - 1) / kPlanThreads));
@@ -410,6 +421,7 @@ cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int w
   PlanArgs a{};
   a.ids = h.topk_ids; a.counts = h.counts; a.offsets = h.offsets; a.s2f = h.sorted_to_flat; a.f2s = h.flat_to_sorted;
   a.hist = h.plan_hist; a.mtiles = h.mtiles; a.tile_list = h.tile_list; a.plan = h.plan; a.status = h.status;
+  a.op = kind_of(h);
   a.slot = slot; a.R = h.n_rows; a.E = E; a.T = h.n_tokens; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows;
   const size_t smem = (size_t)kPlanWarps * E * sizeof(int);
   if (a.R <= kPlanDirectRows) {

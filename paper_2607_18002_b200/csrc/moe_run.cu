@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   grid_dep_wait();             // everything above overlaps the kernel before this one
-  if (warp == 0) begin_unit(&args, &sc->qt, rh, lane, 1);
+  if (warp == 0) begin_unit(&args, &sc->qt, rh, lane, 1, Ring<kMode>::kARows);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

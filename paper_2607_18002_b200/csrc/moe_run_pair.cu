@@ -319,7 +319,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     ti.kind = kEnd;
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
     ti.t_claim = 0;
-    const ClaimWords seen = begin_unit(&args, &sc->qt, rh, lane, kStoreWarps);
+    const ClaimWords seen = begin_unit(&args, &sc->qt, rh, lane, kStoreWarps, kTileRows);
     set_run_off();
     if (lane == 0) mbar_arrive(&sc->began);
     const bool plain = args.static_kind >= 0;             // plain launch: this pair runs one given entry

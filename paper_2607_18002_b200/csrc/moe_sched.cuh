@@ -448,8 +448,8 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
 // unit's first claim (heads: of both halves, the half is only known when they arrive).  All of it is one round trip: lane i reads
 // the plan of op i, the last lanes a word each.  The unit asks for the half with a plain load; the fetch-add that counts it
 // (take_turn) comes later, so that no claim waits behind those of all other units.
-// per_tile: what a committed GEMM entry adds to gemm_done.
-__device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const RunHead* first_half, int lane, int per_tile) {
+// per_tile: what a committed GEMM entry adds to gemm_done.  max_rows: the tallest work tile this kernel has room for.
+__device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const RunHead* first_half, int lane, int per_tile, int max_rows) {
   constexpr int kW = 25;
   static_assert(kMaxOps <= kW, "a lane per op, and one per word");
   const RunHead* second = reinterpret_cast<const RunHead*>(reinterpret_cast<const char*>(first_half) + a->run_bytes);
@@ -461,11 +461,17 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
     word = *reinterpret_cast<const volatile unsigned*>(p);
   }
   PlanState ps{};
-  int cls = 0;
+  int cls = -1;
   if (lane < a->n_ops) {
     ps = *a->plan[lane];
-    cls = a->cls[lane];
+    cls = ps.cls;
+    // The host picks the kernel by the plans it has issued.  A graph replayed in between can have left another plan in the slot.
+    if (ps.planned != 0 && ps.work_rows > max_rows) {
+      report(&a->g->status, MOE_EBOUNDS, slot_of(a, a->slots[lane]), ps.work_rows, max_rows, 5);
+      ps.planned = 0;
+    }
   }
+  const unsigned decode_ops = __ballot_sync(0xffffffffu, cls == MOE_CLASS_DECODE);
   const int entries = ps.planned == 0 ? 0 : ps.n_gemm_tiles + (a->fuse_combine ? ps.n_comb_tiles : 0);
   const int all_gemm = (ps.n_gemm_tiles + ps.n_extra_gemm) * per_tile;
   if (lane == 0) {
@@ -475,15 +481,16 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
   for (int i = 0; i < a->n_ops; ++i) {
     const int ei = __shfl_sync(0xffffffffu, entries, i), ci = __shfl_sync(0xffffffffu, cls, i);
     const int gi = __shfl_sync(0xffffffffu, ps.n_gemm_tiles, i), ai = __shfl_sync(0xffffffffu, all_gemm, i);
+    const int fi = __shfl_sync(0xffffffffu, ps.free_op, i);
     if (lane == 0) {
       const int j = sc->n_cls[ci]++;
       sc->cls_slot[ci][j] = a->slots[i];
-      sc->cls_free[ci][j] = a->free_op[i];
+      sc->cls_free[ci][j] = fi;
       sc->cum[ci][j + 1] = sc->cum[ci][j] + (unsigned)ei;
       sc->n_gemm[ci][j] = (unsigned)gi;
       sc->all_gemm[ci][j] = ai;
       sc->list[ci][j] = a->tile_list[i];
-      sc->carrier[ci][j] = a->carrier[i];
+      sc->carrier[ci][j] = a->carrier[i] < 0 ? -1 : __popc(decode_ops & ((1u << a->carrier[i]) - 1u));
     }
   }
   const unsigned turn = __shfl_sync(0xffffffffu, word, kW);

@@ -255,7 +255,7 @@ def test_a_whole_layer_step_replays_from_a_cuda_graph():
         ctx.plan_pair(0, 1, 0)
         ctx.run([0, 1], fuse_combine=True)
 
-    step()                                     # first calls upload the descriptors: keep them out of the capture
+    step()                                     # first calls may load device code: keep them out of the capture
     ctx.check()
     y0 = [b.y.clone() for b in bound]
     side = torch.cuda.Stream()
