@@ -233,7 +233,7 @@ def moe_plan_static(topk_ids_ptr: int, n_tokens: int, top_k: int, n_experts: int
 
 def moe_route(logits_ptr: int, n_tokens: int, n_experts: int, top_k: int, ids_ptr: int, w_ptr: int,
               stream: int) -> None:
-    rc = (_lib or lib()).moe_route(logits_ptr, int(n_tokens), int(n_experts), int(top_k), ids_ptr, w_ptr, stream)
+    rc = (_lib or lib()).moe_route(logits_ptr, n_tokens, n_experts, top_k, ids_ptr, w_ptr, stream)
     if rc:
         raise MoeError(rc, "moe_route")
 

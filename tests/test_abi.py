@@ -73,16 +73,6 @@ def test_binding_structs_match_what_a_c_compiler_makes_of_the_header(tmp_path):
                    o.layout.offset, o.slab_rows.offset]
 
 
-def test_router_sizes_may_be_any_integer_type(built):
-    """Sizes read from an array are numpy integers; a call of zero tokens launches nothing and needs no GPU."""
-    import numpy as np
-    for t in (int, np.int32, np.int64):
-        moe.moe_route(0, t(0), t(8), t(2), 0, 0, 0)
-        with pytest.raises(moe.MoeError) as ei:
-            moe.moe_route(0, t(0), t(8), t(9), 0, 0, 0)
-        assert ei.value.code == moe.MOE_EINVAL
-
-
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(moe, "_lib", None)
     monkeypatch.setattr(moe, "LIB_PATH", str(tmp_path / "nope.so"))
