@@ -319,7 +319,21 @@ def bind_masked_op(cls: int, x_slabs, counts, w_gate_up, w_down, x_scale=None, s
     return BoundOp(c_op, keep)
 
 
-_get_device = _raw_stream = None   # torch's own, set by the first Context
+def _current_stream() -> int:
+    """The handle of the current stream of the current device."""
+    import torch
+    return int(torch.cuda.current_stream().cuda_stream)
+
+
+def _stream_reader():
+    """The same without a Stream object around it, where this torch has the two functions (they are not public)."""
+    import torch
+    torch.cuda.init()
+    device, raw = (getattr(torch._C, n, None) for n in ("_cuda_getDevice", "_cuda_getCurrentRawStream"))
+    return _current_stream if device is None or raw is None else lambda: raw(device())
+
+
+_read_stream = None                # set by the first call that needs it
 
 
 class Context:
@@ -332,8 +346,6 @@ class Context:
         import torch
         if not torch.cuda.is_available():
             raise RuntimeError("no CUDA device: this library has no CPU path")
-        global _get_device, _raw_stream
-        _get_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
         lib()
         self.cfg = moe_config_t(n_experts, top_k, hidden, inter, dtype, max_tokens_per_op,
                                 max_ops, wait_limit_us, tile_log_entries, n_ctas)
@@ -358,8 +370,10 @@ class Context:
     def _stream(stream) -> int:
         if stream is not None:
             return int(stream.cuda_stream)
-        # the handle of the current stream of the current device, without a Stream object around it
-        return _raw_stream(_get_device())
+        global _read_stream
+        if _read_stream is None:
+            _read_stream = _stream_reader()
+        return _read_stream()
 
     def bind(self, cls, x, topk_ids, topk_w, w_gate_up, w_down, **kw) -> BoundOp:
         return bind_op(cls, x, topk_ids, topk_w, w_gate_up, w_down, self.cfg.top_k,
