@@ -153,6 +153,9 @@ struct RunHead {
   int pad[5];
 };
 
+// the half that the last launch worked on
+__host__ __device__ inline unsigned last_run_off(unsigned turn, unsigned run_bytes) { return (turn >> 31) ? 0u : run_bytes; }
+
 struct RunArgs {
   Global* g;
   OpDev* ops;             // indexed by slot

@@ -205,6 +205,12 @@ __global__ void set_word_kernel(int* p, int v) {
   *reinterpret_cast<volatile int*>(p) = v;
 }
 
+// the tile log of a run without tiles: no records (the ones of the run before are in the half that it worked on)
+__global__ void empty_log_kernel(const Global* g, RunHead* first_half, unsigned run_bytes) {
+  grid_dep_wait();
+  reinterpret_cast<RunHead*>(reinterpret_cast<char*>(first_half) + last_run_off(g->turn, run_bytes))->log_count = 0;
+}
+
 // The op descriptor travels as a kernel parameter (no pageable-memory copy on the stream).
 __global__ void write_op_kernel(const __grid_constant__ OpDev src, OpDev* dst) {
   grid_dep_wait();
@@ -548,7 +554,11 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream) {
   a.tile_list[0] = ctx->host_ops[slot].tile_list;
   a.carrier[0] = -1;
   a.work_rows = ps.work_rows;
-  if (ps.n_gemm_tiles > 0 && launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, st) != cudaSuccess) return MOE_ECUDA;
+  if (ps.n_gemm_tiles > 0) {
+    if (launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, st) != cudaSuccess) return MOE_ECUDA;
+  } else if (launch_after(empty_log_kernel, 1, 1, 0, st, ctx->g(), ctx->rh(), (unsigned)ctx->L.run_bytes) != cudaSuccess) {
+    return MOE_ECUDA;
+  }
   if (ctx->ops[slot].layout == MOE_LAYOUT_GATHERED &&
       launch_combine(ctx->op_dev(slot), ctx->ops[slot].n_tokens, c.top_k, c.hidden, st) != cudaSuccess)
     return MOE_ECUDA;
@@ -700,7 +710,7 @@ int moe_read_tile_log(moe_ctx_t* ctx, moe_tile_rec_t* host_out, int max_records,
   Global g;
   RunHead rh;
   if (cudaMemcpy(&g, ctx->g(), sizeof(g), cudaMemcpyDeviceToHost) != cudaSuccess) return MOE_ECUDA;
-  const size_t half = (g.turn >> 31) ? 0 : ctx->L.run_bytes;            // the one the last launch worked on
+  const size_t half = last_run_off(g.turn, (unsigned)ctx->L.run_bytes);
   if (cudaMemcpy(&rh, reinterpret_cast<unsigned char*>(ctx->rh()) + half, sizeof(rh), cudaMemcpyDeviceToHost) != cudaSuccess)
     return MOE_ECUDA;
   int cnt = (int)rh.log_count;

@@ -112,3 +112,22 @@ def test_a_launch_behind_a_rejected_plan_leaves_a_clean_state(dtype, n_ctas, lau
             ctx.run([0], fuse_combine=True)
             ctx.check()
             assert len(ctx.tile_log()) == n and torch.equal(b.y, want)
+
+
+def test_a_plain_run_without_tiles_has_an_empty_log():
+    spec = synth.Spec("nolog", synth.Shape(8, 2, 512, 256), ((synth.DECODE, 37), (synth.DECODE, 0)), "uniform", None, 1.0, -1.0, 79)
+    ctx = make_ctx(spec, tile_log_entries=1 << 12)
+    bound = bind_ops(ctx, synth.make_ops(spec), weights_to(synth.make_weights(spec)))
+    for s, b in enumerate(bound):
+        ctx.plan(s, b)
+    for _ in range(3):
+        ctx.run([0], fuse_combine=True)
+        ctx.check()
+        n = len(ctx.tile_log())
+        assert n == ctx.footprint(0)[1]
+        ctx.run_plain(1)
+        ctx.check()
+        assert len(ctx.tile_log()) == 0
+        ctx.run_plain(0)
+        ctx.check()
+        assert 0 < len(ctx.tile_log()) < n            # without the combine
