@@ -487,7 +487,7 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const unsigned long long cap = capture_of(st);
   const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
-  bool weights_once = true;
+  bool weights_once = true;              // no op reads a weight byte twice
   for (int i = 0; i < n_ops; ++i) {
     const OpDev& h = ctx->ran_paired[slots[i]] ? ctx->host_pair[slots[i]] : ctx->host_ops[slots[i]];
     a.plan[i] = h.plan;

@@ -97,7 +97,8 @@ __device__ __forceinline__ int quadrant_rows(int rows) { return rows <= 64 ? 16 
 // partials.  The token scales of every k-block are copied by the gather warps into a ring: what the epilogue has not read when
 // a k-block's are written is two groups and the five k-blocks in the stages, of the ring's sixteen.
 // Measured under the power cap (48 tokens, 200 experts of 256): 1245 -> 1108 us a pass at 1.58 -> 1.72 GHz, and
-// 8..10 % on 1 to 64 tokens over 8 to 256 experts.  A weight byte is read once a launch and leaves L2 first (1141 -> 1127 us).
+// 8..10 % on 1 to 64 tokens over 8 to 256 experts.  A weight byte is read once an op and leaves L2 first (1141 -> 1127 us;
+// two ops on the same weights, 48 + 32 tokens on 8 active experts: 122 -> 115).
 // Beyond 64 rows the scale of every column makes the epilogue longer than that of the tokens-as-M form, and a kernel that holds
 // both forms spills.
 constexpr unsigned kIdescF8M128 = (1u << 4) | ((128u >> 4) << 24);
@@ -545,9 +546,9 @@ struct AccUse {
   }
 };
 
-// kOnce: every expert's rows fit one work tile, the launch reads a weight byte once and marks it to leave L2 first (e4m3, 96 tokens on 8
-// experts: 111.1 -> 102.8 us a pass; 128 on 8: 114.5 -> 107.6, on 32: 257.2 -> 251.4).  A kernel of its own: the choice at each load
-// cost launches of larger ops 0.9 %.
+// kOnce: every expert's rows of an op fit one work tile, the op reads a weight byte once and marks it to leave L2 first (e4m3, 96 tokens
+// on 8 experts: 111.1 -> 102.8 us a pass; 128 on 8: 114.5 -> 107.6, on 32: 257.2 -> 251.4; two ops on the same weights, 120 + 100 tokens
+// on 8 experts: 121 -> 109).  A kernel of its own: the choice at each load cost launches of larger ops 0.9 %.
 template <int kMode, bool kOnce>
 __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_constant__ RunArgs args,
                                                               RunHead* rh) {

@@ -193,8 +193,10 @@ __device__ __forceinline__ void issue_kblock(SharedCtl<kTileRows>* sc, unsigned 
                                              unsigned stage, bool leader, unsigned full0_addr) {
   const unsigned sX = stages_addr + stage * (unsigned)Ring<kTileRows>::kSB;
   const unsigned bar = full0_addr + stage * 8u;            // the leader's full[stage]
-  // Where the ops' tokens fit one work tile, a weight byte is read once a launch: marked to leave L2 first, it does not push out what
-  // is read again (one token: 72.7 -> 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  With experts of
+  // Where an op's tokens fit one work tile, the op reads a weight byte once: marked to leave L2 first, it does not push out what
+  // is read again (one token: 72.7 -> 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  Two unpaired ops of a
+  // launch that share their weights read it twice, at different times, and gain too (100 + 64 tokens on 64 experts: 397 -> 383, on 8
+  // active experts: 91 -> 84, on 32 experts of 3 MB: 84 -> 80; 30 + 20 tokens on 32 active experts lose, 213 -> 218).  With experts of
   // several tiles the weights are the data read again, and the mark costs (8192 tokens: 2390 -> 2510).
   constexpr bool kOnce = kTileRows != kWorkRowsBf16;
   pair_issue_kblock<kOnce>(bar, p.tx, smem_u32(&sc->full[stage]),
