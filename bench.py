@@ -742,6 +742,35 @@ def measure(name: str, args, K: int, Wm: int, rank: int, world: int, local: int,
     return res
 
 
+def short_line(full: dict) -> dict:
+    """What goes to standard output: one line that a reader of the last 3000 characters gets whole.  The other fields (tile statistics,
+    how the traffic was taken, every sub-result in full) go to standard error."""
+    def pick(d, keys):
+        return {k: d[k] for k in keys if k in d}
+
+    def rounded(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: rounded(x) for k, x in v.items()}
+        return [rounded(x) for x in v] if isinstance(v, list) else v
+
+    roof = ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "peak_source", "peak_kind", "launch_ms_mean")
+    line = {k: v for k, v in full.items() if k not in ("tiles", "one_launch_for_all_layers", "sub_results")}
+    line["config"] = {k: v for k, v in full["config"].items() if k != "buffers"}
+    line["roofline"] = pick(full["roofline"], roof)
+    for k in ("e2e", "e2e_serial"):
+        if k in full:
+            line[k] = {n: v for n, v in full[k].items() if n != "how"}
+    if "sub_results" in full:
+        line["sub_results"] = {}
+        for name, r in full["sub_results"].items():
+            line["sub_results"][name] = dict(pick(r, ("value", "unit", "ms_per_step", "dtype")),
+                                             roofline=pick(r["roofline"], ("bound", "achieved", "unit", "frac")),
+                                             clocks=pick(r["clocks"], ("sm_mhz", "reasons")))
+    return rounded(line)
+
+
 def run_ours(args):
     from paper_2607_18002_b200 import dist
     if not torch.cuda.is_available():
@@ -772,7 +801,8 @@ def run_ours(args):
         line.setdefault("cpu_baseline", None)
         if sub:
             line["sub_results"] = sub
-        print(json.dumps(line))
+        print(json.dumps(line), file=sys.stderr)
+        print(json.dumps(short_line(line)))
     dist.shutdown()
 
 
