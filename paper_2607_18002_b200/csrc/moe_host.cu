@@ -296,17 +296,19 @@ int moe_create(const moe_config_t* cfg, void* dev_workspace, size_t bytes, moe_c
     if (e == cudaSuccess) e = cudaMemset(ctx->slot_base(s) + L.pplan_off, 0, sizeof(PlanState));
   }
   // A plan that was captured and not replayed yet counts as issued: a launch on its slot has to find a descriptor, of an op without tiles.
-  for (int d = 0; d < 2 * cfg->max_ops && e == cudaSuccess; ++d) {
+  OpDev* first = e == cudaSuccess ? new (std::nothrow) OpDev[2 * cfg->max_ops]() : nullptr;
+  for (int d = 0; d < 2 * cfg->max_ops && first; ++d) {
     const int s = d % cfg->max_ops;
-    OpDev h;
-    memset(&h, 0, sizeof(h));
+    OpDev& h = first[d];
     h.after_op = h.partner = -1;
     h.plan = reinterpret_cast<PlanState*>(ctx->slot_base(s) + (d < cfg->max_ops ? L.plan_off : L.pplan_off));
     h.run = reinterpret_cast<RunState*>(ctx->rs_base(s));
     h.g1_done = reinterpret_cast<int*>(ctx->rs_base(s) + sizeof(RunState));
     h.status = &ctx->g()->status;
-    e = cudaMemcpy(ctx->op_dev(d), &h, sizeof(h), cudaMemcpyHostToDevice);
   }
+  if (e == cudaSuccess && !first) { delete ctx; return MOE_ENOSPC; }
+  if (e == cudaSuccess) e = cudaMemcpy(ctx->op_dev(0), first, sizeof(OpDev) * 2 * cfg->max_ops, cudaMemcpyHostToDevice);
+  delete[] first;
   if (e != cudaSuccess) { delete ctx; return MOE_ECUDA; }
   *out = ctx;
   return MOE_OK;
