@@ -5,6 +5,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "../../include/moe_apk.h"
@@ -57,8 +58,10 @@ struct PlanState {
   int n_extra_gemm;   // paired prefill op: GEMM entries of the decode op's list that carry rows of this op
   int work_rows;      // most rows of a GEMM entry
   int cls;            // of the op that was planned
-  int free_op;        // 1: it has no ready word and no predecessor
+  int flags;          // kOpFree, kOpWatched
 };
+constexpr int kOpFree = 1;      // it has no ready word and no predecessor
+constexpr int kOpWatched = 2;   // somebody looks at its progress: it has a done or a notify word, or it is chained behind another op of the run
 
 // Part of the run state, see RunHead.
 struct RunState {
@@ -125,6 +128,7 @@ struct __align__(128) OpDev {
   int partner;              // paired: descriptor index of the other op of the pair, else -1
   int pad_[2];
 };
+static_assert(offsetof(OpDev, cls) % 128 == 0 && sizeof(OpDev) > offsetof(OpDev, cls) + 256, "touch_ops reads three lines of it");
 constexpr int kRowSlotShift = 27;                       // a flat routed index stays below 2^27 (moe_create checks)
 constexpr int kRowFlatMask = (1 << kRowSlotShift) - 1;
 

@@ -63,9 +63,12 @@ __device__ __forceinline__ int tiles_of(int rows, int tile) { return (rows + til
 
 // what a launch needs to know of the op before it looks at its descriptor
 struct OpKind {
-  int cls, free_op;
+  int cls, flags;
 };
-static OpKind kind_of(const OpDev& h) { return OpKind{h.cls, h.ready == nullptr && h.after_op < 0 ? 1 : 0}; }
+static OpKind kind_of(const OpDev& h) {
+  return OpKind{h.cls, (h.ready == nullptr && h.after_op < 0 ? kOpFree : 0) |
+                           (h.done != nullptr || h.notify != nullptr || h.after_op >= 0 ? kOpWatched : 0)};
+}
 
 // ---------------------------------------------------------------- the ordered tile list of one op
 // Writes this block's share of the queue list of an op whose expert e holds rows [off[e], off[e] + cnt[e]) of the
@@ -123,7 +126,7 @@ __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan,
     ps.n_extra_gemm = n_extra_gemm;
     ps.work_rows = work_rows;
     ps.cls = op.cls;
-    ps.free_op = op.free_op;
+    ps.flags = op.flags;
     *plan = ps;
   }
   return n_gemm;

@@ -602,10 +602,12 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   const unsigned tmem = sc->tmem_base;
   c.run_off = sc->qt.run_off;
   if (warp == 3 && lane == 0) end_turn(&args, take_turn(&args), (int)gridDim.x);
+  const bool watched = sc->qt.watched != 0;
   if (blockIdx.x == 0 && warp == 3) {
     clear_next_run(&args, rh, c.run_off, lane);
-    if (lane == 0) finish_empty_ops(c, -1);
+    if (lane == 0 && watched) finish_empty_ops(c, -1);
   }
+  bool ended = true;           // false: this thread left its role because a wait gave up
   rh = reinterpret_cast<RunHead*>(reinterpret_cast<char*>(rh) + c.run_off);
   // The fp8 epilogue keeps 128 fp32 accumulators per thread: the two epilogue warpgroups take
   // registers from the two others (64 + 192 = 2 x 128 per thread pair).  Each role changes its
@@ -621,6 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     // kClaimAt-th k-block), so the claim's round trips and the first loads of the next tile
     // overlap the current tile's tail instead of draining the pipeline.  A CTA therefore
     // holds at most one claimed tile beyond the one it is executing.
+    ended = false;
     int stage = 0, islot = 0;
     unsigned ph = 0, iph = 0;
     TileInfo ti, nx;
@@ -650,7 +653,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
           mbar_arrive(&sc->ifull[islot]);
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (ti.kind == kEnd || !ok) break;
+        if (ti.kind == kEnd || !ok) { ended = ok; break; }
         if (++islot == kRing) { islot = 0; iph ^= 1u; }
       }
       ti_published = false;
@@ -728,6 +731,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   } else if (warp == 1) {
     control_regs();
     // ============================================================ MMA issuer
+    ended = false;
     int stage = 0, islot = 0;
     unsigned ph = 0, iph = 0, aph[2] = {0, 0}, pph = 0;
     AccUse accs;
@@ -736,7 +740,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       const int kind = sc->info[islot].kind;
       const int kblocks = sc->info[islot].kblocks;
       const int rows = sc->info[islot].rows;
-      if (kind == kEnd) break;
+      if (kind == kEnd) { ended = true; break; }
       bool fail = false;
       if (kFp8 && kind != kCombine) {
         // FP8 with fp32 block scales: the tensor core cannot apply a scale per 128-deep K block,
@@ -846,6 +850,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // rows covered by one cp.async per thread
     constexpr int kPasses = Ring<kMode>::kARows / kRowsPerPass;
     const int chunk = gt % kCpr, rbase = gt / kCpr;       // rows rbase + kRowsPerPass * j
+    ended = false;
     int islot = 0;
     unsigned iph = 0, kiter = 0;                          // kiter: k-blocks of all GEMM tiles so far
     while (true) {
@@ -856,7 +861,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       __syncwarp();
       if (lane == 0) mbar_arrive(&sc->iempty[islot]);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (kind == kEnd) break;
+      if (kind == kEnd) { ended = true; break; }
       if (kind == kCombine) continue;
       if (kind != kGateUp && !kSmall) {   // nothing to gather: hand every stage on empty-handed
         bool failed = false;
@@ -940,6 +945,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     // ============================================================ committer
     // Publishes a tile once all epilogue threads have arrived on the tile's barrier: the
     // barrier orders their stores before this warp's fence and release (cumulativity).
+    ended = false;
     int islot = 0;
     unsigned iph = 0;
     while (true) {
@@ -947,10 +953,10 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       TileInfo ti;
       if (lane == 0) ti = sc->info[islot];
       const int kind = __shfl_sync(0xffffffffu, lane == 0 ? ti.kind : 0, 0);
-      if (kind == kEnd) break;
+      if (kind == kEnd) { ended = true; break; }
       if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->done[islot], iph, 17))) break;
       if (lane == 0) {
-        commit_tile<true>(c, rh, ti);
+        commit_tile<true>(c, rh, ti, watched);
         mbar_arrive(&sc->iempty[islot]);
       }
       __syncwarp();
@@ -967,12 +973,13 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     int islot = 0;
     unsigned iph = 0, aph[2] = {0, 0}, eph = 0, xph = 0, kseq = 0;
     AccUse accs;
+    ended = false;
     unsigned char* scratch = sc->epi_scratch[warp - 8];
     const int srow = lane >> 2, schunk = lane & 3;          // this lane's part of a store
     while (true) {
       if (!__all_sync(0xffffffffu, mbar_wait_inline(c, &sc->ifull[islot], iph, 9))) break;
       const TileInfo ti = sc->info[islot];
-      if (ti.kind == kEnd) break;
+      if (ti.kind == kEnd) { ended = true; break; }
       OpDev* op = &args.ops[ti.slot];
       bool ok = true;
       if (ti.kind == kCombine) {
@@ -1062,10 +1069,9 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     control_regs();        // warp 3: idle, but its warpgroup changes its allowance together
   }
 
-  // teardown: nothing is claimed any more; let asynchronous work settle, then free TMEM
-  if (aborted(c)) __nanosleep(20000);
+  // teardown: nothing is claimed any more.  Where a role gave up, asynchronous work may be under way: let it settle.  Then free TMEM
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(!ended)) __nanosleep(20000);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");

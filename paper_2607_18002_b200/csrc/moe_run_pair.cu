@@ -236,7 +236,6 @@ struct CombineWhenDone {
 // the scheduler hands a tile to the roles of both CTAs
 template <int kTileRows>
 __device__ __forceinline__ void publish(SharedCtl<kTileRows>* sc, int islot, const TileInfo& ti) {
-  fence_async_proxy();
   sc->info[islot] = ti;
   const unsigned ra = map_to_cta(&sc->info[islot], 1);      // same layout as TileInfo
   st_cluster_v4(ra, make_uint4((unsigned)ti.kind, (unsigned)ti.slot, (unsigned)ti.tile, (unsigned)ti.m));
@@ -303,6 +302,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
   // From here to the first loads of a tile everything is latency: tables, first claim, hand-over.  So no barrier of the CTA stands in
   // between, only the scheduler's own two round trips (4300 + 3900 clocks to a claim before, 2750 + 3500 now).
   // The half of the run state is known to the scheduler first; the roles that need it read it behind a barrier.
+  bool ended = true;           // false: this thread left its role because a wait gave up
   const auto set_run_off = [&] {
     c.run_off = sc->qt.run_off;
     rh = reinterpret_cast<RunHead*>(reinterpret_cast<char*>(rh) + c.run_off);
@@ -328,7 +328,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     if (plain) claim_static(&args, (int)(blockIdx.x >> 1), ti);
     else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready, &seen);
     unsigned ticket = 0;
-    if (lane == 0) ticket = take_turn(&args);
+    bool asked = false;
+    ended = false;
     while (true) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
@@ -347,12 +348,15 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           mbar_arrive_cluster(map_to_cta(&sc->rows_in[islot], 1));
           mbar_arrive(&sc->rows_in[islot]);
         }
+        // (asked before the first hand-over, that would wait for the answer: its arrivals release)
+        if (!asked) ticket = take_turn(&args);
+        asked = true;
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
       // The gather warps will read the tile's row list (4 bytes per row) first thing: pull it into L2
       // now, the weight stream has usually pushed it out since the plan wrote it.
       if (ti.kind == kGateUp && lane * 32 < ti.rows) prefetch_l2(op->gather_list + ti.row0 + lane * 32);
-      if (ti.kind == kEnd || !ok) break;
+      if (ti.kind == kEnd || !ok) { ended = ok; break; }
       // A combine tile is handed over at once: its epilogue warps read row indices and router weights and then wait for the op's
       // GEMM tiles themselves.  The next claim waits with them, so that a unit holds one such tile at most.
       if (ti.kind == kCombine) {
@@ -364,11 +368,13 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (plain) ti.kind = kEnd;
       else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready);
     }
-    if (lane == 0) end_turn(&args, ticket, (int)(gridDim.x >> 1));
+    if (lane == 0) end_turn(&args, asked ? ticket : take_turn(&args), (int)(gridDim.x >> 1));
   } else if (warp == 3) {
     // ============================================================ producer (both CTAs)
     // Reads tiles from the ring and issues this CTA's loads, one stage per k-block.  The whole
     // warp runs the loop on warp-uniform values; one elected lane issues each instruction.
+    touch_ops(args, lane);
+    ended = false;
     int islot = 0;
     unsigned iph = 0;
     unsigned stage = 0, par = 1;                           // parity of "stage is free"
@@ -384,7 +390,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       ti.n = __shfl_sync(0xffffffffu, sc->info[islot].n, 0);
       ti.kblocks = __shfl_sync(0xffffffffu, sc->info[islot].kblocks, 0);
       ti.expert = __shfl_sync(0xffffffffu, sc->info[islot].expert, 0);
-      if (ti.kind == kEnd) break;
+      if (ti.kind == kEnd) { ended = true; break; }
       const int tslot = islot;
       const unsigned tph = iph;
       if (leader && lane == 0) mbar_arrive(&sc->taken[tslot]);
@@ -427,6 +433,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // The whole warp runs the loops with warp-uniform values and one elected lane issues each
     // MMA and commit: per k-block one barrier wait, four MMAs and one commit, which keeps
     // issuing ahead of the tensor pipe (about 512 clocks per k-block of a 256-row tile).
+    ended = false;
     int islot = 0;
     unsigned iph = 0, gcount = 0;
     unsigned stage = 0, par = 0;
@@ -436,7 +443,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kind = __shfl_sync(0xffffffffu, sc->info[islot].kind, 0);
       const int kblocks = __shfl_sync(0xffffffffu, sc->info[islot].kblocks, 0);
       const int rows = __shfl_sync(0xffffffffu, sc->info[islot].rows, 0);
-      if (kind == kEnd) break;
+      if (kind == kEnd) { ended = true; break; }
       if (kind != kCombine) {
         const unsigned b = gcount & 1u;
         if (!wwait(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
@@ -471,6 +478,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // ============================================================ gather relay (second CTA)
     // When this CTA's gather threads' copies of a stage have landed it makes them visible to the
     // tensor core (proxy fence) and arrives on the leader's stage barrier.
+    ended = false;
     int islot = 0;
     unsigned iph = 0, kiter = 0, amask = 0;
     while (true) {
@@ -478,7 +486,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kind = sc->info[islot].kind;
       const int kblocks = sc->info[islot].kblocks;
       __syncwarp();
-      if (kind == kEnd) break;
+      if (kind == kEnd) { ended = true; break; }
       if (lane == 0) arrive_at_leader(&sc->iempty[islot], false);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (kind == kCombine) continue;
@@ -508,6 +516,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // 16 rows per cp.async round
     constexpr int kPasses = Ring<kTileRows>::kRows / kRowsPerPass;
     const int chunk = gt % kCpr, rbase = gt / kCpr;
+    ended = false;
     int islot = 0;
     unsigned iph = 0, kiter = 0, gmask = 0;
     while (true) {
@@ -516,7 +525,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kblocks = sc->info[islot].kblocks;
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
       __syncwarp();
-      if (kind == kEnd) break;
+      if (kind == kEnd) { ended = true; break; }
       if (lane == 0) arrive_at_leader(&sc->iempty[islot], leader);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (kind == kCombine) continue;
@@ -577,23 +586,25 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // The scheduler's arrival comes whatever the state of the launch, and the other half has to be cleared in any case (this launch turns
     // the halves over): neither the abort word, which may be set from before, nor a short wait limit ends this wait.
     unsigned long long t0 = 0;
-    bool begun = true;
+    bool begun = true, watched = false;
+    ended = false;
     for (unsigned it = 1; begun && !__all_sync(0xffffffffu, mbar_try(&sc->began, 0u)); ++it)
       if ((it & 63u) == 0) begun = __all_sync(0xffffffffu, in_time(c, t0, kBeginLimitNs, 28));
     if (begun) {
       if (blockIdx.x == 0) clear_next_run(&args, rh, sc->qt.run_off, lane);
       set_run_off();
-      if (blockIdx.x == 0 && lane == 0) finish_empty_ops(c, -1);
+      watched = sc->qt.watched != 0;
+      if (blockIdx.x == 0 && lane == 0 && watched) finish_empty_ops(c, -1);
     }
     while (true) {
       if (!wait_info(c, &sc->ifull[islot], iph, 16, leader)) break;
       TileInfo ti;
       if (lane == 0) ti = sc->info[islot];
       const int kind = __shfl_sync(0xffffffffu, lane == 0 ? ti.kind : 0, 0);
-      if (kind == kEnd) break;
+      if (kind == kEnd) { ended = true; break; }
       if (!wwait_cluster(c, &sc->done[islot], iph, 17)) break;
       if (lane == 0) {
-        commit_tile<false>(c, rh, ti);
+        commit_tile<false>(c, rh, ti, watched);
         mbar_arrive(&sc->iempty[islot]);
       }
       __syncwarp();
@@ -607,6 +618,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     const int q = warp & 3;
     const int half = (warp - 8) >> 2;             // the two warps of a quadrant split the tokens
     const int etid = threadIdx.x - 256;
+    ended = false;
     int islot = 0;
     unsigned iph = 0, gcount = 0, combines = 0;
     bool first = true;
@@ -615,7 +627,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     while (true) {
       if (!wait_info(c, &sc->ifull[islot], iph, 9, leader)) break;
       const TileInfo ti = sc->info[islot];
-      if (ti.kind == kEnd) break;
+      if (ti.kind == kEnd) { ended = true; break; }
       OpDev* op = &args.ops[ti.slot];
       if (first) {
         first = false;
@@ -635,20 +647,22 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (!ok) break;
       } else {
         const int b = (int)(gcount & 1u);
+        // read ahead of the accumulator: behind it these round trips, through a memory system full of weights, delay the tiles that wait
+        // for this one (one token: 2.9 us from accumulator to store)
+        const bool g1 = ti.kind != kDown;                     // gate/up tile: SwiGLU, output to A
+        const StoredWords words = stored_words(c, op, ti);
+        unsigned char* const out0 = reinterpret_cast<unsigned char*>(g1 ? (void*)op->A : (void*)op->D);
         ok = wwait(c, &sc->tfull[b], (gcount >> 1) & 1u, 10);
         if (!ok) break;
         ++gcount;
         tc_fence_after();
-        const bool g1 = ti.kind != kDown;                     // gate/up tile: SwiGLU, output to A
-        const StoredWords words = stored_words(c, op, ti);
         const int cols = tile_cols(ti.rows) / 2;              // this warp's columns
         const int live = min(cols, ti.rows - half * cols);    // ... that hold token rows
         const int passes = (live + 31) / 32;
         if (passes > 0) {
           const unsigned taddr = tmem + (unsigned)(b * kAccCols + half * cols) + ((unsigned)(q * 32) << 16);
           const size_t pitch = (size_t)(g1 ? args.I : args.H) * 2;
-          unsigned char* out = reinterpret_cast<unsigned char*>(g1 ? (void*)op->A : (void*)op->D) +
-                               (size_t)(ti.row0 + half * cols) * pitch +
+          unsigned char* out = out0 + (size_t)(ti.row0 + half * cols) * pitch +
                                (size_t)(g1 ? ti.n * kTileN1 + rank * 64 + q * 16 : ti.n * kTileN2 + rank * 128 + q * 32) * 2;
           unsigned lo[16], hi[16];                            // lanes 0..15 and 16..31 of the quadrant
           tc_ld_frag(taddr, lo);
@@ -720,10 +734,9 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     }
   }
 
-  // teardown: nothing is claimed any more; let asynchronous work settle, then free TMEM
-  if (aborted(c)) __nanosleep(20000);
+  // teardown: nothing is claimed any more.  Where a role gave up, asynchronous work may be under way: let it settle.  Then free TMEM
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(!ended)) __nanosleep(20000);
   cluster_sync_all();          // no CTA leaves while the other may still signal its barriers
   if (warp == 1) {
     tc_fence_after();

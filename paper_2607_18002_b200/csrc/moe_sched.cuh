@@ -24,6 +24,7 @@ struct ClaimWords {
 // per-class queue tables of one launch (built once per CTA in shared memory)
 struct QueueTables {
   unsigned run_off;                // of this launch
+  int watched;                     // an op of the launch is: committed tiles are counted
   int n_cls[2];
   int cls_slot[2][kMaxOps];
   int cls_free[2][kMaxOps];        // 1: the op has no ready word and no predecessor
@@ -212,6 +213,8 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
       takeable = 0;
   }
   if (__shfl_sync(0xffffffffu, takeable, 0) == 0) return -1;
+  // what the op's ready word announced is read by TMA too
+  if (lane == 0 && !sc->cls_free[cls][i]) fence_async_proxy();
   // the 32 entries from the head on are fetched while the fetch-add is in flight
   const unsigned n_op = sc->cum[cls][i + 1] - sc->cum[cls][i];
   int4 e = make_int4(0, 0, 0, 0);
@@ -314,7 +317,7 @@ __device__ inline bool wait_op_ready(const Ctx& c, int lane, const TileInfo& ti)
   while (true) {
     int r = 0;                                   // 1: ready, -1: give up
     if (lane == 0) {
-      if (op_ready(c, &a->ops[ti.slot])) r = 1;
+      if (op_ready(c, &a->ops[ti.slot])) { r = 1; fence_async_proxy(); }
       else if (aborted(c)) r = -1;
       else if ((long long)(gtime_ns() - w0) > a->wait_ns) {
         report(c.st, MOE_ETIMEOUT, 11, (int)blockIdx.x, slot_of(a, ti.slot), ti.tile);
@@ -414,17 +417,20 @@ __device__ inline void count_commit(const Ctx& c, OpDev* op, int desc) {
   }
 }
 
-// Publishing a finished tile: op completion, done word, log, and unless the storing warps have done so (kCounts false) the words that
-// other tiles wait for.  Called by one thread after all writers of the tile have fenced and synchronised.
+// Publishing a finished tile: log, op completion and done word where an op of the launch is watched, and unless the storing warps have
+// done so (kCounts false) the words that other tiles wait for.  Called by one thread after all writers of the tile have fenced and
+// synchronised.  (A launch that nobody watches saves a chain of three round trips behind its last tile.)
 template <bool kCounts>
-__device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti) {
+__device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti, bool watched) {
   const RunArgs* a = c.a;
   OpDev* op = &a->ops[ti.slot];
   const unsigned long long t_commit = a->log_cap > 0 ? gtime_ns() : 0ull;   // before it is published
   if (kCounts && ti.kind != kCombine) count_stored(stored_words(c, op, ti));
-  else fence_acq_rel_gpu();
-  count_commit(c, op, ti.slot);
-  if (op->paired && op->cls == MOE_CLASS_DECODE && ti.kind != kCombine) count_commit(c, &a->ops[op->partner], op->partner);
+  else if (watched) fence_acq_rel_gpu();
+  if (watched) {
+    count_commit(c, op, ti.slot);
+    if (op->paired && op->cls == MOE_CLASS_DECODE && ti.kind != kCombine) count_commit(c, &a->ops[op->partner], op->partner);
+  }
   if (a->log_cap > 0) {
     const unsigned idx = atomicAdd(&rh->log_count, 1u);
     if (idx < (unsigned)a->log_cap) {
@@ -474,14 +480,16 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
   const unsigned decode_ops = __ballot_sync(0xffffffffu, cls == MOE_CLASS_DECODE);
   const int entries = ps.planned == 0 ? 0 : ps.n_gemm_tiles + (a->fuse_combine ? ps.n_comb_tiles : 0);
   const int all_gemm = (ps.n_gemm_tiles + ps.n_extra_gemm) * per_tile;
+  const unsigned watched = __ballot_sync(0xffffffffu, (ps.flags & kOpWatched) != 0);
   if (lane == 0) {
+    sc->watched = watched != 0;
     sc->n_cls[0] = sc->n_cls[1] = 0;
     sc->cum[0][0] = sc->cum[1][0] = 0;
   }
   for (int i = 0; i < a->n_ops; ++i) {
     const int ei = __shfl_sync(0xffffffffu, entries, i), ci = __shfl_sync(0xffffffffu, cls, i);
     const int gi = __shfl_sync(0xffffffffu, ps.n_gemm_tiles, i), ai = __shfl_sync(0xffffffffu, all_gemm, i);
-    const int fi = __shfl_sync(0xffffffffu, ps.free_op, i);
+    const int fi = __shfl_sync(0xffffffffu, ps.flags & kOpFree, i);
     if (lane == 0) {
       const int j = sc->n_cls[ci]++;
       sc->cls_slot[ci][j] = a->slots[i];
@@ -509,6 +517,22 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
 __device__ inline unsigned take_turn(const RunArgs* a) { return atomicAdd(&a->g->turn, 1u); }
 __device__ inline void end_turn(const RunArgs* a, unsigned ticket, int units) {
   if ((ticket & 0x7fffffffu) == (unsigned)units - 1u) atomicExch(&a->g->turn, ~ticket & 0x80000000u);
+}
+// One warp, while the unit's first claim is under way: the tensor maps of the launch's ops, and what the roles read of their descriptors
+// first thing, on their way to this SM.  (An op without rows has no maps.)
+__device__ __forceinline__ void touch_ops(const RunArgs& a, int lane) {
+  const int part = lane & 15;
+  for (int j = lane >> 4; j < a.n_ops; j += 2) {
+    const OpDev* op = &a.ops[a.slots[j]];
+    if (part < 3) {
+      int v;
+      asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<const char*>(&op->cls) + 128 * part) : "memory");
+    } else if (part < 9 && op->n_rows > 0) {
+      if (part < 7) prefetch_tensormap(part == 3 ? &op->tm_p1 : part == 4 ? &op->tm_p2 : part == 5 ? &op->tm_a8 : &op->tm_a32);
+      else if (op->masked) prefetch_tensormap(part == 7 ? &op->tm_x8 : &op->tm_x32);
+    }
+  }
+  __syncwarp();
 }
 // The launch parameters into the constant cache, while the kernel before still runs.
 __device__ __forceinline__ void touch_params(const RunArgs& a) {
