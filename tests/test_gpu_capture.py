@@ -92,6 +92,29 @@ def test_captured_steps_that_share_a_slot(dtype, n_ctas):
         _expect(ctx, bound[j], want[j], lambda: (step(bound[i]), whole[j].replay()))
 
 
+@pytest.mark.parametrize("dtype,n_ctas", [("bf16", 0), ("bf16", 3), ("fp8", 0)], ids=["pairs", "single", "fp8"])
+def test_a_captured_launch_counts_for_the_words_it_finds(dtype, n_ctas):
+    """Committed tiles are counted only where an op of the launch has a done or a notify word or a successor: whether one has is read
+    from the plan that the launch finds, not from the op that it was captured with."""
+    spec, W, ctx, bound, want = _setup(dtype, SIZES, n_ctas=n_ctas)
+    ctx.plan(0, bound[0])
+    g = _capture(lambda: ctx.run([0], fuse_combine=True))
+    words = torch.zeros(2, dtype=torch.int32, device="cuda")
+    d = upload(synth.make_ops(spec)[1], None)
+    args = (synth.PREFILL, d["x"], d["ids"], d["w"], W.w_gate_up, W.w_down)
+    scales = dict(x_scale=d["x_scale"], s_gate_up=W.s_gate_up, s_down=W.s_down)
+    for kw in (dict(done=words[:1]), dict(notify=words[1:], notify_after=3), dict(done=words[:1], notify=words[1:], notify_after=1)):
+        words.zero_()
+        b = ctx.bind(*args, **scales, **kw)
+        ctx.plan(0, b)
+        _expect(ctx, b, want[1], g.replay)
+        assert words.tolist() == [int("done" in kw), int("notify" in kw)]
+        words.zero_()
+        ctx.plan(0, bound[0])
+        _expect(ctx, bound[0], want[0], g.replay)
+        assert words.tolist() == [0, 0]
+
+
 def test_a_captured_pair_and_its_ops_by_themselves():
     spec, W, ctx, bound, want = _setup("bf16", SIZES)
 
