@@ -65,7 +65,7 @@ constexpr int kOpWatched = 2;   // somebody looks at its progress: it has a done
 
 // Part of the run state, see RunHead.
 struct RunState {
-  int gemm_done;      // committed GEMM tiles (CTA pairs: times the warps that store one)
+  int gemm_done;      // committed down tiles (CTA pairs: times the warps that store one)
   int tiles_done;     // committed tiles of any kind
   int done;           // 1 when the op has fully finished
   int pad;

@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         if (lane == 0) {
           // a claimed tile only ever waits on tiles that were claimed before it
           if (ti.kind == kDown) ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
-          if (ti.kind == kCombine) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op), 4);
+          if (ti.kind == kCombine) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_down_tiles(&args, op), 4);
           if (!ok) ti.kind = kEnd;
           fence_async_proxy();
           sc->info[islot] = ti;
@@ -701,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
               int met = 1;
               if (lane == 0) {
                 if (nx.kind == kDown) met = ld_acquire(&g1_done_of(c, nop)[nx.m]) >= args.I / kTileN1;
-                if (nx.kind == kCombine) met = ld_acquire(&run_of(c, nop)->gemm_done) >= op_gemm_tiles(nop);
+                if (nx.kind == kCombine) met = ld_acquire(&run_of(c, nop)->gemm_done) >= op_down_tiles(&args, nop);
                 if (met) {
                   fence_async_proxy();
                   sc->info[islot] = nx;

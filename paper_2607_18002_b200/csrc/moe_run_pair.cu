@@ -216,7 +216,7 @@ struct CombineWhenDone {
   unsigned turn;
   bool look;
   __device__ __forceinline__ bool operator()() const {
-    if (look && wait_counter(*c, &run_of(*c, op)->gemm_done, op_gemm_tiles(op) * kStoreWarps, 4)) st_release_cta(ready, turn);
+    if (look && wait_counter(*c, &run_of(*c, op)->gemm_done, op_down_tiles(c->a, op) * kStoreWarps, 4)) st_release_cta(ready, turn);
     __syncwarp();
     const bool first = (threadIdx.x & 31) == 0;
     unsigned long long t0 = 0;
@@ -360,7 +360,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       // A combine tile is handed over at once: its epilogue warps read row indices and router weights and then wait for the op's
       // GEMM tiles themselves.  The next claim waits with them, so that a unit holds one such tile at most.
       if (ti.kind == kCombine) {
-        if (lane == 0) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_gemm_tiles(op) * kStoreWarps, 4);
+        if (lane == 0) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_down_tiles(&args, op) * kStoreWarps, 4);
         if (__shfl_sync(0xffffffffu, ok, 0) == 0) break;
       }
       if (!wwait(c, &sc->taken[islot], iph, 26)) break;
@@ -724,7 +724,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);
         }
         __syncwarp();
-        if (lane == 0) count_stored(words);
+        const bool alone = ti.rows <= cols;                   // the columns of the quadrant's other warp hold no rows: one counts for both
+        if (lane == 0 && (half == 0 || !alone)) count_stored(words, alone ? 2 : 1);
       }
       // The warp's stores, before the tile is published: the arrival releases them (across the pair: at cluster scope), the
       // committer's fence is cumulative over what it acquires here

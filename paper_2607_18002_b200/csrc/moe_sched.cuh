@@ -135,8 +135,14 @@ __device__ __forceinline__ int op_queue_entries(const OpDev* op, int fuse) {
   if (op->plan->planned == 0) return 0;
   return op->plan->n_gemm_tiles + (fuse ? op->plan->n_comb_tiles : 0);
 }
-// GEMM entries that must have committed before the op's combine may run
-__device__ __forceinline__ int op_gemm_tiles(const OpDev* op) { return op->plan->n_gemm_tiles + op->plan->n_extra_gemm; }
+// Of `gemm` GEMM entries the down tiles.  They are what an op's combine waits for: none of them commits before its gate/up tiles.
+__device__ __forceinline__ int down_tiles(const RunArgs* a, int gemm) {
+  const int nt1 = a->I / kTileN1, nt2 = a->H / kTileN2;
+  return gemm / (nt1 + nt2) * nt2;
+}
+__device__ __forceinline__ int op_down_tiles(const RunArgs* a, const OpDev* op) {
+  return down_tiles(a, op->plan->n_gemm_tiles + op->plan->n_extra_gemm);
+}
 
 // An op without tiles (no tokens, or a plan that was rejected) never commits anything: it counts as
 // finished as soon as its own predecessor has, and its ready word is not consulted.
@@ -380,27 +386,27 @@ __device__ inline void claim_next(const Ctx& c, QueueTables* sc, RunHead* rh, in
   ti.kind = kEnd;
 }
 
-// The words that down and combine tiles wait for, for a tile of `op` (of a combine tile: not counted).  A GEMM entry of a paired
-// decode op carries rows of the prefill op too: it counts for both.
+// The words that wait for a tile of `op` (of a combine tile: not counted): a gate/up tile counts in g1_done of its work tile, where the
+// down tiles of those rows look; a down tile in gemm_done, where the combine tiles look, and if the entry is one of a paired decode op's,
+// which carry rows of the prefill op too, in that op's.  All units count at the end of a wave of tiles, and the words share an L2 slice:
+// gate/up tiles in gemm_done too, and every warp of a tile of one row, made 2400 atomics of what are 600 (one token on 8 experts).
 struct StoredWords {
-  int* rows;           // gate/up tiles: g1_done of the work tile
-  int* op;             // gemm_done
-  int* partner;        // ... of the other op
+  int* own;
+  int* partner;
 };
 __device__ __forceinline__ StoredWords stored_words(const Ctx& c, const OpDev* op, const TileInfo& ti) {
   StoredWords w;
-  w.rows = ti.kind != kDown ? &g1_done_of(c, op)[ti.m] : nullptr;
-  w.op = &run_of(c, op)->gemm_done;
-  w.partner = op->paired && ti.cls == MOE_CLASS_DECODE ? &run_of(c, &c.a->ops[op->partner])->gemm_done : nullptr;
+  const bool down = ti.kind == kDown;
+  w.own = down ? &run_of(c, op)->gemm_done : &g1_done_of(c, op)[ti.m];
+  w.partner = down && op->paired && ti.cls == MOE_CLASS_DECODE ? &run_of(c, &c.a->ops[op->partner])->gemm_done : nullptr;
   return w;
 }
 // By one lane of each warp that stores a tile, after a __syncwarp behind its last store, or by one thread for all of them.
-__device__ __forceinline__ void count_stored(const StoredWords& w) {
+__device__ __forceinline__ void count_stored(const StoredWords& w, int n) {
   fence_acq_rel_gpu();
   fence_async_proxy();
-  if (w.rows) atomicAdd(w.rows, 1);
-  atomicAdd(w.op, 1);
-  if (w.partner) atomicAdd(w.partner, 1);
+  atomicAdd(w.own, n);
+  if (w.partner) atomicAdd(w.partner, n);
 }
 
 // one committed entry counted for `op` (descriptor `desc`): notify word, completion
@@ -425,7 +431,7 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
   const RunArgs* a = c.a;
   OpDev* op = &a->ops[ti.slot];
   const unsigned long long t_commit = a->log_cap > 0 ? gtime_ns() : 0ull;   // before it is published
-  if (kCounts && ti.kind != kCombine) count_stored(stored_words(c, op, ti));
+  if (kCounts && ti.kind != kCombine) count_stored(stored_words(c, op, ti), 1);
   else if (watched) fence_acq_rel_gpu();
   if (watched) {
     count_commit(c, op, ti.slot);
@@ -454,7 +460,7 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
 // unit's first claim (heads: of both halves, the half is only known when they arrive).  All of it is one round trip: lane i reads
 // the plan of op i, the last lanes a word each.  The unit asks for the half with a plain load; the fetch-add that counts it
 // (take_turn) comes later, so that no claim waits behind those of all other units.
-// per_tile: what a committed GEMM entry adds to gemm_done.  max_rows: the tallest work tile this kernel has room for.
+// per_tile: what a committed down tile adds to gemm_done.  max_rows: the tallest work tile this kernel has room for.
 __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const RunHead* first_half, int lane, int per_tile, int max_rows) {
   constexpr int kW = 25;
   static_assert(kMaxOps <= kW, "a lane per op, and one per word");
@@ -479,7 +485,7 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
   }
   const unsigned decode_ops = __ballot_sync(0xffffffffu, cls == MOE_CLASS_DECODE);
   const int entries = ps.planned == 0 ? 0 : ps.n_gemm_tiles + (a->fuse_combine ? ps.n_comb_tiles : 0);
-  const int all_gemm = (ps.n_gemm_tiles + ps.n_extra_gemm) * per_tile;
+  const int all_gemm = down_tiles(a, ps.n_gemm_tiles + ps.n_extra_gemm) * per_tile;
   const unsigned watched = __ballot_sync(0xffffffffu, (ps.flags & kOpWatched) != 0);
   if (lane == 0) {
     sc->watched = watched != 0;
