@@ -9,10 +9,9 @@
 
 namespace moe {
 
-// Tokens [t0, t1) by `nthr` cooperating threads (thread index tid); 8 bf16 per 16-byte access.
-// k <= 8: a group of L adjacent threads (L = 16, 32, ... as many as the thread count allows)
-// owns one token, loads its k routed rows and router weights once, and walks the token's row in
-// steps of L 16-byte slices.  Slots 0..3 and 4..7 are two buffers: as soon as one has been added
+// Columns [v0, v0 + nv) (in units of 8) of tokens [t0, t1) by `nthr` cooperating threads (thread index tid; nthr a power of two); 8 bf16 per
+// 16-byte access.  k <= 8: a group of L adjacent threads (a power of two, as many as there are for a token) owns one token, loads its
+// k routed rows and router weights once, and walks the token's row in steps of L 16-byte slices.  Slots 0..3 and 4..7 are two buffers: as soon as one has been added
 // in, its loads for the next slice are issued, so loads are in flight all the time and the
 // dependent pair (row index, then row) is paid once per token.  The rows are ADDED in slot
 // order j = 0..k-1.
@@ -40,7 +39,7 @@ struct CombineNow {
   __device__ __forceinline__ bool operator()() const { return true; }
 };
 template <class Ready>
-__device__ __noinline__ bool combine_tokens(const OpDev* op, int t0, int t1, int k, int H, int tid, int nthr, Ready ready) {
+__device__ __noinline__ bool combine_tokens(const OpDev* op, int t0, int t1, int v0, int nv, int k, int H, int tid, int nthr, Ready ready) {
   const unsigned n_rows = (unsigned)op->space_rows;    // rows of the packed space D lives in
   // every permutation entry of these tokens is checked once, ahead of the loops that use them
   for (int i = t0 * k + tid; i < t1 * k; i += nthr)
@@ -50,13 +49,13 @@ __device__ __noinline__ bool combine_tokens(const OpDev* op, int t0, int t1, int
   uint4* y = reinterpret_cast<uint4*>(op->y);
   const int* f2s = op->comb_index;
   const float* w = op->topk_w;
-  const int total = (t1 - t0) * vec_per_row;
-  if (k <= 8 && nthr >= 16 && vec_per_row % 16 == 0) {
+  const int total = (t1 - t0) * nv;
+  if (k <= 8 && nthr >= 16) {
     int L = 16;
-    while (2 * L * (t1 - t0) <= nthr && vec_per_row % (2 * L) == 0) L *= 2;
+    while (2 * L * (t1 - t0) <= nthr && L < nv) L *= 2;
     const int tpp = nthr / L;                 // tokens per pass
     const int sub = tid % L, trow = tid / L;      // nthr is a multiple of L: every thread has a group
-    const int nslice = vec_per_row / L;
+    const int nslice = (nv - sub + L - 1) / L;    // (none where the group is wider than the row)
     // row offsets in 16-byte units (moe_create rejects shapes whose D buffer exceeds 2^32 units)
     unsigned off[8];
     float wj[8];
@@ -77,16 +76,16 @@ __device__ __noinline__ bool combine_tokens(const OpDev* op, int t0, int t1, int
     if (!ready()) return false;
     for (int t = t0 + trow; t < t1; t += tpp) {
       if (t > t0 + trow) read_slots(t);
-      const uint4* src = D + sub;
-      uint4* dst = y + (size_t)t * vec_per_row + sub;
+      const uint4* src = D + v0 + sub;
+      uint4* dst = y + (size_t)t * vec_per_row + v0 + sub;
       const int na = k < 4 ? k : 4, nb = k - na;          // slots in the two buffers
       uint4 da[4], db[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         da[i] = make_uint4(0u, 0u, 0u, 0u);
         db[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (i < na) da[i] = src[off[i]];
-        if (i < nb) db[i] = src[off[4 + i]];
+        if (i < na && nslice > 0) da[i] = src[off[i]];
+        if (i < nb && nslice > 0) db[i] = src[off[4 + i]];
       }
       for (int sl = 0; sl < nslice; ++sl) {
         const bool more = sl + 1 < nslice;
@@ -114,7 +113,7 @@ __device__ __noinline__ bool combine_tokens(const OpDev* op, int t0, int t1, int
   }
   if (!ready()) return false;
   for (int idx = tid; idx < total; idx += nthr) {
-    const int t = t0 + idx / vec_per_row, v = idx % vec_per_row;
+    const int t = t0 + idx / nv, v = v0 + idx % nv;
     float acc[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc[i] = 0.f;

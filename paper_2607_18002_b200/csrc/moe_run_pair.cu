@@ -641,9 +641,12 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       }
       bool ok = true;
       if (ti.kind == kCombine) {
-        const int mid = ti.row0 + (ti.rows + 1) / 2;
+        // The two CTAs share the tokens; of one or two, the columns: a thread then walks one or two slices, each a round trip, for three.
+        const int vecs = args.H / 8, mid = ti.row0 + (ti.rows + 1) / 2;
+        const bool by_columns = ti.rows <= 2;
         const CombineWhenDone ready{&c, op, &sc->combine_ready, ++combines, warp == 8 && lane == 0};
-        ok = combine_tokens(op, leader ? ti.row0 : mid, leader ? mid : ti.row0 + ti.rows, args.k, args.H, etid, 256, ready);
+        ok = by_columns ? combine_tokens(op, ti.row0, ti.row0 + ti.rows, leader ? 0 : vecs / 2, vecs / 2, args.k, args.H, etid, 256, ready)
+                        : combine_tokens(op, leader ? ti.row0 : mid, leader ? mid : ti.row0 + ti.rows, 0, vecs, args.k, args.H, etid, 256, ready);
         if (!ok) break;
       } else {
         const int b = (int)(gcount & 1u);
