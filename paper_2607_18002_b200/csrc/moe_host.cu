@@ -9,11 +9,11 @@
 #include "moe_dev.cuh"
 
 namespace moe {
-cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, cudaStream_t stream);
+cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, int read_once, cudaStream_t stream);
 cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
-                               cudaStream_t stream);
+                               int read_once, cudaStream_t stream);
 cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, const OpDev& p, int* gather, int* comb_d,
-                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows,
+                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows, int read_once,
                              int slot_d, int slot_p, cudaStream_t stream);
 cudaError_t launch_combine(const OpDev* d_op, int T, int k, int H, cudaStream_t stream);
 cudaError_t prepare_run_kernel();
@@ -430,8 +430,9 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
   }
   ctx->work_rows[slot] = work_rows;
   ctx->plan_capture[slot] = cap;
-  const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, st)
-                                : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, st);
+  const int read_once = ctx->pair_kernel ? kReadOnce : 0;
+  const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, read_once, st)
+                                : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, read_once, st);
   if (pe != cudaSuccess) {
     ctx->planned[slot] = false;
     return MOE_ECUDA;
@@ -629,7 +630,7 @@ int moe_plan_pair(moe_ctx_t* ctx, int slot_prefill, int slot_decode, int carrier
   }
   if (launch_plan_pair(hd, hp, ctx->host_ops[sd], ctx->host_ops[sp], gather_m, reinterpret_cast<int*>(bd + L.pcomb_off),
                        reinterpret_cast<int*>(bp + L.pcomb_off), c.n_experts, L.NT1, L.NT2,
-                       fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, sd, sp, st) != cudaSuccess)
+                       fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, ctx->pair_kernel ? kReadOnce : 0, sd, sp, st) != cudaSuccess)
     return MOE_ECUDA;
   if (ctx->pair_of[sp] >= 0) ctx->pair_of[ctx->pair_of[sp]] = -1;
   if (ctx->pair_of[sd] >= 0) ctx->pair_of[ctx->pair_of[sd]] = -1;

@@ -55,6 +55,11 @@ __device__ __forceinline__ unsigned long long l2_evict_first() {
   asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
+__device__ __forceinline__ unsigned long long l2_evict_normal() {
+  unsigned long long p;
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
 __device__ __forceinline__ void tma_tile_2d(void* dst, const CUtensorMap* tm, int x, int y,
                                             void* bar) {
   asm volatile(
@@ -383,42 +388,37 @@ __device__ __forceinline__ void mbar_arrive_n_elect(void* bar, unsigned n) {
 // All loads and barrier arrivals of one k-block by one CTA of a pair, as ONE instruction group under a
 // single election: expect_tx on the leader's stage barrier, the box of 128 weight rows, up to three
 // activation boxes (a_rows rows apart), the stand-in arrivals (tiles without a gather) and the go-ahead for the
-// gather warps.  Flags select what is issued; everything is warp-uniform.  kEvictFirst: w_policy is the L2 policy of the weights.
-template <bool kEvictFirst>
+// gather warps.  Flags select what is issued; everything is warp-uniform.  w_policy: the L2 policy of the weights.
 __device__ __forceinline__ void pair_issue_kblock(unsigned bar, unsigned tx, unsigned standin_bar, unsigned standin_n,
                                                   unsigned sW, const CUtensorMap* tmw, int x, int wblk, int expert,
                                                   unsigned sX, const CUtensorMap* tma, int ay, unsigned a_boxes, unsigned a_rows,
                                                   unsigned go_bar, unsigned has_go, unsigned long long w_policy) {
-#define MOE_PAIR_KBLOCK(HINT, POLICY)                                                                                  \
-  asm volatile(                                                                                                        \
-      "{\n\t.reg .pred e, pa1, pa2, pa3, pgo, pst;\n\t.reg .b32 r, st, z, sA1, ay1, sA2, ay2;\n\t"                     \
-      "elect.sync r|e, 0xffffffff;\n\t"                                                                                \
-      "setp.ge.and.u32 pa1, %12, 1, e;\n\t"                                                                            \
-      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"                                                                            \
-      "setp.ge.and.u32 pa3, %12, 3, e;\n\t"                                                                            \
-      "setp.ne.and.b32 pgo, %15, 0, e;\n\t"                                                                            \
-      "setp.ne.and.b32 pst, %3, 0, e;\n\t"                                                                             \
-      "mov.b32 z, 0;\n\t"                                                                                              \
-      "shl.b32 st, %13, 7;\n\t"                                                                                        \
-      "add.u32 sA1, %9, st;\n\t"                                                                                       \
-      "add.s32 ay1, %11, %13;\n\t"                                                                                     \
-      "add.u32 sA2, sA1, st;\n\t"                                                                                      \
-      "add.s32 ay2, ay1, %13;\n\t"                                                                                     \
-      "@e mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;\n\t"                                              \
-      "@pst mbarrier.arrive.shared::cta.b64 _, [%2], %3;\n\t"                                                          \
-      "@e cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes" HINT " [%4], [%5, {%6, z, z, %7, %8}], [%0]" POLICY ";\n\t" \
-      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%9], [%10, {%6, %11}], [%0];\n\t" \
-      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%10, {%6, ay1}], [%0];\n\t" \
-      "@pa3 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA2], [%10, {%6, ay2}], [%0];\n\t" \
-      "@pgo mbarrier.arrive.shared::cta.b64 _, [%14];\n\t}"                                                            \
-      ::"r"(bar), "r"(tx), "r"(standin_bar), "r"(standin_n),                                                           \
-        "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert),                       \
-        "r"(sX), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "r"(a_rows),                   \
-        "r"(go_bar), "r"(has_go), "l"(w_policy)                                                                        \
-      : "memory")
-  if constexpr (kEvictFirst) MOE_PAIR_KBLOCK(".L2::cache_hint", ", %16");
-  else MOE_PAIR_KBLOCK("", "");
-#undef MOE_PAIR_KBLOCK
+  asm volatile(
+      "{\n\t.reg .pred e, pa1, pa2, pa3, pgo, pst;\n\t.reg .b32 r, st, z, sA1, ay1, sA2, ay2;\n\t"
+      "elect.sync r|e, 0xffffffff;\n\t"
+      "setp.ge.and.u32 pa1, %12, 1, e;\n\t"
+      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"
+      "setp.ge.and.u32 pa3, %12, 3, e;\n\t"
+      "setp.ne.and.b32 pgo, %15, 0, e;\n\t"
+      "setp.ne.and.b32 pst, %3, 0, e;\n\t"
+      "mov.b32 z, 0;\n\t"
+      "shl.b32 st, %13, 7;\n\t"
+      "add.u32 sA1, %9, st;\n\t"
+      "add.s32 ay1, %11, %13;\n\t"
+      "add.u32 sA2, sA1, st;\n\t"
+      "add.s32 ay2, ay1, %13;\n\t"
+      "@e mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;\n\t"
+      "@pst mbarrier.arrive.shared::cta.b64 _, [%2], %3;\n\t"
+      "@e cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%4], [%5, {%6, z, z, %7, %8}], [%0], %16;\n\t"
+      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%9], [%10, {%6, %11}], [%0];\n\t"
+      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%10, {%6, ay1}], [%0];\n\t"
+      "@pa3 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA2], [%10, {%6, ay2}], [%0];\n\t"
+      "@pgo mbarrier.arrive.shared::cta.b64 _, [%14];\n\t}"
+      ::"r"(bar), "r"(tx), "r"(standin_bar), "r"(standin_n),
+        "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert),
+        "r"(sX), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "r"(a_rows),
+        "r"(go_bar), "r"(has_go), "l"(w_policy)
+      : "memory");
 }
 
 // The activation boxes alone, for a k-block whose weights and expect_tx went out before

@@ -156,6 +156,7 @@ struct LoadPlan {
   int a_box_rows;
   unsigned tx;
   bool g1;
+  unsigned long long policy;   // L2 policy of the weights
 };
 
 __device__ __forceinline__ LoadPlan make_plan(const OpDev* op, const TileInfo& ti, int rank) {
@@ -165,7 +166,13 @@ __device__ __forceinline__ LoadPlan make_plan(const OpDev* op, const TileInfo& t
   const bool w1 = ti.kind != kDown;          // gate/up weights
   p.tmw = w1 ? &op->tm_p1 : &op->tm_p2;
   p.wblk = w1 ? (ti.n * kTileN1 + 64 * rank) / 8 : (ti.n * kTileN2 + 128 * rank) / 16;
-  p.expert = ti.expert;
+  p.expert = ti.expert & (kReadOnce - 1);
+  // Where one work tile reads an expert's weights, they are marked to leave L2 first and do not push out what is read again (one token: 72.7 ->
+  // 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  Two unpaired ops of a launch that share their weights read
+  // them twice, at different times, and gain too (100 + 64 tokens on 64 experts: 397 -> 383, on 8 active experts: 91 -> 84, on 32
+  // experts of 3 MB: 84 -> 80; 30 + 20 tokens on 32 active experts lose, 213 -> 218).  The weights of experts of several tiles are the data
+  // read again: marked, they cost (8192 tokens: 2390 -> 2510).
+  p.policy = kReadOnce & ti.expert ? l2_evict_first() : l2_evict_normal();
   p.a_boxes = 0;
   p.a_box_rows = 0;
   p.ay = ti.row0 + rank * rpc;
@@ -193,17 +200,11 @@ __device__ __forceinline__ void issue_kblock(SharedCtl<kTileRows>* sc, unsigned 
                                              unsigned stage, bool leader, unsigned full0_addr) {
   const unsigned sX = stages_addr + stage * (unsigned)Ring<kTileRows>::kSB;
   const unsigned bar = full0_addr + stage * 8u;            // the leader's full[stage]
-  // Where an op's tokens fit one work tile, the op reads a weight byte once: marked to leave L2 first, it does not push out what
-  // is read again (one token: 72.7 -> 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  Two unpaired ops of a
-  // launch that share their weights read it twice, at different times, and gain too (100 + 64 tokens on 64 experts: 397 -> 383, on 8
-  // active experts: 91 -> 84, on 32 experts of 3 MB: 84 -> 80; 30 + 20 tokens on 32 active experts lose, 213 -> 218).  With experts of
-  // several tiles the weights are the data read again, and the mark costs (8192 tokens: 2390 -> 2510).
-  constexpr bool kOnce = kTileRows != kWorkRowsBf16;
-  pair_issue_kblock<kOnce>(bar, p.tx, smem_u32(&sc->full[stage]),
+  pair_issue_kblock(bar, p.tx, smem_u32(&sc->full[stage]),
                     (leader && !p.g1) ? (unsigned)kGatherThreads + 1u : 0u,   // nobody gathers for this tile
                     sX + (unsigned)Ring<kTileRows>::kABytes, p.tmw, kb * kBlockK, p.wblk, p.expert,
                     sX, p.tma, p.ay, (unsigned)p.a_boxes, (unsigned)p.a_box_rows,
-                    smem_u32(&sc->goA[stage]), p.g1 ? 1u : 0u, l2_evict_first());
+                    smem_u32(&sc->goA[stage]), p.g1 ? 1u : 0u, p.policy);
 }
 
 // The epilogue warps' wait inside a combine tile: one lane of the CTA looks at the op's counter and counts the tile (its `turn`-th) in
