@@ -147,6 +147,13 @@ __device__ __forceinline__ void arrive_at_leader(void* bar, bool leader) {
   else mbar_arrive_cluster(map_to_cta(bar, 0));
 }
 
+// ... of a role that has read a ring slot or drained an accumulator: nothing that it wrote to memory is handed over, so the arrival does not
+// have to wait, as a release to the other CTA does, for stores and copies that are still under way
+__device__ __forceinline__ void signal_leader(void* bar, bool leader) {
+  if (leader) mbar_arrive(bar);
+  else mbar_arrive_remote(map_to_cta(bar, 0));
+}
+
 // what one CTA loads per k-block of a tile
 struct LoadPlan {
   const CUtensorMap* tmw;
@@ -397,7 +404,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (leader && lane == 0) mbar_arrive(&sc->taken[tslot]);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (ti.kind == kCombine) {
-        if (lane == 0) arrive_at_leader(&sc->iempty[tslot], leader);
+        if (lane == 0) signal_leader(&sc->iempty[tslot], leader);
         continue;
       }
       LoadPlan lp = make_plan(&args.ops[ti.slot], ti, rank);
@@ -421,7 +428,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         }
         lp.a_boxes = (int)boxes;
       }
-      if (lane == 0) arrive_at_leader(&sc->iempty[tslot], leader);   // the ring slot's barriers are not looked at any more
+      if (lane == 0) signal_leader(&sc->iempty[tslot], leader);   // the ring slot's barriers are not looked at any more
       for (; kb < ti.kblocks; ++kb) {
         if (!wwait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
         issue_kblock(sc, stages_addr, lp, kb, stage, leader, full0_addr);
@@ -488,7 +495,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kblocks = sc->info[islot].kblocks;
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
-      if (lane == 0) arrive_at_leader(&sc->iempty[islot], false);
+      if (lane == 0) signal_leader(&sc->iempty[islot], false);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (kind == kCombine) continue;
       if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
@@ -527,7 +534,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
-      if (lane == 0) arrive_at_leader(&sc->iempty[islot], leader);
+      if (lane == 0) signal_leader(&sc->iempty[islot], leader);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (kind == kCombine) continue;
       if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
@@ -678,7 +685,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
             if (last) {                                       // all of it is in registers: the accumulator may be overwritten
               tc_fence_before();
               __syncwarp();
-              if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);
+              if (lane == 0) signal_leader(&sc->tempty[b], leader);
             }
             unsigned o[16];
             if (g1) {
@@ -725,7 +732,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         } else {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) arrive_at_leader(&sc->tempty[b], leader);
+          if (lane == 0) signal_leader(&sc->tempty[b], leader);
         }
         __syncwarp();
         const bool alone = ti.rows <= cols;                   // the columns of the quadrant's other warp hold no rows: one counts for both
