@@ -147,8 +147,8 @@ __device__ __forceinline__ void arrive_at_leader(void* bar, bool leader) {
   else mbar_arrive_cluster(map_to_cta(bar, 0));
 }
 
-// ... of a role that has read a ring slot or drained an accumulator: nothing that it wrote to memory is handed over, so the arrival does not
-// have to wait, as a release to the other CTA does, for stores and copies that are still under way
+// ... of a role that has read a ring slot, drained an accumulator or fenced its stores: nothing that it wrote to memory is handed over by the arrival, which
+// does not have to wait, as a release to the other CTA does, for stores and copies that are still under way
 __device__ __forceinline__ void signal_leader(void* bar, bool leader) {
   if (leader) mbar_arrive(bar);
   else mbar_arrive_remote(map_to_cta(bar, 0));
@@ -738,10 +738,14 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         const bool alone = ti.rows <= cols;                   // the columns of the quadrant's other warp hold no rows: one counts for both
         if (lane == 0 && (half == 0 || !alone)) count_stored(words, alone ? 2 : 1);
       }
-      // The warp's stores, before the tile is published: the arrival releases them (across the pair: at cluster scope), the
-      // committer's fence is cumulative over what it acquires here
+      // The warp's stores, before the tile is published.  Those of a GEMM tile are behind the fence of count_stored (a warp that does not
+      // count stores nothing); of a combine tile the arrival releases them (across the pair: at cluster scope).  The committer's
+      // fence is cumulative over what it sees here.
       __syncwarp();
-      if (lane == 0) arrive_at_leader(&sc->done[islot], leader);
+      if (lane == 0) {
+        if (ti.kind == kCombine) arrive_at_leader(&sc->done[islot], leader);
+        else signal_leader(&sc->done[islot], leader);
+      }
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
   }
