@@ -19,8 +19,8 @@
 // warp 3 producer (TMA loads of its own half, read from the descriptor ring), warps 4-7 gather,
 // warps 8-15 epilogue; second CTA only -- warp 1 relays the completion of its gather to the
 // leader.  Tile descriptors reach the second CTA through distributed shared memory; its barrier
-// arrivals that the leader waits for are remote mbarrier arrivals.  Every wait is bounded, as in
-// the single-CTA kernel.
+// arrivals that the leader waits for are remote mbarrier arrivals.  Its roles give a ring slot back to
+// warp 2 (second CTA), which tells the leader.  Every wait is bounded, as in the single-CTA kernel.
 #include "moe_combine.cuh"
 #include "moe_ptx.cuh"
 #include "moe_sched.cuh"
@@ -66,7 +66,8 @@ struct SharedCtl {
   unsigned long long tfull[2];       // both (multicast commit): accumulator complete
   unsigned long long tempty[2];      // leader's: accumulator drained by the 16 epilogue warps
   unsigned long long ifull[kRing];   // own: tile descriptor published
-  unsigned long long iempty[kRing];  // leader's: ring slot released by the roles of both CTAs
+  unsigned long long iempty[kRing];  // leader's: ring slot released by its roles and, once for all of its own, by the other CTA
+  unsigned long long iread[kRing];   // second CTA's: its roles have read the tile descriptor
   unsigned long long done[kRing];    // leader's: the 16 epilogue warps have stored the tile
   unsigned long long taken[kRing];   // leader's: its producer has started on the tile
   unsigned long long rows_in[kRing]; // own: the rows that the tile reads are in place (down tiles: its gate/up tiles are committed)
@@ -147,7 +148,16 @@ __device__ __forceinline__ void arrive_at_leader(void* bar, bool leader) {
   else mbar_arrive_cluster(map_to_cta(bar, 0));
 }
 
-// ... of a role that has read a ring slot, drained an accumulator or fenced its stores: nothing that it wrote to memory is handed over by the arrival, which
+// A role has read what it needs of a ring slot.  In the second CTA it says so to warp 2 of its own CTA, which nothing waits for and which
+// orders all of these reads before the leader's next descriptor with one release to the cluster.  A release by the role itself
+// waits for its stores and copies: a round trip at the start of every tile, ahead of the gather (one token 57.8 us a pass in place
+// of 55.4); arrivals without one, which left that order to the hardware, take as long as this (56.5, now 55.7).
+template <int kTileRows>
+__device__ __forceinline__ void release_slot(SharedCtl<kTileRows>* sc, int islot, bool leader) {
+  mbar_arrive(leader ? &sc->iempty[islot] : &sc->iread[islot]);
+}
+
+// ... of a role that has drained an accumulator or fenced its stores: nothing that it wrote to memory is handed over by the arrival, which
 // does not have to wait, as a release to the other CTA does, for stores and copies that are still under way
 __device__ __forceinline__ void signal_leader(void* bar, bool leader) {
   if (leader) mbar_arrive(bar);
@@ -279,11 +289,12 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       mbar_init(&sc->tfull[s], 1);
       mbar_init(&sc->tempty[s], 16);
     }
-    // a ring slot is released by: MMA warp, committer, producer, 4 gather warps (leader); producer,
-    // relay, 4 gather warps (other CTA)
+    // a ring slot is released by: MMA warp, committer, producer, 4 gather warps (leader); warp 2 of the other CTA, where it is read by
+    // producer, relay, 4 gather and 8 epilogue warps (the leader's are behind the committer)
     for (int s = 0; s < kRing; ++s) {
       mbar_init(&sc->ifull[s], 1);
-      mbar_init(&sc->iempty[s], 13);
+      mbar_init(&sc->iempty[s], 8);
+      mbar_init(&sc->iread[s], 14);
       mbar_init(&sc->done[s], 16);
       mbar_init(&sc->taken[s], 1);
       mbar_init(&sc->rows_in[s], 1);
@@ -324,6 +335,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // loads are being issued.
     int islot = 0;
     unsigned iph = 0;
+    bool lapped = false;                                  // every ring slot has been used
     TileInfo ti;
     bool need_ready = false;
     ti.kind = kEnd;
@@ -341,7 +353,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     while (true) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
-      if (!wwait(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
+      if (lapped && !wwait_cluster(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
       if (ti.kind != kEnd && need_ready && !wait_op_ready(c, lane, ti)) ti.kind = kEnd;
       // A down tile is handed over at once: the producers fill the free stages with its weights and add the rows when its gate/up
       // tiles are committed (one token: 67.6 -> 67.0 us a pass, 128 tokens on 8 experts: 80.3 -> 79.1).
@@ -372,7 +384,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (__shfl_sync(0xffffffffu, ok, 0) == 0) break;
       }
       if (!wwait(c, &sc->taken[islot], iph, 26)) break;
-      if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      if (++islot == kRing) { islot = 0; iph ^= 1u; lapped = true; }
       if (plain) ti.kind = kEnd;
       else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready);
     }
@@ -404,7 +416,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (leader && lane == 0) mbar_arrive(&sc->taken[tslot]);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (ti.kind == kCombine) {
-        if (lane == 0) signal_leader(&sc->iempty[tslot], leader);
+        if (lane == 0) release_slot(sc, tslot, leader);
         continue;
       }
       LoadPlan lp = make_plan(&args.ops[ti.slot], ti, rank);
@@ -428,7 +440,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         }
         lp.a_boxes = (int)boxes;
       }
-      if (lane == 0) signal_leader(&sc->iempty[tslot], leader);   // the ring slot's barriers are not looked at any more
+      if (lane == 0) release_slot(sc, tslot, leader);   // the ring slot's barriers are not looked at any more
       for (; kb < ti.kblocks; ++kb) {
         if (!wwait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
         issue_kblock(sc, stages_addr, lp, kb, stage, leader, full0_addr);
@@ -495,7 +507,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kblocks = sc->info[islot].kblocks;
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
-      if (lane == 0) signal_leader(&sc->iempty[islot], false);
+      if (lane == 0) release_slot(sc, islot, false);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (kind == kCombine) continue;
       if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
@@ -534,7 +546,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
-      if (lane == 0) signal_leader(&sc->iempty[islot], leader);
+      if (lane == 0) release_slot(sc, islot, leader);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (kind == kCombine) continue;
       if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
@@ -618,6 +630,19 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       __syncwarp();
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
+  } else if (warp == 2) {
+    // ============================================================ ring slots of the second CTA
+    ended = false;
+    int islot = 0;
+    unsigned iph = 0;
+    while (true) {
+      if (!wait_info(c, &sc->ifull[islot], iph, 30, false)) break;
+      const int kind = __shfl_sync(0xffffffffu, sc->info[islot].kind, 0);
+      if (kind == kEnd) { ended = true; break; }
+      if (!wait_info(c, &sc->iread[islot], iph, 31, true)) break;       // (an arrival of this CTA)
+      if (lane == 0) mbar_arrive_cluster(map_to_cta(&sc->iempty[islot], 0));
+      if (++islot == kRing) { islot = 0; iph ^= 1u; }
+    }
   } else if (warp >= 8) {
     // ============================================================ epilogue (8 warps per CTA)
     // Warp w reads TMEM lanes 32 (w % 4) .. +31 (weight rows: 2 x (8 gate + 8 up), or 32 down features) and one half of the
@@ -636,6 +661,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (!wait_info(c, &sc->ifull[islot], iph, 9, leader)) break;
       const TileInfo ti = sc->info[islot];
       if (ti.kind == kEnd) { ended = true; break; }
+      __syncwarp();
+      if (!leader && lane == 0) release_slot(sc, islot, false);
       OpDev* op = &args.ops[ti.slot];
       if (first) {
         first = false;
