@@ -284,10 +284,17 @@ __device__ __forceinline__ void mbar_arrive_cluster(unsigned cluster_addr) {
 __device__ __forceinline__ void mbar_expect_tx_cluster(unsigned cluster_addr, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.release.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
 }
-// the same two without cluster-scope release: for pipeline barriers whose data moves by TMA or cp.async
-__device__ __forceinline__ void mbar_arrive_remote(unsigned cluster_addr) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+// behind a fence of the caller's that orders what the arrival hands over
+__device__ __forceinline__ void mbar_arrive_relaxed(unsigned cluster_addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+// A stage's rows are in place in the shared memory of the CTA that says so, where the pair's MMAs read them: written by cp.async of this
+// CTA's threads, seen complete by the caller and fenced for the tensor core, so the release is to this CTA.  (To the cluster, once a
+// k-block, it takes longer than the k-block: one token 56 -> 129 us a pass, 777 tokens 1120 -> 2604.)
+__device__ __forceinline__ void mbar_arrive_remote(unsigned cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// the bytes of a stage: the barrier itself counts them
 __device__ __forceinline__ void mbar_expect_tx_remote(unsigned cluster_addr, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
 }

@@ -21,3 +21,16 @@ def test_a_ring_slot_is_given_back_by_a_release_to_the_cluster():
     # the roles of the second CTA meet on a barrier of their own
     assert _uses("moe_run_pair.cu", "iread") == {"mbar_init", "wait_info"}
     assert "mbar_arrive(leader ? &sc->iempty[islot] : &sc->iread[islot]);" in _code("moe_run_pair.cu")
+
+
+def test_a_stored_tile_is_handed_over_at_cluster_scope():
+    code, ptx = _code("moe_run_pair.cu"), _code("moe_ptx.cuh")
+    # behind the fence of the warps that count, a relaxed arrival that the other CTA's wait can meet; behind no fence, a release
+    assert _uses("moe_run_pair.cu", "done") == {"mbar_init", "arrive_at_leader", "signal_leader", "wwait_cluster"}
+    body = lambda text, name: re.search(name + r"\([^)]*\) \{(.*?)\n\}", text, re.S).group(1)
+    assert "mbar_arrive_relaxed(map_to_cta(bar, 0))" in body(code, "void signal_leader")
+    assert "mbar_arrive_cluster(map_to_cta(bar, 0))" in body(code, "void arrive_at_leader")
+    assert body(_code("moe_sched.cuh"), "void count_stored").strip().startswith("fence_acq_rel_gpu();")
+    # every arrival on a barrier of the other CTA says what it orders and for whom; one of them is for this CTA: gathered rows
+    assert set(re.findall(r"mbarrier\.arrive(\S*)\.shared::cluster\.b64 _, \[%0\];", ptx)) == {".release.cluster", ".relaxed.cluster", ".release.cta"}
+    assert re.findall(r"mbar_arrive_remote\((.*?)\);", code) == ["map_to_cta(&sc->full[stage], 0)"]
