@@ -310,6 +310,18 @@ __device__ __forceinline__ bool mbar_try_cluster(void* bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
+// wait for relaxed arrivals of the other CTA: a fence of the caller's orders what follows
+__device__ __forceinline__ bool mbar_try_relaxed(void* bar, unsigned parity) {
+  unsigned ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // non-blocking test that also synchronises with arrivals of the other CTA
 __device__ __forceinline__ bool mbar_test_cluster(void* bar, unsigned parity) {
   unsigned ok;

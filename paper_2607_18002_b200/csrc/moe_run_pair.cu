@@ -82,11 +82,12 @@ static_assert(sizeof(TileInfo) == 48, "descriptor is copied as three 16-byte wor
 template <int kTileRows>
 constexpr size_t kSmemBytes = 1024 + (size_t)Ring<kTileRows>::kNS * Ring<kTileRows>::kSB + sizeof(SharedCtl<kTileRows>);
 
-// bounded wait that also synchronises with arrivals of the other CTA
+// bounded wait on arrivals of the other CTA.  kTry: mbar_try_cluster, or mbar_try_relaxed where a fence of the caller's follows
+template <bool (*kTry)(void*, unsigned)>
 __device__ __noinline__ bool wait_slow(const Ctx& c, void* bar, unsigned parity, int where) {
   unsigned long long t0 = 0;
   for (unsigned it = 1;; ++it) {
-    if (mbar_try_cluster(bar, parity)) return true;
+    if (kTry(bar, parity)) return true;
     if ((it & 63u) == 0) {
       if (aborted(c)) return false;
       const unsigned long long now = gtime_ns();
@@ -98,15 +99,19 @@ __device__ __noinline__ bool wait_slow(const Ctx& c, void* bar, unsigned parity,
     }
   }
 }
+template <bool (*kTry)(void*, unsigned)>
 __device__ __forceinline__ bool bwait(const Ctx& c, void* bar, unsigned parity, int where) {
-  if (mbar_try_cluster(bar, parity)) return true;
-  return wait_slow(c, bar, parity, where);
+  if (kTry(bar, parity)) return true;
+  return wait_slow<kTry>(c, bar, parity, where);
 }
 // whole-warp forms.  The cluster-scope wait is for the hand-offs where this thread then reads
 // data the other CTA's threads wrote (the tile descriptor, stored outputs); pipeline barriers,
 // whose data moves by TMA, tensor core or this CTA's own threads, take the plain wait.
 __device__ __forceinline__ bool wwait_cluster(const Ctx& c, void* bar, unsigned parity, int where) {
-  return __all_sync(0xffffffffu, bwait(c, bar, parity, where));
+  return __all_sync(0xffffffffu, bwait<mbar_try_cluster>(c, bar, parity, where));
+}
+__device__ __forceinline__ bool wwait_relaxed(const Ctx& c, void* bar, unsigned parity, int where) {
+  return __all_sync(0xffffffffu, bwait<mbar_try_relaxed>(c, bar, parity, where));
 }
 __device__ __forceinline__ bool wwait(const Ctx& c, void* bar, unsigned parity, int where) {
   return __all_sync(0xffffffffu, mbar_wait(c, bar, parity, where));
@@ -466,7 +471,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (kind == kEnd) { ended = true; break; }
       if (kind != kCombine) {
         const unsigned b = gcount & 1u;
-        if (!wwait(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
+        if (!wwait_relaxed(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
         tc_fence_after();
         const unsigned d = __shfl_sync(0xffffffffu, tmem, 0) + b * (unsigned)kAccCols;
         const unsigned idesc = kIdescM256 | ((unsigned)tile_cols(rows) >> 3) << 17;

@@ -34,3 +34,12 @@ def test_a_stored_tile_is_handed_over_at_cluster_scope():
     # every arrival on a barrier of the other CTA says what it orders and for whom; one of them is for this CTA: gathered rows
     assert set(re.findall(r"mbarrier\.arrive(\S*)\.shared::cluster\.b64 _, \[%0\];", ptx)) == {".release.cluster", ".relaxed.cluster", ".release.cta"}
     assert re.findall(r"mbar_arrive_remote\((.*?)\);", code) == ["map_to_cta(&sc->full[stage], 0)"]
+
+
+def test_a_drained_accumulator_is_handed_back_between_tcgen05_fences():
+    code = _code("moe_run_pair.cu")
+    assert _uses("moe_run_pair.cu", "tempty") == {"mbar_init", "signal_leader", "wwait_relaxed"}
+    assert re.search(r"wwait_relaxed\(c, &sc->tempty.*\n\s*tc_fence_after\(\);", code)
+    arrivals = re.findall(r"(.*)\n(.*)\n.*signal_leader\(&sc->tempty", code)
+    assert len(arrivals) == 2 and all("tc_fence_before" in a and "__syncwarp" in b for a, b in arrivals)
+    assert ".relaxed.cluster" in re.search(r"mbar_try_relaxed.*?mbarrier\.try_wait\.parity(\S*) ", _code("moe_ptx.cuh"), re.S).group(1)
