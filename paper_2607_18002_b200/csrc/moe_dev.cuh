@@ -5,7 +5,6 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
-#include <stddef.h>
 #include <stdint.h>
 
 #include "../../include/moe_apk.h"
@@ -130,7 +129,6 @@ struct __align__(128) OpDev {
   int partner;              // paired: descriptor index of the other op of the pair, else -1
   int pad_[2];
 };
-static_assert(offsetof(OpDev, cls) % 128 == 0 && sizeof(OpDev) > offsetof(OpDev, cls) + 256, "touch_ops reads three lines of it");
 constexpr int kRowSlotShift = 27;                       // a flat routed index stays below 2^27 (moe_create checks)
 constexpr int kRowFlatMask = (1 << kRowSlotShift) - 1;
 

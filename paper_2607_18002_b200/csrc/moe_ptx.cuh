@@ -194,9 +194,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
-__device__ __forceinline__ void prefetch_tensormap(const void* p) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(p) : "memory");
-}
 __device__ __forceinline__ void cp_async_4(unsigned dst_smem, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_smem), "l"(src) : "memory");
 }

@@ -398,7 +398,6 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // ============================================================ producer (both CTAs)
     // Reads tiles from the ring and issues this CTA's loads, one stage per k-block.  The whole
     // warp runs the loop on warp-uniform values; one elected lane issues each instruction.
-    touch_ops(args, lane);
     ended = false;
     int islot = 0;
     unsigned iph = 0;

@@ -524,22 +524,6 @@ __device__ inline unsigned take_turn(const RunArgs* a) { return atomicAdd(&a->g-
 __device__ inline void end_turn(const RunArgs* a, unsigned ticket, int units) {
   if ((ticket & 0x7fffffffu) == (unsigned)units - 1u) atomicExch(&a->g->turn, ~ticket & 0x80000000u);
 }
-// One warp, while the unit's first claim is under way: the tensor maps of the launch's ops, and what the roles read of their descriptors
-// first thing, on their way to this SM.  (An op without rows has no maps.)
-__device__ __forceinline__ void touch_ops(const RunArgs& a, int lane) {
-  const int part = lane & 15;
-  for (int j = lane >> 4; j < a.n_ops; j += 2) {
-    const OpDev* op = &a.ops[a.slots[j]];
-    if (part < 3) {
-      int v;
-      asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<const char*>(&op->cls) + 128 * part) : "memory");
-    } else if (part < 9 && op->n_rows > 0) {
-      if (part < 7) prefetch_tensormap(part == 3 ? &op->tm_p1 : part == 4 ? &op->tm_p2 : part == 5 ? &op->tm_a8 : &op->tm_a32);
-      else if (op->masked) prefetch_tensormap(part == 7 ? &op->tm_x8 : &op->tm_x32);
-    }
-  }
-  __syncwarp();
-}
 // The launch parameters into the constant cache, while the kernel before still runs.
 __device__ __forceinline__ void touch_params(const RunArgs& a) {
   const int* p = reinterpret_cast<const int*>(&a);
