@@ -680,9 +680,11 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       }
       bool ok = true;
       if (ti.kind == kCombine) {
-        // The two CTAs share the tokens; of one or two, the columns: a thread then walks one or two slices, each a round trip, for three.
+        // The two CTAs share the tokens; of one, the columns: a thread then walks one slice of its row, a round trip, where it would walk two
+        // and the other CTA none (one token: 56.5 -> 56.0 us a pass).  Two tokens are two slices a thread either way, and by columns both
+        // CTAs read the rows and weights of both (82.1-83.1 us either way).
         const int vecs = args.H / 8, mid = ti.row0 + (ti.rows + 1) / 2;
-        const bool by_columns = ti.rows <= 2;
+        const bool by_columns = ti.rows == 1;
         const CombineWhenDone ready{&c, op, &sc->combine_ready, ++combines, warp == 8 && lane == 0};
         ok = by_columns ? combine_tokens(op, ti.row0, ti.row0 + ti.rows, leader ? 0 : vecs / 2, vecs / 2, args.k, args.H, etid, 256, ready)
                         : combine_tokens(op, leader ? ti.row0 : mid, leader ? mid : ti.row0 + ti.rows, 0, vecs, args.k, args.H, etid, 256, ready);
