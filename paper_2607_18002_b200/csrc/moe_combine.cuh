@@ -10,11 +10,10 @@
 namespace moe {
 
 // Columns [v0, v0 + nv) (in units of 8) of tokens [t0, t1) by `nthr` cooperating threads (thread index tid; nthr a power of two); 8 bf16 per
-// 16-byte access.  k <= 8: a group of L adjacent threads (a power of two, as many as there are for a token) owns one token, loads its
-// k routed rows and router weights once, and walks the token's row in steps of L 16-byte slices.  Slots 0..3 and 4..7 are two buffers: as soon as one has been added
-// in, its loads for the next slice are issued, so loads are in flight all the time and the
-// dependent pair (row index, then row) is paid once per token.  The rows are ADDED in slot
-// order j = 0..k-1.
+// 16-byte access.  k <= 8: a group of L adjacent threads (a power of two, as many as there are for a token, so that short tiles walk
+// few slices) owns one token, loads its k routed rows and router weights once, and walks the token's columns in steps of L 16-byte
+// slices.  Slots 0..3 and 4..7 are two buffers: as soon as one has been added in, its loads for the next slice are issued, so loads are in
+// flight all the time and the dependent pair (row index, then row) is paid once per token.  The rows are ADDED in slot order j = 0..k-1.
 __device__ __forceinline__ void combine_add4(float (&acc)[8], const uint4 (&d)[4], const float* wj, int n) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {

@@ -190,10 +190,13 @@ __device__ __forceinline__ LoadPlan make_plan(const OpDev* op, const TileInfo& t
   p.wblk = w1 ? (ti.n * kTileN1 + 64 * rank) / 8 : (ti.n * kTileN2 + 128 * rank) / 16;
   p.expert = ti.expert & (kReadOnce - 1);
   // Where one work tile reads an expert's weights, they are marked to leave L2 first and do not push out what is read again (one token: 72.7 ->
-  // 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  Two unpaired ops of a launch that share their weights read
-  // them twice, at different times, and gain too (100 + 64 tokens on 64 experts: 397 -> 383, on 8 active experts: 91 -> 84, on 32
-  // experts of 3 MB: 84 -> 80; 30 + 20 tokens on 32 active experts lose, 213 -> 218).  The weights of experts of several tiles are the data
-  // read again: marked, they cost (8192 tokens: 2390 -> 2510).
+  // 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  A plan knows its own op only: of two unpaired ops of a launch
+  // that share their weights both mark what the other reads too, at another time, and mostly gain.  Small ops (unmarked -> marked): 100 + 64
+  // tokens on 64 experts 397 -> 383, on 8 active experts 91 -> 84, on 32 experts of 3 MB 84 -> 80, but 30 + 20 on 32 active experts 213 ->
+  // 218.  Launches of 256-row tiles: 600 + 16 tokens on 64 experts 526 -> 505, 1000 + 32 1613 -> 1591, 300 + 200 1938 -> 1915, 1000 + 200
+  // 2205 -> 2170, 8192 + 128 3140 -> 3067, 12288 + 64 3695 -> 3597, 4096 + 64 on 64 experts 1226 -> 1213 (within the spread), but 2048 + 256
+  // on 128 experts 1255 -> 1274.  The weights of experts of several tiles are the data read again: marked, they cost (8192 tokens: 2390 ->
+  // 2510).
   p.policy = kReadOnce & ti.expert ? l2_evict_first() : l2_evict_normal();
   p.a_boxes = 0;
   p.a_box_rows = 0;
