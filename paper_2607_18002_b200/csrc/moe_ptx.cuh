@@ -1,6 +1,5 @@
-// Inline-PTX wrappers for the sm_100a features the persistent kernel uses: mbarriers, tiled
-// and gather4 TMA loads, tcgen05 (UMMA) issue / commit / TMEM loads, proxy fences and
-// scoped loads and stores.
+// Inline-PTX wrappers for the sm_100a features the persistent kernels use: mbarriers, tiled TMA loads,
+// tcgen05 (UMMA) issue / commit / TMEM loads, proxy fences and scoped loads and stores.
 #pragma once
 #include <cuda.h>
 #include <stdint.h>
@@ -18,11 +17,6 @@ __device__ __forceinline__ void mbar_arrive(void* bar) {
 }
 __device__ __forceinline__ void mbar_arrive_n(void* bar, unsigned n) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(void* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
 }
 __device__ __forceinline__ bool mbar_try(void* bar, unsigned parity) {
   unsigned ok;
@@ -60,22 +54,6 @@ __device__ __forceinline__ unsigned long long l2_evict_normal() {
   asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-__device__ __forceinline__ void tma_tile_2d(void* dst, const CUtensorMap* tm, int x, int y,
-                                            void* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
-      "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tma_gather4(void* dst, const CUtensorMap* tm, int x, int4 rows,
-                                            void* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(smem_u32(dst)),
-      "l"(tm), "r"(x), "r"(rows.x), "r"(rows.y), "r"(rows.z), "r"(rows.w), "r"(smem_u32(bar))
-      : "memory");
-}
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -97,30 +75,6 @@ __device__ __forceinline__ void tc_mma_bf16(unsigned d_tmem, unsigned long long 
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void tc_mma_f8(unsigned d_tmem, unsigned long long adesc,
-                                          unsigned long long bdesc, unsigned idesc,
-                                          unsigned accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void tc_st32(unsigned taddr, const unsigned (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-      "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-      "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
-__device__ __forceinline__ void tc_wait_st() {
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tc_ld32(unsigned taddr, unsigned (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -131,16 +85,6 @@ __device__ __forceinline__ void tc_ld32(unsigned taddr, unsigned (&r)[32]) {
         "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
         "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
         "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tc_ld16(unsigned taddr, unsigned (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
 }
@@ -191,9 +135,6 @@ __device__ __forceinline__ void tc_wait_ld() {
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
 __device__ __forceinline__ void cp_async_4(unsigned dst_smem, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_smem), "l"(src) : "memory");
 }
@@ -203,11 +144,6 @@ __device__ __forceinline__ void cp_async_16(unsigned dst_smem, const void* src) 
 // the mbarrier receives one arrival when all cp.async issued so far by this thread have landed
 __device__ __forceinline__ void cp_async_arrive_noinc(void* bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int kPending>
-__device__ __forceinline__ void cp_async_wait_group() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -278,9 +214,6 @@ __device__ __forceinline__ unsigned map_to_cta(const void* p, unsigned rank) {
 __device__ __forceinline__ void mbar_arrive_cluster(unsigned cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx_cluster(unsigned cluster_addr, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.release.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
-}
 // behind a fence of the caller's that orders what the arrival hands over
 __device__ __forceinline__ void mbar_arrive_relaxed(unsigned cluster_addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -290,10 +223,6 @@ __device__ __forceinline__ void mbar_arrive_relaxed(unsigned cluster_addr) {
 // k-block, it takes longer than the k-block: one token 56 -> 129 us a pass, 777 tokens 1120 -> 2604.)
 __device__ __forceinline__ void mbar_arrive_remote(unsigned cluster_addr) {
   asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// the bytes of a stage: the barrier itself counts them
-__device__ __forceinline__ void mbar_expect_tx_remote(unsigned cluster_addr, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
 }
 // wait that synchronises with arrivals made by the other CTA of the pair
 __device__ __forceinline__ bool mbar_try_cluster(void* bar, unsigned parity) {
@@ -334,70 +263,17 @@ __device__ __forceinline__ bool mbar_test_cluster(void* bar, unsigned parity) {
 __device__ __forceinline__ void st_cluster_v4(unsigned cluster_addr, uint4 v) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-// tiled TMA load by either CTA of a pair; the transaction bytes go to the barrier at `bar_cluster_addr`
-// (the pair leader's), the data to this CTA's own shared memory
-__device__ __forceinline__ void tma_tile_2d_pair(void* dst, const CUtensorMap* tm, int x, int y, unsigned bar_cluster_addr) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<unsigned long long>(tm)), "r"(bar_cluster_addr), "r"(x), "r"(y)
-      : "memory");
-}
-// one MMA of the pair: M = 256 or 128 rows split over the two CTAs, both halves of B read from the two CTAs
-__device__ __forceinline__ void tc_mma2_bf16(unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc,
-                                             unsigned idesc, unsigned accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// arrives on the barrier at the same shared-memory offset in both CTAs once the pair's MMAs so far retire
-__device__ __forceinline__ void tc_commit_pair(void* bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
-}
 
 // ---- warp-uniform issue: the whole warp executes these, one elected lane issues the instruction.
 // Their operands then stay warp-uniform for the compiler (no per-thread staging of descriptors),
 // which keeps the issue loops of the MMA and producer warps short.
-__device__ __forceinline__ void tc_mma2_bf16_elect(unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc,
-                                                   unsigned idesc, unsigned accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, e;\n\t.reg .b32 r;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
+// arrives on the barrier at the same shared-memory offset in both CTAs once the pair's MMAs so far retire
 __device__ __forceinline__ void tc_commit_pair_elect(void* bar) {
   asm volatile(
       "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
       "elect.sync r|e, 0xffffffff;\n\t"
       "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
       "h"((unsigned short)3)
-      : "memory");
-}
-__device__ __forceinline__ void tma_tile_2d_pair_elect(unsigned dst_smem, const CUtensorMap* tm, int x, int y, unsigned bar_cluster_addr) {
-  asm volatile(
-      "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n\t}" ::"r"(dst_smem),
-      "l"(reinterpret_cast<unsigned long long>(tm)), "r"(bar_cluster_addr), "r"(x), "r"(y)
-      : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx_addr_elect(unsigned cluster_addr, unsigned bytes) {
-  asm volatile(
-      "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "@e mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;\n\t}" ::"r"(cluster_addr), "r"(bytes)
-      : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_n_elect(void* bar, unsigned n) {
-  asm volatile(
-      "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "@e mbarrier.arrive.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(bar)), "r"(n)
       : "memory");
 }
 
