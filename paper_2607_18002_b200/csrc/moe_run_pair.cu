@@ -162,8 +162,9 @@ __device__ __forceinline__ void release_slot(SharedCtl<kTileRows>* sc, int islot
   mbar_arrive(leader ? &sc->iempty[islot] : &sc->iread[islot]);
 }
 
-// ... behind a fence that orders what the arrival hands over: the fence.acq_rel.gpu of a warp that counts a stored tile (one that does not
-// count has stored nothing), the tcgen05.fence of a warp that has drained an accumulator.  A release would wait for the stores again.
+// Arrival at the leader behind a fence that orders what it hands over: the fence.acq_rel.gpu of a warp that counts a stored tile (one that
+// does not count has stored nothing), the tcgen05.fence of a warp that has drained an accumulator.  A release would wait for the
+// stores again.
 __device__ __forceinline__ void signal_leader(void* bar, bool leader) {
   if (leader) mbar_arrive(bar);
   else mbar_arrive_relaxed(map_to_cta(bar, 0));
