@@ -264,64 +264,53 @@ __device__ __forceinline__ void st_cluster_v4(unsigned cluster_addr, uint4 v) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// ---- warp-uniform issue: the whole warp executes these, one elected lane issues the instruction.
-// Their operands then stay warp-uniform for the compiler (no per-thread staging of descriptors),
-// which keeps the issue loops of the MMA and producer warps short.
-// arrives on the barrier at the same shared-memory offset in both CTAs once the pair's MMAs so far retire
-__device__ __forceinline__ void tc_commit_pair_elect(void* bar) {
-  asm volatile(
-      "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
-      "h"((unsigned short)3)
-      : "memory");
+// one lane of a converged warp.  The compiler knows a branch on elect.sync for a region of one thread: instructions that take uniform
+// registers (TMA, MMA, commit) are then issued as they stand
+__device__ __forceinline__ bool elect_one() {
+  unsigned e;
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 r;\n\telect.sync r|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0;
+}
+// arrives on the barrier at the same shared-memory offset in both CTAs once this thread's MMAs of the pair so far retire
+__device__ __forceinline__ void tc_commit_pair(void* bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+               "h"((unsigned short)3)
+               : "memory");
 }
 
-// All loads and barrier arrivals of one k-block by one CTA of a pair, as ONE instruction group under a
-// single election: expect_tx on the leader's stage barrier, the box of 128 weight rows, up to three
-// activation boxes (a_rows rows apart), the stand-in arrivals (tiles without a gather) and the go-ahead for the
-// gather warps.  Flags select what is issued; everything is warp-uniform.  w_policy: the L2 policy of the weights.
-__device__ __forceinline__ void pair_issue_kblock(unsigned bar, unsigned tx, unsigned standin_bar, unsigned standin_n,
-                                                  unsigned sW, const CUtensorMap* tmw, int x, int wblk, int expert,
-                                                  unsigned sX, const CUtensorMap* tma, int ay, unsigned a_boxes, unsigned a_rows,
-                                                  unsigned go_bar, unsigned has_go, unsigned long long w_policy) {
+// The weights of one k-block by one CTA of a pair, by one thread: expect_tx (of the rows' bytes too) on the leader's stage barrier, the
+// stand-in arrivals (tiles without a gather), the go-ahead for those that bring the rows, and the box of 128 weight rows with its L2
+// policy.  The next stage's barrier is tested first and the result read last, as with the MMAs: returns whether that stage is free.
+__device__ __forceinline__ bool pair_issue_kblock(unsigned bar, unsigned tx, unsigned standin_bar, unsigned standin_n, unsigned go_bar,
+                                                  unsigned has_go, unsigned sW, const CUtensorMap* tmw, int x, int wblk, int expert,
+                                                  unsigned long long w_policy, unsigned next_empty_bar, unsigned next_parity) {
+  unsigned ready;
   asm volatile(
-      "{\n\t.reg .pred e, pa1, pa2, pa3, pgo, pst;\n\t.reg .b32 r, st, z, sA1, ay1, sA2, ay2;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "setp.ge.and.u32 pa1, %12, 1, e;\n\t"
-      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"
-      "setp.ge.and.u32 pa3, %12, 3, e;\n\t"
-      "setp.ne.and.b32 pgo, %15, 0, e;\n\t"
-      "setp.ne.and.b32 pst, %3, 0, e;\n\t"
+      "{\n\t.reg .pred pgo, pst, pn;\n\t.reg .b32 z;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 pn, [%13], %14;\n\t"
+      "setp.ne.b32 pst, %4, 0;\n\t"
+      "setp.ne.b32 pgo, %6, 0;\n\t"
       "mov.b32 z, 0;\n\t"
-      "shl.b32 st, %13, 7;\n\t"
-      "add.u32 sA1, %9, st;\n\t"
-      "add.s32 ay1, %11, %13;\n\t"
-      "add.u32 sA2, sA1, st;\n\t"
-      "add.s32 ay2, ay1, %13;\n\t"
-      "@e mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;\n\t"
-      "@pst mbarrier.arrive.shared::cta.b64 _, [%2], %3;\n\t"
-      "@e cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%4], [%5, {%6, z, z, %7, %8}], [%0], %16;\n\t"
-      "@pa1 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%9], [%10, {%6, %11}], [%0];\n\t"
-      "@pa2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA1], [%10, {%6, ay1}], [%0];\n\t"
-      "@pa3 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [sA2], [%10, {%6, ay2}], [%0];\n\t"
-      "@pgo mbarrier.arrive.shared::cta.b64 _, [%14];\n\t}"
-      ::"r"(bar), "r"(tx), "r"(standin_bar), "r"(standin_n),
-        "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert),
-        "r"(sX), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "r"(a_rows),
-        "r"(go_bar), "r"(has_go), "l"(w_policy)
+      "mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%1], %2;\n\t"
+      "@pgo mbarrier.arrive.shared::cta.b64 _, [%5];\n\t"
+      "@pst mbarrier.arrive.shared::cta.b64 _, [%3], %4;\n\t"
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%7], [%8, {%9, z, z, %10, %11}], [%1], %12;\n\t"
+      "selp.u32 %0, 1, 0, pn;\n\t}"
+      : "=r"(ready)
+      : "r"(bar), "r"(tx), "r"(standin_bar), "r"(standin_n), "r"(go_bar), "r"(has_go), "r"(sW),
+        "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert), "l"(w_policy), "r"(next_empty_bar), "r"(next_parity)
       : "memory");
+  return ready != 0;
 }
 
-// The activation boxes alone, for a k-block whose weights and expect_tx went out before
+// The activation boxes of one k-block by one CTA of a pair, by one thread: up to three, a_rows rows apart
 __device__ __forceinline__ void pair_issue_rows(unsigned bar, int x, unsigned sX, const CUtensorMap* tma, int ay, unsigned a_boxes,
                                                 unsigned a_rows) {
   asm volatile(
-      "{\n\t.reg .pred e, pa1, pa2, pa3;\n\t.reg .b32 r, st, sA1, ay1, sA2, ay2;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "setp.ge.and.u32 pa1, %5, 1, e;\n\t"
-      "setp.ge.and.u32 pa2, %5, 2, e;\n\t"
-      "setp.ge.and.u32 pa3, %5, 3, e;\n\t"
+      "{\n\t.reg .pred pa1, pa2, pa3;\n\t.reg .b32 st, sA1, ay1, sA2, ay2;\n\t"
+      "setp.ge.u32 pa1, %5, 1;\n\t"
+      "setp.ge.u32 pa2, %5, 2;\n\t"
+      "setp.ge.u32 pa3, %5, 3;\n\t"
       "shl.b32 st, %6, 7;\n\t"
       "add.u32 sA1, %2, st;\n\t"
       "add.s32 ay1, %4, %6;\n\t"
@@ -334,28 +323,26 @@ __device__ __forceinline__ void pair_issue_rows(unsigned bar, int x, unsigned sX
       : "memory");
 }
 
-// One k-block of the pair's MMAs as ONE instruction group: the next stage's barrier is tested first and
+// One k-block of the pair's MMAs, by one thread: the next stage's barrier is tested first and
 // the result is only read after the four MMAs and the commit have been issued, so that the barrier's
-// shared-memory round trip hides behind the issue of the MMAs.  Whole warp, warp-uniform operands; one
-// elected lane issues the MMAs and the commit.  Returns whether the next stage is already full.
+// shared-memory round trip hides behind the issue of the MMAs.  Returns whether the next stage is already full.
 __device__ __forceinline__ bool pair_mma_kblock(unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc,
                                                 unsigned idesc, unsigned accumulate_first, unsigned empty_bar,
                                                 unsigned next_full_bar, unsigned next_parity) {
   unsigned ready;
   asm volatile(
-      "{\n\t.reg .pred e, p0, p1, pn;\n\t.reg .b32 r;\n\t.reg .b16 m;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "{\n\t.reg .pred p0, p1, pn;\n\t.reg .b16 m;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
       "mov.b16 m, 3;\n\t"
       "mbarrier.test_wait.parity.shared::cta.b64 pn, [%7], %8;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
       "setp.ne.b32 p0, %5, 0;\n\t"
       "setp.eq.b32 p1, 0, 0;\n\t"
       "add.u64 a1, %2, 2;\n\tadd.u64 a2, %2, 4;\n\tadd.u64 a3, %2, 6;\n\t"
       "add.u64 b1, %3, 2;\n\tadd.u64 b2, %3, 4;\n\tadd.u64 b3, %3, 6;\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%1], %2, %3, %4, p0;\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%1], a1, b1, %4, p1;\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%1], a2, b2, %4, p1;\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%1], a3, b3, %4, p1;\n\t"
-      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%6], m;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%1], %2, %3, %4, p0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%1], a1, b1, %4, p1;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%1], a2, b2, %4, p1;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%1], a3, b3, %4, p1;\n\t"
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%6], m;\n\t"
       "selp.u32 %0, 1, 0, pn;\n\t}"
       : "=r"(ready)
       : "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate_first), "r"(empty_bar),

@@ -16,7 +16,7 @@
 //   - a tile uses up to 256 of the 512 TMEM columns, so the epilogue of one tile overlaps the MMAs of the next.
 // Roles per CTA (16 warps): leader only -- warp 0 scheduler (claims, waits for dependencies,
 // publishes tile descriptors to both CTAs), warp 1 MMA issuer, warp 2 committer; both CTAs --
-// warp 3 producer (TMA loads of its own half, read from the descriptor ring), warps 4-7 gather,
+// warp 3 producer (TMA loads of its own half of the weights), warps 4-7 gather (a thread of warp 4 loads consecutive rows as boxes),
 // warps 8-15 epilogue; second CTA only -- warp 1 relays the completion of its gather to the
 // leader.  Tile descriptors reach the second CTA through distributed shared memory; its barrier
 // arrivals that the leader waits for are remote mbarrier arrivals.  Its roles give a ring slot back to
@@ -24,7 +24,6 @@
 #include "moe_combine.cuh"
 #include "moe_ptx.cuh"
 #include "moe_sched.cuh"
-#include <climits>
 
 namespace moe {
 namespace pairk {
@@ -61,7 +60,8 @@ struct SharedCtl {
   // place); on tiles without a gather the leader's producer arrives in their place
   unsigned long long full[Ring<kTileRows>::kNS];
   unsigned long long fullA[Ring<kTileRows>::kNS];     // second CTA: completion of its own gather threads' copies
-  unsigned long long goA[Ring<kTileRows>::kNS];       // producer -> gather warps: the stage may be overwritten
+  unsigned long long goA[Ring<kTileRows>::kNS];       // producer -> gather warps: the stage may be overwritten (gathered rows)
+  unsigned long long goR[Ring<kTileRows>::kNS];       // ... (consecutive rows: the thread that loads their boxes)
   unsigned long long empty[Ring<kTileRows>::kNS];     // both (multicast commit): the stage's MMAs retired
   unsigned long long tfull[2];       // both (multicast commit): accumulator complete
   unsigned long long tempty[2];      // leader's: accumulator drained by the 16 epilogue warps
@@ -110,8 +110,9 @@ __device__ __forceinline__ bool bwait(const Ctx& c, void* bar, unsigned parity, 
 __device__ __forceinline__ bool wwait_cluster(const Ctx& c, void* bar, unsigned parity, int where) {
   return __all_sync(0xffffffffu, bwait<mbar_try_cluster>(c, bar, parity, where));
 }
+// by the one thread that issues the MMAs
 __device__ __forceinline__ bool wwait_relaxed(const Ctx& c, void* bar, unsigned parity, int where) {
-  return __all_sync(0xffffffffu, bwait<mbar_try_relaxed>(c, bar, parity, where));
+  return bwait<mbar_try_relaxed>(c, bar, parity, where);
 }
 __device__ __forceinline__ bool wwait(const Ctx& c, void* bar, unsigned parity, int where) {
   return __all_sync(0xffffffffu, mbar_wait(c, bar, parity, where));
@@ -140,13 +141,6 @@ __device__ __forceinline__ bool wait_info(const Ctx& c, void* bar, unsigned pari
   return __all_sync(0xffffffffu, info_wait_one(c, bar, parity, where, leader));
 }
 
-// whether the scheduler has seen the rows of the tile in ring slot `islot` in place
-template <int kTileRows>
-__device__ __forceinline__ bool rows_in_place(SharedCtl<kTileRows>* sc, int islot, unsigned parity, bool leader) {
-  const bool in = leader ? mbar_test(&sc->rows_in[islot], parity) : mbar_test_cluster(&sc->rows_in[islot], parity);
-  return __all_sync(0xffffffffu, in);
-}
-
 // arrival on a barrier that lives in the leader's shared memory
 __device__ __forceinline__ void arrive_at_leader(void* bar, bool leader) {
   if (leader) mbar_arrive(bar);
@@ -170,25 +164,35 @@ __device__ __forceinline__ void signal_leader(void* bar, bool leader) {
   else mbar_arrive_relaxed(map_to_cta(bar, 0));
 }
 
-// what one CTA loads per k-block of a tile
-struct LoadPlan {
-  const CUtensorMap* tmw;
-  const CUtensorMap* tma;
-  int wblk, expert;   // place of the 128 weight rows (see OpDev)
-  int ay, a_boxes;    // first activation row, number of boxes (0: none or gathered)
-  int a_box_rows;
-  unsigned tx;
-  bool g1;
-  unsigned long long policy;   // L2 policy of the weights
+// The consecutive rows that one CTA loads per k-block of a tile, as boxes: of the packed intermediate (down tile) or of x itself
+// (masked-layout gate/up tile).  None where the rows are gathered.
+struct RowPlan {
+  const CUtensorMap* map;
+  int y, boxes, box_rows;      // first row, number of boxes and their rows
+  __device__ __forceinline__ unsigned bytes() const { return (unsigned)(boxes * box_rows * kRowBytes); }
 };
+__device__ __forceinline__ RowPlan row_plan(const OpDev* op, int kind, int row0, int rows, int rank) {
+  const int rpc = tile_cols(rows) / 2;       // rows per CTA
+  const int mine = kind == kGateUp ? 0 : min(rows - rank * rpc, rpc);
+  const bool fromx = kind != kDown;
+  RowPlan p{&op->tm_a8, row0 + rank * rpc, 0, 0};
+  if (mine > 96) p = RowPlan{fromx ? &op->tm_x128 : &op->tm_a128, p.y, 1, 128};
+  else if (mine > 16) p = RowPlan{fromx ? &op->tm_x32 : &op->tm_a32, p.y, (mine + 31) / 32, 32};
+  else if (mine > 0) p = RowPlan{fromx ? &op->tm_x8 : &op->tm_a8, p.y, (mine + 7) / 8, 8};
+  return p;
+}
 
-__device__ __forceinline__ LoadPlan make_plan(const OpDev* op, const TileInfo& ti, int rank) {
-  LoadPlan p;
-  const int rpc = tile_cols(ti.rows) / 2;    // rows per CTA
-  p.g1 = ti.kind == kGateUp;                 // activation rows come from the gather warps
+// The place of a tile's 128 weight rows of one CTA, and their L2 policy
+struct WeightPlan {
+  const CUtensorMap* map;
+  int blk, expert;             // (see OpDev)
+  unsigned long long policy;
+};
+__device__ __forceinline__ WeightPlan weight_plan(const OpDev* op, const TileInfo& ti, int rank) {
+  WeightPlan p;
   const bool w1 = ti.kind != kDown;          // gate/up weights
-  p.tmw = w1 ? &op->tm_p1 : &op->tm_p2;
-  p.wblk = w1 ? (ti.n * kTileN1 + 64 * rank) / 8 : (ti.n * kTileN2 + 128 * rank) / 16;
+  p.map = w1 ? &op->tm_p1 : &op->tm_p2;
+  p.blk = w1 ? (ti.n * kTileN1 + 64 * rank) / 8 : (ti.n * kTileN2 + 128 * rank) / 16;
   p.expert = ti.expert & (kReadOnce - 1);
   // Where one work tile reads an expert's weights, they are marked to leave L2 first and do not push out what is read again (one token: 72.7 ->
   // 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  A plan knows its own op only: of two unpaired ops of a launch
@@ -199,38 +203,7 @@ __device__ __forceinline__ LoadPlan make_plan(const OpDev* op, const TileInfo& t
   // on 128 experts 1255 -> 1274.  The weights of experts of several tiles are the data read again: marked, they cost (8192 tokens: 2390 ->
   // 2510).
   p.policy = kReadOnce & ti.expert ? l2_evict_first() : l2_evict_normal();
-  p.a_boxes = 0;
-  p.a_box_rows = 0;
-  p.ay = ti.row0 + rank * rpc;
-  p.tma = &op->tm_a8;
-  unsigned a_bytes = 0;
-  if (!p.g1) {
-    // consecutive rows: of the packed intermediate (down tile) or of x itself (masked-layout gate/up tile)
-    const bool fromx = w1;
-    const int mine = min(ti.rows - rank * rpc, rpc);
-    if (mine > 0) {
-      if (mine <= 16) { p.tma = fromx ? &op->tm_x8 : &op->tm_a8; p.a_boxes = (mine + 7) / 8; p.a_box_rows = 8; }
-      else if (mine <= 96) { p.tma = fromx ? &op->tm_x32 : &op->tm_a32; p.a_boxes = (mine + 31) / 32; p.a_box_rows = 32; }
-      else { p.tma = fromx ? &op->tm_x128 : &op->tm_a128; p.a_boxes = 1; p.a_box_rows = 128; }
-      a_bytes = (unsigned)(p.a_boxes * p.a_box_rows * kRowBytes);
-    }
-  }
-  p.tx = (unsigned)kBBytes + a_bytes;
   return p;
-}
-
-// one k-block of loads, executed by the whole producer warp with warp-uniform arguments; one
-// elected lane issues each instruction (the stage is known to be free)
-template <int kTileRows>
-__device__ __forceinline__ void issue_kblock(SharedCtl<kTileRows>* sc, unsigned stages_addr, const LoadPlan& p, int kb,
-                                             unsigned stage, bool leader, unsigned full0_addr) {
-  const unsigned sX = stages_addr + stage * (unsigned)Ring<kTileRows>::kSB;
-  const unsigned bar = full0_addr + stage * 8u;            // the leader's full[stage]
-  pair_issue_kblock(bar, p.tx, smem_u32(&sc->full[stage]),
-                    (leader && !p.g1) ? (unsigned)kGatherThreads + 1u : 0u,   // nobody gathers for this tile
-                    sX + (unsigned)Ring<kTileRows>::kABytes, p.tmw, kb * kBlockK, p.wblk, p.expert,
-                    sX, p.tma, p.ay, (unsigned)p.a_boxes, (unsigned)p.a_box_rows,
-                    smem_u32(&sc->goA[stage]), p.g1 ? 1u : 0u, p.policy);
 }
 
 // The epilogue warps' wait inside a combine tile: one lane of the CTA looks at the op's counter and counts the tile (its `turn`-th) in
@@ -292,6 +265,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       mbar_init(&sc->full[s], kFullCount);
       mbar_init(&sc->fullA[s], kGatherThreads);
       mbar_init(&sc->goA[s], 1);
+      mbar_init(&sc->goR[s], 1);
       mbar_init(&sc->empty[s], 1);
     }
     for (int s = 0; s < 2; ++s) {
@@ -400,138 +374,119 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     if (lane == 0) end_turn(&args, asked ? ticket : take_turn(&args), (int)(gridDim.x >> 1));
   } else if (warp == 3) {
     // ============================================================ producer (both CTAs)
-    // Reads tiles from the ring and issues this CTA's loads, one stage per k-block.  The whole
-    // warp runs the loop on warp-uniform values; one elected lane issues each instruction.
-    ended = false;
-    int islot = 0;
-    unsigned iph = 0;
-    unsigned stage = 0, par = 1;                           // parity of "stage is free"
-    const unsigned stages_addr = smem_u32(stages);
-    const unsigned full0_addr = leader ? smem_u32(&sc->full[0]) : map_to_cta(&sc->full[0], 0);
-    while (true) {
-      if (!wait_info(c, &sc->ifull[islot], iph, 21, leader)) break;
-      TileInfo ti;
-      ti.kind = __shfl_sync(0xffffffffu, sc->info[islot].kind, 0);
-      ti.slot = __shfl_sync(0xffffffffu, sc->info[islot].slot, 0);
-      ti.row0 = __shfl_sync(0xffffffffu, sc->info[islot].row0, 0);
-      ti.rows = __shfl_sync(0xffffffffu, sc->info[islot].rows, 0);
-      ti.n = __shfl_sync(0xffffffffu, sc->info[islot].n, 0);
-      ti.kblocks = __shfl_sync(0xffffffffu, sc->info[islot].kblocks, 0);
-      ti.expert = __shfl_sync(0xffffffffu, sc->info[islot].expert, 0);
-      if (ti.kind == kEnd) { ended = true; break; }
-      const int tslot = islot;
-      const unsigned tph = iph;
-      if (leader && lane == 0) mbar_arrive(&sc->taken[tslot]);
-      if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (ti.kind == kCombine) {
-        if (lane == 0) release_slot(sc, tslot, leader);
-        continue;
-      }
-      LoadPlan lp = make_plan(&args.ops[ti.slot], ti, rank);
-      bool fail = false;
-      int kb = 0;
-      if (ti.kind == kDown && !rows_in_place(sc, tslot, tph, leader)) {
-        const unsigned boxes = (unsigned)lp.a_boxes, stage0 = stage;
-        lp.a_boxes = 0;
-        bool in = false;
-        do {
-          if (!wwait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
-          issue_kblock(sc, stages_addr, lp, kb, stage, leader, full0_addr);
-          if (++stage == kNS) { stage = 0; par ^= 1u; }
-          in = rows_in_place(sc, tslot, tph, leader);
-        } while (++kb < min(ti.kblocks, kNS) && !in);
-        if (fail || !wait_info(c, &sc->rows_in[tslot], tph, 27, leader)) break;
-        for (int j = 0, s = (int)stage0; j < kb; ++j) {
-          pair_issue_rows(full0_addr + s * 8u, j * kBlockK, stages_addr + s * (unsigned)kSB, lp.tma, lp.ay, boxes,
-                          (unsigned)lp.a_box_rows);
-          if (++s == kNS) s = 0;
-        }
-        lp.a_boxes = (int)boxes;
-      }
-      if (lane == 0) release_slot(sc, tslot, leader);   // the ring slot's barriers are not looked at any more
-      for (; kb < ti.kblocks; ++kb) {
-        if (!wwait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
-        issue_kblock(sc, stages_addr, lp, kb, stage, leader, full0_addr);
-        if (++stage == kNS) { stage = 0; par ^= 1u; }
-      }
-      if (fail) break;
-    }
-  } else if (warp == 1 && leader) {
-    // ============================================================ MMA issuer (leader)
-    // The whole warp runs the loops with warp-uniform values and one elected lane issues each
-    // MMA and commit: per k-block one barrier wait, four MMAs and one commit, which keeps
-    // issuing ahead of the tensor pipe (about 512 clocks per k-block of a 256-row tile).
-    ended = false;
-    int islot = 0;
-    unsigned iph = 0, gcount = 0;
-    unsigned stage = 0, par = 0;
-    const unsigned sbase = smem_u32(stages);
-    while (true) {
-      if (!wait_info(c, &sc->ifull[islot], iph, 6, true)) break;
-      const int kind = __shfl_sync(0xffffffffu, sc->info[islot].kind, 0);
-      const int kblocks = __shfl_sync(0xffffffffu, sc->info[islot].kblocks, 0);
-      const int rows = __shfl_sync(0xffffffffu, sc->info[islot].rows, 0);
-      if (kind == kEnd) { ended = true; break; }
-      if (kind != kCombine) {
-        const unsigned b = gcount & 1u;
-        if (!wwait_relaxed(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
-        tc_fence_after();
-        const unsigned d = __shfl_sync(0xffffffffu, tmem, 0) + b * (unsigned)kAccCols;
-        const unsigned idesc = kIdescM256 | ((unsigned)tile_cols(rows) >> 3) << 17;
-        const bool g1 = kind == kGateUp;
+    // Reads tiles from the ring and loads this CTA's weights, one stage per k-block; the rows are loaded by the gather warps, because a TMA
+    // instruction holds its thread for some 140 clocks.  One thread runs the whole role (see the MMA issuer).
+    if (elect_one()) {
+      ended = false;
+      int islot = 0;
+      unsigned iph = 0;
+      unsigned stage = 0, par = 1;                           // parity of "stage is free"
+      bool ready = false;                                    // the stage was seen free by the look-ahead test
+      const unsigned w0 = smem_u32(stages) + (unsigned)kABytes, go_rows = smem_u32(&sc->goR[0]), go_gather = smem_u32(&sc->goA[0]);
+      const unsigned full0 = leader ? smem_u32(&sc->full[0]) : map_to_cta(&sc->full[0], 0), empty0 = smem_u32(&sc->empty[0]);
+      while (true) {
+        if (!info_wait_one(c, &sc->ifull[islot], iph, 21, leader)) break;
+        const TileInfo ti = sc->info[islot];
+        if (ti.kind == kEnd) { ended = true; break; }
+        if (leader) mbar_arrive(&sc->taken[islot]);
+        release_slot(sc, islot, leader);
+        if (++islot == kRing) { islot = 0; iph ^= 1u; }
+        if (ti.kind == kCombine) continue;
+        const OpDev* op = &args.ops[ti.slot];
+        const WeightPlan wp = weight_plan(op, ti, rank);
+        const unsigned row_bytes = row_plan(op, ti.kind, ti.row0, ti.rows, rank).bytes();
+        const bool g1 = ti.kind == kGateUp;
+        const unsigned standin = leader && !g1 ? (unsigned)kGatherThreads + 1u : 0u;   // nobody gathers for this tile
+        const unsigned go = g1 ? go_gather : go_rows, has_go = g1 || row_bytes ? 1u : 0u;
         bool fail = false;
-        bool ready = false;                           // the current stage was seen full by the look-ahead test
-        const unsigned full0 = smem_u32(&sc->full[0]), empty0 = smem_u32(&sc->empty[0]);
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!ready && !wwait(c, &sc->full[stage], par, 8)) { fail = true; break; }
-          if (g1) fence_async_proxy_smem();            // this CTA's cp.async-written rows -> tensor core reads
-          const unsigned sA = sbase + stage * (unsigned)kSB;
-          const unsigned long long wd = umma_desc(sA + kABytes, kRowBytes), xd = umma_desc(sA, kRowBytes);
+        for (int kb = 0; kb < ti.kblocks; ++kb) {
+          if (!ready && !mbar_wait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
           const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
-          // four MMAs (+32 bytes along K per step: the descriptor's address field counts 16 bytes), the
-          // commit that frees the stage in both CTAs, and the test of the next stage's barrier
-          ready = pair_mma_kblock(d, wd, xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u, full0 + nstage * 8u, npar);
-          ready = __all_sync(0xffffffffu, ready) && kb + 1 < kblocks;
+          ready = pair_issue_kblock(full0 + stage * 8u, (unsigned)kBBytes + row_bytes, smem_u32(&sc->full[stage]), standin, go + stage * 8u, has_go,
+                                    w0 + stage * (unsigned)kSB, wp.map, kb * kBlockK, wp.blk, wp.expert, wp.policy, empty0 + nstage * 8u, npar);
           stage = nstage;
           par = npar;
         }
         if (fail) break;
-        tc_commit_pair_elect(&sc->tfull[b]);            // accumulator complete, both CTAs
-        ++gcount;
       }
-      if (lane == 0) mbar_arrive(&sc->iempty[islot]);
-      if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
+    __syncwarp();
+  } else if (warp == 1 && leader) {
+    // ============================================================ MMA issuer (leader)
+    // One thread runs the whole role.  Inside a branch on elect.sync the compiler knows that a single thread is there and feeds the
+    // instructions from uniform registers as they are.  With the whole warp in the loop and an election around each group, the same four MMAs
+    // and commit took 300 clocks to issue (350 with the fence of a gathered tile), whatever the tile's rows, now 240 (260); a probe without
+    // loads issues them in 155, and in 315 that way.  A k-block of up to 64 gathered rows went from 445 to 390 clocks (4096 tokens on 16
+    // experts), 16 384 + 256 paired from 4330 to 4300 us: the 1000 W cap takes most of it back as clock.  One token: 56.0 -> 54.9 us a pass.
+    if (elect_one()) {
+      ended = false;
+      int islot = 0;
+      unsigned iph = 0, gcount = 0;
+      unsigned stage = 0, par = 0;
+      bool ready = false;                             // the current stage was seen full by the look-ahead test
+      const unsigned full0 = smem_u32(&sc->full[0]), empty0 = smem_u32(&sc->empty[0]);
+      const unsigned long long desc0 = umma_desc(smem_u32(stages), kRowBytes);
+      while (true) {
+        if (!info_wait_one(c, &sc->ifull[islot], iph, 6, true)) break;
+        const int kind = sc->info[islot].kind, kblocks = sc->info[islot].kblocks, rows = sc->info[islot].rows;
+        if (kind == kEnd) { ended = true; break; }
+        if (kind != kCombine) {
+          const unsigned b = gcount & 1u;
+          if (!wwait_relaxed(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
+          tc_fence_after();
+          const unsigned d = tmem + b * (unsigned)kAccCols;
+          const unsigned idesc = kIdescM256 | ((unsigned)tile_cols(rows) >> 3) << 17;
+          const bool g1 = kind == kGateUp;
+          bool fail = false;
+          for (int kb = 0; kb < kblocks; ++kb) {
+            if (!ready && !mbar_wait(c, &sc->full[stage], par, 8)) { fail = true; break; }
+            if (g1) fence_async_proxy_smem();          // this CTA's cp.async-written rows -> tensor core reads
+            const unsigned long long xd = desc0 + stage * (unsigned)(kSB / 16), wd = xd + (unsigned)(kABytes / 16);
+            const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
+            // four MMAs (+32 bytes along K per step: the descriptor's address field counts 16 bytes), the
+            // commit that frees the stage in both CTAs, and the test of the next stage's barrier (of the next tile's first one too)
+            ready = pair_mma_kblock(d, wd, xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u, full0 + nstage * 8u, npar);
+            stage = nstage;
+            par = npar;
+          }
+          if (fail) break;
+          tc_commit_pair(&sc->tfull[b]);                // accumulator complete, both CTAs
+          ++gcount;
+        }
+        mbar_arrive(&sc->iempty[islot]);
+        if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      }
+    }
+    __syncwarp();
   } else if (warp == 1) {
     // ============================================================ gather relay (second CTA)
     // When this CTA's gather threads' copies of a stage have landed it makes them visible to the
     // tensor core (proxy fence) and arrives on the leader's stage barrier.
-    ended = false;
-    int islot = 0;
-    unsigned iph = 0, kiter = 0, amask = 0;
-    while (true) {
-      if (!wait_info(c, &sc->ifull[islot], iph, 24, false)) break;
-      const int kind = sc->info[islot].kind;
-      const int kblocks = sc->info[islot].kblocks;
-      __syncwarp();
-      if (kind == kEnd) { ended = true; break; }
-      if (lane == 0) release_slot(sc, islot, false);
-      if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (kind == kCombine) continue;
-      if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
-      bool fail = false;
-      for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
-        const int stage = (int)(kiter % kNS);
-        if (!wwait(c, &sc->fullA[stage], (amask >> stage) & 1u, 25)) { fail = true; break; }
-        amask ^= 1u << stage;
-        if (lane == 0) {
+    if (elect_one()) {
+      ended = false;
+      int islot = 0;
+      unsigned iph = 0, kiter = 0, amask = 0;
+      while (true) {
+        if (!info_wait_one(c, &sc->ifull[islot], iph, 24, false)) break;
+        const int kind = sc->info[islot].kind;
+        const int kblocks = sc->info[islot].kblocks;
+        if (kind == kEnd) { ended = true; break; }
+        release_slot(sc, islot, false);
+        if (++islot == kRing) { islot = 0; iph ^= 1u; }
+        if (kind == kCombine) continue;
+        if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
+        bool fail = false;
+        for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
+          const int stage = (int)(kiter % kNS);
+          if (!mbar_wait(c, &sc->fullA[stage], (amask >> stage) & 1u, 25)) { fail = true; break; }
+          amask ^= 1u << stage;
           fence_async_proxy_smem();
           mbar_arrive_remote(map_to_cta(&sc->full[stage], 0));
         }
-        __syncwarp();
+        if (fail) break;
       }
-      if (fail) break;
     }
+    __syncwarp();
   } else if (warp >= 4 && warp < 4 + kGatherThreads / 32) {
     // ============================================================ gather warps (cp.async)
     // This CTA's rows of a gate/up tile: row r of the tile is token sorted_to_flat[row0 + r] / k.
@@ -544,9 +499,13 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // 16 rows per cp.async round
     constexpr int kPasses = Ring<kTileRows>::kRows / kRowsPerPass;
     const int chunk = gt % kCpr, rbase = gt / kCpr;
+    // the swizzle XORs the chunk index with the row's place in its 8-row group, which is the same in every pass
+    static_assert(kRowsPerPass % 8 == 0, "");
+    const unsigned dst0 = smem_u32(stages) + rbase * kRowBytes + ((chunk ^ (rbase & 7)) << 4);
     ended = false;
     int islot = 0;
-    unsigned iph = 0, kiter = 0, gmask = 0;
+    unsigned iph = 0, kiter = 0, gmask = 0, rmask = 0;
+    const unsigned rows0 = smem_u32(stages), full0 = leader ? smem_u32(&sc->full[0]) : map_to_cta(&sc->full[0], 0);
     while (true) {
       if (!wait_info(c, &sc->ifull[islot], iph, 13, leader)) break;
       const int kind = sc->info[islot].kind;
@@ -554,13 +513,38 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
-      if (lane == 0) release_slot(sc, islot, leader);
+      const int tslot = islot;
+      const unsigned tph = iph;
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (kind == kCombine) continue;
-      if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
       const OpDev* op = &args.ops[slot];
+      // Consecutive rows: one thread of one warp loads their boxes, once the scheduler has seen them in place (the weights of a down tile
+      // are loaded meanwhile) and the producer has the stage.
+      if (kind == kDown || kind == kGateUpDirect) {
+        bool fail = false;
+        if (warp == 4 && elect_one()) {
+          fail = !info_wait_one(c, &sc->rows_in[tslot], tph, 27, leader);
+          release_slot(sc, tslot, leader);
+          const RowPlan rp = row_plan(op, kind, row0, rows, rank);
+          unsigned stage = kiter % (unsigned)kNS;
+          if (rp.boxes > 0)
+            for (int kb = 0; kb < kblocks && !fail; ++kb) {
+              if (!mbar_wait(c, &sc->goR[stage], (rmask >> stage) & 1u, 32)) { fail = true; break; }
+              rmask ^= 1u << stage;
+              pair_issue_rows(full0 + stage * 8u, kb * kBlockK, rows0 + stage * (unsigned)kSB, rp.map, rp.y, (unsigned)rp.boxes,
+                              (unsigned)rp.box_rows);
+              if (++stage == kNS) stage = 0;
+            }
+        } else if (warp != 4 && lane == 0) {
+          release_slot(sc, tslot, leader);
+        }
+        if (__any_sync(0xffffffffu, fail)) break;
+        kiter += (unsigned)kblocks;
+        continue;
+      }
+      if (lane == 0) release_slot(sc, tslot, leader);
+      if (kind == kCombine) continue;
       // a paired op's gather list also holds rows of its partner, tagged with their slot: those come from
-      // the partner's activations (kept as the complement of the token index)
+      // the partner's activations
       const bool paired = op->paired != 0;
       const OpDev* pop = paired ? &args.ops[op->partner] : op;
       const unsigned char* X = static_cast<const unsigned char*>(op->x) + chunk * 16;
@@ -568,7 +552,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const size_t pitch = (size_t)args.H * 2;
       const int rpc = tile_cols(rows) / 2;
       const int first = rank * rpc;                       // this CTA's first row of the tile
-      int tok[kPasses];
+      const unsigned char* src[kPasses];                  // this thread's 16 bytes of the row's first k-block
       const int n_rows = op->n_rows, n_rows_p = pop->n_rows;
       const int own_tag = paired ? slot_of(&args, slot) : 0, partner_tag = paired ? slot_of(&args, op->partner) : 0;
       bool bad = false;
@@ -582,7 +566,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         // an index the plan never wrote is reported below and its row is skipped
         const bool in_range = v >= 0 && (tag == own_tag || tag == partner_tag) && flat < (theirs ? n_rows_p : n_rows);
         bad |= mine && !in_range;
-        tok[j] = (mine && in_range) ? (theirs ? ~(flat / args.k) : flat / args.k) : INT_MIN;
+        src[j] = mine && in_range ? (theirs ? Xp : X) + (size_t)(flat / args.k) * pitch : nullptr;
       }
       if (bad) report(c.st, MOE_EBOUNDS, slot_of(&args, slot), row0, rows, 0);
       unsigned long long* landed = leader ? sc->full : sc->fullA;
@@ -591,17 +575,10 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         const int stage = (int)(kiter % kNS);
         if (!wwait(c, &sc->goA[stage], (gmask >> stage) & 1u, 14)) { fail = true; break; }
         gmask ^= 1u << stage;
-        const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-        const unsigned char* Xk = X + (size_t)kb * kRowBytes;
-        const unsigned char* Xpk = Xp + (size_t)kb * kRowBytes;
+        const unsigned sA = dst0 + stage * (unsigned)kSB;
 #pragma unroll
-        for (int j = 0; j < kPasses; ++j) {
-          const int r = rbase + kRowsPerPass * j;
-          const int t = tok[j];
-          if (t != INT_MIN)    // the swizzle XORs the chunk index with the row's place in its 8-row group
-            cp_async_16(sA + r * kRowBytes + ((chunk ^ (r & 7)) << 4),
-                        (t >= 0 ? Xk : Xpk) + (size_t)(t >= 0 ? t : ~t) * pitch);
-        }
+        for (int j = 0; j < kPasses; ++j)
+          if (src[j]) cp_async_16(sA + j * (kRowsPerPass * kRowBytes), src[j] + (size_t)kb * kRowBytes);
         cp_async_arrive_noinc(&landed[stage]);
       }
       if (fail) break;
