@@ -178,7 +178,7 @@ int make_map(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t rows, size
   return r == CUDA_SUCCESS ? MOE_OK : MOE_ECUDA;
 }
 
-// The weights of one GEMM as the M operand: a 5-D view whose box is 128 rows x 128 bytes in one copy.
+// The weights of one GEMM: a 5-D view whose box is the 128 or 256 rows x 128 bytes of a stage in one copy.
 // rows: what one step of dimensions 1..4 moves by, in weight rows.
 int make_map_m(moe_ctx* ctx, CUtensorMap* out, const void* base, size_t cols, const size_t (&size)[4], const size_t (&rows)[4],
                   const cuuint32_t (&boxes)[4]) {
@@ -399,12 +399,12 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
       if (!rc && ctx->pair_kernel)                 // 8 gate rows, the 8 matching up rows, the next 8 gate rows, ...
         rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, I / 8, E}, {1, I, 8, 2 * I}, {8, 2, 8, 1});
       if (!rc && fp8)                              // ... of 16 rows: 8 even gate, 8 even up, 8 odd gate, 8 odd up rows
-        rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, 2 * E * I, 4}, {2, I, 1, 16}, {8, 2, 2, 4});
+        rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, 2 * E * I, 8}, {2, I, 1, 16}, {8, 2, 2, 8});
       if (!rc && (ctx->pair_kernel || fp8))
-        rc = make_map_m(ctx, &h.tm_p2, op->w_down, I, {8, 2, H / 16, E}, {1, 8, 16, H}, {8, 2, 8, 1});
+        rc = make_map_m(ctx, &h.tm_p2, op->w_down, I, {8, 2, H / 16, E}, {1, 8, 16, H}, {8, 2, fp8 ? 16u : 8u, 1});
       if (!ctx->pair_kernel) {
-        if (!rc) rc = make_map(ctx, &h.tm_w1, op->w_gate_up, E * 2 * I, H, 128);
-        if (!rc) rc = make_map(ctx, &h.tm_w2, op->w_down, E * H, I, 128);
+        if (!rc) rc = make_map_m(ctx, &h.tm_w1, op->w_gate_up, H, {I, 2, E, 1}, {1, I, 2 * I, 2 * I}, {128, 2, 1, 1});
+        if (!rc) rc = make_map_m(ctx, &h.tm_w2, op->w_down, I, {128, H / 128, E, 1}, {1, 128, H, H}, {128, 2, 1, 1});
       }
       if (masked) {
         const size_t xr = (size_t)c.n_experts * op->slab_rows;

@@ -15,9 +15,6 @@ __device__ __forceinline__ void mbar_init(void* bar, int count) {
 __device__ __forceinline__ void mbar_arrive(void* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_n(void* bar, unsigned n) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n) : "memory");
-}
 __device__ __forceinline__ bool mbar_try(void* bar, unsigned parity) {
   unsigned ok;
   asm volatile(
@@ -371,109 +368,101 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
   return v;
 }
-// One e4m3 k-block of a small tile: both halves of the weight tile as M = 128 operands against the same few token rows, into
+// One e4m3 k-block of a small tile, by one thread: both halves of the weight tile as M = 128 operands against the same few token rows, into
 // the columns from d and from d + half on; the commit that frees the stage and (end_of_group) the one that hands the group of partials over.
-__device__ __forceinline__ void f8_small_kblock(unsigned d_tmem, unsigned long long w0desc, unsigned long long w1desc,
+// Returns whether the next stage is already full (tested first, read last, as in pair_mma_kblock).
+__device__ __forceinline__ bool f8_small_kblock(unsigned d_tmem, unsigned long long w0desc, unsigned long long w1desc,
                                                 unsigned long long xdesc, unsigned idesc, unsigned half, unsigned pfull_bar, unsigned end_of_group,
-                                                unsigned empty_bar) {
+                                                unsigned empty_bar, unsigned next_full_bar, unsigned next_parity) {
+  unsigned ready;
   asm volatile(
-      "{\n\t.reg .pred e, p0, p1, pg;\n\t.reg .b32 r, d1;\n\t.reg .b64 x1, x2, x3, a1, a2, a3, b1, b2, b3;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
+      "{\n\t.reg .pred p0, p1, pg, pn;\n\t.reg .b32 d1;\n\t.reg .b64 x1, x2, x3, a1, a2, a3, b1, b2, b3;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 pn, [%10], %11;\n\t"
       "setp.ne.b32 p0, 0, 0;\n\t"
       "setp.eq.b32 p1, 0, 0;\n\t"
-      "setp.ne.and.b32 pg, %6, 0, e;\n\t"
-      "add.u32 d1, %0, %8;\n\t"
-      "add.u64 x1, %3, 2;\n\tadd.u64 x2, %3, 4;\n\tadd.u64 x3, %3, 6;\n\t"
-      "add.u64 a1, %1, 2;\n\tadd.u64 a2, %1, 4;\n\tadd.u64 a3, %1, 6;\n\t"
-      "add.u64 b1, %2, 2;\n\tadd.u64 b2, %2, 4;\n\tadd.u64 b3, %2, 6;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %3, %4, p0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a1, x1, %4, p1;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a2, x2, %4, p1;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a3, x3, %4, p1;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], %2, %3, %4, p0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b1, x1, %4, p1;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b2, x2, %4, p1;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b3, x3, %4, p1;\n\t"
-      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n\t"
-      "@pg tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}"
-      ::"r"(d_tmem), "l"(w0desc), "l"(w1desc), "l"(xdesc), "r"(idesc), "r"(pfull_bar), "r"(end_of_group), "r"(empty_bar), "r"(half)
+      "setp.ne.b32 pg, %7, 0;\n\t"
+      "add.u32 d1, %1, %9;\n\t"
+      "add.u64 x1, %4, 2;\n\tadd.u64 x2, %4, 4;\n\tadd.u64 x3, %4, 6;\n\t"
+      "add.u64 a1, %2, 2;\n\tadd.u64 a2, %2, 4;\n\tadd.u64 a3, %2, 6;\n\t"
+      "add.u64 b1, %3, 2;\n\tadd.u64 b2, %3, 4;\n\tadd.u64 b3, %3, 6;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%1], %2, %4, %5, p0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%1], a1, x1, %5, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%1], a2, x2, %5, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%1], a3, x3, %5, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], %3, %4, %5, p0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b1, x1, %5, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b2, x2, %5, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [d1], b3, x3, %5, p1;\n\t"
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n\t"
+      "@pg tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t"
+      "selp.u32 %0, 1, 0, pn;\n\t}"
+      : "=r"(ready)
+      : "r"(d_tmem), "l"(w0desc), "l"(w1desc), "l"(xdesc), "r"(idesc), "r"(pfull_bar), "r"(end_of_group), "r"(empty_bar), "r"(half),
+        "r"(next_full_bar), "r"(next_parity)
       : "memory");
+  return ready != 0;
 }
-// One e4m3 k-block (128 elements = four 32-element MMAs) into a fresh partial buffer, then the two
-// commits (partial full, stage empty), as one group.  Whole warp, warp-uniform operands; one elected
-// lane issues: instructions issued from a divergent single-lane branch cost about 100 clocks each.
+// One e4m3 k-block (128 elements = four 32-element MMAs) into a fresh partial buffer, by one thread, then the two commits (partial full, stage
+// empty).  The barriers of the next k-block, its stage and its partial buffer, are tested first and the results read last.
 __device__ __forceinline__ void f8_mma_kblock(unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc,
-                                              unsigned idesc, unsigned pfull_bar, unsigned empty_bar) {
+                                              unsigned idesc, unsigned pfull_bar, unsigned empty_bar, unsigned next_full_bar, unsigned next_parity,
+                                              unsigned next_pempty_bar, unsigned next_pparity, bool& ready, bool& drained) {
+  unsigned r, d;
   asm volatile(
-      "{\n\t.reg .pred e, p0, p1;\n\t.reg .b32 r;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
+      "{\n\t.reg .pred p0, p1, pn, pp;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 pn, [%8], %9;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 pp, [%10], %11;\n\t"
       "setp.ne.b32 p0, 0, 0;\n\t"
       "setp.eq.b32 p1, 0, 0;\n\t"
-      "add.u64 a1, %1, 2;\n\tadd.u64 a2, %1, 4;\n\tadd.u64 a3, %1, 6;\n\t"
-      "add.u64 b1, %2, 2;\n\tadd.u64 b2, %2, 4;\n\tadd.u64 b3, %2, 6;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a1, b1, %3, p1;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a2, b2, %3, p1;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a3, b3, %3, p1;\n\t"
-      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%4];\n\t"
-      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(pfull_bar), "r"(empty_bar)
+      "add.u64 a1, %3, 2;\n\tadd.u64 a2, %3, 4;\n\tadd.u64 a3, %3, 6;\n\t"
+      "add.u64 b1, %4, 2;\n\tadd.u64 b2, %4, 4;\n\tadd.u64 b3, %4, 6;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%2], %3, %4, %5, p0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%2], a1, b1, %5, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%2], a2, b2, %5, p1;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%2], a3, b3, %5, p1;\n\t"
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t"
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n\t"
+      "selp.u32 %0, 1, 0, pn;\n\t"
+      "selp.u32 %1, 1, 0, pp;\n\t}"
+      : "=r"(r), "=r"(d)
+      : "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(pfull_bar), "r"(empty_bar), "r"(next_full_bar), "r"(next_parity),
+        "r"(next_pempty_bar), "r"(next_pparity)
       : "memory");
+  ready = r != 0;
+  drained = d != 0;
 }
-// The loads of one k-block of the single-CTA kernel as ONE group: expect_tx, the two halves of the
-// weight tile and (down tiles) the box of packed intermediate rows.  Whole warp, warp-uniform
-// operands; one elected lane issues.
-// kOnce: the weights are marked to leave L2 first.
-template <bool kOnce>
-__device__ __forceinline__ void single_issue_kblock(unsigned bar, unsigned tx, unsigned sB0, unsigned sB1,
-                                                    const CUtensorMap* tmw, int x, int wy0, int wy1, unsigned sA,
-                                                    const CUtensorMap* tma, int ay, unsigned has_a) {
-  if constexpr (kOnce) {
-    asm volatile(
-        "{\n\t.reg .pred e, pa;\n\t.reg .b32 r;\n\t"
-        "elect.sync r|e, 0xffffffff;\n\t"
-        "setp.ne.and.b32 pa, %11, 0, e;\n\t"
-        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
-        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%2], [%4, {%5, %6}], [%0], %12;\n\t"
-        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%3], [%4, {%5, %7}], [%0], %12;\n\t"
-        "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%5, %10}], [%0];\n\t}"
-        ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wy0),
-          "r"(wy1), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(has_a), "l"(l2_evict_first())
-        : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred e, pa;\n\t.reg .b32 r;\n\t"
-        "elect.sync r|e, 0xffffffff;\n\t"
-        "setp.ne.and.b32 pa, %11, 0, e;\n\t"
-        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
-        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%4, {%5, %6}], [%0];\n\t"
-        "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%3], [%4, {%5, %7}], [%0];\n\t"
-        "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%8], [%9, {%5, %10}], [%0];\n\t}"
-        ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wy0),
-          "r"(wy1), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(has_a)
-        : "memory");
-  }
-}
-// ... with the two halves of the weight tile as boxes of a 5-D map (coordinates 1 and 2 zero), and up to two activation
-// boxes of 32 rows; w_policy is the L2 policy of the weights
-__device__ __forceinline__ void single_issue_kblock_5d(unsigned bar, unsigned tx, unsigned sB0, unsigned sB1,
-                                                       const CUtensorMap* tmw, int x, int c3_0, int c3_1, int c4, unsigned sA,
-                                                       const CUtensorMap* tma, int ay, unsigned a_boxes, unsigned long long w_policy) {
+// The weights of one k-block of the single-CTA kernel, by one thread: expect_tx (of the rows' bytes too), the stand-in arrivals (tiles whose
+// rows one thread loads), the go-ahead for those that bring the rows, and the box of 256 weight rows with its L2 policy.  Returns whether
+// the next stage is already free.
+__device__ __forceinline__ bool single_issue_kblock(unsigned bar, unsigned tx, unsigned standin_n, unsigned go_bar, unsigned sW,
+                                                    const CUtensorMap* tmw, int x, int c1, int c2, int c3, int c4, unsigned long long w_policy,
+                                                    unsigned next_empty_bar, unsigned next_parity) {
+  unsigned ready;
   asm volatile(
-      "{\n\t.reg .pred e, pa, pa2;\n\t.reg .b32 r, z, sA1, ay1;\n\t"
-      "elect.sync r|e, 0xffffffff;\n\t"
-      "mov.b32 z, 0;\n\t"
-      "setp.ge.and.u32 pa, %12, 1, e;\n\t"
-      "setp.ge.and.u32 pa2, %12, 2, e;\n\t"
-      "add.u32 sA1, %9, 4096;\n\t"
-      "add.s32 ay1, %11, 32;\n\t"
-      "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
-      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%2], [%4, {%5, z, z, %6, %8}], [%0], %13;\n\t"
-      "@e cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%3], [%4, {%5, z, z, %7, %8}], [%0], %13;\n\t"
-      "@pa cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%9], [%10, {%5, %11}], [%0];\n\t"
-      "@pa2 cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [sA1], [%10, {%5, ay1}], [%0];\n\t}"
-      ::"r"(bar), "r"(tx), "r"(sB0), "r"(sB1), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(c3_0), "r"(c3_1),
-        "r"(c4), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes), "l"(w_policy)
+      "{\n\t.reg .pred pst, pn;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 pn, [%13], %14;\n\t"
+      "setp.ne.b32 pst, %3, 0;\n\t"
+      "mbarrier.arrive.expect_tx.shared::cta.b64 _, [%1], %2;\n\t"
+      "mbarrier.arrive.shared::cta.b64 _, [%4];\n\t"
+      "@pst mbarrier.arrive.shared::cta.b64 _, [%1], %3;\n\t"
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%5], [%6, {%7, %8, %9, %10, %11}], [%1], %12;\n\t"
+      "selp.u32 %0, 1, 0, pn;\n\t}"
+      : "=r"(ready)
+      : "r"(bar), "r"(tx), "r"(standin_n), "r"(go_bar), "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(c1), "r"(c2),
+        "r"(c3), "r"(c4), "l"(w_policy), "r"(next_empty_bar), "r"(next_parity)
+      : "memory");
+  return ready != 0;
+}
+// The activation rows of a k-block, by one thread: a box, and behind it a second one of 32 rows
+__device__ __forceinline__ void single_issue_rows(unsigned bar, int x, unsigned sA, const CUtensorMap* tma, int ay, unsigned a_boxes) {
+  asm volatile(
+      "{\n\t.reg .pred pa2;\n\t.reg .b32 sA1, ay1;\n\t"
+      "setp.ge.u32 pa2, %5, 2;\n\t"
+      "add.u32 sA1, %2, 4096;\n\t"
+      "add.s32 ay1, %4, 32;\n\t"
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%2], [%3, {%1, %4}], [%0];\n\t"
+      "@pa2 cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [sA1], [%3, {%1, ay1}], [%0];\n\t}"
+      ::"r"(bar), "r"(x), "r"(sA), "l"(reinterpret_cast<unsigned long long>(tma)), "r"(ay), "r"(a_boxes)
       : "memory");
 }
 }  // namespace moe

@@ -3,24 +3,23 @@
 // grids with an odd number of CTAs; bf16 on an even grid runs on CTA pairs (moe_run_pair.cu).
 //
 // One CTA per SM, 16 warps with fixed roles:
-//   warp 0      scheduler + producer.  At every tile boundary it reads the decode budget
+//   warp 0      scheduler.  At every tile boundary it reads the decode budget
 //               word and the two queue heads, claims the next tile (decode first for CTAs
 //               below the budget, prefill first for the others, each falling back to the
-//               other class: Sections 4.2 and 6.4), hands the tile to the other warps
+//               other class: Sections 4.2 and 6.4), waits for the tile's dependencies and hands the tile to the other warps
 //               through a shared-memory ring guarded by mbarriers (the hand-off of
-//               Section 4.3: the first pipeline warp decides, later warps follow), waits for
-//               the tile's dependencies, then feeds the pipeline: weight tiles (and the
-//               packed intermediate rows of a down tile) by tiled TMA.
-//   warp 1      issues tcgen05.mma (128 x 256 x 16, bf16 -> fp32) into the TMEM accumulators;
+//               Section 4.3: the first pipeline warp decides, later warps follow).  The next claim starts when the producer
+//               has started on the published tile, so a CTA holds one claimed tile beyond the one being loaded.
+//   warp 1      one thread issues tcgen05.mma (128 x 256 x 16, bf16 -> fp32) into the TMEM accumulators;
 //               tcgen05.commit releases pipeline stages and publishes the accumulators.  A
 //               tile of up to 256 rows runs as two 128-row MMAs per k-step against the SAME
 //               weight tile in shared memory, which halves the weight bytes moved per flop.
 //   warp 2      committer: when the epilogue threads have stored a tile it fences and bumps the
 //               dependency counters, the op's done word and the tile log.
-//   warp 3      idle (it only joins the final barrier).
+//   warp 3      one thread loads the weights, one stage per k-block, by tiled TMA.
 //   warps 4-7   gather: the activation rows of a gate/up tile are scattered tokens; they are
 //               copied through the permutation with 16-byte cp.async into the swizzled
-//               layout the tensor core reads.
+//               layout the tensor core reads.  Consecutive rows (down tiles, masked layout) one thread of warp 4 loads as boxes.
 //   warps 8-15  epilogue: tcgen05.ld, SwiGLU (gate/up tiles), bf16 stores transposed through
 //               shared memory into row segments.  They also run the combine tiles.
 // A phase switch happens only between tiles, so no accumulator, TMA transaction or buffer is
@@ -32,7 +31,6 @@
 #include "moe_ptx.cuh"
 #include "moe_sched.cuh"
 #include <cuda_fp8.h>
-#include <climits>
 #include <type_traits>
 
 namespace moe {
@@ -59,12 +57,16 @@ struct F8Small {
 };
 template <int kMode>
 struct SharedCtl {
-  unsigned long long full[kMaxStages], fullA[kMaxStages], empty[kMaxStages];
+  unsigned long long full[kMaxStages];             // the weights, and 128 arrivals of the gather threads (or of the producer in their place)
+  unsigned long long empty[kMaxStages];
+  // producer: the stage may be overwritten (by the gather warps; by the thread that loads boxes)
+  unsigned long long goA[kMaxStages], goR[kMaxStages];
   unsigned long long tfull[2], tempty[2];
   unsigned long long pfull[2], pempty[2];          // fp8: per-k-block partial products, two 256-column buffers
   unsigned long long xbar[4];                      // fp8: amax exchange between the two warps of a quadrant (small tiles: [0], all eight)
   std::conditional_t<kMode == kF8Small, F8Small, F8Big> f8;
   unsigned long long ifull[kRing], iempty[kRing], done[kRing];
+  unsigned long long taken[kRing];                 // the producer has started on the tile
   TileInfo info[kRing];
   unsigned tmem_base;
   alignas(16) unsigned char epi_scratch[8][2048];   // per epilogue warp: 32 rows x 64 bytes
@@ -534,6 +536,19 @@ __device__ __forceinline__ void take_registers() {
   else if constexpr (n > 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(n));
 }
 
+// The boxes of consecutive rows that a tile's k-block takes: of 8, 32, 128 or 256 rows, the smallest that holds them (small tiles: up to
+// two of 32)
+struct RowBoxes {
+  int rows, boxes;
+  __device__ __forceinline__ unsigned bytes() const { return (unsigned)(rows * boxes * kRowBytes); }
+};
+template <int kMode>
+__device__ __forceinline__ RowBoxes row_boxes(int rows) {
+  if (rows <= 8) return RowBoxes{8, 1};
+  if (kMode == kF8Small) return RowBoxes{32, rows > 32 ? 2 : 1};
+  return RowBoxes{rows <= 32 ? 32 : rows <= 128 ? 128 : 256, 1};
+}
+
 // ------------------------------------------------------------------ the persistent kernel
 // which accumulator(s) a tile uses: a tile of up to 128 rows alternates between the two, a
 // tile of up to 256 rows takes both (rows 0..127 -> accumulator 0, rows 128..255 -> 1).
@@ -565,8 +580,9 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kNS; ++s) {
-      mbar_init(&sc->full[s], 1);
-      mbar_init(&sc->fullA[s], kGatherThreads);
+      mbar_init(&sc->full[s], 1 + kGatherThreads);
+      mbar_init(&sc->goA[s], 1);
+      mbar_init(&sc->goR[s], 1);
       mbar_init(&sc->empty[s], 1);
     }
     for (int s = 0; s < 2; ++s) {
@@ -578,10 +594,11 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       mbar_init(&sc->pempty[s], 8);
     }
     for (int s = 0; s < 4; ++s) mbar_init(&sc->xbar[s], kSmall ? 8 : 64);
-    // a ring slot is released by the MMA warp, the committer and each gather warp
+    // a ring slot is released by the MMA thread, the committer, the producer and each gather warp
     for (int s = 0; s < kRing; ++s) {
       mbar_init(&sc->ifull[s], 1);
-      mbar_init(&sc->iempty[s], 2 + kGatherThreads / 32);
+      mbar_init(&sc->iempty[s], 3 + kGatherThreads / 32);
+      mbar_init(&sc->taken[s], 1);
       mbar_init(&sc->done[s], 256);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -601,9 +618,9 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   tc_fence_after();
   const unsigned tmem = sc->tmem_base;
   c.run_off = sc->qt.run_off;
-  if (warp == 3 && lane == 0) end_turn(&args, take_turn(&args), (int)gridDim.x);
+  if (warp == 2 && lane == 0) end_turn(&args, take_turn(&args), (int)gridDim.x);
   const bool watched = sc->qt.watched != 0;
-  if (blockIdx.x == 0 && warp == 3) {
+  if (blockIdx.x == 0 && warp == 2) {
     clear_next_run(&args, rh, c.run_off, lane);
     if (lane == 0 && watched) finish_empty_ops(c, -1);
   }
@@ -618,227 +635,189 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
 
   if (warp == 0) {
     control_regs();
-    // ============================================================ scheduler + TMA producer
-    // The next tile is claimed while the current one is still being loaded (after its
-    // kClaimAt-th k-block), so the claim's round trips and the first loads of the next tile
-    // overlap the current tile's tail instead of draining the pipeline.  A CTA therefore
-    // holds at most one claimed tile beyond the one it is executing.
+    // ============================================================ scheduler
+    // The next tile is claimed while the current one is being loaded, so the claim's round trips do not drain the pipeline.
     ended = false;
-    int stage = 0, islot = 0;
-    unsigned ph = 0, iph = 0;
-    TileInfo ti, nx;
-    bool ti_need_ready = false, nx_need_ready = false, have_nx = false;
-    bool ti_published = false, nx_published = false;
+    int islot = 0;
+    unsigned iph = 0;
+    TileInfo ti;
+    bool need_ready = false;
     ti.kind = kEnd;
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
     ti.t_claim = 0;
-    nx = ti;
-    claim_next<false>(c, &sc->qt, rh, lane, ti, ti_need_ready);
     while (true) {
+      claim_next<false>(c, &sc->qt, rh, lane, ti, need_ready);
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);      // the claim loops exit warp-uniformly
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
-      if (!ti_published) {
-        // blocking hand-off: a free ring slot, the op ready, the tile's dependencies met
-        if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->iempty[islot], iph ^ 1u, 2))) break;
-        if (ti.kind != kEnd && ti_need_ready && !wait_op_ready(c, lane, ti)) ti.kind = kEnd;
-        int ok = 1;
-        if (lane == 0) {
-          // a claimed tile only ever waits on tiles that were claimed before it
-          if (ti.kind == kDown) ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
-          if (ti.kind == kCombine) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_down_tiles(&args, op), 4);
-          if (!ok) ti.kind = kEnd;
-          fence_async_proxy();
-          sc->info[islot] = ti;
-          __threadfence_block();
-          mbar_arrive(&sc->ifull[islot]);
-        }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (ti.kind == kEnd || !ok) { ended = ok; break; }
-        if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      // a free ring slot, the op ready, the tile's dependencies met
+      if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->iempty[islot], iph ^ 1u, 2))) break;
+      if (ti.kind != kEnd && need_ready && !wait_op_ready(c, lane, ti)) ti.kind = kEnd;
+      int ok = 1;
+      if (lane == 0) {
+        // a claimed tile only ever waits on tiles that were claimed before it
+        if (ti.kind == kDown) ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1, 3);
+        if (ti.kind == kCombine) ok = wait_counter(c, &run_of(c, op)->gemm_done, op_down_tiles(&args, op), 4);
+        if (!ok) ti.kind = kEnd;
+        fence_async_proxy();
+        sc->info[islot] = ti;
+        __threadfence_block();
+        mbar_arrive(&sc->ifull[islot]);
       }
-      ti_published = false;
-
-      if (ti.kind != kCombine) {
-        // Weight tiles by tiled TMA.  The A operand of a down tile is the packed intermediate:
-        // consecutive rows, one TMA box (8, 32, 128 or 256 rows high, the smallest that holds
-        // the tile's rows); the A operand of a gate/up tile is gathered by the gather warps.
-        const bool g1 = ti.kind != kDown;                  // gate/up weights
-        const bool gathered = ti.kind == kGateUp;          // activation rows come from the gather warps
-        const bool fromx = ti.kind == kGateUpDirect;       // ... or are consecutive rows of x (masked layout)
-        const CUtensorMap* tmw = g1 ? &op->tm_w1 : &op->tm_w2;
-        const int wrow0 = g1 ? ti.expert * 2 * args.I + ti.n * kTileN1 : ti.expert * args.H + ti.n * kTileN2;
-        const int wrow1 = g1 ? wrow0 + args.I : wrow0 + 128;
-        const int box = ti.rows <= 8 ? 8 : (ti.rows <= 32 || kSmall ? 32 : (ti.rows <= 128 ? 128 : 256));
-        const int boxes = kSmall && ti.rows > 32 ? 2 : 1;
-        const CUtensorMap* tma = fromx ? (box == 8 ? &op->tm_x8 : (box == 32 ? &op->tm_x32 : (box == 128 ? &op->tm_x128 : &op->tm_x256)))
-                                       : (box == 8 ? &op->tm_a8 : (box == 32 ? &op->tm_a32 : (box == 128 ? &op->tm_a128 : &op->tm_a256)));
-        const unsigned tx = (unsigned)kBBytes + (gathered ? 0u : (unsigned)(boxes * box * kRowBytes));
-        const int claim_at = min(kClaimAt, ti.kblocks - 1);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (ti.kind == kEnd || !ok) { ended = ok; break; }
+      if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->taken[islot], iph, 26))) break;
+      if (++islot == kRing) { islot = 0; iph ^= 1u; }
+    }
+  } else if (warp == 3) {
+    control_regs();
+    // ============================================================ producer
+    // The weights of the tiles in the ring, and the go-ahead for those that bring the rows.  One thread runs the whole role, see elect_one.
+    if (elect_one()) {
+      ended = false;
+      int islot = 0;
+      unsigned iph = 0;
+      unsigned stage = 0, par = 1;                         // parity of "stage is free"
+      bool ready = false;                                  // the stage was seen free by the look-ahead test
+      const unsigned stages0 = smem_u32(stages), full0 = smem_u32(&sc->full[0]), empty0 = smem_u32(&sc->empty[0]);
+      const unsigned long long policy = kOnce ? l2_evict_first() : l2_evict_normal();
+      while (true) {
+        if (!mbar_wait(c, &sc->ifull[islot], iph, 21)) break;
+        const int kind = sc->info[islot].kind, kblocks = sc->info[islot].kblocks, rows = sc->info[islot].rows;
+        const int n = sc->info[islot].n, expert = sc->info[islot].expert, slot = sc->info[islot].slot;
+        if (kind == kEnd) { ended = true; break; }
+        mbar_arrive(&sc->taken[islot]);
+        mbar_arrive(&sc->iempty[islot]);
+        if (++islot == kRing) { islot = 0; iph ^= 1u; }
+        if (kind == kCombine) continue;
+        const OpDev* op = &args.ops[slot];
+        const bool g1 = kind != kDown;                     // gate/up weights
+        const bool gathered = kind == kGateUp;             // activation rows come from the gather warps
+        const CUtensorMap* tmw = kSmall ? (g1 ? &op->tm_p1 : &op->tm_p2) : (g1 ? &op->tm_w1 : &op->tm_w2);
+        // the box of 256 weight rows of this tile, see OpDev
+        const int c1 = kSmall || !g1 ? 0 : n * kTileN1;
+        const int c2 = kSmall || g1 ? 0 : n * (kTileN2 / 128);
+        const int c3 = !kSmall ? expert : g1 ? expert * 2 * args.I + n * kTileN1 : n * kTileN2 / 16;
+        const int c4 = kSmall && !g1 ? expert : 0;
+        const unsigned tx = (unsigned)kBBytes + (gathered ? 0u : row_boxes<kMode>(rows).bytes());
+        const bool all_gather = gathered || kSmall;        // the gather warps arrive for every k-block (small tiles: with the scales)
+        const unsigned go = all_gather ? smem_u32(&sc->goA[0]) : smem_u32(&sc->goR[0]), standin = all_gather ? 0u : (unsigned)kGatherThreads;
         bool fail = false;
-        for (int kb = 0; kb < ti.kblocks; ++kb) {
-          if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->empty[stage], ph ^ 1u, 5))) { fail = true; break; }
-          if constexpr (kSmall) {
-            const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-            const int c3 = g1 ? ti.expert * 2 * args.I + ti.n * kTileN1 : ti.n * kTileN2 / 16;
-            single_issue_kblock_5d(smem_u32(&sc->full[stage]), tx, sA + kBOff, sA + kBOff + kBHalfBytes, g1 ? &op->tm_p1 : &op->tm_p2,
-                                   kb * kKb, c3, c3 + (g1 ? 64 : 8), g1 ? 0 : ti.expert, sA, tma, ti.row0, gathered ? 0u : (unsigned)boxes,
-                                   l2_evict_first());
-          } else {
-            const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-            single_issue_kblock<kOnce>(smem_u32(&sc->full[stage]), tx, sA + kBOff, sA + kBOff + kBHalfBytes, tmw, kb * kKb, wrow0, wrow1, sA,
-                                       tma, ti.row0, gathered ? 0u : 1u);
-          }
-          if (++stage == kNS) { stage = 0; ph ^= 1u; }
-          if (kb == claim_at)              // claim ahead (never blocks here)
-            have_nx = claim_once<false>(c, &sc->qt, rh, lane, nx, nx_need_ready) == 1;
-          if (have_nx && !nx_published && kb > claim_at && kb >= ti.kblocks - kPublishLead) {
-            // Hand the next tile to the other warps before this one's last loads go out, if that
-            // takes no waiting: free ring slot, op ready, dependencies already met.
-            const OpDev* nop = &args.ops[nx.slot];
-            bool can = __all_sync(0xffffffffu, mbar_try(&sc->iempty[islot], iph ^ 1u));
-            if (can && nx_need_ready) can = __shfl_sync(0xffffffffu, op_ready(c, nop) ? 1 : 0, 0) != 0;   // lane 0's look
-            if (can) {
-              int met = 1;
-              if (lane == 0) {
-                if (nx.kind == kDown) met = ld_acquire(&g1_done_of(c, nop)[nx.m]) >= args.I / kTileN1;
-                if (nx.kind == kCombine) met = ld_acquire(&run_of(c, nop)->gemm_done) >= op_down_tiles(&args, nop);
-                if (met) {
-                  fence_async_proxy();
-                  sc->info[islot] = nx;
-                  __threadfence_block();
-                  mbar_arrive(&sc->ifull[islot]);
-                }
-              }
-              met = __shfl_sync(0xffffffffu, met, 0);
-              if (met) {
-                nx_published = true;
-                if (++islot == kRing) { islot = 0; iph ^= 1u; }
-              }
-            }
-          }
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!ready && !mbar_wait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
+          const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
+          ready = single_issue_kblock(full0 + stage * 8u, tx, standin, go + stage * 8u, stages0 + stage * (unsigned)kSB + (unsigned)kBOff, tmw,
+                                      kb * kKb, c1, c2, c3, c4, policy, empty0 + nstage * 8u, npar);
+          stage = nstage;
+          par = npar;
         }
         if (fail) break;
       }
-      if (have_nx) {
-        ti = nx;
-        ti_need_ready = nx_need_ready;
-        ti_published = nx_published;
-        have_nx = nx_published = false;
-      } else {
-        claim_next<false>(c, &sc->qt, rh, lane, ti, ti_need_ready);
-      }
     }
+    __syncwarp();
   } else if (warp == 1) {
     control_regs();
     // ============================================================ MMA issuer
-    ended = false;
-    int stage = 0, islot = 0;
-    unsigned ph = 0, iph = 0, aph[2] = {0, 0}, pph = 0;
-    AccUse accs;
-    while (true) {
-      if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->ifull[islot], iph, 6))) break;
-      const int kind = sc->info[islot].kind;
-      const int kblocks = sc->info[islot].kblocks;
-      const int rows = sc->info[islot].rows;
-      if (kind == kEnd) { ended = true; break; }
-      bool fail = false;
-      if (kFp8 && kind != kCombine) {
-        // FP8 with fp32 block scales: the tensor core cannot apply a scale per 128-deep K block,
-        // so every k-block (= one scale block) is multiplied into a FRESH partial buffer, one
-        // per 128-column half of the weight tile (each half has a single weight scale), and the
-        // epilogue warps scale-and-add it into the fp32 accumulator columns of TMEM.
-        const unsigned idesc8 = rows <= 64 ? kIdescF8M64 : kIdescF8;
-        const unsigned idesc_small = kIdescF8M128 | ((unsigned)small_cols(rows) >> 3) << 17;
-        const int slot = small_slot(rows), last_of_group = 128 / slot - 1;
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->full[stage], ph, 8))) { fail = true; break; }
-          if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->fullA[stage], ph, 12))) { fail = true; break; }
-          if constexpr (kSmall) {
-            const int g = kb & last_of_group, pb = (kb / (last_of_group + 1)) & 1;
-            if (g == 0) {
-              if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->pempty[pb], ((pph >> pb) & 1u) ^ 1u, 18))) { fail = true; break; }
-              pph ^= 1u << pb;
-            }
-            tc_fence_after();
-            fence_async_proxy_smem();
-            const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-            f8_small_kblock(tmem + (unsigned)(pb * 256 + g * 2 * slot), umma_desc(sA + kBOff, kRowBytes),
-                            umma_desc(sA + kBOff + kBHalfBytes, kRowBytes), umma_desc(sA, kRowBytes), idesc_small, (unsigned)slot,
-                            smem_u32(&sc->pfull[pb]), g == last_of_group || kb + 1 == kblocks ? 1u : 0u, smem_u32(&sc->empty[stage]));
-          } else {
-            const int pb = kb & 1;                        // partial buffer of this k-block
-            if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->pempty[pb], ((pph >> pb) & 1u) ^ 1u, 18))) { fail = true; break; }
-            pph ^= 1u << pb;
-            tc_fence_after();
-            {
+    // One thread runs the whole role (see elect_one), and the barriers of the next k-block are tested while the MMAs of one are issued.  (The
+    // whole warp in the loop, an election around each group and a wait for each of three barriers: 1090 clocks a k-block of up to 64
+    // rows, 1240 above, now 1045 and 1190, of which the MMAs need 512; what is left is the partial buffers' way to the epilogue and back.)
+    // With the scheduler, the loads of weights and those of rows on threads of their own: 48 tokens 1164 -> 1134 us a pass, 4096 + 512
+    // paired 3412 -> 3389.
+    if (elect_one()) {
+      ended = false;
+      unsigned stage = 0, par = 0, iph = 0, aph[2] = {0, 0}, pph = 0;
+      int islot = 0;
+      bool ready = false;                                  // the stage was seen full by the look-ahead test
+      AccUse accs;
+      const unsigned full0 = smem_u32(&sc->full[0]), empty0 = smem_u32(&sc->empty[0]), pfull0 = smem_u32(&sc->pfull[0]),
+                     pempty0 = smem_u32(&sc->pempty[0]);
+      const unsigned long long desc0 = umma_desc(smem_u32(stages), kRowBytes);
+      while (true) {
+        if (!mbar_wait(c, &sc->ifull[islot], iph, 6)) break;
+        const int kind = sc->info[islot].kind;
+        const int kblocks = sc->info[islot].kblocks;
+        const int rows = sc->info[islot].rows;
+        if (kind == kEnd) { ended = true; break; }
+        bool fail = false;
+        if (kFp8 && kind != kCombine) {
+          // FP8 with fp32 block scales: the tensor core cannot apply a scale per 128-deep K block,
+          // so every k-block (= one scale block) is multiplied into a FRESH partial buffer, one
+          // per 128-column half of the weight tile (each half has a single weight scale), and the
+          // epilogue warps scale-and-add it into their fp32 accumulators.
+          const unsigned idesc8 = rows <= 64 ? kIdescF8M64 : kIdescF8;
+          const unsigned idesc_small = kIdescF8M128 | ((unsigned)small_cols(rows) >> 3) << 17;
+          const int slot = small_slot(rows), last_of_group = 128 / slot - 1;
+          bool drained = false;                            // the next partial buffer was seen free
+          for (int kb = 0; kb < kblocks; ++kb) {
+            if (!ready && !mbar_wait(c, &sc->full[stage], par, 8)) { fail = true; break; }
+            const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
+            const unsigned long long xd = desc0 + stage * (unsigned)(kSB / 16), wd = xd + (unsigned)(kBOff / 16);
+            if constexpr (kSmall) {
+              const int g = kb & last_of_group, pb = (kb / (last_of_group + 1)) & 1;
+              if (g == 0) {
+                if (!mbar_wait(c, &sc->pempty[pb], ((pph >> pb) & 1u) ^ 1u, 18)) { fail = true; break; }
+                pph ^= 1u << pb;
+              }
+              tc_fence_after();
               fence_async_proxy_smem();
-              const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-              const unsigned long long ad = umma_desc(sA, kRowBytes);
-              const unsigned long long bd = umma_desc(sA + kBOff, kRowBytes);
+              ready = f8_small_kblock(tmem + (unsigned)(pb * 256 + g * 2 * slot), wd, wd + (unsigned)(kBHalfBytes / 16), xd, idesc_small,
+                                      (unsigned)slot, pfull0 + pb * 8u, g == last_of_group || kb + 1 == kblocks ? 1u : 0u,
+                                      empty0 + stage * 8u, full0 + nstage * 8u, npar);
+            } else {
+              const unsigned pb = kb & 1u;                 // partial buffer of this k-block
+              if (!drained && !mbar_wait(c, &sc->pempty[pb], ((pph >> pb) & 1u) ^ 1u, 18)) { fail = true; break; }
+              pph ^= 1u << pb;
+              tc_fence_after();
+              fence_async_proxy_smem();
               // four MMAs of 32 e4m3 elements (32 bytes) each, partial full, stage empty
-              f8_mma_kblock(tmem + (unsigned)(pb * 256), ad, bd, idesc8, smem_u32(&sc->pfull[pb]),
-                            smem_u32(&sc->empty[stage]));
+              f8_mma_kblock(tmem + pb * 256u, xd, wd, idesc8, pfull0 + pb * 8u, empty0 + stage * 8u, full0 + nstage * 8u, npar,
+                            pempty0 + (pb ^ 1u) * 8u, ((pph >> (pb ^ 1u)) & 1u) ^ 1u, ready, drained);
             }
+            stage = nstage;
+            par = npar;
           }
           if (fail) break;
-          if (++stage == kNS) { stage = 0; ph ^= 1u; }
-        }
-        if (fail) break;
-      } else if (kind != kCombine) {
-        bool use0, use1;
-        accs.take(rows, use0, use1);
-        // A 256-row tile takes both accumulators: it waits for accumulator 1 only when its first
-        // MMA into it is due, so the drain of accumulator 1 overlaps the tile's first MMAs.
-        const bool pair = use0 && use1;
-        if (use0 && !__all_sync(0xffffffffu, mbar_wait(c, &sc->tempty[0], aph[0] ^ 1u, 7))) break;
-        if (use1 && !pair && !__all_sync(0xffffffffu, mbar_wait(c, &sc->tempty[1], aph[1] ^ 1u, 7))) break;
-        tc_fence_after();
-        const unsigned d0 = tmem + (use0 ? 0u : (unsigned)kAccCols);     // accumulator of rows 0..127
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->full[stage], ph, 8))) { fail = true; break; }
-          // The gather warps arrive on fullA for every k-block (with the copied rows of a
-          // gate/up tile, empty-handed otherwise): being part of every stage hand-off keeps them
-          // within one phase of the stage barriers they wait on.
-          if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->fullA[stage], ph, 12))) { fail = true; break; }
+        } else if (kind != kCombine) {
+          bool use0, use1;
+          accs.take(rows, use0, use1);
+          // A 256-row tile takes both accumulators: it waits for accumulator 1 only when its first
+          // MMA into it is due, so the drain of accumulator 1 overlaps the tile's first MMAs.
+          const bool pair = use0 && use1;
+          if (use0 && !mbar_wait(c, &sc->tempty[0], aph[0] ^ 1u, 7)) break;
+          if (use1 && !pair && !mbar_wait(c, &sc->tempty[1], aph[1] ^ 1u, 7)) break;
           tc_fence_after();
-          if (lane == 0) {
-            fence_async_proxy_smem();                    // cp.async-written rows -> tensor core reads
-            const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-            const unsigned long long ad = umma_desc(sA, kRowBytes), bd = umma_desc(sA + kBOff, kRowBytes);
-#pragma unroll
-            for (int k4 = 0; k4 < kBlockK / 16; ++k4)   // +32 bytes along K per step (>>4 = 2)
-              tc_mma_bf16(d0, ad + 2ull * k4, bd + 2ull * k4, kIdesc, (kb | k4) ? 1u : 0u);
-          }
-          if (pair && kb == 0) {                         // accumulator 1 is needed from here on
-            if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->tempty[1], aph[1] ^ 1u, 7))) { fail = true; break; }
+          const unsigned d0 = tmem + (use0 ? 0u : (unsigned)kAccCols);     // accumulator of rows 0..127
+          for (int kb = 0; kb < kblocks; ++kb) {
+            if (!mbar_wait(c, &sc->full[stage], par, 8)) { fail = true; break; }
             tc_fence_after();
-          }
-          if (lane == 0) {
-            const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-            const unsigned long long bd = umma_desc(sA + kBOff, kRowBytes);
-            if (pair) {                                  // rows 128..255 against the same weight tile
-              const unsigned long long ad1 = umma_desc(sA + kAHalfBytes, kRowBytes);
+            fence_async_proxy_smem();                      // cp.async-written rows -> tensor core reads
+            const unsigned long long ad = desc0 + stage * (unsigned)(kSB / 16), bd = ad + (unsigned)(kBOff / 16);
+#pragma unroll
+            for (int k4 = 0; k4 < kBlockK / 16; ++k4)      // +32 bytes along K per step (>>4 = 2)
+              tc_mma_bf16(d0, ad + 2ull * k4, bd + 2ull * k4, kIdesc, (kb | k4) ? 1u : 0u);
+            if (pair) {                                    // rows 128..255 against the same weight tile
+              if (kb == 0) {                               // accumulator 1 is needed from here on
+                if (!mbar_wait(c, &sc->tempty[1], aph[1] ^ 1u, 7)) { fail = true; break; }
+                tc_fence_after();
+              }
+              const unsigned long long ad1 = ad + (unsigned)(kAHalfBytes / 16);
 #pragma unroll
               for (int k4 = 0; k4 < kBlockK / 16; ++k4)
                 tc_mma_bf16(tmem + (unsigned)kAccCols, ad1 + 2ull * k4, bd + 2ull * k4, kIdesc, (kb | k4) ? 1u : 0u);
             }
-            tc_commit(&sc->empty[stage]);               // frees the stage when the MMAs retire
+            tc_commit(&sc->empty[stage]);                  // frees the stage when the MMAs retire
+            if (++stage == kNS) { stage = 0; par ^= 1u; }
           }
-          __syncwarp();
-          if (++stage == kNS) { stage = 0; ph ^= 1u; }
-        }
-        if (fail) break;
-        if (lane == 0) {                                 // accumulator(s) complete
-          if (use0) tc_commit(&sc->tfull[0]);
+          if (fail) break;
+          if (use0) tc_commit(&sc->tfull[0]);              // accumulator(s) complete
           if (use1) tc_commit(&sc->tfull[1]);
+          if (use0) aph[0] ^= 1u;
+          if (use1) aph[1] ^= 1u;
         }
-        __syncwarp();
-        if (use0) aph[0] ^= 1u;
-        if (use1) aph[1] ^= 1u;
+        mbar_arrive(&sc->iempty[islot]);
+        if (++islot == kRing) { islot = 0; iph ^= 1u; }
       }
-      if (lane == 0) mbar_arrive(&sc->iempty[islot]);
-      if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
+    __syncwarp();
   } else if (warp >= 4 && warp < 4 + kGatherThreads / 32) {
     gather_regs();
     // ============================================================ gather warps (cp.async)
@@ -850,39 +829,53 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // rows covered by one cp.async per thread
     constexpr int kPasses = Ring<kMode>::kARows / kRowsPerPass;
     const int chunk = gt % kCpr, rbase = gt / kCpr;       // rows rbase + kRowsPerPass * j
+    // the swizzle XORs the 16-byte chunk index with the row's place in its 8-row group, which is the same in every pass
+    static_assert(kRowsPerPass % 8 == 0 && kRowBytes == 128, "");
+    const unsigned stages0 = smem_u32(stages), full0 = smem_u32(&sc->full[0]);
+    const unsigned dst0 = stages0 + rbase * kRowBytes + ((chunk ^ (rbase & 7)) << 4);
     ended = false;
     int islot = 0;
-    unsigned iph = 0, kiter = 0;                          // kiter: k-blocks of all GEMM tiles so far
+    unsigned iph = 0, stage = 0, gmask = 0, rmask = 0, kiter = 0;      // kiter: k-blocks of all GEMM tiles so far
     while (true) {
       if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->ifull[islot], iph, 13))) break;
       const int kind = sc->info[islot].kind;
       const int kblocks = sc->info[islot].kblocks;
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
       __syncwarp();
+      if (kind == kEnd) { ended = true; break; }
       if (lane == 0) mbar_arrive(&sc->iempty[islot]);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (kind == kEnd) { ended = true; break; }
       if (kind == kCombine) continue;
-      if (kind != kGateUp && !kSmall) {   // nothing to gather: hand every stage on empty-handed
-        bool failed = false;
-        for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
-          const int stage = (int)(kiter % kNS);
-          if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->empty[stage], ((kiter / kNS) & 1u) ^ 1u, 15))) { failed = true; break; }
-          if (lane == 0) mbar_arrive_n(&sc->fullA[stage], 32);   // the whole warp's share in one arrival
+      const OpDev* op = &args.ops[slot];
+      const RowBoxes rb = row_boxes<kMode>(rows);
+      const bool fromx = kind == kGateUpDirect;           // masked layout: rows of x, otherwise of the packed intermediate
+      const CUtensorMap* tma = rb.rows == 8    ? (fromx ? &op->tm_x8 : &op->tm_a8)
+                               : rb.rows == 32 ? (fromx ? &op->tm_x32 : &op->tm_a32)
+                               : rb.rows == 128 ? (fromx ? &op->tm_x128 : &op->tm_a128) : (fromx ? &op->tm_x256 : &op->tm_a256);
+      if (kind != kGateUp && !kSmall) {   // consecutive rows, the smallest box that holds them
+        bool fail = false;
+        if (warp == 4 && elect_one()) {
+          for (int kb = 0, s = (int)stage; kb < kblocks; ++kb) {
+            if (!mbar_wait(c, &sc->goR[s], (rmask >> s) & 1u, 32)) { fail = true; break; }
+            rmask ^= 1u << s;
+            single_issue_rows(full0 + s * 8u, kb * kKb, stages0 + s * (unsigned)kSB, tma, row0, (unsigned)rb.boxes);
+            if (++s == kNS) s = 0;
+          }
         }
-        if (failed) break;
+        if (__any_sync(0xffffffffu, fail)) break;
+        kiter += (unsigned)kblocks;
+        stage = kiter % (unsigned)kNS;
         continue;
       }
-      const OpDev* op = &args.ops[slot];
       // a paired op's gather list also holds rows of its partner, tagged with their slot: those come from
-      // the partner's activations (kept as the complement of the token index)
+      // the partner's activations
       const bool paired = op->paired != 0;
       const OpDev* pop = paired ? &args.ops[op->partner] : op;
       const unsigned char* X = static_cast<const unsigned char*>(op->x) + chunk * 16;
       const unsigned char* Xp = static_cast<const unsigned char*>(pop->x) + chunk * 16;
       const size_t pitch = (size_t)args.H * kEl;
       const int n_gather = kind == kGateUp ? rows : 0;
-      int tok[kPasses];
+      const unsigned char* src[kPasses];                  // this thread's 16 bytes of the row's first k-block
       const int n_rows = op->n_rows, n_rows_p = pop->n_rows;
       const int own_tag = paired ? slot_of(&args, slot) : 0, partner_tag = paired ? slot_of(&args, op->partner) : 0;
       bool bad = false;
@@ -895,7 +888,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         // an index the plan never wrote is reported below and its row is skipped
         const bool in_range = v >= 0 && (tag == own_tag || tag == partner_tag) && flat < (theirs ? n_rows_p : n_rows);
         bad |= r < n_gather && !in_range;
-        tok[j] = (r < n_gather && in_range) ? (theirs ? ~(flat / args.k) : flat / args.k) : INT_MIN;
+        src[j] = r < n_gather && in_range ? (theirs ? Xp : X) + (size_t)(flat / args.k) * pitch : nullptr;
       }
       if (bad) report(c.st, MOE_EBOUNDS, slot_of(&args, slot), row0, rows, 0);
       // a small e4m3 tile: the scale of token gt of every k-block
@@ -904,9 +897,9 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
         if (kind == kGateUp) {
           const int v = op->gather_list[row0 + gt];
           const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
-          const OpDev* src = tag != own_tag && tag == partner_tag ? pop : op;
-          const bool in_range = v >= 0 && (tag == own_tag || src != op) && flat < src->n_rows;   // reported above if not
-          sx = src->x_scale + (size_t)(in_range ? flat / args.k : 0) * (args.H / 128);
+          const OpDev* from = tag != own_tag && tag == partner_tag ? pop : op;
+          const bool in_range = v >= 0 && (tag == own_tag || from != op) && flat < from->n_rows;   // reported above if not
+          sx = from->x_scale + (size_t)(in_range ? flat / args.k : 0) * (args.H / 128);
         } else {
           sx = kind == kDown ? op->a_scale + (size_t)(row0 + gt) * (args.I / 128) : op->x_scale + (size_t)(row0 + gt) * (args.H / 128);
         }
@@ -915,27 +908,22 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       if constexpr (kSmall) scale_at = smem_u32(sc->f8.scale) + (unsigned)scale_index(gt & 63) * 4u;
       bool fail = false;
       for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
-        const int stage = (int)(kiter % kNS);
-        if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->empty[stage], ((kiter / kNS) & 1u) ^ 1u, 14))) { fail = true; break; }
+        if (!__all_sync(0xffffffffu, mbar_wait(c, &sc->goA[stage], (gmask >> stage) & 1u, 14))) { fail = true; break; }
+        gmask ^= 1u << stage;
+        if (kSmall && kind != kGateUp && warp == 4 && elect_one())
+          single_issue_rows(full0 + stage * 8u, kb * kKb, stages0 + stage * (unsigned)kSB, tma, row0, (unsigned)rb.boxes);
         if (kSmall && sx) cp_async_4(scale_at + (kiter & 15u) * 256u, sx + kb);
-        const unsigned sA = smem_u32(stages + (size_t)stage * kSB);
-        const unsigned char* Xk = X + (size_t)kb * kRowBytes;
-        const unsigned char* Xpk = Xp + (size_t)kb * kRowBytes;
+        const unsigned dst = dst0 + stage * (unsigned)kSB;
         const auto copy_row = [&](int j) {
-          const int r = rbase + kRowsPerPass * j;
-          // the swizzle XORs the 16-byte chunk index with the row's position in its 8-row group
-          const int sw = kRowBytes == 128 ? (r & 7) : ((r >> 1) & 3);
-          const int t = tok[j];
-          if (t != INT_MIN)
-            cp_async_16(sA + r * kRowBytes + ((chunk ^ sw) << 4),
-                        (t >= 0 ? Xk : Xpk) + (size_t)(t >= 0 ? t : ~t) * pitch);
+          if (src[j]) cp_async_16(dst + j * (kRowsPerPass * kRowBytes), src[j] + (size_t)kb * kRowBytes);
         };
         copy_row(0);
         if (!kSmall || n_gather > kRowsPerPass) {        // most small tiles need one pass
 #pragma unroll
           for (int j = 1; j < kPasses; ++j) copy_row(j);
         }
-        cp_async_arrive_noinc(&sc->fullA[stage]);
+        cp_async_arrive_noinc(&sc->full[stage]);
+        if (++stage == kNS) stage = 0;
       }
       if (fail) break;
     }
@@ -1063,10 +1051,6 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       mbar_arrive(&sc->done[islot]);              // this thread's part of the tile is stored
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
-  }
-
-  else {
-    control_regs();        // warp 3: idle, but its warpgroup changes its allowance together
   }
 
   // teardown: nothing is claimed any more.  Where a role gave up, asynchronous work may be under way: let it settle.  Then free TMEM

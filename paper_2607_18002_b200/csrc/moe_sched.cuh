@@ -8,8 +8,6 @@ namespace moe {
 
 constexpr int kRing = 4;                               // tile-info ring depth
 constexpr int kEnd = -1;
-constexpr int kClaimAt = 2;                             // claim the next tile after this k-block
-constexpr int kPublishLead = 5;                         // try to hand the next tile on from this many k-blocks before the end
 
 struct TileInfo {
   int kind, slot, tile, m, row0, rows, n, kblocks, expert, cls;
