@@ -37,7 +37,7 @@ enum TileKind : int { kGateUp = 0, kDown = 1, kCombine = 2, kGateUpDirect = 3 };
 
 // Queue entry (16 bytes, one load per claim): x = kind | n-tile << 4 | m-tile << 12,
 // y = first packed row (first token for a combine tile), z = valid rows, w = expert (| kReadOnce: no other work tile of the op, or of the
-// pair, reads its weights; in plans for the CTA-pair kernel only).
+// pair, reads its weights; not in bf16 plans for the single-CTA kernel).
 constexpr int kReadOnce = 1 << 16;
 __host__ __device__ inline int4 make_entry(int kind, int n, int m, int row0, int rows, int expert) {
   return make_int4(kind | (n << 4) | (m << 12), row0, rows, expert);

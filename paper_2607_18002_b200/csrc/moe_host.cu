@@ -17,7 +17,7 @@ cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, c
                              int slot_d, int slot_p, cudaStream_t stream);
 cudaError_t launch_combine(const OpDev* d_op, int T, int k, int H, cudaStream_t stream);
 cudaError_t prepare_run_kernel();
-cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, bool weights_once, cudaStream_t stream);
+cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream);
 cudaError_t prepare_pair_kernel();
 cudaError_t prepare_plan_kernels();
 cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream);
@@ -430,7 +430,7 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
   }
   ctx->work_rows[slot] = work_rows;
   ctx->plan_capture[slot] = cap;
-  const int read_once = ctx->pair_kernel ? kReadOnce : 0;
+  const int read_once = ctx->pair_kernel || c.dtype == MOE_DTYPE_FP8_E4M3 ? kReadOnce : 0;
   const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, read_once, st)
                                 : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, read_once, st);
   if (pe != cudaSuccess) {
@@ -490,7 +490,6 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const unsigned long long cap = capture_of(st);
   const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
-  bool weights_once = true;              // no op reads a weight byte twice
   for (int i = 0; i < n_ops; ++i) {
     const OpDev& h = ctx->ran_paired[slots[i]] ? ctx->host_pair[slots[i]] : ctx->host_ops[slots[i]];
     a.plan[i] = h.plan;
@@ -504,8 +503,6 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     const bool any_plan = ctx->ran_paired[slots[i]] || ctx->plan_capture[slots[i]] != cap;
     const int rows = any_plan ? full : ctx->work_rows[slots[i]];
     a.work_rows = rows > a.work_rows ? rows : a.work_rows;
-    const moe_op_t& op = ctx->ops[slots[i]];
-    if (any_plan || (op.layout == MOE_LAYOUT_MASKED ? op.slab_rows : op.n_tokens) > rows) weights_once = false;
   }
   if (ctx->poison) {
     for (int i = 0; i < n_ops; ++i) {
@@ -516,7 +513,7 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     }
   }
   const cudaError_t le = ctx->pair_kernel ? launch_pair(a, ctx->rh(), ctx->n_ctas, st)
-                                          : launch_run(a, ctx->rh(), ctx->n_ctas, weights_once, st);
+                                          : launch_run(a, ctx->rh(), ctx->n_ctas, st);
   if (le != cudaSuccess) return MOE_ECUDA;
   return MOE_OK;
 }
@@ -630,7 +627,7 @@ int moe_plan_pair(moe_ctx_t* ctx, int slot_prefill, int slot_decode, int carrier
   }
   if (launch_plan_pair(hd, hp, ctx->host_ops[sd], ctx->host_ops[sp], gather_m, reinterpret_cast<int*>(bd + L.pcomb_off),
                        reinterpret_cast<int*>(bp + L.pcomb_off), c.n_experts, L.NT1, L.NT2,
-                       fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, ctx->pair_kernel ? kReadOnce : 0, sd, sp, st) != cudaSuccess)
+                       fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, ctx->pair_kernel || fp8 ? kReadOnce : 0, sd, sp, st) != cudaSuccess)
     return MOE_ECUDA;
   if (ctx->pair_of[sp] >= 0) ctx->pair_of[ctx->pair_of[sp]] = -1;
   if (ctx->pair_of[sd] >= 0) ctx->pair_of[ctx->pair_of[sd]] = -1;

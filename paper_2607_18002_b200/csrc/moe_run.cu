@@ -127,10 +127,10 @@ __device__ __forceinline__ bool epilogue_fp8_small(const Ctx& c, SharedCtl<kF8Sm
   // weight scales: one per k-block and 128 rows of the matrix
   const float *sw0, *sw1;
   if (g1) {
-    sw0 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + ti.n) * HB;
+    sw0 = op->s_gate_up + ((size_t)expert_of(ti) * (2 * IB) + ti.n) * HB;
     sw1 = sw0 + (size_t)IB * HB;
   } else {
-    sw0 = sw1 = op->s_down + ((size_t)ti.expert * HB + 2 * ti.n + half) * IB;
+    sw0 = sw1 = op->s_down + ((size_t)expert_of(ti) * HB + 2 * ti.n + half) * IB;
   }
   unsigned long long acc[kChunks][4][2];
 #pragma unroll
@@ -284,10 +284,10 @@ __device__ __forceinline__ const float* row_scales(const Ctx& c, const OpDev* op
 __device__ __forceinline__ void weight_scales(const RunArgs& a, const OpDev* op, const TileInfo& ti, const float*& sw0, const float*& sw1) {
   const int HB = a.H / 128, IB = a.I / 128;
   if (ti.kind != kDown) {
-    sw0 = op->s_gate_up + ((size_t)ti.expert * (2 * IB) + ti.n) * HB;
+    sw0 = op->s_gate_up + ((size_t)expert_of(ti) * (2 * IB) + ti.n) * HB;
     sw1 = sw0 + (size_t)IB * HB;
   } else {
-    sw0 = op->s_down + ((size_t)ti.expert * HB + 2 * ti.n) * IB;
+    sw0 = op->s_down + ((size_t)expert_of(ti) * HB + 2 * ti.n) * IB;
     sw1 = sw0 + IB;
   }
 }
@@ -561,10 +561,7 @@ struct AccUse {
   }
 };
 
-// kOnce: every expert's rows of an op fit one work tile, the op reads a weight byte once and marks it to leave L2 first (e4m3, 96 tokens
-// on 8 experts: 111.1 -> 102.8 us a pass; 128 on 8: 114.5 -> 107.6, on 32: 257.2 -> 251.4; two ops on the same weights, 120 + 100 tokens
-// on 8 experts: 121 -> 109).  A kernel of its own: the choice at each load cost launches of larger ops 0.9 %.
-template <int kMode, bool kOnce>
+template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_constant__ RunArgs args,
                                                               RunHead* rh) {
   constexpr bool kFp8 = kMode != kBf16, kSmall = kMode == kF8Small;
@@ -679,11 +676,14 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       unsigned stage = 0, par = 1;                         // parity of "stage is free"
       bool ready = false;                                  // the stage was seen free by the look-ahead test
       const unsigned stages0 = smem_u32(stages), full0 = smem_u32(&sc->full[0]), empty0 = smem_u32(&sc->empty[0]);
-      const unsigned long long policy = kOnce ? l2_evict_first() : l2_evict_normal();
       while (true) {
         if (!mbar_wait(c, &sc->ifull[islot], iph, 21)) break;
         const int kind = sc->info[islot].kind, kblocks = sc->info[islot].kblocks, rows = sc->info[islot].rows;
-        const int n = sc->info[islot].n, expert = sc->info[islot].expert, slot = sc->info[islot].slot;
+        const int n = sc->info[islot].n, expert = expert_of(sc->info[islot]), slot = sc->info[islot].slot;
+        // As in the CTA-pair kernel, the weights of an expert with one work tile leave L2 first (2000 tokens: 2075 -> 2038 us a pass, 4096 + 512
+        // paired 3060 -> 3021, 512 on 64 experts 500 -> 485, 1000 + 200 unpaired 1744 -> 1713).  A kernel of its own for launches
+        // without a second tile, with the whole producer warp choosing, was 0.9 % slower for the others.
+        const unsigned long long policy = sc->info[islot].expert & kReadOnce ? l2_evict_first() : l2_evict_normal();
         if (kind == kEnd) { ended = true; break; }
         mbar_arrive(&sc->taken[islot]);
         mbar_arrive(&sc->iempty[islot]);
@@ -1062,27 +1062,24 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
   }
 }
 
-template <int kMode, bool kOnce>
+template <int kMode>
 static cudaError_t prepare_mode() {
-  return cudaFuncSetAttribute(moe_apk_kernel<kMode, kOnce>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes<kMode>);
+  return cudaFuncSetAttribute(moe_apk_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes<kMode>);
 }
 cudaError_t prepare_run_kernel() {
-  cudaError_t e = prepare_mode<kBf16, false>();
-  if (e == cudaSuccess) e = prepare_mode<kF8, false>();
-  if (e == cudaSuccess) e = prepare_mode<kF8, true>();
-  return e == cudaSuccess ? prepare_mode<kF8Small, true>() : e;
+  cudaError_t e = prepare_mode<kBf16>();
+  if (e == cudaSuccess) e = prepare_mode<kF8>();
+  return e == cudaSuccess ? prepare_mode<kF8Small>() : e;
 }
 
-template <int kMode, bool kOnce>
+template <int kMode>
 static cudaError_t launch_mode(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
-  return launch_after(moe_apk_kernel<kMode, kOnce>, n_ctas, kThreads, kSmemBytes<kMode>, stream, args, rh);
+  return launch_after(moe_apk_kernel<kMode>, n_ctas, kThreads, kSmemBytes<kMode>, stream, args, rh);
 }
-// weights_once: of an e4m3 launch, every op is unpaired and has no more tokens (slab rows) than a work tile has rows
-cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, bool weights_once, cudaStream_t stream) {
-  return args.dtype != MOE_DTYPE_FP8_E4M3            ? launch_mode<kBf16, false>(args, rh, n_ctas, stream)
-         : args.work_rows <= kWorkRowsFp8Small ? launch_mode<kF8Small, true>(args, rh, n_ctas, stream)
-         : weights_once                        ? launch_mode<kF8, true>(args, rh, n_ctas, stream)
-                                               : launch_mode<kF8, false>(args, rh, n_ctas, stream);
+cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
+  return args.dtype != MOE_DTYPE_FP8_E4M3            ? launch_mode<kBf16>(args, rh, n_ctas, stream)
+         : args.work_rows <= kWorkRowsFp8Small ? launch_mode<kF8Small>(args, rh, n_ctas, stream)
+                                               : launch_mode<kF8>(args, rh, n_ctas, stream);
 }
 
 }  // namespace moe

@@ -193,7 +193,7 @@ __device__ __forceinline__ WeightPlan weight_plan(const OpDev* op, const TileInf
   const bool w1 = ti.kind != kDown;          // gate/up weights
   p.map = w1 ? &op->tm_p1 : &op->tm_p2;
   p.blk = w1 ? (ti.n * kTileN1 + 64 * rank) / 8 : (ti.n * kTileN2 + 128 * rank) / 16;
-  p.expert = ti.expert & (kReadOnce - 1);
+  p.expert = expert_of(ti);
   // Where one work tile reads an expert's weights, they are marked to leave L2 first and do not push out what is read again (one token: 72.7 ->
   // 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  A plan knows its own op only: of two unpaired ops of a launch
   // that share their weights both mark what the other reads too, at another time, and mostly gain.  Small ops (unmarked -> marked): 100 + 64

@@ -14,6 +14,8 @@ struct TileInfo {
   unsigned long long t_claim;
 };
 
+__device__ __forceinline__ int expert_of(const TileInfo& ti) { return ti.expert & (kReadOnce - 1); }
+
 // what a unit reads before it claims
 struct ClaimWords {
   unsigned abort, budget, head[2];
