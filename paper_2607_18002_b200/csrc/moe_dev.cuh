@@ -39,6 +39,12 @@ enum TileKind : int { kGateUp = 0, kDown = 1, kCombine = 2, kGateUpDirect = 3 };
 // y = first packed row (first token for a combine tile), z = valid rows, w = expert (| kReadOnce: no other work tile of the op, or of the
 // pair, reads its weights; not in bf16 plans for the single-CTA kernel).
 constexpr int kReadOnce = 1 << 16;
+// ... in a tile descriptor only: the tile runs together with the one behind it, see moe_run_pair.cu
+constexpr int kDualFirst = 1 << 17;
+// what a plan's list is made for: kReadOnce or 0, and whether a launch may hand its GEMM entries out in twos
+struct ListForm {
+  int read_once, twos;
+};
 __host__ __device__ inline int4 make_entry(int kind, int n, int m, int row0, int rows, int expert) {
   return make_int4(kind | (n << 4) | (m << 12), row0, rows, expert);
 }
@@ -79,6 +85,7 @@ struct __align__(128) OpDev {
   CUtensorMap tm_a32;   // [Rmax, I]   box {64, 32}
   CUtensorMap tm_w1;    // gate/up weights as [1][E][gate, up][I][H], box of 128 gate rows and the 128 matching up rows x 128 bytes
   CUtensorMap tm_w2;    // down weights as [1][E][H/128][128][I], box of 256 consecutive rows x 128 bytes
+                        // (CTA pairs: views of tm_p1 and tm_p2 with boxes of 256 rows)
   CUtensorMap tm_a128;  // [Rmax, I]   box {64, 128}
   CUtensorMap tm_a256;  // [Rmax, I]   box {64, 256}
   CUtensorMap tm_p1;    // weights as the M operand: gate/up rows x 128 bytes, a box holds 64 gate rows and the matching up rows in

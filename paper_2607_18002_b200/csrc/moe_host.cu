@@ -9,23 +9,25 @@
 #include "moe_dev.cuh"
 
 namespace moe {
-cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, int read_once, cudaStream_t stream);
+cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, ListForm form, cudaStream_t stream);
 cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
-                               int read_once, cudaStream_t stream);
+                               ListForm form, cudaStream_t stream);
 cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, const OpDev& p, int* gather, int* comb_d,
-                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows, int read_once,
+                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows, ListForm form,
                              int slot_d, int slot_p, cudaStream_t stream);
 cudaError_t launch_combine(const OpDev* d_op, int T, int k, int H, cudaStream_t stream);
 cudaError_t prepare_run_kernel();
 cudaError_t launch_run(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream);
 cudaError_t prepare_pair_kernel();
 cudaError_t prepare_plan_kernels();
-cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream);
+cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, bool dual, cudaStream_t stream);
 }  // namespace moe
 
 using namespace moe;
 
 namespace {
+
+constexpr int kDualRounds = 3, kDualBlocks = 8;        // see moe_run
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -220,6 +222,10 @@ __global__ void write_op_kernel(const __grid_constant__ OpDev src, OpDev* dst) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
 }
 
+ListForm list_form(const moe_ctx* ctx) {
+  return ListForm{ctx->pair_kernel || ctx->cfg.dtype == MOE_DTYPE_FP8_E4M3 ? kReadOnce : 0, ctx->pair_kernel ? 1 : 0};
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
@@ -398,6 +404,10 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
       const bool fp8 = c.dtype == MOE_DTYPE_FP8_E4M3;
       if (!rc && ctx->pair_kernel)                 // 8 gate rows, the 8 matching up rows, the next 8 gate rows, ...
         rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, I / 8, E}, {1, I, 8, 2 * I}, {8, 2, 8, 1});
+      if (!rc && ctx->pair_kernel)                 // ... two n-blocks' rows at once
+        rc = make_map_m(ctx, &h.tm_w1, op->w_gate_up, H, {8, 2, I / 8, E}, {1, I, 8, 2 * I}, {8, 2, 16, 1});
+      if (!rc && ctx->pair_kernel)
+        rc = make_map_m(ctx, &h.tm_w2, op->w_down, I, {8, 2, H / 16, E}, {1, 8, 16, H}, {8, 2, 16, 1});
       if (!rc && fp8)                              // ... of 16 rows: 8 even gate, 8 even up, 8 odd gate, 8 odd up rows
         rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, 2 * E * I, 8}, {2, I, 1, 16}, {8, 2, 2, 8});
       if (!rc && (ctx->pair_kernel || fp8))
@@ -430,9 +440,9 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
   }
   ctx->work_rows[slot] = work_rows;
   ctx->plan_capture[slot] = cap;
-  const int read_once = ctx->pair_kernel || c.dtype == MOE_DTYPE_FP8_E4M3 ? kReadOnce : 0;
-  const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, read_once, st)
-                                : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, read_once, st);
+  const ListForm form = list_form(ctx);
+  const cudaError_t pe = masked ? launch_plan_masked(h, slot, c.n_experts, L.NT1, L.NT2, op->slab_rows, work_rows, form, st)
+                                : launch_plan(h, slot, c.n_experts, L.NT1, L.NT2, work_rows, form, st);
   if (pe != cudaSuccess) {
     ctx->planned[slot] = false;
     return MOE_ECUDA;
@@ -490,6 +500,7 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const unsigned long long cap = capture_of(st);
   const int full = c.dtype == MOE_DTYPE_FP8_E4M3 ? kWorkRowsFp8 : kWorkRowsBf16;
+  long long routed = 0;                  // rows of the launch's ops
   for (int i = 0; i < n_ops; ++i) {
     const OpDev& h = ctx->ran_paired[slots[i]] ? ctx->host_pair[slots[i]] : ctx->host_ops[slots[i]];
     a.plan[i] = h.plan;
@@ -503,6 +514,7 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     const bool any_plan = ctx->ran_paired[slots[i]] || ctx->plan_capture[slots[i]] != cap;
     const int rows = any_plan ? full : ctx->work_rows[slots[i]];
     a.work_rows = rows > a.work_rows ? rows : a.work_rows;
+    if (ctx->ops[slots[i]].layout != MOE_LAYOUT_MASKED) routed += (long long)ctx->ops[slots[i]].n_tokens * c.top_k;
   }
   if (ctx->poison) {
     for (int i = 0; i < n_ops; ++i) {
@@ -512,7 +524,14 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
       if (cudaMemsetAsync(sb + ctx->L.D_off, 0xff, d_bytes, st) != cudaSuccess) return MOE_ECUDA;
     }
   }
-  const cudaError_t le = ctx->pair_kernel ? launch_pair(a, ctx->rh(), ctx->n_ctas, st)
+  // Two tiles at a time (see moe_run_pair.cu) pay where there are enough of them for the units to share out and where their k-blocks outlast
+  // the stores that nothing overlaps.  What is known here are the rows: a lower bound of the tiles.  us a pass, one by one / two at a time:
+  // 350 tokens on 256 experts (240 tiles at least) 1091 / 1082, 777 1166 / 1149, 8192 2367 / 2271, 4096 on 32 experts with 16 k-blocks a tile
+  // 266 / 257, 8000 on 32 with 16 and 8 187 / 184; but 256 on 64 active experts (192 tiles at least) 307 / 309, 200 on 8 (144) 76 / 78, 1000 on
+  // 32 with 16 and 8 k-blocks (120) 69 / 73, 5000 on 8 with 4 and 8 k-blocks 61 / 65.
+  const bool dual = routed / kWorkRowsBf16 * (ctx->L.NT1 + ctx->L.NT2) >= kDualRounds * (ctx->n_ctas / 2) &&
+                    a.kb_gate_up >= kDualBlocks && a.kb_down >= kDualBlocks;
+  const cudaError_t le = ctx->pair_kernel ? launch_pair(a, ctx->rh(), ctx->n_ctas, dual, st)
                                           : launch_run(a, ctx->rh(), ctx->n_ctas, st);
   if (le != cudaSuccess) return MOE_ECUDA;
   return MOE_OK;
@@ -555,7 +574,7 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream) {
   a.carrier[0] = -1;
   a.work_rows = ps.work_rows;
   if (ps.n_gemm_tiles > 0) {
-    if (launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, st) != cudaSuccess) return MOE_ECUDA;
+    if (launch_pair(a, ctx->rh(), 2 * ps.n_gemm_tiles, false, st) != cudaSuccess) return MOE_ECUDA;
   } else if (launch_after(empty_log_kernel, 1, 1, 0, st, ctx->g(), ctx->rh(), (unsigned)ctx->L.run_bytes) != cudaSuccess) {
     return MOE_ECUDA;
   }
@@ -627,7 +646,7 @@ int moe_plan_pair(moe_ctx_t* ctx, int slot_prefill, int slot_decode, int carrier
   }
   if (launch_plan_pair(hd, hp, ctx->host_ops[sd], ctx->host_ops[sp], gather_m, reinterpret_cast<int*>(bd + L.pcomb_off),
                        reinterpret_cast<int*>(bp + L.pcomb_off), c.n_experts, L.NT1, L.NT2,
-                       fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, ctx->pair_kernel || fp8 ? kReadOnce : 0, sd, sp, st) != cudaSuccess)
+                       fp8 ? kWorkRowsFp8 : kWorkRowsBf16, carrier_rows, list_form(ctx), sd, sp, st) != cudaSuccess)
     return MOE_ECUDA;
   if (ctx->pair_of[sp] >= 0) ctx->pair_of[ctx->pair_of[sp]] = -1;
   if (ctx->pair_of[sd] >= 0) ctx->pair_of[ctx->pair_of[sd]] = -1;

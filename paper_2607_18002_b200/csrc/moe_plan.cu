@@ -70,10 +70,19 @@ static OpKind kind_of(const OpDev& h) {
                            (h.done != nullptr || h.notify != nullptr || h.after_op >= 0 ? kOpWatched : 0)};
 }
 
+// Entry i of the wx work tiles x nt n-blocks of one expert's GEMM: n-major over the work tiles, so that they share a weight tile in L2; in
+// lists that are handed out in twos, two n-blocks of a work tile lie next to one another.
+__device__ __forceinline__ void place(int i, int wx, int nt, int twos, int& n, int& j) {
+  if (wx == 1) { n = i; j = 0; return; }
+  const int p = twos ? i / (2 * wx) : 0;
+  if (!twos || 2 * p + 1 >= nt) { n = i / wx; j = i - n * wx; }
+  else { n = 2 * p + (i & 1); j = (i - 2 * p * wx) >> 1; }
+}
+
 // ---------------------------------------------------------------- the ordered tile list of one op
 // Writes this block's share of the queue list of an op whose expert e holds rows [off[e], off[e] + cnt[e]) of the
 // packed row space (cnt / off / work in shared memory; work[e]: work tiles of the experts before e), and (block 0) its
-// PlanState.  All blocks of the grid call it.  read_once: kReadOnce or 0, the mark of entries whose weights no other entry reads; other_work: the
+// PlanState.  All blocks of the grid call it.  form.read_once: the mark of entries whose weights no other entry reads; other_work: the
 // work tiles of the other list of a pair, like work.
 // Work tiles (the unit the queues hand out): up to `work_rows` consecutive rows of one
 // expert, i.e. one or two adjacent m-tiles that share each weight tile they read.
@@ -82,7 +91,7 @@ static OpKind kind_of(const OpDev& h) {
 // depends on were claimed long before.  Every entry's place follows from the prefix sum of the work tiles.
 __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan, OpKind op, const int* cnt, const int* off, const int* work,
                                                 int E, int NT1, int NT2, int T, int work_rows, int x_moe, int planned,
-                                                int n_extra_gemm, int read_once, const int* other_work = nullptr, int g1_kind = kGateUp) {
+                                                int n_extra_gemm, ListForm form, const int* other_work = nullptr, int g1_kind = kGateUp) {
   const int n_work = work[E];
   // Inside an expert: n-major over its work tiles, so an expert's entries of one GEMM are one
   // contiguous run of the list.  One warp per expert writes them (a popular expert has hundreds).
@@ -91,7 +100,7 @@ __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan,
     const int mx = work[x], wx = work[x + 1] - mx;
     if (wx == 0) continue;
     const int cx = cnt[x], ox = off[x];
-    const int ex = x | (wx == 1 && (!other_work || other_work[x + 1] == other_work[x]) ? read_once : 0);
+    const int ex = x | (wx == 1 && (!other_work || other_work[x + 1] == other_work[x]) ? form.read_once : 0);
     // Work tiles whose down entries come before expert x's gate/up entries (those of the experts that end kLagWork tiles
     // ahead of it), and whose gate/up entries come before its down entries (up to the first expert that starts kLagWork tiles
     // after its end): the largest work[i] <= mx - kLagWork, and the smallest work[i] >= mx + wx + kLagWork.
@@ -106,11 +115,13 @@ __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan,
     int4* g1 = tile_list + (size_t)mx * NT1 + (size_t)down_before * NT2;
     int4* g2 = tile_list + (size_t)up_before * NT1 + (size_t)mx * NT2;
     for (int i = lane; i < wx * NT1; i += 32) {
-      const int n = wx == 1 ? i : i / wx, j = i - n * wx;
+      int n, j;
+      place(i, wx, NT1, form.twos, n, j);
       g1[i] = make_entry(g1_kind, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), ex);
     }
     for (int i = lane; i < wx * NT2; i += 32) {
-      const int n = wx == 1 ? i : i / wx, j = i - n * wx;
+      int n, j;
+      place(i, wx, NT2, form.twos, n, j);
       g2[i] = make_entry(kDown, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), ex);
     }
   }
@@ -149,7 +160,7 @@ struct PlanArgs {
   Status* status;
   OpKind op;
   int slot, R, E, T, NT1, NT2, work_rows;
-  int read_once;        // kReadOnce or 0: the mark of the entries of experts with one work tile
+  ListForm form;
   int own;              // rows per block: block b owns rows [b * own, (b + 1) * own)
 };
 
@@ -275,7 +286,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_rank_kernel(const __grid_co
     for (int j = 0, m0 = s_mtile[tid], me = s_mtile[tid + 1] - m0; j < me; ++j)
       a.mtiles[m0 + j] = MTile{tid, off + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
   build_tile_list(a.tile_list, a.plan, a.op, s_cnt, s_off, s_work, E, a.NT1, a.NT2, a.T, a.work_rows, s_mtile[E], total == R ? 1 : 0, 0,
-                  a.read_once);
+                  a.form);
 }
 
 // ---------------------------------------------------------------- masked layout
@@ -308,7 +319,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_masked_kernel(const __grid_
       for (int j = 0, m0 = s_mtile[e], me = s_mtile[e + 1] - m0; j < me; ++j)
         a.mtiles[m0 + j] = MTile{e, e * slab_rows + j * kTileM, min(kTileM, cnt - j * kTileM), 0};
   }
-  build_tile_list(a.tile_list, a.plan, a.op, s_cnt, s_off, s_work, E, a.NT1, a.NT2, 0, a.work_rows, s_mtile[E], 1, 0, a.read_once, nullptr,
+  build_tile_list(a.tile_list, a.plan, a.op, s_cnt, s_off, s_work, E, a.NT1, a.NT2, 0, a.work_rows, s_mtile[E], 1, 0, a.form, nullptr,
                   kGateUpDirect);
 }
 
@@ -335,7 +346,8 @@ struct PairSide {
 struct PairArgs {
   PairSide d, p;
   int* gather;                // row of the shared space -> flat routed index, tagged with its slot
-  int E, NT1, NT2, work_rows, carrier_rows, read_once;
+  int E, NT1, NT2, work_rows, carrier_rows;
+  ListForm form;
 };
 
 // One launch: every block scans the experts and writes its share of both lists, then moves its share of the rows
@@ -373,10 +385,10 @@ __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_co
   else if (e < 64) warp_scan(work_p, cnt_p, E, [&](int rows) { return tiles_of(rows, a.work_rows); });
   __syncthreads();
   const int n_dec = build_tile_list(a.d.tile_list, a.d.plan, a.d.op, cnt_d, off_d, work_d, E, a.NT1, a.NT2, a.d.T, rows_d,
-                                    a.d.plain->n_mtiles, ok, 0, a.read_once, work_p);
+                                    a.d.plain->n_mtiles, ok, 0, a.form, work_p);
   // every GEMM entry of the decode list may carry prefill rows: the prefill op is complete when they are too
   build_tile_list(a.p.tile_list, a.p.plan, a.p.op, cnt_p, off_p, work_p, E, a.NT1, a.NT2, a.p.T, a.work_rows, a.p.plain->n_mtiles, ok,
-                  n_dec, a.read_once, work_d);
+                  n_dec, a.form, work_d);
   // the shared row space's permutation
   for (int i = (int)(blockIdx.x * kPlanThreads + threadIdx.x); i < a.d.R + a.p.R; i += (int)gridDim.x * kPlanThreads) {
     const bool dec = i < a.d.R;
@@ -397,23 +409,23 @@ __global__ void __launch_bounds__(kPlanThreads) plan_pair_kernel(const __grid_co
 static int list_blocks(int E) { return (E + kPlanListExperts - 1) / kPlanListExperts; }
 
 cudaError_t launch_plan_masked(const OpDev& h, int slot, int E, int NT1, int NT2, int slab_rows, int work_rows,
-                               int read_once, cudaStream_t stream) {
+                               ListForm form, cudaStream_t stream) {
   PlanArgs a{};
   a.counts = h.counts; a.offsets = h.offsets; a.mtiles = h.mtiles; a.tile_list = h.tile_list; a.plan = h.plan;
   a.status = h.status;
   a.op = kind_of(h);
-  a.slot = slot; a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows; a.read_once = read_once;
+  a.slot = slot; a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows; a.form = form;
   return launch_after(plan_masked_kernel, list_blocks(E), kPlanThreads, 0, stream, a, slab_rows);
 }
 
 cudaError_t launch_plan_pair(const OpDev& hd, const OpDev& hp, const OpDev& d, const OpDev& p, int* gather, int* comb_d,
-                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows, int read_once,
+                             int* comb_p, int E, int NT1, int NT2, int work_rows, int carrier_rows, ListForm form,
                              int slot_d, int slot_p, cudaStream_t stream) {
   PairArgs a{};
   a.d = PairSide{d.topk_ids, d.counts, d.offsets, d.flat_to_sorted, d.plan, hd.tile_list, hd.plan, comb_d, d.n_rows, d.n_tokens, slot_d, kind_of(d)};
   a.p = PairSide{p.topk_ids, p.counts, p.offsets, p.flat_to_sorted, p.plan, hp.tile_list, hp.plan, comb_p, p.n_rows, p.n_tokens, slot_p, kind_of(p)};
   a.gather = gather;
-  a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows; a.carrier_rows = carrier_rows; a.read_once = read_once;
+  a.E = E; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows; a.carrier_rows = carrier_rows; a.form = form;
   const int blocks = max(list_blocks(E), min(kPlanMaxBlocks, (d.n_rows + p.n_rows + kPlanThreads - 1) / kPlanThreads));
   return launch_after(plan_pair_kernel, blocks, kPlanThreads, 0, stream, a);
 }
@@ -425,13 +437,13 @@ cudaError_t prepare_plan_kernels() {
 }
 
 // h: the op's descriptor as the host holds it
-cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, int read_once, cudaStream_t stream) {
+cudaError_t launch_plan(const OpDev& h, int slot, int E, int NT1, int NT2, int work_rows, ListForm form, cudaStream_t stream) {
   PlanArgs a{};
   a.ids = h.topk_ids; a.counts = h.counts; a.offsets = h.offsets; a.s2f = h.sorted_to_flat; a.f2s = h.flat_to_sorted;
   a.hist = h.plan_hist; a.mtiles = h.mtiles; a.tile_list = h.tile_list; a.plan = h.plan; a.status = h.status;
   a.op = kind_of(h);
   a.slot = slot; a.R = h.n_rows; a.E = E; a.T = h.n_tokens; a.NT1 = NT1; a.NT2 = NT2; a.work_rows = work_rows;
-  a.read_once = read_once;
+  a.form = form;
   const size_t smem = (size_t)kPlanWarps * E * sizeof(int);
   if (a.R <= kPlanDirectRows) {
     const int blocks = list_blocks(E);

@@ -320,6 +320,23 @@ __device__ __forceinline__ void pair_issue_rows(unsigned bar, int x, unsigned sX
       : "memory");
 }
 
+// The four MMAs of one tile's k-block, where another tile's follow against the same rows
+__device__ __forceinline__ void pair_mma_half(unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc, unsigned idesc,
+                                              unsigned accumulate_first) {
+  asm volatile(
+      "{\n\t.reg .pred p0, p1;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "setp.ne.b32 p0, %4, 0;\n\t"
+      "setp.eq.b32 p1, 0, 0;\n\t"
+      "add.u64 a1, %1, 2;\n\tadd.u64 a2, %1, 4;\n\tadd.u64 a3, %1, 6;\n\t"
+      "add.u64 b1, %2, 2;\n\tadd.u64 b2, %2, 4;\n\tadd.u64 b3, %2, 6;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a1, b1, %3, p1;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a2, b2, %3, p1;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a3, b3, %3, p1;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate_first)
+      : "memory");
+}
+
 // One k-block of the pair's MMAs, by one thread: the next stage's barrier is tested first and
 // the result is only read after the four MMAs and the commit have been issued, so that the barrier's
 // shared-memory round trip hides behind the issue of the MMAs.  Returns whether the next stage is already full.

@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   grid_dep_wait();             // everything above overlaps the kernel before this one
-  if (warp == 0) begin_unit(&args, &sc->qt, rh, lane, 1, Ring<kMode>::kARows);
+  if (warp == 0) begin_unit<false>(&args, &sc->qt, rh, lane, 1, Ring<kMode>::kARows);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -638,12 +638,12 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     int islot = 0;
     unsigned iph = 0;
     TileInfo ti;
-    bool need_ready = false;
+    bool need_ready = false, one = false;
     ti.kind = kEnd;
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
     ti.t_claim = 0;
     while (true) {
-      claim_next<false>(c, &sc->qt, rh, lane, ti, need_ready);
+      claim_next<false, false>(c, &sc->qt, rh, lane, ti, need_ready, nullptr, one);
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);      // the claim loops exit warp-uniformly
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
       // a free ring slot, the op ready, the tile's dependencies met

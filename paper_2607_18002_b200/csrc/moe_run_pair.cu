@@ -13,7 +13,14 @@
 //     for 128, eleven for 32 (the launch's ops decide).  Where few units have work the rate of a unit is its bytes in
 //     flight over the load latency (one token, 96 tiles on 74 units: 80 -> 73 us a pass with eleven stages for six), and where all
 //     have, more bytes in flight keep HBM busier (128 tokens on 252 experts: 1085 -> 1040 us with eight);
-//   - a tile uses up to 256 of the 512 TMEM columns, so the epilogue of one tile overlaps the MMAs of the next.
+//   - a tile uses up to 256 of the 512 TMEM columns, so the epilogue of one tile overlaps the MMAs of the next;
+//   - one form of the kernel for tiles of up to 256 rows takes two neighbouring n-blocks of a work tile at a time where the list has them (kDual,
+//     chosen in moe_run): a stage then holds 256 weight rows per CTA and the rows once, four stages of 48 KB, and both accumulators run side
+//     by side.  Large launches run at the 1000 W limit, where time is energy, and a 256-row k-block came to 580 clocks of the SMs' intake from L2
+//     for 513 of the tensor pipe (both measured without the other): two of them now take in 96 KB a pair instead of 128, and hand-overs,
+//     TMA instructions and gather serve twice the weights.  Nothing overlaps the stores of two accumulators but the first MMAs of the next two
+//     tiles.  us a pass, before and after: 8192 tokens 2440 -> 2260, 16 384 + 256 paired 4170 -> 3930, 4096 + 64 on 64 experts 1220 -> 1175,
+//     777 1166 -> 1149.
 // Roles per CTA (16 warps): leader only -- warp 0 scheduler (claims, waits for dependencies,
 // publishes tile descriptors to both CTAs), warp 1 MMA issuer, warp 2 committer; both CTAs --
 // warp 3 producer (TMA loads of its own half of the weights), warps 4-7 gather (a thread of warp 4 loads consecutive rows as boxes),
@@ -30,14 +37,16 @@ namespace pairk {
 
 constexpr int kThreads = 512;
 constexpr int kGatherThreads = 128;
-constexpr int kBBytes = 128 * kRowBytes;                 // this CTA's 128 weight rows of a stage
+constexpr int kBBytes = 128 * kRowBytes;                 // this CTA's 128 weight rows of a tile's k-block
 // the pipeline for work tiles of up to kTileRows rows
-template <int kTileRows>
+// kDual: two tiles at a time
+template <int kTileRows, bool kDual>
 struct Ring {
   static constexpr int kRows = kTileRows / 2;            // activation rows of this CTA
   static constexpr int kABytes = kRows * kRowBytes;
-  static constexpr int kSB = kABytes + kBBytes;
-  static constexpr int kNS = kTileRows == 256 ? 6 : kTileRows == 128 ? 8 : 11;
+  static constexpr int kSB = kABytes + (kDual ? 2 : 1) * kBBytes;
+  static constexpr int kNS = kDual ? 4 : kTileRows == 256 ? 6 : kTileRows == 128 ? 8 : 11;
+  static constexpr int kInfos = kDual ? 8 : 4;           // tile descriptors: those being loaded, claimed ahead and being stored
 };
 constexpr int kAccCols = 256;
 // Warps that store a tile, in both CTAs.  Each counts the tile in the words that down and combine tiles wait for as soon as its own
@@ -51,18 +60,19 @@ constexpr unsigned kIdescM256 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4
 // accumulator columns of a tile (16 is the instruction's step), half of them from each CTA's shared memory
 __device__ __forceinline__ int tile_cols(int rows) { return (rows + 15) & ~15; }
 
-template <int kTileRows>
+template <int kTileRows, bool kDual>
 struct SharedCtl {
+  static constexpr int kRing = Ring<kTileRows, kDual>::kInfos;
   alignas(16) TileInfo info[kRing];
   // leader's: everything the MMAs of a stage read is in place.  kFullCount arrivals: one expect_tx
   // per producer (TMA bytes of both CTAs), one per gather thread of the leader (completion of its
   // cp.async copies) and one from the other CTA's relay warp (that CTA's gathered rows are in
   // place); on tiles without a gather the leader's producer arrives in their place
-  unsigned long long full[Ring<kTileRows>::kNS];
-  unsigned long long fullA[Ring<kTileRows>::kNS];     // second CTA: completion of its own gather threads' copies
-  unsigned long long goA[Ring<kTileRows>::kNS];       // producer -> gather warps: the stage may be overwritten (gathered rows)
-  unsigned long long goR[Ring<kTileRows>::kNS];       // ... (consecutive rows: the thread that loads their boxes)
-  unsigned long long empty[Ring<kTileRows>::kNS];     // both (multicast commit): the stage's MMAs retired
+  unsigned long long full[Ring<kTileRows, kDual>::kNS];
+  unsigned long long fullA[Ring<kTileRows, kDual>::kNS];     // second CTA: completion of its own gather threads' copies
+  unsigned long long goA[Ring<kTileRows, kDual>::kNS];       // producer -> gather warps: the stage may be overwritten (gathered rows)
+  unsigned long long goR[Ring<kTileRows, kDual>::kNS];       // ... (consecutive rows: the thread that loads their boxes)
+  unsigned long long empty[Ring<kTileRows, kDual>::kNS];     // both (multicast commit): the stage's MMAs retired
   unsigned long long tfull[2];       // both (multicast commit): accumulator complete
   unsigned long long tempty[2];      // leader's: accumulator drained by the 16 epilogue warps
   unsigned long long ifull[kRing];   // own: tile descriptor published
@@ -79,8 +89,8 @@ struct SharedCtl {
 };
 static_assert(sizeof(TileInfo) == 48, "descriptor is copied as three 16-byte words");
 
-template <int kTileRows>
-constexpr size_t kSmemBytes = 1024 + (size_t)Ring<kTileRows>::kNS * Ring<kTileRows>::kSB + sizeof(SharedCtl<kTileRows>);
+template <int kTileRows, bool kDual>
+constexpr size_t kSmemBytes = 1024 + (size_t)Ring<kTileRows, kDual>::kNS * Ring<kTileRows, kDual>::kSB + sizeof(SharedCtl<kTileRows, kDual>);
 
 // bounded wait on arrivals of the other CTA.  kTry: mbar_try_cluster, or mbar_try_relaxed where a fence of the caller's follows
 template <bool (*kTry)(void*, unsigned)>
@@ -151,8 +161,8 @@ __device__ __forceinline__ void arrive_at_leader(void* bar, bool leader) {
 // orders all of these reads before the leader's next descriptor with one release to the cluster.  A release by the role itself
 // waits for its stores and copies: a round trip at the start of every tile, ahead of the gather (one token 57.8 us a pass in place
 // of 55.4); arrivals without one, which left that order to the hardware, take as long as this (56.5, now 55.7).
-template <int kTileRows>
-__device__ __forceinline__ void release_slot(SharedCtl<kTileRows>* sc, int islot, bool leader) {
+template <int kTileRows, bool kDual>
+__device__ __forceinline__ void release_slot(SharedCtl<kTileRows, kDual>* sc, int islot, bool leader) {
   mbar_arrive(leader ? &sc->iempty[islot] : &sc->iread[islot]);
 }
 
@@ -182,17 +192,28 @@ __device__ __forceinline__ RowPlan row_plan(const OpDev* op, int kind, int row0,
   return p;
 }
 
-// The place of a tile's 128 weight rows of one CTA, and their L2 policy
+// The first feature that CTA `rank` computes of a tile.  Of two tiles that run together the first CTA takes the first half of the features of
+// both, so that its weight rows are one box.
+__device__ __forceinline__ int first_feature(const TileInfo& ti, int rank, bool dual) {
+  const int w = ti.kind == kDown ? kTileN2 / 2 : kTileN1 / 2;             // of a CTA and tile
+  return (2 * ti.n + (dual ? 2 * rank : rank)) * w;
+}
+// two entries that run together
+__device__ __forceinline__ bool runs_with(const TileInfo& a, const TileInfo& b) {
+  return a.kind == b.kind && a.kind != kCombine && a.row0 == b.row0 && a.rows == b.rows && a.expert == b.expert && a.n + 1 == b.n;
+}
+
+// The place of the weight rows of one CTA, and their L2 policy
 struct WeightPlan {
   const CUtensorMap* map;
   int blk, expert;             // (see OpDev)
   unsigned long long policy;
 };
-__device__ __forceinline__ WeightPlan weight_plan(const OpDev* op, const TileInfo& ti, int rank) {
+__device__ __forceinline__ WeightPlan weight_plan(const OpDev* op, const TileInfo& ti, int rank, bool dual) {
   WeightPlan p;
   const bool w1 = ti.kind != kDown;          // gate/up weights
-  p.map = w1 ? &op->tm_p1 : &op->tm_p2;
-  p.blk = w1 ? (ti.n * kTileN1 + 64 * rank) / 8 : (ti.n * kTileN2 + 128 * rank) / 16;
+  p.map = dual ? (w1 ? &op->tm_w1 : &op->tm_w2) : (w1 ? &op->tm_p1 : &op->tm_p2);
+  p.blk = first_feature(ti, rank, dual) / (w1 ? 8 : 16);
   p.expert = expert_of(ti);
   // Where one work tile reads an expert's weights, they are marked to leave L2 first and do not push out what is read again (one token: 72.7 ->
   // 68.8 us; 128 tokens on 8 experts: 88.1 -> 84.3, on 252: 1067 -> 1060).  A plan knows its own op only: of two unpaired ops of a launch
@@ -234,8 +255,8 @@ struct CombineWhenDone {
 };
 
 // the scheduler hands a tile to the roles of both CTAs
-template <int kTileRows>
-__device__ __forceinline__ void publish(SharedCtl<kTileRows>* sc, int islot, const TileInfo& ti) {
+template <int kTileRows, bool kDual>
+__device__ __forceinline__ void publish(SharedCtl<kTileRows, kDual>* sc, int islot, const TileInfo& ti) {
   sc->info[islot] = ti;
   const unsigned ra = map_to_cta(&sc->info[islot], 1);      // same layout as TileInfo
   st_cluster_v4(ra, make_uint4((unsigned)ti.kind, (unsigned)ti.slot, (unsigned)ti.tile, (unsigned)ti.m));
@@ -247,14 +268,15 @@ __device__ __forceinline__ void publish(SharedCtl<kTileRows>* sc, int islot, con
   mbar_arrive(&sc->ifull[islot]);
 }
 
-template <int kTileRows>
+template <int kTileRows, bool kDual>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
-  constexpr int kNS = Ring<kTileRows>::kNS, kSB = Ring<kTileRows>::kSB, kABytes = Ring<kTileRows>::kABytes;
+  using R = Ring<kTileRows, kDual>;
+  constexpr int kNS = R::kNS, kSB = R::kSB, kABytes = R::kABytes, kRing = R::kInfos;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* stages = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  SharedCtl<kTileRows>* sc = reinterpret_cast<SharedCtl<kTileRows>*>(stages + (size_t)kNS * kSB);
+  SharedCtl<kTileRows, kDual>* sc = reinterpret_cast<SharedCtl<kTileRows, kDual>*>(stages + (size_t)kNS * kSB);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const bool leader = rank == 0;
@@ -318,31 +340,37 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // loads are being issued.
     int islot = 0;
     unsigned iph = 0;
-    bool lapped = false;                                  // every ring slot has been used
-    TileInfo ti;
-    bool need_ready = false;
+    int published = 0;                                    // tiles so far, to kRing: every ring slot has been used
+    TileInfo ti, nx;                                      // nx: the ticket's second tile
+    bool need_ready = false, have_nx = false;
     ti.kind = kEnd;
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
     ti.t_claim = 0;
-    const ClaimWords seen = begin_unit(&args, &sc->qt, rh, lane, kStoreWarps, kTileRows);
+    nx = ti;
+    const ClaimWords seen = begin_unit<kDual>(&args, &sc->qt, rh, lane, kStoreWarps, kTileRows);
     set_run_off();
     if (lane == 0) mbar_arrive(&sc->began);
     const bool plain = args.static_kind >= 0;             // plain launch: this pair runs one given entry
     if (plain) claim_static(&args, (int)(blockIdx.x >> 1), ti);
-    else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready, &seen);
+    else claim_next<true, kDual>(c, &sc->qt, rh, lane, ti, need_ready, &nx, have_nx, &seen);
     unsigned ticket = 0;
     bool asked = false;
     ended = false;
     while (true) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
-      if (lapped && !wwait_cluster(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
+      const bool dual = kDual && have_nx && ti.kind != kEnd && runs_with(ti, nx);
+      const int second = islot + 1 == kRing ? 0 : islot + 1;
+      if (published >= kRing && !wwait_cluster(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
+      if (dual && published + 1 >= kRing && !wwait_cluster(c, &sc->iempty[second], second == 0 ? iph : iph ^ 1u, 2)) break;
+      if (dual) ti.expert |= kDualFirst;
       if (ti.kind != kEnd && need_ready && !wait_op_ready(c, lane, ti)) ti.kind = kEnd;
       // A down tile is handed over at once: the producers fill the free stages with its weights and add the rows when its gate/up
       // tiles are committed (one token: 67.6 -> 67.0 us a pass, 128 tokens on 8 experts: 80.3 -> 79.1).
       int ok = 1;
       if (lane == 0) {
         publish(sc, islot, ti);
+        if (dual && ti.kind != kEnd) publish(sc, second, nx);
         if (ti.kind == kDown) {
           ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1 * kStoreWarps, 3);
           fence_async_proxy();
@@ -350,6 +378,10 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (ok) {
           mbar_arrive_cluster(map_to_cta(&sc->rows_in[islot], 1));
           mbar_arrive(&sc->rows_in[islot]);
+          if (dual) {                                     // (nobody waits there)
+            mbar_arrive_cluster(map_to_cta(&sc->rows_in[second], 1));
+            mbar_arrive(&sc->rows_in[second]);
+          }
         }
         // (asked before the first hand-over, that would wait for the answer: its arrivals release)
         if (!asked) ticket = take_turn(&args);
@@ -367,9 +399,18 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (__shfl_sync(0xffffffffu, ok, 0) == 0) break;
       }
       if (!wwait(c, &sc->taken[islot], iph, 26)) break;
-      if (++islot == kRing) { islot = 0; iph ^= 1u; lapped = true; }
-      if (plain) ti.kind = kEnd;
-      else claim_next<true>(c, &sc->qt, rh, lane, ti, need_ready);
+      published = min(published + (dual ? 2 : 1), kRing);
+      if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      if (dual && ++islot == kRing) { islot = 0; iph ^= 1u; }
+      if (plain) {
+        ti.kind = kEnd;
+      } else if (have_nx && !dual) {
+        ti = nx;
+        have_nx = need_ready = false;
+      } else {
+        have_nx = false;
+        claim_next<true, kDual>(c, &sc->qt, rh, lane, ti, need_ready, &nx, have_nx);
+      }
     }
     if (lane == 0) end_turn(&args, asked ? ticket : take_turn(&args), (int)(gridDim.x >> 1));
   } else if (warp == 3) {
@@ -388,13 +429,21 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (!info_wait_one(c, &sc->ifull[islot], iph, 21, leader)) break;
         const TileInfo ti = sc->info[islot];
         if (ti.kind == kEnd) { ended = true; break; }
+        const bool dual = kDual && (ti.expert & kDualFirst) != 0;
         if (leader) mbar_arrive(&sc->taken[islot]);
         release_slot(sc, islot, leader);
         if (++islot == kRing) { islot = 0; iph ^= 1u; }
+        if (dual) {                                          // the descriptor behind it is for those that store the tiles
+          if (!info_wait_one(c, &sc->ifull[islot], iph, 21, leader)) break;
+          if (leader) mbar_arrive(&sc->taken[islot]);
+          release_slot(sc, islot, leader);
+          if (++islot == kRing) { islot = 0; iph ^= 1u; }
+        }
         if (ti.kind == kCombine) continue;
         const OpDev* op = &args.ops[ti.slot];
-        const WeightPlan wp = weight_plan(op, ti, rank);
+        const WeightPlan wp = weight_plan(op, ti, rank, dual);
         const unsigned row_bytes = row_plan(op, ti.kind, ti.row0, ti.rows, rank).bytes();
+        const unsigned w_bytes = (unsigned)(dual ? 2 * kBBytes : kBBytes);
         const bool g1 = ti.kind == kGateUp;
         const unsigned standin = leader && !g1 ? (unsigned)kGatherThreads + 1u : 0u;   // nobody gathers for this tile
         const unsigned go = g1 ? go_gather : go_rows, has_go = g1 || row_bytes ? 1u : 0u;
@@ -402,7 +451,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         for (int kb = 0; kb < ti.kblocks; ++kb) {
           if (!ready && !mbar_wait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
           const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
-          ready = pair_issue_kblock(full0 + stage * 8u, (unsigned)kBBytes + row_bytes, smem_u32(&sc->full[stage]), standin, go + stage * 8u, has_go,
+          ready = pair_issue_kblock(full0 + stage * 8u, w_bytes + row_bytes, smem_u32(&sc->full[stage]), standin, go + stage * 8u, has_go,
                                     w0 + stage * (unsigned)kSB, wp.map, kb * kBlockK, wp.blk, wp.expert, wp.policy, empty0 + nstage * 8u, npar);
           stage = nstage;
           par = npar;
@@ -429,7 +478,13 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       while (true) {
         if (!info_wait_one(c, &sc->ifull[islot], iph, 6, true)) break;
         const int kind = sc->info[islot].kind, kblocks = sc->info[islot].kblocks, rows = sc->info[islot].rows;
+        const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
         if (kind == kEnd) { ended = true; break; }
+        if (dual) {                                       // the second tile's descriptor
+          mbar_arrive(&sc->iempty[islot]);
+          if (++islot == kRing) { islot = 0; iph ^= 1u; }
+          if (!info_wait_one(c, &sc->ifull[islot], iph, 6, true)) break;
+        }
         if (kind != kCombine) {
           const unsigned b = gcount & 1u;
           if (!wwait_relaxed(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
@@ -438,19 +493,46 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           const unsigned idesc = kIdescM256 | ((unsigned)tile_cols(rows) >> 3) << 17;
           const bool g1 = kind == kGateUp;
           bool fail = false;
+          // Two tiles: while the other accumulator is still being stored, the first tile's MMAs of the k-blocks that are there are issued.  (With
+          // this, and both tiles stored before either is counted: 8192 tokens 2365 -> 2290 us a pass, 12 288 3175 -> 2990.)
+          int ahead = 0;
+          if (dual) {
+            unsigned st = stage, pa = par;
+            unsigned long long* const other = sc->tempty + (b ^ 1u);
+            for (; ahead < min(kNS, kblocks) && !mbar_try_relaxed(other, (((gcount + 1) >> 1) & 1u) ^ 1u); ++ahead) {
+              if (!(ahead == 0 && ready) && !mbar_wait(c, &sc->full[st], pa, 8)) { fail = true; break; }
+              if (g1) fence_async_proxy_smem();
+              const unsigned long long xd = desc0 + st * (unsigned)(kSB / 16);
+              pair_mma_half(d, xd + (unsigned)(kABytes / 16), xd, idesc, ahead ? 1u : 0u);
+              if (++st == kNS) { st = 0; pa ^= 1u; }
+            }
+            if (fail) break;
+            if (!wwait_relaxed(c, &sc->tempty[b ^ 1u], (((gcount + 1) >> 1) & 1u) ^ 1u, 7)) break;
+            tc_fence_after();
+          }
           for (int kb = 0; kb < kblocks; ++kb) {
-            if (!ready && !mbar_wait(c, &sc->full[stage], par, 8)) { fail = true; break; }
-            if (g1) fence_async_proxy_smem();          // this CTA's cp.async-written rows -> tensor core reads
+            if (kb >= ahead) {
+              if (!ready && !mbar_wait(c, &sc->full[stage], par, 8)) { fail = true; break; }
+              if (g1) fence_async_proxy_smem();        // this CTA's cp.async-written rows -> tensor core reads
+            }
             const unsigned long long xd = desc0 + stage * (unsigned)(kSB / 16), wd = xd + (unsigned)(kABytes / 16);
             const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
             // four MMAs (+32 bytes along K per step: the descriptor's address field counts 16 bytes), the
             // commit that frees the stage in both CTAs, and the test of the next stage's barrier (of the next tile's first one too)
-            ready = pair_mma_kblock(d, wd, xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u, full0 + nstage * 8u, npar);
+            if (dual) {
+              if (kb >= ahead) pair_mma_half(d, wd, xd, idesc, kb ? 1u : 0u);
+              if (kb + 1 == kblocks) tc_commit_pair(&sc->tfull[b]);
+              ready = pair_mma_kblock(d ^ (unsigned)kAccCols, wd + (unsigned)(kBBytes / 16), xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u,
+                                      full0 + nstage * 8u, npar);
+            } else {
+              ready = pair_mma_kblock(d, wd, xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u, full0 + nstage * 8u, npar);
+            }
             stage = nstage;
             par = npar;
           }
           if (fail) break;
-          tc_commit_pair(&sc->tfull[b]);                // accumulator complete, both CTAs
+          if (dual) ++gcount;
+          tc_commit_pair(&sc->tfull[gcount & 1u]);      // accumulator complete, both CTAs
           ++gcount;
         }
         mbar_arrive(&sc->iempty[islot]);
@@ -470,9 +552,15 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (!info_wait_one(c, &sc->ifull[islot], iph, 24, false)) break;
         const int kind = sc->info[islot].kind;
         const int kblocks = sc->info[islot].kblocks;
+        const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
         if (kind == kEnd) { ended = true; break; }
         release_slot(sc, islot, false);
         if (++islot == kRing) { islot = 0; iph ^= 1u; }
+        if (dual) {
+          if (!info_wait_one(c, &sc->ifull[islot], iph, 24, false)) break;
+          release_slot(sc, islot, false);
+          if (++islot == kRing) { islot = 0; iph ^= 1u; }
+        }
         if (kind == kCombine) continue;
         if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
         bool fail = false;
@@ -497,7 +585,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     const int gt = threadIdx.x - 128;
     constexpr int kCpr = kRowBytes / 16;                  // 16-byte chunks per row slice
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // 16 rows per cp.async round
-    constexpr int kPasses = Ring<kTileRows>::kRows / kRowsPerPass;
+    constexpr int kPasses = Ring<kTileRows, kDual>::kRows / kRowsPerPass;
     const int chunk = gt % kCpr, rbase = gt / kCpr;
     // the swizzle XORs the chunk index with the row's place in its 8-row group, which is the same in every pass
     static_assert(kRowsPerPass % 8 == 0, "");
@@ -511,18 +599,24 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kind = sc->info[islot].kind;
       const int kblocks = sc->info[islot].kblocks;
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
+      const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
       const int tslot = islot;
       const unsigned tph = iph;
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      if (dual) {
+        if (!wait_info(c, &sc->ifull[islot], iph, 13, leader)) break;
+        if (lane == 0) release_slot(sc, islot, leader);
+        if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      }
       const OpDev* op = &args.ops[slot];
       // Consecutive rows: one thread of one warp loads their boxes, once the scheduler has seen them in place (the weights of a down tile
       // are loaded meanwhile) and the producer has the stage.
       if (kind == kDown || kind == kGateUpDirect) {
         bool fail = false;
         if (warp == 4 && elect_one()) {
-          fail = !info_wait_one(c, &sc->rows_in[tslot], tph, 27, leader);
+          if (kind == kDown) fail = !info_wait_one(c, &sc->rows_in[tslot], tph, 27, leader);
           release_slot(sc, tslot, leader);
           const RowPlan rp = row_plan(op, kind, row0, rows, rank);
           unsigned stage = kiter % (unsigned)kNS;
@@ -648,6 +742,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (ti.kind == kEnd) { ended = true; break; }
       __syncwarp();
       if (!leader && lane == 0) release_slot(sc, islot, false);
+      const bool dual = kDual && (ti.expert & kDualFirst) != 0;
       OpDev* op = &args.ops[ti.slot];
       if (first) {
         first = false;
@@ -671,86 +766,92 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
                         : combine_tokens(op, leader ? ti.row0 : mid, leader ? mid : ti.row0 + ti.rows, 0, vecs, args.k, args.H, etid, 256, ready);
         if (!ok) break;
       } else {
-        const int b = (int)(gcount & 1u);
         // read ahead of the accumulator: behind it these round trips, through a memory system full of weights, delay the tiles that wait
         // for this one (one token: 2.9 us from accumulator to store)
         const bool g1 = ti.kind != kDown;                     // gate/up tile: SwiGLU, output to A
         const StoredWords words = stored_words(c, op, ti);
         unsigned char* const out0 = reinterpret_cast<unsigned char*>(g1 ? (void*)op->A : (void*)op->D);
-        ok = wwait(c, &sc->tfull[b], (gcount >> 1) & 1u, 10);
-        if (!ok) break;
-        ++gcount;
-        tc_fence_after();
         const int cols = tile_cols(ti.rows) / 2;              // this warp's columns
         const int live = min(cols, ti.rows - half * cols);    // ... that hold token rows
         const int passes = (live + 31) / 32;
-        if (passes > 0) {
-          const unsigned taddr = tmem + (unsigned)(b * kAccCols + half * cols) + ((unsigned)(q * 32) << 16);
-          const size_t pitch = (size_t)(g1 ? args.I : args.H) * 2;
-          unsigned char* out = out0 + (size_t)(ti.row0 + half * cols) * pitch +
-                               (size_t)(g1 ? ti.n * kTileN1 + rank * 64 + q * 16 : ti.n * kTileN2 + rank * 128 + q * 32) * 2;
-          unsigned lo[16], hi[16];                            // lanes 0..15 and 16..31 of the quadrant
-          tc_ld_frag(taddr, lo);
-          tc_ld_frag(taddr + (16u << 16), hi);
+        // Of two tiles that run together both are stored before either is counted: the fence there waits for the stores, and the second
+        // accumulator is to be handed back.
 #pragma unroll 1
-          for (int p = 0; p < passes; ++p) {
-            tc_wait_ld();
-            const bool last = p + 1 == passes;
-            if (last) {                                       // all of it is in registers: the accumulator may be overwritten
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) signal_leader(&sc->tempty[b], leader);
-            }
-            unsigned o[16];
-            if (g1) {
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                o[j] = pack_bf16(silu_mul(__uint_as_float(lo[4 * j]), __uint_as_float(lo[4 * j + 2])),
-                                 silu_mul(__uint_as_float(lo[4 * j + 1]), __uint_as_float(lo[4 * j + 3])));
-                o[4 + j] = pack_bf16(silu_mul(__uint_as_float(hi[4 * j]), __uint_as_float(hi[4 * j + 2])),
-                                     silu_mul(__uint_as_float(hi[4 * j + 1]), __uint_as_float(hi[4 * j + 3])));
+        for (int t = 0; t < (dual ? 2 : 1); ++t) {
+          const int b = (int)(gcount & 1u);
+          ok = wwait(c, &sc->tfull[b], (gcount >> 1) & 1u, 10);
+          if (!ok) break;
+          ++gcount;
+          tc_fence_after();
+          if (passes > 0) {
+            const unsigned taddr = tmem + (unsigned)(b * kAccCols + half * cols) + ((unsigned)(q * 32) << 16);
+            const size_t pitch = (size_t)(g1 ? args.I : args.H) * 2;
+            unsigned char* out = out0 + (size_t)(ti.row0 + half * cols) * pitch +
+                                 (size_t)(first_feature(ti, rank, dual) + t * (g1 ? kTileN1 / 2 : kTileN2 / 2) + q * (g1 ? 16 : 32)) * 2;
+            unsigned lo[16], hi[16];                            // lanes 0..15 and 16..31 of the quadrant
+            tc_ld_frag(taddr, lo);
+            tc_ld_frag(taddr + (16u << 16), hi);
+#pragma unroll 1
+            for (int p = 0; p < passes; ++p) {
+              tc_wait_ld();
+              const bool last = p + 1 == passes;
+              if (last) {                                       // all of it is in registers: the accumulator may be overwritten
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) signal_leader(&sc->tempty[b], leader);
               }
-            } else {
+              unsigned o[16];
+              if (g1) {
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < 4; ++j) {
+                  o[j] = pack_bf16(silu_mul(__uint_as_float(lo[4 * j]), __uint_as_float(lo[4 * j + 2])),
+                                   silu_mul(__uint_as_float(lo[4 * j + 1]), __uint_as_float(lo[4 * j + 3])));
+                  o[4 + j] = pack_bf16(silu_mul(__uint_as_float(hi[4 * j]), __uint_as_float(hi[4 * j + 2])),
+                                       silu_mul(__uint_as_float(hi[4 * j + 1]), __uint_as_float(hi[4 * j + 3])));
+                }
+              } else {
 #pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                  o[4 * r + j] = pack_bf16(__uint_as_float(lo[4 * j + 2 * r]), __uint_as_float(lo[4 * j + 2 * r + 1]));
-                  o[8 + 4 * r + j] = pack_bf16(__uint_as_float(hi[4 * j + 2 * r]), __uint_as_float(hi[4 * j + 2 * r + 1]));
+                for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                  for (int r = 0; r < 2; ++r) {
+                    o[4 * r + j] = pack_bf16(__uint_as_float(lo[4 * j + 2 * r]), __uint_as_float(lo[4 * j + 2 * r + 1]));
+                    o[8 + 4 * r + j] = pack_bf16(__uint_as_float(hi[4 * j + 2 * r]), __uint_as_float(hi[4 * j + 2 * r + 1]));
+                  }
                 }
               }
-            }
-            if (!last) {
-              tc_ld_frag(taddr + (unsigned)((p + 1) * 32), lo);
-              tc_ld_frag(taddr + (unsigned)((p + 1) * 32) + (16u << 16), hi);
-            }
-            unsigned char* dst = out + (size_t)(p * 32) * pitch;
-            const int left = live - p * 32;
-            if (g1) {
-              __syncwarp();                                   // scratch free again
-              // matrix i / 8 of a store is token group i / 8, its row i % 8 is token `lane` of the pass
-#pragma unroll
-              for (int f = 0; f < 2; ++f)
-                st_matrix4_trans(scratch_addr + lane * 32 + f * 16, o[4 * f], o[4 * f + 1], o[4 * f + 2], o[4 * f + 3]);
-              __syncwarp();
-#pragma unroll
-              for (int j = 0; j < 2; ++j) {
-                const int r = 16 * j + (lane >> 1), f = lane & 1;
-                const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 32 + f * 16);
-                if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + f * 16) = v4;
+              if (!last) {
+                tc_ld_frag(taddr + (unsigned)((p + 1) * 32), lo);
+                tc_ld_frag(taddr + (unsigned)((p + 1) * 32) + (16u << 16), hi);
               }
-            } else {
-              store_features32(scratch, scratch_addr, o, lane, dst, pitch, left, lane);
+              unsigned char* dst = out + (size_t)(p * 32) * pitch;
+              const int left = live - p * 32;
+              if (g1) {
+                __syncwarp();                                   // scratch free again
+                // matrix i / 8 of a store is token group i / 8, its row i % 8 is token `lane` of the pass
+#pragma unroll
+                for (int f = 0; f < 2; ++f)
+                  st_matrix4_trans(scratch_addr + lane * 32 + f * 16, o[4 * f], o[4 * f + 1], o[4 * f + 2], o[4 * f + 3]);
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                  const int r = 16 * j + (lane >> 1), f = lane & 1;
+                  const uint4 v4 = *reinterpret_cast<const uint4*>(scratch + r * 32 + f * 16);
+                  if (r < left) *reinterpret_cast<uint4*>(dst + (size_t)r * pitch + f * 16) = v4;
+                }
+              } else {
+                store_features32(scratch, scratch_addr, o, lane, dst, pitch, left, lane);
+              }
             }
+          } else {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) signal_leader(&sc->tempty[b], leader);
           }
-        } else {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) signal_leader(&sc->tempty[b], leader);
         }
+        if (!ok) break;
         __syncwarp();
         const bool alone = ti.rows <= cols;                   // the columns of the quadrant's other warp hold no rows: one counts for both
-        if (lane == 0 && (half == 0 || !alone)) count_stored(words, alone ? 2 : 1);
+        if (lane == 0 && (half == 0 || !alone)) count_stored(words, (alone ? 2 : 1) * (dual ? 2 : 1));
       }
       // The warp's stores, before the tile is published.  Those of a GEMM tile are behind the fence of count_stored (a warp that does not
       // count stores nothing); of a combine tile the arrival releases them (across the pair: at cluster scope).  The committer's
@@ -761,6 +862,14 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         else signal_leader(&sc->done[islot], leader);
       }
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      if (dual) {                                             // the second tile's descriptor says nothing new
+        if (!wait_info(c, &sc->ifull[islot], iph, 9, leader)) break;
+        if (lane == 0) {
+          if (!leader) release_slot(sc, islot, false);
+          signal_leader(&sc->done[islot], leader);
+        }
+        if (++islot == kRing) { islot = 0; iph ^= 1u; }
+      }
     }
   }
 
@@ -776,26 +885,29 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
 
 }  // namespace pairk
 
-template <int kTileRows>
+template <int kTileRows, bool kDual>
 static cudaError_t prepare_one() {
-  return cudaFuncSetAttribute(pairk::moe_apk_pair_kernel<kTileRows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)pairk::kSmemBytes<kTileRows>);
+  return cudaFuncSetAttribute(pairk::moe_apk_pair_kernel<kTileRows, kDual>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)pairk::kSmemBytes<kTileRows, kDual>);
 }
 cudaError_t prepare_pair_kernel() {
-  cudaError_t e = prepare_one<kWorkRowsBf16>();
-  if (e == cudaSuccess) e = prepare_one<kWorkRowsMid>();
-  return e == cudaSuccess ? prepare_one<kWorkRowsSmall>() : e;
+  cudaError_t e = prepare_one<kWorkRowsBf16, true>();
+  if (e == cudaSuccess) e = prepare_one<kWorkRowsBf16, false>();
+  if (e == cudaSuccess) e = prepare_one<kWorkRowsMid, false>();
+  return e == cudaSuccess ? prepare_one<kWorkRowsSmall, false>() : e;
 }
 
 // n_ctas: the persistent grid, or 2 x the number of queue entries for a plain launch
-template <int kTileRows>
+template <int kTileRows, bool kDual>
 static cudaError_t launch_one(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
-  return launch_after(pairk::moe_apk_pair_kernel<kTileRows>, n_ctas, pairk::kThreads, pairk::kSmemBytes<kTileRows>, stream, args, rh);
+  return launch_after(pairk::moe_apk_pair_kernel<kTileRows, kDual>, n_ctas, pairk::kThreads, pairk::kSmemBytes<kTileRows, kDual>, stream, args, rh);
 }
-cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, cudaStream_t stream) {
-  return args.work_rows <= kWorkRowsSmall ? launch_one<kWorkRowsSmall>(args, rh, n_ctas, stream)
-         : args.work_rows <= kWorkRowsMid ? launch_one<kWorkRowsMid>(args, rh, n_ctas, stream)
-                                          : launch_one<kWorkRowsBf16>(args, rh, n_ctas, stream);
+// dual: of a launch with work tiles of up to 256 rows
+cudaError_t launch_pair(const RunArgs& args, RunHead* rh, int n_ctas, bool dual, cudaStream_t stream) {
+  return args.work_rows <= kWorkRowsSmall ? launch_one<kWorkRowsSmall, false>(args, rh, n_ctas, stream)
+         : args.work_rows <= kWorkRowsMid ? launch_one<kWorkRowsMid, false>(args, rh, n_ctas, stream)
+         : dual                           ? launch_one<kWorkRowsBf16, true>(args, rh, n_ctas, stream)
+                                          : launch_one<kWorkRowsBf16, false>(args, rh, n_ctas, stream);
 }
 
 }  // namespace moe
