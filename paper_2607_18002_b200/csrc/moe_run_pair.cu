@@ -81,6 +81,9 @@ struct SharedCtl {
   unsigned long long done[kRing];    // leader's: the 16 epilogue warps have stored the tile
   unsigned long long taken[kRing];   // leader's: its producer has started on the tile
   unsigned long long rows_in[kRing]; // own: the rows that the tile reads are in place (down tiles: its gate/up tiles are committed)
+  // two tiles at a time: the rows of a gathered tile are in `list` (nullptr: none)
+  unsigned long long listed[kRing];
+  const unsigned char* list[kRing][kDual ? Ring<kTileRows, kDual>::kRows : 1];
   unsigned long long began;          // leader's: the queue tables and qt.run_off are in place
   unsigned combine_ready;            // own: combine tiles so far whose op's expert outputs were seen in place
   unsigned tmem_base;
@@ -254,6 +257,41 @@ struct CombineWhenDone {
   }
 };
 
+// Two tiles at a time: one warp lists this CTA's rows for the gather warps while the tiles before are still being loaded.  By the gather warps
+// themselves, four round trips behind one another at the start of a tile, the MMAs wait 4500 clocks for the first rows of 256.  Where the power
+// limit has settled most of that comes back as clock: 8192 tokens 2472 -> 2458 us a pass, 12 288 3190 -> 3178, 4096 + 64 on 64 experts 1245 ->
+// 1238; before it has, 2370 -> 2330 and 3030 -> 2940.  (Where tiles are short the scheduler, whose work this is in the leader, is what is
+// waited for: 300 + 20 tokens on 32 experts of 3 MB 62.6 -> 64.1, the toy layer 30.5 -> 31.2.  There the gather warps do it.)
+template <int kTileRows, bool kDual>
+__device__ __forceinline__ void list_rows(const Ctx& c, SharedCtl<kTileRows, kDual>* sc, int islot, int slot, int row0, int rows, int rank,
+                                          int lane) {
+  const RunArgs& a = *c.a;
+  const OpDev* op = &a.ops[slot];
+  const bool paired = op->paired != 0;
+  const OpDev* pop = paired ? &a.ops[op->partner] : op;
+  const unsigned char* X = static_cast<const unsigned char*>(op->x);
+  const unsigned char* Xp = static_cast<const unsigned char*>(pop->x);
+  const int n_rows = op->n_rows, n_rows_p = pop->n_rows;
+  const int own_tag = paired ? slot_of(&a, slot) : 0, partner_tag = paired ? slot_of(&a, op->partner) : 0;
+  const int rpc = tile_cols(rows) / 2, first = rank * rpc;         // this CTA's first row of the tile
+  const int* list = op->gather_list + row0 + first;
+  bool bad = false;
+#pragma unroll
+  for (int i = 0; i < Ring<kTileRows, kDual>::kRows / 32; ++i) {
+    const int r = lane + 32 * i;
+    const bool mine = r < rpc && first + r < rows;
+    const int v = mine ? list[r] : 0;
+    const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
+    const bool theirs = tag != own_tag;
+    const bool in_range = v >= 0 && (tag == own_tag || tag == partner_tag) && flat < (theirs ? n_rows_p : n_rows);   // as by the gather warps
+    bad |= mine && !in_range;
+    if (r < rpc) sc->list[islot][r] = mine && in_range ? (theirs ? Xp : X) + (size_t)(flat / a.k) * ((size_t)a.H * 2) : nullptr;
+  }
+  if (bad) report(c.st, MOE_EBOUNDS, slot_of(c.a, slot), row0, rows, 0);
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&sc->listed[islot]);
+}
+
 // the scheduler hands a tile to the roles of both CTAs
 template <int kTileRows, bool kDual>
 __device__ __forceinline__ void publish(SharedCtl<kTileRows, kDual>* sc, int islot, const TileInfo& ti) {
@@ -295,14 +333,15 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       mbar_init(&sc->tempty[s], 16);
     }
     // a ring slot is released by: MMA warp, committer, producer, 4 gather warps (leader); warp 2 of the other CTA, where it is read by
-    // producer, relay, 4 gather and 8 epilogue warps (the leader's are behind the committer)
+    // producer, relay, 4 gather and 8 epilogue warps (the leader's are behind the committer), and the warp that lists rows
     for (int s = 0; s < kRing; ++s) {
       mbar_init(&sc->ifull[s], 1);
       mbar_init(&sc->iempty[s], 8);
-      mbar_init(&sc->iread[s], 14);
+      mbar_init(&sc->iread[s], kDual ? 15 : 14);
       mbar_init(&sc->done[s], 16);
       mbar_init(&sc->taken[s], 1);
       mbar_init(&sc->rows_in[s], 1);
+      mbar_init(&sc->listed[s], 1);
     }
     mbar_init(&sc->began, 1);
     sc->combine_ready = 0;
@@ -388,9 +427,13 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         asked = true;
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
-      // The gather warps will read the tile's row list (4 bytes per row) first thing: pull it into L2
-      // now, the weight stream has usually pushed it out since the plan wrote it.
-      if (ti.kind == kGateUp && lane * 32 < ti.rows) prefetch_l2(op->gather_list + ti.row0 + lane * 32);
+      if constexpr (kDual) {
+        if (ti.kind == kGateUp && ok) list_rows(c, sc, islot, ti.slot, ti.row0, ti.rows, 0, lane);
+      } else {
+        // The gather warps will read the tile's row list (4 bytes per row) first thing: pull it into L2
+        // now, the weight stream has usually pushed it out since the plan wrote it.
+        if (ti.kind == kGateUp && lane * 32 < ti.rows) prefetch_l2(op->gather_list + ti.row0 + lane * 32);
+      }
       if (ti.kind == kEnd || !ok) { ended = ok; break; }
       // A combine tile is handed over at once: its epilogue warps read row indices and router weights and then wait for the op's
       // GEMM tiles themselves.  The next claim waits with them, so that a unit holds one such tile at most.
@@ -413,6 +456,23 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       }
     }
     if (lane == 0) end_turn(&args, asked ? ticket : take_turn(&args), (int)(gridDim.x >> 1));
+  } else if (kDual && warp == 0) {
+    // ============================================================ lists of rows (second CTA; the leader's are its scheduler's)
+    ended = false;
+    int islot = 0;
+    unsigned iph = 0;
+    bool second = false;                                  // of two tiles that run together
+    while (true) {
+      if (!wait_info(c, &sc->ifull[islot], iph, 34, false)) break;
+      const int kind = sc->info[islot].kind, slot = sc->info[islot].slot, row0 = sc->info[islot].row0, rows = sc->info[islot].rows;
+      const bool dual = (sc->info[islot].expert & kDualFirst) != 0;
+      __syncwarp();
+      if (kind == kEnd) { ended = true; break; }
+      if (kind == kGateUp && !second) list_rows(c, sc, islot, slot, row0, rows, 1, lane);
+      second = dual;
+      if (lane == 0) release_slot(sc, islot, false);
+      if (++islot == kRing) { islot = 0; iph ^= 1u; }
+    }
   } else if (warp == 3) {
     // ============================================================ producer (both CTAs)
     // Reads tiles from the ring and loads this CTA's weights, one stage per k-block; the rows are loaded by the gather warps, because a TMA
@@ -577,7 +637,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     __syncwarp();
   } else if (warp >= 4 && warp < 4 + kGatherThreads / 32) {
     // ============================================================ gather warps (cp.async)
-    // This CTA's rows of a gate/up tile: row r of the tile is token sorted_to_flat[row0 + r] / k.
+    // This CTA's rows of a gate/up tile: row r of the tile is token gather_list[row0 + r] / k.
     // Eight adjacent lanes copy one 128-byte row slice.  Completion is asynchronous: every
     // thread's copies arrive on a barrier when they land (the leader's stage barrier in the
     // leader, a local one that the relay warp forwards in the other CTA), so these warps never
@@ -592,7 +652,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     const unsigned dst0 = smem_u32(stages) + rbase * kRowBytes + ((chunk ^ (rbase & 7)) << 4);
     ended = false;
     int islot = 0;
-    unsigned iph = 0, kiter = 0, gmask = 0, rmask = 0;
+    unsigned iph = 0, kiter = 0, gmask = 0, rmask = 0, lmask = 0;
     const unsigned rows0 = smem_u32(stages), full0 = leader ? smem_u32(&sc->full[0]) : map_to_cta(&sc->full[0], 0);
     while (true) {
       if (!wait_info(c, &sc->ifull[islot], iph, 13, leader)) break;
@@ -635,34 +695,49 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         kiter += (unsigned)kblocks;
         continue;
       }
-      if (lane == 0) release_slot(sc, tslot, leader);
-      if (kind == kCombine) continue;
-      // a paired op's gather list also holds rows of its partner, tagged with their slot: those come from
-      // the partner's activations
-      const bool paired = op->paired != 0;
-      const OpDev* pop = paired ? &args.ops[op->partner] : op;
-      const unsigned char* X = static_cast<const unsigned char*>(op->x) + chunk * 16;
-      const unsigned char* Xp = static_cast<const unsigned char*>(pop->x) + chunk * 16;
-      const size_t pitch = (size_t)args.H * 2;
-      const int rpc = tile_cols(rows) / 2;
-      const int first = rank * rpc;                       // this CTA's first row of the tile
-      const unsigned char* src[kPasses];                  // this thread's 16 bytes of the row's first k-block
-      const int n_rows = op->n_rows, n_rows_p = pop->n_rows;
-      const int own_tag = paired ? slot_of(&args, slot) : 0, partner_tag = paired ? slot_of(&args, op->partner) : 0;
-      bool bad = false;
-#pragma unroll
-      for (int j = 0; j < kPasses; ++j) {
-        const int r = rbase + kRowsPerPass * j;
-        const bool mine = r < rpc && first + r < rows;
-        const int v = mine ? op->gather_list[row0 + first + r] : 0;
-        const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
-        const bool theirs = tag != own_tag;
-        // an index the plan never wrote is reported below and its row is skipped
-        const bool in_range = v >= 0 && (tag == own_tag || tag == partner_tag) && flat < (theirs ? n_rows_p : n_rows);
-        bad |= mine && !in_range;
-        src[j] = mine && in_range ? (theirs ? Xp : X) + (size_t)(flat / args.k) * pitch : nullptr;
+      if (kind == kCombine) {
+        if (lane == 0) release_slot(sc, tslot, leader);
+        continue;
       }
-      if (bad) report(c.st, MOE_EBOUNDS, slot_of(&args, slot), row0, rows, 0);
+      const int rpc = tile_cols(rows) / 2, first = rank * rpc;      // this CTA's first row of the tile
+      const unsigned char* src[kPasses];                  // this thread's 16 bytes of the row's first k-block
+      if constexpr (kDual) {
+        if (!wwait(c, &sc->listed[tslot], (lmask >> tslot) & 1u, 35)) break;
+        lmask ^= 1u << tslot;
+#pragma unroll
+        for (int j = 0; j < kPasses; ++j) {
+          const int r = rbase + kRowsPerPass * j;
+          const unsigned char* row = r < rpc ? sc->list[tslot][r] : nullptr;
+          src[j] = row ? row + chunk * 16 : nullptr;
+        }
+        __syncwarp();
+        if (lane == 0) release_slot(sc, tslot, leader);
+      } else {
+        if (lane == 0) release_slot(sc, tslot, leader);
+        // a paired op's gather list also holds rows of its partner, tagged with their slot: those come from
+        // the partner's activations
+        const bool paired = op->paired != 0;
+        const OpDev* pop = paired ? &args.ops[op->partner] : op;
+        const unsigned char* X = static_cast<const unsigned char*>(op->x) + chunk * 16;
+        const unsigned char* Xp = static_cast<const unsigned char*>(pop->x) + chunk * 16;
+        const size_t pitch = (size_t)args.H * 2;
+        const int n_rows = op->n_rows, n_rows_p = pop->n_rows;
+        const int own_tag = paired ? slot_of(&args, slot) : 0, partner_tag = paired ? slot_of(&args, op->partner) : 0;
+        bool bad = false;
+#pragma unroll
+        for (int j = 0; j < kPasses; ++j) {
+          const int r = rbase + kRowsPerPass * j;
+          const bool mine = r < rpc && first + r < rows;
+          const int v = mine ? op->gather_list[row0 + first + r] : 0;
+          const int tag = v >> kRowSlotShift, flat = v & kRowFlatMask;
+          const bool theirs = tag != own_tag;
+          // an index the plan never wrote is reported below and its row is skipped
+          const bool in_range = v >= 0 && (tag == own_tag || tag == partner_tag) && flat < (theirs ? n_rows_p : n_rows);
+          bad |= mine && !in_range;
+          src[j] = mine && in_range ? (theirs ? Xp : X) + (size_t)(flat / args.k) * pitch : nullptr;
+        }
+        if (bad) report(c.st, MOE_EBOUNDS, slot_of(&args, slot), row0, rows, 0);
+      }
       unsigned long long* landed = leader ? sc->full : sc->fullA;
       bool fail = false;
       for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
