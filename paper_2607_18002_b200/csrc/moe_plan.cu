@@ -70,13 +70,20 @@ static OpKind kind_of(const OpDev& h) {
                            (h.done != nullptr || h.notify != nullptr || h.after_op >= 0 ? kOpWatched : 0)};
 }
 
-// Entry i of the wx work tiles x nt n-blocks of one expert's GEMM: n-major over the work tiles, so that they share a weight tile in L2; in
-// lists that are handed out in twos, two n-blocks of a work tile lie next to one another.
+// Entry i of the wx work tiles x nt n-blocks of one expert's GEMM: n-major over the work tiles, so that they share a weight tile in L2.  In
+// lists that are handed out in twos two n-blocks of a work tile lie next to one another, and the sweeps over n go over kSweep work tiles
+// at a time: the rows of a popular expert's tiles (1.6 MB each) are still in L2 for the next n-block, and its weights for the next tiles
+// (16 384 + 256 tokens paired: 12.8 -> 12.3 GB read from DRAM, 4130 -> 4066 us a pass; 4 or 16 tiles 4073, 4089.  4096 + 512 tokens in e4m3, tiles
+// of 0.8 MB: 13.0 -> 13.1 GB, 3289 -> 3307, so the lists of that kernel are swept whole).
+constexpr int kSweep = 8;
 __device__ __forceinline__ void place(int i, int wx, int nt, int twos, int& n, int& j) {
   if (wx == 1) { n = i; j = 0; return; }
-  const int p = twos ? i / (2 * wx) : 0;
-  if (!twos || 2 * p + 1 >= nt) { n = i / wx; j = i - n * wx; }
-  else { n = 2 * p + (i & 1); j = (i - 2 * p * wx) >> 1; }
+  if (!twos) { n = i / wx; j = i - n * wx; return; }
+  const int j0 = i / (kSweep * nt) * kSweep, w = min(kSweep, wx - j0);
+  i -= j0 * nt;
+  const int p = i / (2 * w);
+  if (2 * p + 1 >= nt) { n = i / w; j = j0 + i - n * w; }
+  else { n = 2 * p + (i & 1); j = j0 + ((i - 2 * p * w) >> 1); }
 }
 
 // ---------------------------------------------------------------- the ordered tile list of one op
