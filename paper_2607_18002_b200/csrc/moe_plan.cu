@@ -70,20 +70,35 @@ static OpKind kind_of(const OpDev& h) {
                            (h.done != nullptr || h.notify != nullptr || h.after_op >= 0 ? kOpWatched : 0)};
 }
 
-// Entry i of the wx work tiles x nt n-blocks of one expert's GEMM: n-major over the work tiles, so that they share a weight tile in L2.  In
+// The entries of the wx work tiles x nt n-blocks of one expert's GEMM, by one warp: put(i, n, j) for entry i, n-block n of work tile j.
+// n-major over the work tiles, so that they share a weight tile in L2.  In
 // lists that are handed out in twos two n-blocks of a work tile lie next to one another, and the sweeps over n go over kSweep work tiles
 // at a time: the rows of a popular expert's tiles (1.6 MB each) are still in L2 for the next n-block, and its weights for the next tiles
 // (16 384 + 256 tokens paired: 12.8 -> 12.3 GB read from DRAM, 4130 -> 4066 us a pass; 4 or 16 tiles 4073, 4089.  4096 + 512 tokens in e4m3, tiles
 // of 0.8 MB: 13.0 -> 13.1 GB, 3289 -> 3307, so the lists of that kernel are swept whole).
 constexpr int kSweep = 8;
-__device__ __forceinline__ void place(int i, int wx, int nt, int twos, int& n, int& j) {
-  if (wx == 1) { n = i; j = 0; return; }
-  if (!twos) { n = i / wx; j = i - n * wx; return; }
-  const int j0 = i / (kSweep * nt) * kSweep, w = min(kSweep, wx - j0);
-  i -= j0 * nt;
-  const int p = i / (2 * w);
-  if (2 * p + 1 >= nt) { n = i / w; j = j0 + i - n * w; }
-  else { n = 2 * p + (i & 1); j = j0 + ((i - 2 * p * w) >> 1); }
+template <class Put>
+__device__ __forceinline__ void sweep(int wx, int nt, int twos, int lane, Put put) {
+  if (!twos) {
+    for (int i = lane; i < wx * nt; i += 32) {
+      const int n = wx == 1 ? i : i / wx;
+      put(i, n, i - n * wx);
+    }
+    return;
+  }
+  for (int j0 = 0; j0 < wx; j0 += kSweep) {
+    const int w = min(kSweep, wx - j0), pairs = nt / 2 * 2 * w;               // entries whose n-blocks lie two and two
+    for (int i = lane; i < w * nt; i += 32) {
+      int n, j;
+      if (w == 1) { n = i; j = 0; }
+      else if (i < pairs) {
+        const int p = w == kSweep ? i / (2 * kSweep) : i / (2 * w);           // (a division takes as long as the rest)
+        n = 2 * p + (i & 1);
+        j = (i - 2 * p * w) >> 1;
+      } else { n = i / w; j = i - n * w; }
+      put(j0 * nt + i, n, j0 + j);
+    }
+  }
 }
 
 // ---------------------------------------------------------------- the ordered tile list of one op
@@ -121,16 +136,11 @@ __device__ __forceinline__ int build_tile_list(int4* tile_list, PlanState* plan,
     up_before = __reduce_min_sync(0xffffffffu, up_before);
     int4* g1 = tile_list + (size_t)mx * NT1 + (size_t)down_before * NT2;
     int4* g2 = tile_list + (size_t)up_before * NT1 + (size_t)mx * NT2;
-    for (int i = lane; i < wx * NT1; i += 32) {
-      int n, j;
-      place(i, wx, NT1, form.twos, n, j);
-      g1[i] = make_entry(g1_kind, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), ex);
-    }
-    for (int i = lane; i < wx * NT2; i += 32) {
-      int n, j;
-      place(i, wx, NT2, form.twos, n, j);
-      g2[i] = make_entry(kDown, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), ex);
-    }
+    const auto entry = [&](int kind, int n, int j) {
+      return make_entry(kind, n, mx + j, ox + j * work_rows, min(work_rows, cx - j * work_rows), ex);
+    };
+    sweep(wx, NT1, form.twos, lane, [&](int i, int n, int j) { g1[i] = entry(g1_kind, n, j); });
+    sweep(wx, NT2, form.twos, lane, [&](int i, int n, int j) { g2[i] = entry(kDown, n, j); });
   }
   const int n_gemm = n_work * (NT1 + NT2);
   const int ct = combine_tile_tokens(T);
