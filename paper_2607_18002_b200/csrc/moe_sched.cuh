@@ -476,8 +476,9 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
 // the plan of op i, the last lanes a word each.  The unit asks for the half with a plain load; the fetch-add that counts it
 // (take_turn) comes later, so that no claim waits behind those of all other units.
 // per_tile: what a committed down tile adds to gemm_done.  max_rows: the tallest work tile this kernel has room for.
-// kTwos: it runs two tiles at a time.  The last entries of a list, two a unit, are handed out one by one all the same: the units end closer to one
-// another (256 tokens on 64 experts: 314 us a pass without, 305).
+// kTwos: it runs two tiles at a time.  The last entries of a list, two a unit but a quarter of it at most, are handed out one by one all the same:
+// the units end closer to one another (256 tokens on 64 experts: 314 us a pass without, 305).  (Two a unit of a short list is most of it, and
+// single tiles are slow in four stages: 128 decode tokens on 8 experts next to 8192 of prefill, budget 16, done after 535 us, now 443.)
 template <bool kTwos>
 __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const RunHead* first_half, int lane, int per_tile, int max_rows) {
   constexpr int kW = 25;
@@ -518,7 +519,7 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
       const int j = sc->n_cls[ci]++;
       sc->cls_slot[ci][j] = a->slots[i];
       sc->cls_free[ci][j] = fi;
-      const int twos = kTwos ? max(0, gi - (int)gridDim.x) / 2 : 0;
+      const int twos = kTwos ? (gi - min((int)gridDim.x, gi / 4)) / 2 : 0;
       if constexpr (kTwos) sc->twos[ci][j] = (unsigned)twos;
       sc->n_gemm[ci][j] = (unsigned)(gi - twos);
       sc->cum[ci][j + 1] = sc->cum[ci][j] + (unsigned)(gi - twos + ei);
