@@ -41,7 +41,8 @@ enum TileKind : int { kGateUp = 0, kDown = 1, kCombine = 2, kGateUpDirect = 3 };
 constexpr int kReadOnce = 1 << 16;
 // ... in a tile descriptor only: the tile runs together with the one behind it, see moe_run_pair.cu
 constexpr int kDualFirst = 1 << 17;
-// what a plan's list is made for: kReadOnce or 0, and whether a launch may hand its GEMM entries out in twos
+// what a plan's list is made for: kReadOnce or 0, and whether a launch may hand its GEMM entries out in twos: two n-blocks of a work tile, which run
+// together
 struct ListForm {
   int read_once, twos;
 };

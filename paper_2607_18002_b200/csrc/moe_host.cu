@@ -222,8 +222,13 @@ __global__ void write_op_kernel(const __grid_constant__ OpDev src, OpDev* dst) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
 }
 
+// Whether launches may run two neighbouring n-blocks at a time.  Only where both GEMMs have an even number of them: every expert's entries then
+// start at an even place of the list and each ticket holds two that run together.  (In twos by place alone, most tickets of a layer
+// with odd numbers held two that do not, which then ran singly in the stages made for two, the second without a look at the budget: us a
+// pass, 4096 tokens on 64 experts: 13 and 13 n-blocks 1193 that way, 1176 tile by tile; 13 and 12 1092 / 1060, 12 and 13 1107 / 1068.)
+bool may_run_twos(const moe_ctx* ctx) { return ctx->pair_kernel && ctx->L.NT1 % 2 == 0 && ctx->L.NT2 % 2 == 0; }
 ListForm list_form(const moe_ctx* ctx) {
-  return ListForm{ctx->pair_kernel || ctx->cfg.dtype == MOE_DTYPE_FP8_E4M3 ? kReadOnce : 0, ctx->pair_kernel ? 1 : 0};
+  return ListForm{ctx->pair_kernel || ctx->cfg.dtype == MOE_DTYPE_FP8_E4M3 ? kReadOnce : 0, may_run_twos(ctx) ? 1 : 0};
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -529,7 +534,7 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   // 350 tokens on 256 experts (240 tiles at least) 1091 / 1082, 777 1166 / 1149, 8192 2367 / 2271, 4096 on 32 experts with 16 k-blocks a tile
   // 266 / 257, 8000 on 32 with 16 and 8 187 / 184; but 256 on 64 active experts (192 tiles at least) 307 / 309, 200 on 8 (144) 76 / 78, 1000 on
   // 32 with 16 and 8 k-blocks (120) 69 / 73, 5000 on 8 with 4 and 8 k-blocks 61 / 65.
-  const bool dual = routed / kWorkRowsBf16 * (ctx->L.NT1 + ctx->L.NT2) >= kDualRounds * (ctx->n_ctas / 2) &&
+  const bool dual = may_run_twos(ctx) && routed / kWorkRowsBf16 * (ctx->L.NT1 + ctx->L.NT2) >= kDualRounds * (ctx->n_ctas / 2) &&
                     a.kb_gate_up >= kDualBlocks && a.kb_down >= kDualBlocks;
   const cudaError_t le = ctx->pair_kernel ? launch_pair(a, ctx->rh(), ctx->n_ctas, dual, st)
                                           : launch_run(a, ctx->rh(), ctx->n_ctas, st);

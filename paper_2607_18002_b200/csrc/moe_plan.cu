@@ -72,7 +72,7 @@ static OpKind kind_of(const OpDev& h) {
 
 // The entries of the wx work tiles x nt n-blocks of one expert's GEMM, by one warp: put(i, n, j) for entry i, n-block n of work tile j.
 // n-major over the work tiles, so that they share a weight tile in L2.  In
-// lists that are handed out in twos two n-blocks of a work tile lie next to one another, and the sweeps over n go over kSweep work tiles
+// lists that are handed out in twos (nt is even) two n-blocks of a work tile lie next to one another, and the sweeps over n go over kSweep work tiles
 // at a time: the rows of a popular expert's tiles (1.6 MB each) are still in L2 for the next n-block, and its weights for the next tiles
 // (16 384 + 256 tokens paired: 12.8 -> 12.3 GB read from DRAM, 4130 -> 4066 us a pass; 4 or 16 tiles 4073, 4089.  4096 + 512 tokens in e4m3, tiles
 // of 0.8 MB: 13.0 -> 13.1 GB, 3289 -> 3307, so the lists of that kernel are swept whole).
@@ -87,15 +87,14 @@ __device__ __forceinline__ void sweep(int wx, int nt, int twos, int lane, Put pu
     return;
   }
   for (int j0 = 0; j0 < wx; j0 += kSweep) {
-    const int w = min(kSweep, wx - j0), pairs = nt / 2 * 2 * w;               // entries whose n-blocks lie two and two
+    const int w = min(kSweep, wx - j0);
     for (int i = lane; i < w * nt; i += 32) {
-      int n, j;
-      if (w == 1) { n = i; j = 0; }
-      else if (i < pairs) {
+      int n = i, j = 0;
+      if (w > 1) {
         const int p = w == kSweep ? i / (2 * kSweep) : i / (2 * w);           // (a division takes as long as the rest)
         n = 2 * p + (i & 1);
         j = (i - 2 * p * w) >> 1;
-      } else { n = i / w; j = i - n * w; }
+      }
       put(j0 * nt + i, n, j0 + j);
     }
   }

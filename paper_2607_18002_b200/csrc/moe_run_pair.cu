@@ -201,10 +201,6 @@ __device__ __forceinline__ int first_feature(const TileInfo& ti, int rank, bool 
   const int w = ti.kind == kDown ? kTileN2 / 2 : kTileN1 / 2;             // of a CTA and tile
   return (2 * ti.n + (dual ? 2 * rank : rank)) * w;
 }
-// two entries that run together
-__device__ __forceinline__ bool runs_with(const TileInfo& a, const TileInfo& b) {
-  return a.kind == b.kind && a.kind != kCombine && a.row0 == b.row0 && a.rows == b.rows && a.expert == b.expert && a.n + 1 == b.n;
-}
 
 // The place of the weight rows of one CTA, and their L2 policy
 struct WeightPlan {
@@ -380,7 +376,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     int islot = 0;
     unsigned iph = 0;
     int published = 0;                                    // tiles so far, to kRing: every ring slot has been used
-    TileInfo ti, nx;                                      // nx: the ticket's second tile
+    TileInfo ti, nx;                                      // nx: the ticket's second tile, which runs together with the first
     bool need_ready = false, have_nx = false;
     ti.kind = kEnd;
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
@@ -398,7 +394,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     while (true) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
-      const bool dual = kDual && have_nx && ti.kind != kEnd && runs_with(ti, nx);
+      const bool dual = kDual && have_nx && ti.kind != kEnd;
       const int second = islot + 1 == kRing ? 0 : islot + 1;
       if (published >= kRing && !wwait_cluster(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
       if (dual && published + 1 >= kRing && !wwait_cluster(c, &sc->iempty[second], second == 0 ? iph : iph ^ 1u, 2)) break;
@@ -445,15 +441,9 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       published = min(published + (dual ? 2 : 1), kRing);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
       if (dual && ++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (plain) {
-        ti.kind = kEnd;
-      } else if (have_nx && !dual) {
-        ti = nx;
-        have_nx = need_ready = false;
-      } else {
-        have_nx = false;
-        claim_next<true, kDual>(c, &sc->qt, rh, lane, ti, need_ready, &nx, have_nx);
-      }
+      have_nx = false;
+      if (plain) ti.kind = kEnd;
+      else claim_next<true, kDual>(c, &sc->qt, rh, lane, ti, need_ready, &nx, have_nx);
     }
     if (lane == 0) end_turn(&args, asked ? ticket : take_turn(&args), (int)(gridDim.x >> 1));
   } else if (kDual && warp == 0) {
