@@ -27,7 +27,7 @@ using namespace moe;
 
 namespace {
 
-constexpr int kDualRounds = 3, kDualBlocks = 8;        // see moe_run
+constexpr int kDualRounds = 10, kDualRoundsFew = 5, kDualFewRows = 64, kDualBlocks = 8;        // see moe_run
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -530,11 +530,17 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
     }
   }
   // Two tiles at a time (see moe_run_pair.cu) pay where there are enough of them for the units to share out and where their k-blocks outlast
-  // the stores that nothing overlaps.  What is known here are the rows: a lower bound of the tiles.  us a pass, one by one / two at a time:
-  // 350 tokens on 256 experts (240 tiles at least) 1091 / 1082, 777 1166 / 1149, 8192 2367 / 2271, 4096 on 32 experts with 16 k-blocks a tile
-  // 266 / 257, 8000 on 32 with 16 and 8 187 / 184; but 256 on 64 active experts (192 tiles at least) 307 / 309, 200 on 8 (144) 76 / 78, 1000 on
-  // 32 with 16 and 8 k-blocks (120) 69 / 73, 5000 on 8 with 4 and 8 k-blocks 61 / 65.
-  const bool dual = may_run_twos(ctx) && routed / kWorkRowsBf16 * (ctx->L.NT1 + ctx->L.NT2) >= kDualRounds * (ctx->n_ctas / 2) &&
+  // the stores that nothing overlaps.  What is known here are the rows: a lower bound of the tiles, counted below in rounds of the units.
+  // With few rounds the longer tickets leave units idle at the end.  us a pass, one by one / two at a time (rounds):
+  //   48 and 24 k-blocks a tile, 8 experts: 500 tokens 130 / 141 (4.9), 800 214 / 219 (8.1), 1200 274 / 277 (12); 16 experts: 400 145 / 149 (3.9),
+  //   700 203 / 213 (6.8); 32: 600 241 / 249 (5.8), 1000 309 / 310 (10); 256: 8192 2367 / 2271 (83);
+  //   32 and 16, 32 experts: 700 137 / 146 (4.5), 1000 168 / 171 (6.7), 1500 214 / 212 (10); 64: 500 173 / 175 (3.2), 1000 220 / 222 (6.7);
+  //   16 and 8, 32 experts: 2400 83 / 88 (4.0), 4000 112 / 117 (6.7), 6000 144 / 142 (10), 12 000 256 / 249 (20).
+  // Where experts get few rows most tiles are short ones that the bound does not count, and two at a time pay earlier:
+  //   48 and 24: 777 tokens on 256 experts 1134 / 1127 (7.8), 600 on 128 632 / 626 (5.8); 16 and 8: 1500 on 128 142 / 141 (5.0); but 32 and 16: 700
+  //   on 128 315 / 320 (4.5).  8 or more k-blocks: 5000 tokens on 8 experts with 4 and 8 of them take 61 / 65.
+  const long long rounds = routed <= (long long)kDualFewRows * c.n_experts ? kDualRoundsFew : kDualRounds;
+  const bool dual = may_run_twos(ctx) && routed / kWorkRowsBf16 * (ctx->L.NT1 + ctx->L.NT2) >= rounds * (ctx->n_ctas / 2) &&
                     a.kb_gate_up >= kDualBlocks && a.kb_down >= kDualBlocks;
   const cudaError_t le = ctx->pair_kernel ? launch_pair(a, ctx->rh(), ctx->n_ctas, dual, st)
                                           : launch_run(a, ctx->rh(), ctx->n_ctas, st);

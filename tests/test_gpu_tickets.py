@@ -40,3 +40,11 @@ def test_two_entries_of_a_ticket_always_run_together(H, I, twos):
     assert len(two) * 2 > len(got) if twos else not two
     for a, b in two:                                    # n-blocks 2 p and 2 p + 1 of a work tile lie at places 2 t and 2 t + 1 of the list
         assert a["kind"] == b["kind"] and a["tile"] % 2 == 0 and b["tile"] == a["tile"] + 1
+
+
+@pytest.mark.parametrize("E,T,twos", [(32, 1000, True), (16, 1000, False), (16, 2000, True)])
+def test_two_at_a_time_where_units_have_many_tiles(E, T, twos):
+    """Ten rounds of the 16 units by the rows, five where experts get 64 rows or fewer: 5.3, 5.3 and 11 rounds here."""
+    spec = synth.Spec("rounds", synth.Shape(E, 2, 1024, 1024), ((synth.PREFILL, T),), "zipf", 1.0, 1.0, -1.0, 89)
+    ctx, _ = run(spec, n_ctas=32)
+    assert any(len(t) > 1 for t in tickets(ctx.tile_log(), 0)) == twos
