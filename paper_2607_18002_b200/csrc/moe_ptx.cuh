@@ -300,6 +300,16 @@ __device__ __forceinline__ bool pair_issue_kblock(unsigned bar, unsigned tx, uns
   return ready != 0;
 }
 
+// ... the weights of a second k-block in the same stage
+__device__ __forceinline__ void pair_issue_weights(unsigned bar, unsigned sW, const CUtensorMap* tmw, int x, int wblk, int expert,
+                                                   unsigned long long w_policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+      "[%1], [%2, {%3, %6, %6, %4, %5}], [%0], %7;"
+      ::"r"(bar), "r"(sW), "l"(reinterpret_cast<unsigned long long>(tmw)), "r"(x), "r"(wblk), "r"(expert), "r"(0), "l"(w_policy)
+      : "memory");
+}
+
 // The activation boxes of one k-block by one CTA of a pair, by one thread: up to three, a_rows rows apart
 __device__ __forceinline__ void pair_issue_rows(unsigned bar, int x, unsigned sX, const CUtensorMap* tma, int ay, unsigned a_boxes,
                                                 unsigned a_rows) {

@@ -48,6 +48,12 @@ struct Ring {
   static constexpr int kNS = kDual ? 4 : kTileRows == 256 ? 6 : kTileRows == 128 ? 8 : 11;
   static constexpr int kInfos = kDual ? 8 : 4;           // tile descriptors: those being loaded, claimed ahead and being stored
 };
+// Two tiles at a time: of a tile that runs alone and has so few rows (a decode tile, the end of a list) a stage takes two k-blocks, the second's
+// weights and rows in the second half of either part.  With one a stage, half of it was unused and four were in flight where six are
+// in the other form: us from claim to commit of decode tiles next to 8192 prefill tokens, 128 tokens on 8 experts 43 that way, 31 now, 36 in the
+// other form; 256 on all of 256 experts next to 16 384 37, 25, 31.
+constexpr int kWideRows = 128;
+constexpr int kWideBytes = kWideRows / 2 * kRowBytes;    // from the rows of the first k-block of a stage to those of the second
 constexpr int kAccCols = 256;
 // Warps that store a tile, in both CTAs.  Each counts the tile in the words that down and combine tiles wait for as soon as its own
 // part is out: one token takes 63.9 us a pass where 65.9 with one thread that counts for all of them after they have met.  (In the
@@ -59,6 +65,11 @@ constexpr int kFullCount = 2 + kGatherThreads + 1;
 constexpr unsigned kIdescM256 = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4) << 24);
 // accumulator columns of a tile (16 is the instruction's step), half of them from each CTA's shared memory
 __device__ __forceinline__ int tile_cols(int rows) { return (rows + 15) & ~15; }
+// k-blocks of a tile that share a stage.  (A launch that runs two tiles at a time has an even number of them in either GEMM: even numbers of n-blocks
+// are multiples of 512 in H and of 256 in I.)
+static_assert(2 * kTileN2 % (2 * kBlockK) == 0 && 2 * kTileN1 % (2 * kBlockK) == 0, "");
+template <bool kDual>
+__device__ __forceinline__ int kblocks_a_stage(int rows, bool dual) { return kDual && !dual && tile_cols(rows) <= kWideRows ? 2 : 1; }
 
 template <int kTileRows, bool kDual>
 struct SharedCtl {
@@ -497,12 +508,17 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         const bool g1 = ti.kind == kGateUp;
         const unsigned standin = leader && !g1 ? (unsigned)kGatherThreads + 1u : 0u;   // nobody gathers for this tile
         const unsigned go = g1 ? go_gather : go_rows, has_go = g1 || row_bytes ? 1u : 0u;
+        const int step = kblocks_a_stage<kDual>(ti.rows, dual);
         bool fail = false;
-        for (int kb = 0; kb < ti.kblocks; ++kb) {
+        for (int kb = 0; kb < ti.kblocks; kb += step) {
           if (!ready && !mbar_wait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
           const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
-          ready = pair_issue_kblock(full0 + stage * 8u, w_bytes + row_bytes, smem_u32(&sc->full[stage]), standin, go + stage * 8u, has_go,
-                                    w0 + stage * (unsigned)kSB, wp.map, kb * kBlockK, wp.blk, wp.expert, wp.policy, empty0 + nstage * 8u, npar);
+          ready = pair_issue_kblock(full0 + stage * 8u, (w_bytes + row_bytes) * (unsigned)step, smem_u32(&sc->full[stage]), standin,
+                                    go + stage * 8u, has_go, w0 + stage * (unsigned)kSB, wp.map, kb * kBlockK, wp.blk, wp.expert, wp.policy,
+                                    empty0 + nstage * 8u, npar);
+          if (step == 2)
+            pair_issue_weights(full0 + stage * 8u, w0 + stage * (unsigned)kSB + (unsigned)kBBytes, wp.map, (kb + 1) * kBlockK, wp.blk, wp.expert,
+                               wp.policy);
           stage = nstage;
           par = npar;
         }
@@ -560,7 +576,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
             if (!wwait_relaxed(c, &sc->tempty[b ^ 1u], (((gcount + 1) >> 1) & 1u) ^ 1u, 7)) break;
             tc_fence_after();
           }
-          for (int kb = 0; kb < kblocks; ++kb) {
+          const int step = kblocks_a_stage<kDual>(rows, dual);
+          for (int kb = 0; kb < kblocks; kb += step) {
             if (kb >= ahead) {
               if (!ready && !mbar_wait(c, &sc->full[stage], par, 8)) { fail = true; break; }
               if (g1) fence_async_proxy_smem();        // this CTA's cp.async-written rows -> tensor core reads
@@ -573,6 +590,10 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
               if (kb >= ahead) pair_mma_half(d, wd, xd, idesc, kb ? 1u : 0u);
               if (kb + 1 == kblocks) tc_commit_pair(&sc->tfull[b]);
               ready = pair_mma_kblock(d ^ (unsigned)kAccCols, wd + (unsigned)(kBBytes / 16), xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u,
+                                      full0 + nstage * 8u, npar);
+            } else if (step == 2) {
+              pair_mma_half(d, wd, xd, idesc, kb ? 1u : 0u);
+              ready = pair_mma_kblock(d, wd + (unsigned)(kBBytes / 16), xd + (unsigned)(kWideBytes / 16), idesc, 1u, empty0 + stage * 8u,
                                       full0 + nstage * 8u, npar);
             } else {
               ready = pair_mma_kblock(d, wd, xd, idesc, kb ? 1u : 0u, empty0 + stage * 8u, full0 + nstage * 8u, npar);
@@ -601,8 +622,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       while (true) {
         if (!info_wait_one(c, &sc->ifull[islot], iph, 24, false)) break;
         const int kind = sc->info[islot].kind;
-        const int kblocks = sc->info[islot].kblocks;
         const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
+        const int n_stages = sc->info[islot].kblocks / kblocks_a_stage<kDual>(sc->info[islot].rows, dual);
         if (kind == kEnd) { ended = true; break; }
         release_slot(sc, islot, false);
         if (++islot == kRing) { islot = 0; iph ^= 1u; }
@@ -612,9 +633,9 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           if (++islot == kRing) { islot = 0; iph ^= 1u; }
         }
         if (kind == kCombine) continue;
-        if (kind != kGateUp) { kiter += (unsigned)kblocks; continue; }
+        if (kind != kGateUp) { kiter += (unsigned)n_stages; continue; }
         bool fail = false;
-        for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
+        for (int i = 0; i < n_stages; ++i, ++kiter) {
           const int stage = (int)(kiter % kNS);
           if (!mbar_wait(c, &sc->fullA[stage], (amask >> stage) & 1u, 25)) { fail = true; break; }
           amask ^= 1u << stage;
@@ -636,6 +657,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     constexpr int kCpr = kRowBytes / 16;                  // 16-byte chunks per row slice
     constexpr int kRowsPerPass = kGatherThreads / kCpr;   // 16 rows per cp.async round
     constexpr int kPasses = Ring<kTileRows, kDual>::kRows / kRowsPerPass;
+    constexpr int kWidePasses = kWideRows / 2 / kRowsPerPass < kPasses ? kWideRows / 2 / kRowsPerPass : kPasses;
     const int chunk = gt % kCpr, rbase = gt / kCpr;
     // the swizzle XORs the chunk index with the row's place in its 8-row group, which is the same in every pass
     static_assert(kRowsPerPass % 8 == 0, "");
@@ -650,6 +672,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kblocks = sc->info[islot].kblocks;
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
       const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
+      const int step = kblocks_a_stage<kDual>(rows, dual);
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
       const int tslot = islot;
@@ -671,18 +694,21 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           const RowPlan rp = row_plan(op, kind, row0, rows, rank);
           unsigned stage = kiter % (unsigned)kNS;
           if (rp.boxes > 0)
-            for (int kb = 0; kb < kblocks && !fail; ++kb) {
+            for (int kb = 0; kb < kblocks && !fail; kb += step) {
               if (!mbar_wait(c, &sc->goR[stage], (rmask >> stage) & 1u, 32)) { fail = true; break; }
               rmask ^= 1u << stage;
               pair_issue_rows(full0 + stage * 8u, kb * kBlockK, rows0 + stage * (unsigned)kSB, rp.map, rp.y, (unsigned)rp.boxes,
                               (unsigned)rp.box_rows);
+              if (step == 2)
+                pair_issue_rows(full0 + stage * 8u, (kb + 1) * kBlockK, rows0 + stage * (unsigned)kSB + (unsigned)kWideBytes, rp.map, rp.y,
+                                (unsigned)rp.boxes, (unsigned)rp.box_rows);
               if (++stage == kNS) stage = 0;
             }
         } else if (warp != 4 && lane == 0) {
           release_slot(sc, tslot, leader);
         }
         if (__any_sync(0xffffffffu, fail)) break;
-        kiter += (unsigned)kblocks;
+        kiter += (unsigned)(kblocks / step);
         continue;
       }
       if (kind == kCombine) {
@@ -730,7 +756,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       }
       unsigned long long* landed = leader ? sc->full : sc->fullA;
       bool fail = false;
-      for (int kb = 0; kb < kblocks; ++kb, ++kiter) {
+      for (int kb = 0; kb < kblocks; kb += step, ++kiter) {
         const int stage = (int)(kiter % kNS);
         if (!wwait(c, &sc->goA[stage], (gmask >> stage) & 1u, 14)) { fail = true; break; }
         gmask ^= 1u << stage;
@@ -738,6 +764,11 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
 #pragma unroll
         for (int j = 0; j < kPasses; ++j)
           if (src[j]) cp_async_16(sA + j * (kRowsPerPass * kRowBytes), src[j] + (size_t)kb * kRowBytes);
+        if (step == 2) {
+#pragma unroll
+          for (int j = 0; j < kWidePasses; ++j)
+            if (src[j]) cp_async_16(sA + kWideBytes + j * (kRowsPerPass * kRowBytes), src[j] + (size_t)(kb + 1) * kRowBytes);
+        }
         cp_async_arrive_noinc(&landed[stage]);
       }
       if (fail) break;

@@ -477,8 +477,13 @@ __device__ inline void commit_tile(const Ctx& c, RunHead* rh, const TileInfo& ti
 // (take_turn) comes later, so that no claim waits behind those of all other units.
 // per_tile: what a committed down tile adds to gemm_done.  max_rows: the tallest work tile this kernel has room for.
 // kTwos: it runs two tiles at a time.  The last entries of a list, two a unit but a quarter of it at most, are handed out one by one all the same:
-// the units end closer to one another (256 tokens on 64 experts: 314 us a pass without, 305).  (Two a unit of a short list is most of it, and
-// single tiles are slow in four stages: 128 decode tokens on 8 experts next to 8192 of prefill, budget 16, done after 535 us, now 443.)
+// the units end closer to one another (256 tokens on 64 experts: 314 us a pass without, 305).  (Two a unit of a short list is most of it: 128
+// decode tokens on 8 experts next to 8192 of prefill, budget 16, done after 535 us, 443 with a quarter.)
+// A decode op next to prefill ops is handed out one by one: latency is what its budget is bought for.  128 decode tokens on 8 experts next to
+// 8192 of prefill, us from claim to commit of a tile at the 99th percentile and until the op is done, in twos / one by one: budget 16 80,
+// 504 / 42, 452, budget 32 80, 276 / 43, 262, budget 64 82, 182 / 46, 190; 64 on 64 experts next to 4096, budget 64 69, 630 / 36, 598; launches as
+// long as before (2320 / 2325, 1190 / 1187).  Not where its tiles carry prefill rows: those of more than 128 rows are slow one by one (16 384 + 256
+// paired 3728 / 3862 us a launch, decode done 2483 / 2856).
 template <bool kTwos>
 __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const RunHead* first_half, int lane, int per_tile, int max_rows) {
   constexpr int kW = 25;
@@ -503,6 +508,12 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
     }
   }
   const unsigned decode_ops = __ballot_sync(0xffffffffu, cls == MOE_CLASS_DECODE);
+  unsigned singly = 0;                             // decode ops next to prefill ops whose tiles carry no prefill rows
+  if constexpr (kTwos) {
+    const int carrier = lane < a->n_ops ? a->carrier[lane] : -1;
+    const unsigned carriers = __reduce_or_sync(0xffffffffu, carrier < 0 ? 0u : 1u << carrier);
+    if (__popc(decode_ops) < a->n_ops) singly = decode_ops & ~carriers;
+  }
   const int combines = ps.planned != 0 && a->fuse_combine ? ps.n_comb_tiles : 0, gemms = ps.planned != 0 ? ps.n_gemm_tiles : 0;
   const int all_gemm = down_tiles(a, ps.n_gemm_tiles + ps.n_extra_gemm) * per_tile;
   const unsigned watched = __ballot_sync(0xffffffffu, (ps.flags & kOpWatched) != 0);
@@ -519,7 +530,7 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
       const int j = sc->n_cls[ci]++;
       sc->cls_slot[ci][j] = a->slots[i];
       sc->cls_free[ci][j] = fi;
-      const int twos = kTwos ? (gi - min((int)gridDim.x, gi / 4)) / 2 : 0;
+      const int twos = kTwos && !((singly >> i) & 1u) ? (gi - min((int)gridDim.x, gi / 4)) / 2 : 0;
       if constexpr (kTwos) sc->twos[ci][j] = (unsigned)twos;
       sc->n_gemm[ci][j] = (unsigned)(gi - twos);
       sc->cum[ci][j + 1] = sc->cum[ci][j] + (unsigned)(gi - twos + ei);

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+import paper_2607_18002_b200 as moe
 from workloads import synth
 
 from gpu_util import bind_ops, make_ctx, weights_to
@@ -48,3 +49,41 @@ def test_two_at_a_time_where_units_have_many_tiles(E, T, twos):
     spec = synth.Spec("rounds", synth.Shape(E, 2, 1024, 1024), ((synth.PREFILL, T),), "zipf", 1.0, 1.0, -1.0, 89)
     ctx, _ = run(spec, n_ctas=32)
     assert any(len(t) > 1 for t in tickets(ctx.tile_log(), 0)) == twos
+
+
+@pytest.mark.parametrize("decode,masked", [(40, False), (300, False), (48, True)])
+def test_decode_entries_go_one_by_one_next_to_prefill(decode, masked):
+    """In a launch that hands prefill entries out in twos, the decode op's tickets are single entries.  Its tiles (rows below and above the 128 up to
+    which two k-blocks share a stage, gathered or consecutive) and those at the end of the prefill list give bit for bit what each op gives
+    by itself in the plain launch, or the masked op in a launch of its own."""
+    E, H, I = 6, 1024, 768
+    spec = synth.Spec("latency", synth.Shape(E, 2, H, I), ((synth.PREFILL, 1800), (synth.DECODE, decode)), "zipf", 1.0, 1.0, -1.0, 97)
+    W = weights_to(synth.make_weights(spec))
+    ops = synth.make_ops(spec)
+    ctx = make_ctx(spec, max_tokens=1800, n_ctas=6, tile_log_entries=1 << 14)
+    bound = bind_ops(ctx, ops, W)
+    alone = make_ctx(spec, max_tokens=1800, max_ops=1)
+    if masked:
+        x = torch.randn(E, decode, H, generator=torch.Generator().manual_seed(5)).to(torch.bfloat16).cuda()
+        counts = torch.tensor([48, 0, 1, 17, 33, 40], dtype=torch.int32, device="cuda")
+        bound[1] = moe.bind_masked_op(moe.MOE_CLASS_DECODE, x, counts, W.w_gate_up, W.w_down)
+        valid = torch.arange(decode, device="cuda")[None, :] < counts[:, None]
+    else:
+        valid = slice(None)
+    want = []
+    for s, b in enumerate(bound):
+        b.y.fill_(7.0)
+        alone.plan(0, b)
+        alone.run([0]) if masked and s == 1 else alone.run_plain(0)
+        alone.check()
+        want.append(b.y.clone())
+    ctx.set_budget(2)
+    for s, b in enumerate(bound):
+        b.y.fill_(7.0)
+        ctx.plan(s, b)
+    for _ in range(2):
+        ctx.run([0, 1], fuse_combine=True)
+    ctx.check()
+    log = ctx.tile_log()
+    assert any(len(t) == 2 for t in tickets(log, 0)) and all(len(t) == 1 for t in tickets(log, 1))
+    assert torch.equal(bound[0].y, want[0]) and torch.equal(bound[1].y[valid], want[1][valid])
