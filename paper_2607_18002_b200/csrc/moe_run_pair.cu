@@ -213,6 +213,15 @@ __device__ __forceinline__ int first_feature(const TileInfo& ti, int rank, bool 
   return (2 * ti.n + (dual ? 2 * rank : rank)) * w;
 }
 
+// Two tiles at a time, in launches with ops of both classes: the k-block of two tiles at which the scheduler may claim what comes after them.  A
+// claim at their start is held for twice their time, and that long a unit does not turn to the other class: 128 decode tokens on 8
+// experts that arrive in the middle of 8192 of prefill were done after 521, 236 and 211 us at budgets 16, 64 and 128, tile by tile after 508, 175
+// and 148, now after 442, 173 and 119.  It leaves the claim and the list of rows the time of a dozen k-blocks (with 8 or 4 to go the MMAs wait
+// for them: 8192 + 128 tokens 3047 and 3090 us a launch where half the tile takes 2961 and its start 2916).  Launches of one class have
+// nothing to turn to.
+constexpr int kClaimBlocks = 12;
+__device__ __forceinline__ int late_claim(int kblocks) { return max(0, min(kblocks / 2, kblocks - kClaimBlocks)); }
+
 // The place of the weight rows of one CTA, and their L2 policy
 struct WeightPlan {
   const CUtensorMap* map;
@@ -382,8 +391,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // ============================================================ scheduler (leader)
     // Claims a tile, waits (bounded) for a free ring slot, the op's ready word and the tile's
     // dependencies, and publishes it to both CTAs.  The next claim starts when the producer has
-    // taken the published tile, so the pair holds at most one claimed tile beyond the one whose
-    // loads are being issued.
+    // taken the published tile (see late_claim), so the pair holds at most one claimed ticket, a tile or two that run
+    // together, beyond the one whose loads are being issued.
     int islot = 0;
     unsigned iph = 0;
     int published = 0;                                    // tiles so far, to kRing: every ring slot has been used
@@ -491,7 +500,9 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         const TileInfo ti = sc->info[islot];
         if (ti.kind == kEnd) { ended = true; break; }
         const bool dual = kDual && (ti.expert & kDualFirst) != 0;
-        if (leader) mbar_arrive(&sc->taken[islot]);
+        unsigned long long* const taken = &sc->taken[islot];
+        const int claim_at = dual && leader && sc->qt.two_classes != 0 ? late_claim(ti.kblocks) : 0;
+        if (leader && claim_at == 0) mbar_arrive(taken);
         release_slot(sc, islot, leader);
         if (++islot == kRing) { islot = 0; iph ^= 1u; }
         if (dual) {                                          // the descriptor behind it is for those that store the tiles
@@ -512,6 +523,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         bool fail = false;
         for (int kb = 0; kb < ti.kblocks; kb += step) {
           if (!ready && !mbar_wait(c, &sc->empty[stage], par, 5)) { fail = true; break; }
+          if (claim_at > 0 && kb == claim_at) mbar_arrive(taken);
           const unsigned nstage = stage + 1 == kNS ? 0u : stage + 1, npar = stage + 1 == kNS ? par ^ 1u : par;
           ready = pair_issue_kblock(full0 + stage * 8u, (w_bytes + row_bytes) * (unsigned)step, smem_u32(&sc->full[stage]), standin,
                                     go + stage * 8u, has_go, w0 + stage * (unsigned)kSB, wp.map, kb * kBlockK, wp.blk, wp.expert, wp.policy,

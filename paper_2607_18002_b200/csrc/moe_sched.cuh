@@ -25,6 +25,7 @@ struct ClaimWords {
 struct QueueTables {
   unsigned run_off;                // of this launch
   int watched;                     // an op of the launch is: committed tiles are counted
+  int two_classes;                 // (two tiles at a time) it has ops of both
   int n_cls[2];
   int cls_slot[2][kMaxOps];
   int cls_free[2][kMaxOps];        // 1: the op has no ready word and no predecessor
@@ -512,7 +513,9 @@ __device__ inline ClaimWords begin_unit(const RunArgs* a, QueueTables* sc, const
   if constexpr (kTwos) {
     const int carrier = lane < a->n_ops ? a->carrier[lane] : -1;
     const unsigned carriers = __reduce_or_sync(0xffffffffu, carrier < 0 ? 0u : 1u << carrier);
-    if (__popc(decode_ops) < a->n_ops) singly = decode_ops & ~carriers;
+    const bool both = decode_ops != 0 && __popc(decode_ops) < a->n_ops;
+    if (both) singly = decode_ops & ~carriers;
+    if (lane == 0) sc->two_classes = both;
   }
   const int combines = ps.planned != 0 && a->fuse_combine ? ps.n_comb_tiles : 0, gemms = ps.planned != 0 ? ps.n_gemm_tiles : 0;
   const int all_gemm = down_tiles(a, ps.n_gemm_tiles + ps.n_extra_gemm) * per_tile;

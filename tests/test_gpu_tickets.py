@@ -87,3 +87,18 @@ def test_decode_entries_go_one_by_one_next_to_prefill(decode, masked):
     log = ctx.tile_log()
     assert any(len(t) == 2 for t in tickets(log, 0)) and all(len(t) == 1 for t in tickets(log, 1))
     assert torch.equal(bound[0].y, want[0]) and torch.equal(bound[1].y[valid], want[1][valid])
+
+
+def test_a_unit_next_to_another_class_claims_late():
+    """In a launch with both classes a unit asks for its next ticket half-way through the loads of two prefill tiles, so that it holds a ticket
+    for one and a half times what one takes.  (Asked for at their start it is held for two.)"""
+    spec = synth.Spec("late", synth.Shape(4, 2, 3072, 1536), ((synth.PREFILL, 1500), (synth.DECODE, 8)), "uniform", None, 1.0, -1.0, 101)
+    ctx, _ = run(spec, n_ctas=6, budget=2)
+    got = [t for t in tickets(ctx.tile_log(), 0) if len(t) == 2 and t[0]["kind"] == 0]       # 48 k-blocks each
+    held, period = [], []
+    for u in {int(t[0]["cta"]) for t in got} - {0}:                    # the unit inside the budget starts with decode tiles
+        mine = sorted((t for t in got if t[0]["cta"] == u), key=lambda t: t[0]["t_claim"])[2:]
+        end = [max(int(r["t_commit"]) for r in t) for t in mine]
+        held += [e - int(t[0]["t_claim"]) for e, t in zip(end, mine)]
+        period += list(np.diff(end))
+    assert len(period) > 10 and np.median(held) < 1.75 * np.median(period), (np.median(held), np.median(period))
