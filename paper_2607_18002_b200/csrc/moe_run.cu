@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
     ti.slot = ti.tile = ti.m = ti.row0 = ti.rows = ti.n = ti.kblocks = ti.expert = ti.cls = 0;
     ti.t_claim = 0;
     while (true) {
-      claim_next<false, false>(c, &sc->qt, rh, lane, ti, need_ready, nullptr, one);
+      claim_next<false, false>(c, &sc->qt, rh, lane, ti, need_ready, one);
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);      // the claim loops exit warp-uniformly
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
       // a free ring slot, the op ready, the tile's dependencies met

@@ -214,10 +214,10 @@ __device__ __forceinline__ unsigned first_entry(const QueueTables* sc, int cls, 
 // early_combine: also take a combine entry whose GEMM entries are still running -- all of them must have been claimed, or every unit
 // could end up holding such an entry with none left for what they wait for.  The op's own are (the head stands behind them); those of
 // the decode list that carry rows of a paired prefill op are once the head of the decode queue, other_head, has passed them.
-// more, have_more (kTwos): the ticket's second entry.
+// two (kTwos): the ticket holds the entry behind it too, the next n-block of the same work tile.
 template <bool kTwos>
 __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int cls, unsigned h, unsigned other_head,
-                                int lane, TileInfo& ti, bool& need_ready, TileInfo* more, bool& have_more, bool early_combine = false) {
+                                int lane, TileInfo& ti, bool& need_ready, bool& two, bool early_combine = false) {
   const RunArgs* a = c.a;
   const int n = sc->n_cls[cls];
   if (n == 0) return 0;
@@ -266,22 +266,16 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
   // the op is instantiated by the claim of its first tile: its budget field takes effect now
   if (local == 0 && lane == 0 && op->op_budget > 0) atomicExch(&a->g->budget, op->op_budget);
   const unsigned at = first_entry<kTwos>(sc, cls, i, local);
-  const auto entry = [&](unsigned at, TileInfo& to) {
-    const unsigned d = at - first;
-    const bool hit = same_op && d < 32u;
-    int4 got;
-    got.x = __shfl_sync(0xffffffffu, e.x, hit ? d : 0);
-    got.y = __shfl_sync(0xffffffffu, e.y, hit ? d : 0);
-    got.z = __shfl_sync(0xffffffffu, e.z, hit ? d : 0);
-    got.w = __shfl_sync(0xffffffffu, e.w, hit ? d : 0);
-    if (!hit) got = sc->list[cls][i][at];
-    fill_tile(a, got, slot, (int)at, cls, to);
-  };
-  entry(at, ti);
-  if constexpr (kTwos) {
-    have_more = local < sc->twos[cls][i];
-    if (have_more) entry(at + 1, *more);
-  }
+  const unsigned d = at - first;
+  const bool hit = same_op && d < 32u;
+  int4 got;
+  got.x = __shfl_sync(0xffffffffu, e.x, hit ? d : 0);
+  got.y = __shfl_sync(0xffffffffu, e.y, hit ? d : 0);
+  got.z = __shfl_sync(0xffffffffu, e.z, hit ? d : 0);
+  got.w = __shfl_sync(0xffffffffu, e.w, hit ? d : 0);
+  if (!hit) got = sc->list[cls][i][at];
+  fill_tile(a, got, slot, (int)at, cls, ti);
+  if constexpr (kTwos) two = local < sc->twos[cls][i];
   return 1;
 }
 
@@ -292,10 +286,10 @@ __device__ inline int try_claim(const Ctx& c, QueueTables* sc, RunHead* rh, int 
 // kEarlyCombine: a unit that finds nothing to run in either class takes a combine entry that has to wait for GEMM entries running
 // elsewhere (see try_claim), so that the wait for the last of them starts with the entry in hand.  It claims nothing more meanwhile.
 // seen: the words as the unit's start read them (its first claim); they only tell where to look, the fetch-add decides.
-// kTwos: more, have_more: the second entry of the ticket.
+// kTwos: two: see try_claim.
 template <bool kEarlyCombine, bool kTwos>
 __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int lane, TileInfo& ti,
-                                 bool& need_ready, TileInfo* more, bool& have_more, const ClaimWords* seen = nullptr) {
+                                 bool& need_ready, bool& two, const ClaimWords* seen = nullptr) {
   const RunArgs* a = c.a;
   ClaimWords w{};
   if (seen) {
@@ -325,16 +319,15 @@ __device__ inline int claim_once(const Ctx& c, QueueTables* sc, RunHead* rh, int
     for (int p = 0; p < 4; ++p) {
       if (p >= 2 && none[p & 1] == 0) continue;
       const int cls = (p & 1) ? 1 - first : first;
-      none[p & 1] = try_claim<kTwos>(c, sc, rh, cls, cls == 0 ? h0 : h1, cls == 0 ? h1 : h0, lane, ti, need_ready, more, have_more, p >= 2);
+      none[p & 1] = try_claim<kTwos>(c, sc, rh, cls, cls == 0 ? h0 : h1, cls == 0 ? h1 : h0, lane, ti, need_ready, two, p >= 2);
       if (none[p & 1] == 1) break;
     }
   } else {                                       // (in a loop this kernel's scheduler spills)
-    none[0] = try_claim<kTwos>(c, sc, rh, first, first == 0 ? h0 : h1, 0u, lane, ti, need_ready, more, have_more);
-    if (none[0] != 1) none[1] = try_claim<kTwos>(c, sc, rh, 1 - first, first == 0 ? h1 : h0, 0u, lane, ti, need_ready, more, have_more);
+    none[0] = try_claim<kTwos>(c, sc, rh, first, first == 0 ? h0 : h1, 0u, lane, ti, need_ready, two);
+    if (none[0] != 1) none[1] = try_claim<kTwos>(c, sc, rh, 1 - first, first == 0 ? h1 : h0, 0u, lane, ti, need_ready, two);
   }
   if (none[0] == 1 || none[1] == 1) {
     if (a->log_cap > 0) ti.t_claim = gtime_ns();
-    if (kTwos && have_more) more->t_claim = ti.t_claim;
     return 1;
   }
   return (none[0] | none[1]) == 0 ? 0 : -1;
@@ -378,10 +371,10 @@ __device__ inline void claim_static(const RunArgs* a, int unit, TileInfo& ti) {
 // ti.kind == kEnd when nothing is left (or the run was aborted).
 template <bool kEarlyCombine, bool kTwos>
 __device__ inline void claim_next(const Ctx& c, QueueTables* sc, RunHead* rh, int lane, TileInfo& ti,
-                                  bool& need_ready, TileInfo* more, bool& have_more, const ClaimWords* seen = nullptr) {
+                                  bool& need_ready, bool& two, const ClaimWords* seen = nullptr) {
   unsigned long long t0 = 0;
   for (unsigned it = 0;; ++it) {
-    const int r = claim_once<kEarlyCombine, kTwos>(c, sc, rh, lane, ti, need_ready, more, have_more, seen);
+    const int r = claim_once<kEarlyCombine, kTwos>(c, sc, rh, lane, ti, need_ready, two, seen);
     seen = nullptr;
     if (r == 1) return;
     if (r == 0) break;
