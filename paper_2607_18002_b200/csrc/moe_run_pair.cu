@@ -215,11 +215,11 @@ __device__ __forceinline__ int first_feature(const TileInfo& ti, int rank, bool 
 
 // Two tiles at a time, in launches with ops of both classes: the k-block of two tiles at which the scheduler may claim what comes after them.  A
 // claim at their start is held for twice their time, and that long a unit does not turn to the other class: 128 decode tokens on 8
-// experts that arrive in the middle of 8192 of prefill were done after 521, 236 and 211 us at budgets 16, 64 and 128, tile by tile after 508, 175
-// and 148, now after 442, 173 and 119.  It leaves the claim and the list of rows the time of a dozen k-blocks (with 8 or 4 to go the MMAs wait
-// for them: 8192 + 128 tokens 3047 and 3090 us a launch where half the tile takes 2961 and its start 2916).  Launches of one class have
-// nothing to turn to.
-constexpr int kClaimBlocks = 12;
+// experts that arrive in the middle of 8192 of prefill were done after 512, 235 and 210 us at budgets 16, 64 and 128, tile by tile after 479, 183
+// and 140, and so after 439, 174 and 134.  The claim and the list of rows need the time of some 16 k-blocks: us a launch with 16, 12, 8 and 4 to go
+// (half the tile at most) 2048 + 128 tokens paired 1400, 1410, 1450, 1466, claimed at the start 1403; 1000 + 200 2211, 2221, 2285, 2313 /
+// 2228; 2048 + 256 on 128 experts 1339, 1343, 1405, 1436 / 1318.  Launches of one class have nothing to turn to.
+constexpr int kClaimBlocks = 16;
 __device__ __forceinline__ int late_claim(int kblocks) { return max(0, min(kblocks / 2, kblocks - kClaimBlocks)); }
 
 // The place of the weight rows of one CTA, and their L2 policy
@@ -885,8 +885,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         const int vecs = args.H / 8, mid = ti.row0 + (ti.rows + 1) / 2;
         const bool by_columns = ti.rows == 1;
         const CombineWhenDone ready{&c, op, &sc->combine_ready, ++combines, warp == 8 && lane == 0};
-        ok = by_columns ? combine_tokens(op, ti.row0, ti.row0 + ti.rows, leader ? 0 : vecs / 2, vecs / 2, args.k, args.H, etid, 256, ready)
-                        : combine_tokens(op, leader ? ti.row0 : mid, leader ? mid : ti.row0 + ti.rows, 0, vecs, args.k, args.H, etid, 256, ready);
+        const int t0 = by_columns || leader ? ti.row0 : mid, t1 = by_columns || !leader ? ti.row0 + ti.rows : mid;
+        ok = combine_tokens(op, t0, t1, by_columns && !leader ? vecs / 2 : 0, by_columns ? vecs / 2 : vecs, args.k, args.H, etid, 256, ready);
         if (!ok) break;
       } else {
         // read ahead of the accumulator: behind it these round trips, through a memory system full of weights, delay the tiles that wait
