@@ -157,6 +157,12 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream);
  * ready (Section 6.4) -- and runs it: gate/up grouped GEMM with fused SwiGLU, then the
  * down grouped GEMM, on rows gathered through the permutation.  A phase switch happens
  * only between tiles (Section 4.2), so results do not depend on the schedule.
+ * The claiming unit is a CTA, for bf16 on an even grid a pair of CTAs.  What a unit claims
+ * at a time -- a ticket -- is one tile.  In large bf16 launches a ticket of a prefill op, and
+ * of a decode op that is alone in its launch or whose tiles carry prefill rows
+ * (moe_plan_pair), is two neighbouring tiles that run together: the same rows, the next
+ * columns.  A unit holds one claimed ticket beyond the one it is loading; next to ops of the
+ * other class it claims that one half-way through the loads of two tiles.
  * Ops of one class are served in the order given.  With fuse_combine != 0 the
  * router-weighted combine runs as tiles of the same launch and y is final when the
  * kernel ends; otherwise call moe_combine.
@@ -202,7 +208,8 @@ int moe_run_plain(moe_ctx_t* ctx, int slot, void* stream);
 int moe_combine(moe_ctx_t* ctx, int slot, void* stream);
 
 /* Decode SM budget q of Section 6.4: a stream-ordered 4-byte write to the device word
- * the running kernel reads at every tile boundary.  0 <= decode_sms. */
+ * the running kernel reads at every claim, i.e. at every tile boundary, or every second one
+ * where two tiles run together (see moe_run).  0 <= decode_sms. */
 int moe_set_budget(moe_ctx_t* ctx, int decode_sms, void* stream);
 
 /* Online SM reallocation (Section 6.4, "Online SM Reallocation"): sets the budget word to
