@@ -86,9 +86,9 @@ struct __align__(128) OpDev {
   CUtensorMap tm_a32;   // [Rmax, I]   box {64, 32}
   CUtensorMap tm_w1;    // gate/up weights as [1][E][gate, up][I][H], box of 128 gate rows and the 128 matching up rows x 128 bytes
   CUtensorMap tm_w2;    // down weights as [1][E][H/128][128][I], box of 256 consecutive rows x 128 bytes
-                        // (CTA pairs: views of tm_p1 and tm_p2 with boxes of 256 rows)
+                        // (CTA pairs: views of tm_p1 and tm_p2 with boxes of 256 rows, where two tiles may run together)
   CUtensorMap tm_a128;  // [Rmax, I]   box {64, 128}
-  CUtensorMap tm_a256;  // [Rmax, I]   box {64, 256}
+  CUtensorMap tm_a256;  // [Rmax, I]   box {64, 256} (as tm_x256 not for CTA pairs)
   CUtensorMap tm_p1;    // weights as the M operand: gate/up rows x 128 bytes, a box holds 64 gate rows and the matching up rows in
                         // groups of eight (bf16: [E][I/8][gate, up][8][H]), or 128 of each (e4m3: [8][2 E I][gate, up][8 every other][H])
   CUtensorMap tm_p2;    // ... down, as [E][H/16][2][8][I], box of 128 (e4m3: 256) consecutive rows x 128 bytes

@@ -392,7 +392,7 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
   ctx->pair_of[slot] = -1;
   ctx->ran_paired[slot] = false;
   // Re-planning a slot with the same buffers (the usual serving loop) reuses the descriptors
-  // already on the device: encoding seven tensor maps and uploading them is host time.
+  // already on the device: encoding its tensor maps and uploading them is host time.
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const unsigned long long cap = capture_of(st);
   const bool same = ctx->up[slot].sent && memcmp(&ctx->ops[slot], op, sizeof(moe_op_t)) == 0;
@@ -404,14 +404,14 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
       rc = make_map(ctx, &h.tm_a8, h.A, (size_t)L.max_rows, (size_t)c.inter, 8);
       if (!rc) rc = make_map(ctx, &h.tm_a32, h.A, (size_t)L.max_rows, (size_t)c.inter, 32);
       if (!rc) rc = make_map(ctx, &h.tm_a128, h.A, (size_t)L.max_rows, (size_t)c.inter, 128);
-      if (!rc) rc = make_map(ctx, &h.tm_a256, h.A, (size_t)L.max_rows, (size_t)c.inter, 256);
+      if (!rc && !ctx->pair_kernel) rc = make_map(ctx, &h.tm_a256, h.A, (size_t)L.max_rows, (size_t)c.inter, 256);
       const size_t E = c.n_experts, H = c.hidden, I = c.inter;
       const bool fp8 = c.dtype == MOE_DTYPE_FP8_E4M3;
       if (!rc && ctx->pair_kernel)                 // 8 gate rows, the 8 matching up rows, the next 8 gate rows, ...
         rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, I / 8, E}, {1, I, 8, 2 * I}, {8, 2, 8, 1});
-      if (!rc && ctx->pair_kernel)                 // ... two n-blocks' rows at once
+      if (!rc && may_run_twos(ctx))                // ... two n-blocks' rows at once
         rc = make_map_m(ctx, &h.tm_w1, op->w_gate_up, H, {8, 2, I / 8, E}, {1, I, 8, 2 * I}, {8, 2, 16, 1});
-      if (!rc && ctx->pair_kernel)
+      if (!rc && may_run_twos(ctx))
         rc = make_map_m(ctx, &h.tm_w2, op->w_down, I, {8, 2, H / 16, E}, {1, 8, 16, H}, {8, 2, 16, 1});
       if (!rc && fp8)                              // ... of 16 rows: 8 even gate, 8 even up, 8 odd gate, 8 odd up rows
         rc = make_map_m(ctx, &h.tm_p1, op->w_gate_up, H, {8, 2, 2 * E * I, 8}, {2, I, 1, 16}, {8, 2, 2, 8});
@@ -426,7 +426,7 @@ int moe_plan(moe_ctx_t* ctx, int slot, const moe_op_t* op, void* stream) {
         if (!rc) rc = make_map(ctx, &h.tm_x8, op->x, xr, (size_t)c.hidden, 8);
         if (!rc) rc = make_map(ctx, &h.tm_x32, op->x, xr, (size_t)c.hidden, 32);
         if (!rc) rc = make_map(ctx, &h.tm_x128, op->x, xr, (size_t)c.hidden, 128);
-        if (!rc) rc = make_map(ctx, &h.tm_x256, op->x, xr, (size_t)c.hidden, 256);
+        if (!rc && !ctx->pair_kernel) rc = make_map(ctx, &h.tm_x256, op->x, xr, (size_t)c.hidden, 256);
       }
       if (rc) return rc;
     }

@@ -26,18 +26,6 @@ __device__ __forceinline__ bool mbar_try(void* bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
-// non-blocking test of a phase (try_wait may suspend the thread for a while)
-__device__ __forceinline__ bool mbar_test(void* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
 // orders what this thread wrote or saw before what it writes after, for all of the device
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // L2 policy of bytes that nobody reads a second time
@@ -239,18 +227,6 @@ __device__ __forceinline__ bool mbar_try_relaxed(void* bar, unsigned parity) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// non-blocking test that also synchronises with arrivals of the other CTA
-__device__ __forceinline__ bool mbar_test_cluster(void* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
       : "r"(smem_u32(bar)), "r"(parity)

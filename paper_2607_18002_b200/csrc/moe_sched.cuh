@@ -132,11 +132,6 @@ __device__ __forceinline__ int op_total_tiles(const OpDev* op, int fuse) {
   if (op->plan->planned == 0) return 0;
   return op->plan->n_gemm_tiles + op->plan->n_extra_gemm + (fuse ? op->plan->n_comb_tiles : 0);
 }
-// entries of the op's own queue list
-__device__ __forceinline__ int op_queue_entries(const OpDev* op, int fuse) {
-  if (op->plan->planned == 0) return 0;
-  return op->plan->n_gemm_tiles + (fuse ? op->plan->n_comb_tiles : 0);
-}
 // Of `gemm` GEMM entries the down tiles.  They are what an op's combine waits for: none of them commits before its gate/up tiles.
 __device__ __forceinline__ int down_tiles(const RunArgs* a, int gemm) {
   const int nt1 = a->I / kTileN1, nt2 = a->H / kTileN2;
