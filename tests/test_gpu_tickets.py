@@ -102,3 +102,71 @@ def test_a_unit_next_to_another_class_claims_late():
         held += [e - int(t[0]["t_claim"]) for e, t in zip(end, mine)]
         period += list(np.diff(end))
     assert len(period) > 10 and np.median(held) < 1.75 * np.median(period), (np.median(held), np.median(period))
+
+
+def test_masked_entries_in_twos():
+    """A masked op next to a large gathered op of its own class: its gate/up tiles (consecutive rows of x) and down tiles run in twos as well, at 1 to
+    200 rows; bit for bit the op in a launch of its own."""
+    E, H, I, slab = 6, 1024, 768, 200
+    spec = synth.Spec("masked2", synth.Shape(E, 2, H, I), ((synth.DECODE, 1800), (synth.DECODE, 600)), "zipf", 1.0, 1.0, -1.0, 103)
+    W = weights_to(synth.make_weights(spec))
+    ctx = make_ctx(spec, max_tokens=1800, n_ctas=6, tile_log_entries=1 << 14)
+    x = torch.randn(E, slab, H, generator=torch.Generator().manual_seed(7)).to(torch.bfloat16).cuda()
+    counts = torch.tensor([200, 1, 0, 129, 128, 33], dtype=torch.int32, device="cuda")
+    op = moe.bind_masked_op(moe.MOE_CLASS_DECODE, x, counts, W.w_gate_up, W.w_down)
+    alone = make_ctx(spec, max_tokens=600, max_ops=1)
+    alone.plan(0, op)
+    alone.run([0])
+    alone.check()
+    want = op.y.clone()
+    op.y.fill_(7.0)
+    ctx.plan(0, bind_ops(ctx, synth.make_ops(spec)[:1], W)[0])
+    ctx.plan(1, op)
+    ctx.run([0, 1], fuse_combine=True)
+    ctx.check()
+    two = [t for t in tickets(ctx.tile_log(), 1) if len(t) == 2]
+    assert {int(t[0]["kind"]) for t in two} == {1, 3}
+    valid = torch.arange(slab, device="cuda")[None, :] < counts[:, None]
+    assert torch.equal(op.y[valid], want[valid]) and torch.all(op.y[~valid] == 7.0)
+
+
+def test_a_captured_step_in_twos_and_an_entry_out_of_range():
+    """A layer step of both classes that runs two tiles at a time, captured and replayed on other routing in the same buffers: the same as when called.
+    A permutation entry out of range, met by the warp that lists the rows of the next tiles, ends the launch with MOE_EBOUNDS, and the step behind
+    it is right again."""
+    spec = synth.Spec("cap2", synth.Shape(6, 2, 1024, 768), ((synth.PREFILL, 1800), (synth.DECODE, 40)), "zipf", 1.0, 1.0, -1.0, 107)
+    W = weights_to(synth.make_weights(spec))
+    ctx = make_ctx(spec, max_tokens=1800, n_ctas=6, tile_log_entries=1 << 14, wait_limit_us=20000)
+    bound = bind_ops(ctx, synth.make_ops(spec), W)
+
+    def step():
+        ctx.set_budget(2)
+        for s, b in enumerate(bound):
+            ctx.plan(s, b)
+        ctx.run([0, 1], fuse_combine=True)
+
+    step()
+    ctx.check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+    for shift in (0, 1):
+        for b in bound:
+            b.topk_ids.copy_((b.topk_ids + shift) % 6)
+        step()
+        ctx.check()
+        want = [b.y.clone() for b in bound]
+        for b in bound:
+            b.y.fill_(7.0)
+        graph.replay()
+        ctx.check()
+        assert any(len(t) == 2 for t in tickets(ctx.tile_log(), 0))
+        assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
+    for at in (0, 700, 3599):
+        bound[0].sorted_to_flat[at] = 1 << 28
+        ctx.run([0, 1], fuse_combine=True)
+        torch.cuda.synchronize()
+        assert ctx.status()[0] == moe.MOE_EBOUNDS
+        step()
+        ctx.check()
+        assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
