@@ -533,11 +533,11 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   // the stores that nothing overlaps.  What is known here are the rows: a lower bound of the tiles, counted below in rounds of the units.
   // With few rounds the longer tickets leave units idle at the end.  us a pass, one by one / two at a time (rounds):
   //   48 and 24 k-blocks a tile, 8 experts: 500 tokens 130 / 141 (4.9), 800 214 / 219 (8.1), 1200 274 / 277 (12); 16 experts: 400 145 / 149 (3.9),
-  //   700 203 / 213 (6.8); 32: 600 241 / 249 (5.8), 1000 309 / 310 (10); 256: 8192 2367 / 2271 (83);
+  //   700 203 / 213 (6.8); 32: 600 241 / 249 (5.8), 1000 309 / 310 (10); 256: 8192 2458 / 2389 (83);
   //   32 and 16, 32 experts: 700 137 / 146 (4.5), 1000 168 / 171 (6.7), 1500 214 / 212 (10); 64: 500 173 / 175 (3.2), 1000 220 / 222 (6.7);
   //   16 and 8, 32 experts: 2400 83 / 88 (4.0), 4000 112 / 117 (6.7), 6000 144 / 142 (10), 12 000 256 / 249 (20).
   // Where experts get few rows most tiles are short ones that the bound does not count, and two at a time pay earlier:
-  //   48 and 24: 777 tokens on 256 experts 1134 / 1127 (7.8), 600 on 128 632 / 626 (5.8); 16 and 8: 1500 on 128 142 / 141 (5.0); but 32 and 16: 700
+  //   48 and 24: 777 tokens on 256 experts 1181 / 1159 (7.8), 600 on 128 632 / 626 (5.8); 16 and 8: 1500 on 128 142 / 141 (5.0); but 32 and 16: 700
   //   on 128 315 / 320 (4.5).  8 or more k-blocks: 5000 tokens on 8 experts with 4 and 8 of them take 61 / 65.
   const long long rounds = routed <= (long long)kDualFewRows * c.n_experts ? kDualRoundsFew : kDualRounds;
   const bool dual = may_run_twos(ctx) && routed / kWorkRowsBf16 * (ctx->L.NT1 + ctx->L.NT2) >= rounds * (ctx->n_ctas / 2) &&

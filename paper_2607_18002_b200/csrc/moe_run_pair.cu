@@ -19,8 +19,9 @@
 //     by side.  Large launches run at the 1000 W limit, where time is energy, and a 256-row k-block came to 580 clocks of the SMs' intake from L2
 //     for 513 of the tensor pipe (both measured without the other): two of them now take in 96 KB a pair instead of 128, and hand-overs,
 //     TMA instructions and gather serve twice the weights.  Nothing overlaps the stores of two accumulators but the first MMAs of the next two
-//     tiles.  us a pass, before and after: 8192 tokens 2440 -> 2260, 16 384 + 256 paired 4170 -> 3930, 4096 + 64 on 64 experts 1220 -> 1175,
-//     777 1166 -> 1149.
+//     tiles.  us a pass, one by one / two at a time, in turn on one GPU: 8192 tokens 2458 / 2389, 12 288 3174 / 3065, 16 384 + 256 paired
+//     4236 / 4113, 4096 + 64 on 64 experts 1254 / 1210, 777 1181 / 1159.  (What comes from DRAM does not shrink: 2048 tokens on 64 experts 2.01 GB /
+//     2.03.)
 // Roles per CTA (16 warps): leader only -- warp 0 scheduler (claims, waits for dependencies,
 // publishes tile descriptors to both CTAs), warp 1 MMA issuer, warp 2 committer; both CTAs --
 // warp 3 producer (TMA loads of its own half of the weights), warps 4-7 gather (a thread of warp 4 loads consecutive rows as boxes),
@@ -577,7 +578,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
           const bool g1 = kind == kGateUp;
           bool fail = false;
           // Two tiles: while the other accumulator is still being stored, the first tile's MMAs of the k-blocks that are there are issued.  (With
-          // this, and both tiles stored before either is counted: 8192 tokens 2365 -> 2290 us a pass, 12 288 3175 -> 2990.)
+          // this, and both tiles stored before either is counted: 8192 tokens 2365 -> 2290 us a pass, 12 288 3175 -> 2990.  Asked with
+          // test_wait, which does not suspend the thread, the same or a little slower: 8192 2203 / 2205, 4096 + 64 on 64 experts 1126 / 1137.)
           int ahead = 0;
           if (dual) {
             unsigned st = stage, pa = par;
