@@ -39,8 +39,8 @@ enum TileKind : int { kGateUp = 0, kDown = 1, kCombine = 2, kGateUpDirect = 3 };
 // y = first packed row (first token for a combine tile), z = valid rows, w = expert (| kReadOnce: no other work tile of the op, or of the
 // pair, reads its weights; not in bf16 plans for the single-CTA kernel).
 constexpr int kReadOnce = 1 << 16;
-// ... in a tile descriptor only: the tile runs together with the one behind it, see moe_run_pair.cu
-constexpr int kDualFirst = 1 << 17;
+// ... in a tile descriptor only: the tile and the next n-block run together, see moe_run_pair.cu
+constexpr int kTwoTiles = 1 << 17;
 // what a plan's list is made for: kReadOnce or 0, and whether a launch may hand its GEMM entries out in twos: two n-blocks of a work tile, which run
 // together
 struct ListForm {

@@ -47,7 +47,6 @@ struct Ring {
   static constexpr int kABytes = kRows * kRowBytes;
   static constexpr int kSB = kABytes + (kDual ? 2 : 1) * kBBytes;
   static constexpr int kNS = kDual ? 4 : kTileRows == 256 ? 6 : kTileRows == 128 ? 8 : 11;
-  static constexpr int kInfos = kDual ? 8 : 4;           // tile descriptors: those being loaded, claimed ahead and being stored
 };
 // Two tiles at a time: of a tile that runs alone and has so few rows (a decode tile, the end of a list) a stage takes two k-blocks, the second's
 // weights and rows in the second half of either part.  With one a stage, half of it was unused and four were in flight where six are
@@ -74,7 +73,9 @@ __device__ __forceinline__ int kblocks_a_stage(int rows, bool dual) { return kDu
 
 template <int kTileRows, bool kDual>
 struct SharedCtl {
-  static constexpr int kRing = Ring<kTileRows, kDual>::kInfos;
+  // One descriptor a ticket, of two tiles too: the second is the next n-block.  (With one a tile and eight of them a unit claimed up to eight single
+  // tiles while its epilogue was at a combine tile: of 256 decode tokens that become ready in the middle of 16 384 of prefill, budget 16, the
+  // slowest hundredth of the tiles took 157 us from claim to commit, with four 80.)
   alignas(16) TileInfo info[kRing];
   // leader's: everything the MMAs of a stage read is in place.  kFullCount arrivals: one expect_tx
   // per producer (TMA bytes of both CTAs), one per gather thread of the leader (completion of its
@@ -327,7 +328,7 @@ template <int kTileRows, bool kDual>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
   using R = Ring<kTileRows, kDual>;
-  constexpr int kNS = R::kNS, kSB = R::kSB, kABytes = R::kABytes, kRing = R::kInfos;
+  constexpr int kNS = R::kNS, kSB = R::kSB, kABytes = R::kABytes;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* stages = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -396,7 +397,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     // together, beyond the one whose loads are being issued.
     int islot = 0;
     unsigned iph = 0;
-    int published = 0;                                    // tiles so far, to kRing: every ring slot has been used
+    bool lapped = false;                                  // every ring slot has been used
     TileInfo ti;
     bool need_ready = false, two = false;                 // two: the ticket's second tile is the next n-block and runs together with the first
     ti.kind = kEnd;
@@ -415,23 +416,14 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       ti.kind = __shfl_sync(0xffffffffu, ti.kind, 0);
       const OpDev* op = &args.ops[ti.kind == kEnd ? args.slots[0] : ti.slot];
       const bool dual = kDual && two && ti.kind != kEnd;
-      const int second = islot + 1 == kRing ? 0 : islot + 1;
-      if (published >= kRing && !wwait_cluster(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
-      if (dual && published + 1 >= kRing && !wwait_cluster(c, &sc->iempty[second], second == 0 ? iph : iph ^ 1u, 2)) break;
-      if (dual) ti.expert |= kDualFirst;
+      if (lapped && !wwait_cluster(c, &sc->iempty[islot], iph ^ 1u, 2)) break;
+      if (dual) ti.expert |= kTwoTiles;
       if (ti.kind != kEnd && need_ready && !wait_op_ready(c, lane, ti)) ti.kind = kEnd;
       // A down tile is handed over at once: the producers fill the free stages with its weights and add the rows when its gate/up
       // tiles are committed (one token: 67.6 -> 67.0 us a pass, 128 tokens on 8 experts: 80.3 -> 79.1).
       int ok = 1;
       if (lane == 0) {
         publish(sc, islot, ti);
-        if (dual && ti.kind != kEnd) {
-          TileInfo nx = ti;
-          nx.expert &= ~kDualFirst;
-          ++nx.n;
-          ++nx.tile;
-          publish(sc, second, nx);
-        }
         if (ti.kind == kDown) {
           ok = wait_counter(c, &g1_done_of(c, op)[ti.m], args.I / kTileN1 * kStoreWarps, 3);
           fence_async_proxy();
@@ -439,10 +431,6 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (ok) {
           mbar_arrive_cluster(map_to_cta(&sc->rows_in[islot], 1));
           mbar_arrive(&sc->rows_in[islot]);
-          if (dual) {                                     // (nobody waits there)
-            mbar_arrive_cluster(map_to_cta(&sc->rows_in[second], 1));
-            mbar_arrive(&sc->rows_in[second]);
-          }
         }
         // (asked before the first hand-over, that would wait for the answer: its arrivals release)
         if (!asked) ticket = take_turn(&args);
@@ -464,9 +452,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (__shfl_sync(0xffffffffu, ok, 0) == 0) break;
       }
       if (!wwait(c, &sc->taken[islot], iph, 26)) break;
-      published = min(published + (dual ? 2 : 1), kRing);
-      if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (dual && ++islot == kRing) { islot = 0; iph ^= 1u; }
+      if (++islot == kRing) { islot = 0; iph ^= 1u; lapped = true; }
       two = false;
       if (plain) ti.kind = kEnd;
       else claim_next<true, kDual>(c, &sc->qt, rh, lane, ti, need_ready, two);
@@ -477,15 +463,12 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
     ended = false;
     int islot = 0;
     unsigned iph = 0;
-    bool second = false;                                  // of two tiles that run together
     while (true) {
       if (!wait_info(c, &sc->ifull[islot], iph, 34, false)) break;
       const int kind = sc->info[islot].kind, slot = sc->info[islot].slot, row0 = sc->info[islot].row0, rows = sc->info[islot].rows;
-      const bool dual = (sc->info[islot].expert & kDualFirst) != 0;
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
-      if (kind == kGateUp && !second) list_rows(c, sc, islot, slot, row0, rows, 1, lane);
-      second = dual;
+      if (kind == kGateUp) list_rows(c, sc, islot, slot, row0, rows, 1, lane);
       if (lane == 0) release_slot(sc, islot, false);
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
     }
@@ -505,18 +488,12 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         if (!info_wait_one(c, &sc->ifull[islot], iph, 21, leader)) break;
         const TileInfo ti = sc->info[islot];
         if (ti.kind == kEnd) { ended = true; break; }
-        const bool dual = kDual && (ti.expert & kDualFirst) != 0;
+        const bool dual = kDual && (ti.expert & kTwoTiles) != 0;
         unsigned long long* const taken = &sc->taken[islot];
         const int claim_at = dual && leader && sc->qt.two_classes != 0 ? late_claim(ti.kblocks) : 0;
         if (leader && claim_at == 0) mbar_arrive(taken);
         release_slot(sc, islot, leader);
         if (++islot == kRing) { islot = 0; iph ^= 1u; }
-        if (dual) {                                          // the descriptor behind it is for those that store the tiles
-          if (!info_wait_one(c, &sc->ifull[islot], iph, 21, leader)) break;
-          if (leader) mbar_arrive(&sc->taken[islot]);
-          release_slot(sc, islot, leader);
-          if (++islot == kRing) { islot = 0; iph ^= 1u; }
-        }
         if (ti.kind == kCombine) continue;
         const OpDev* op = &args.ops[ti.slot];
         const WeightPlan wp = weight_plan(op, ti, rank, dual);
@@ -562,13 +539,8 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       while (true) {
         if (!info_wait_one(c, &sc->ifull[islot], iph, 6, true)) break;
         const int kind = sc->info[islot].kind, kblocks = sc->info[islot].kblocks, rows = sc->info[islot].rows;
-        const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
+        const bool dual = kDual && (sc->info[islot].expert & kTwoTiles) != 0;
         if (kind == kEnd) { ended = true; break; }
-        if (dual) {                                       // the second tile's descriptor
-          mbar_arrive(&sc->iempty[islot]);
-          if (++islot == kRing) { islot = 0; iph ^= 1u; }
-          if (!info_wait_one(c, &sc->ifull[islot], iph, 6, true)) break;
-        }
         if (kind != kCombine) {
           const unsigned b = gcount & 1u;
           if (!wwait_relaxed(c, &sc->tempty[b], ((gcount >> 1) & 1u) ^ 1u, 7)) break;
@@ -651,16 +623,11 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       while (true) {
         if (!info_wait_one(c, &sc->ifull[islot], iph, 24, false)) break;
         const int kind = sc->info[islot].kind;
-        const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
+        const bool dual = kDual && (sc->info[islot].expert & kTwoTiles) != 0;
         const int n_stages = sc->info[islot].kblocks >> (kblocks_a_stage<kDual>(sc->info[islot].rows, dual) - 1);
         if (kind == kEnd) { ended = true; break; }
         release_slot(sc, islot, false);
         if (++islot == kRing) { islot = 0; iph ^= 1u; }
-        if (dual) {
-          if (!info_wait_one(c, &sc->ifull[islot], iph, 24, false)) break;
-          release_slot(sc, islot, false);
-          if (++islot == kRing) { islot = 0; iph ^= 1u; }
-        }
         if (kind == kCombine) continue;
         if (kind != kGateUp) { kiter += (unsigned)n_stages; continue; }
         bool fail = false;
@@ -700,18 +667,13 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       const int kind = sc->info[islot].kind;
       const int kblocks = sc->info[islot].kblocks;
       const int rows = sc->info[islot].rows, row0 = sc->info[islot].row0, slot = sc->info[islot].slot;
-      const bool dual = kDual && (sc->info[islot].expert & kDualFirst) != 0;
+      const bool dual = kDual && (sc->info[islot].expert & kTwoTiles) != 0;
       const int step = kblocks_a_stage<kDual>(rows, dual);
       __syncwarp();
       if (kind == kEnd) { ended = true; break; }
       const int tslot = islot;
       const unsigned tph = iph;
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (dual) {
-        if (!wait_info(c, &sc->ifull[islot], iph, 13, leader)) break;
-        if (lane == 0) release_slot(sc, islot, leader);
-        if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      }
       const OpDev* op = &args.ops[slot];
       // Consecutive rows: one thread of one warp loads their boxes, once the scheduler has seen them in place (the weights of a down tile
       // are loaded meanwhile) and the producer has the stage.
@@ -829,6 +791,10 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (!wwait_cluster(c, &sc->done[islot], iph, 17)) break;
       if (lane == 0) {
         commit_tile<false>(c, rh, ti, watched);
+        if (kDual && (ti.expert & kTwoTiles) != 0) {
+          ++ti.tile;
+          commit_tile<false>(c, rh, ti, watched);
+        }
         mbar_arrive(&sc->iempty[islot]);
       }
       __syncwarp();
@@ -867,7 +833,7 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
       if (ti.kind == kEnd) { ended = true; break; }
       __syncwarp();
       if (!leader && lane == 0) release_slot(sc, islot, false);
-      const bool dual = kDual && (ti.expert & kDualFirst) != 0;
+      const bool dual = kDual && (ti.expert & kTwoTiles) != 0;
       OpDev* op = &args.ops[ti.slot];
       if (first) {
         first = false;
@@ -987,14 +953,6 @@ moe_apk_pair_kernel(const __grid_constant__ RunArgs args, RunHead* rh) {
         else signal_leader(&sc->done[islot], leader);
       }
       if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      if (dual) {                                             // the second tile's descriptor says nothing new
-        if (!wait_info(c, &sc->ifull[islot], iph, 9, leader)) break;
-        if (lane == 0) {
-          if (!leader) release_slot(sc, islot, false);
-          signal_leader(&sc->done[islot], leader);
-        }
-        if (++islot == kRing) { islot = 0; iph ^= 1u; }
-      }
     }
   }
 

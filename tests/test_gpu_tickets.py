@@ -170,3 +170,18 @@ def test_a_captured_step_in_twos_and_an_entry_out_of_range():
         step()
         ctx.check()
         assert all(torch.equal(b.y, w) for b, w in zip(bound, want))
+
+
+@pytest.mark.parametrize("n_ctas,T,H,I", [(6, 1800, 1024, 1024), (6, 1800, 1024, 1152), (0, 16384, 4096, 512)])
+def test_a_unit_holds_at_most_five_tickets(n_ctas, T, H, I):
+    """Four in the descriptor ring and the one that waits for a place, also where the epilogue is behind (combine tiles of many long rows, all units
+    at once) and in launches that run two tiles at a time."""
+    spec = synth.Spec("held", synth.Shape(6, 2, H, I), ((synth.PREFILL, T), (synth.DECODE, 300)), "zipf", 1.0, 1.0, -1.0, 109)
+    ctx, _ = run(spec, n_ctas=n_ctas, budget=2)
+    log = ctx.tile_log()
+    for u in np.unique(log["cta"]):
+        mine = log[log["cta"] == u]
+        claim = np.unique(mine["t_claim"])
+        end = np.array([mine["t_commit"][mine["t_claim"] == t].max() for t in claim])
+        held = [int((end[:i] > t).sum()) + 1 for i, t in enumerate(claim)]
+        assert len(claim) > 8 and max(held) <= 5, max(held)
