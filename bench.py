@@ -47,14 +47,14 @@ DEFAULT_STEPS = {"c2": (200, 10), "c3": (30, 5), "c4": (4, 3), "c5": (30, 5), "c
 # save/restore is too large); the full-size figures scale them by the number of active experts, because the
 # traffic is the weights of the active experts, read about once (c3: 256/64, c2: 251/63, c5: 256/32).
 NCU_DRAM_BYTES = {
-    ("c3s", "moe_apk_pair_kernel"): 2.040e9 + 0.154e9,
-    ("c3", "moe_apk_pair_kernel"): (2.040e9 + 0.154e9) * 256 / 64,
-    ("c2s", "moe_apk_pair_kernel"): 1.812e9 + 0.006e9,
-    ("c2", "moe_apk_pair_kernel"): (1.812e9 + 0.006e9) * 251 / 63,
-    ("c4s", "moe_apk_pair_kernel"): 3.053e9 + 0.329e9,           # decode + prefill op paired (carrier tiles)
-    ("c4", "moe_apk_pair_kernel"): (3.053e9 + 0.329e9) * 256 / 64,
-    ("c5s", "moe_apk_kernel"): 1.546e9 + 0.056e9,                # paired, decode budget 96
-    ("c5", "moe_apk_kernel"): (1.546e9 + 0.056e9) * 256 / 32,
+    ("c3s", "moe_apk_pair_kernel"): 2.033e9 + 0.151e9,
+    ("c3", "moe_apk_pair_kernel"): (2.033e9 + 0.151e9) * 256 / 64,
+    ("c2s", "moe_apk_pair_kernel"): 1.812e9 + 0.005e9,
+    ("c2", "moe_apk_pair_kernel"): (1.812e9 + 0.005e9) * 251 / 63,
+    ("c4s", "moe_apk_pair_kernel"): 3.028e9 + 0.326e9,           # decode + prefill op paired (carrier tiles)
+    ("c4", "moe_apk_pair_kernel"): (3.028e9 + 0.326e9) * 256 / 64,
+    ("c5s", "moe_apk_kernel"): 1.543e9 + 0.059e9,                # paired, decode budget 96
+    ("c5", "moe_apk_kernel"): (1.543e9 + 0.059e9) * 256 / 32,
 }
 
 def load_peaks():
