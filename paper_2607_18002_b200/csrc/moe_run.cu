@@ -971,7 +971,8 @@ __global__ void __launch_bounds__(kThreads, 1) moe_apk_kernel(const __grid_const
       OpDev* op = &args.ops[ti.slot];
       bool ok = true;
       if (ti.kind == kCombine) {
-        combine_tokens(op, ti.row0, ti.row0 + ti.rows, 0, args.H / 8, args.k, args.H, etid, 256, CombineNow{});
+        if constexpr (kSmall) combine_tokens_called(op, ti.row0, ti.row0 + ti.rows, args.k, args.H, etid, 256);
+        else combine_tokens(op, ti.row0, ti.row0 + ti.rows, 0, args.H / 8, args.k, args.H, etid, 256, CombineNow{});
       } else if constexpr (kSmall) {
         ok = ti.rows <= 32 ? epilogue_fp8_small<32>(c, sc, op, ti, tmem, warp, lane, eph, xph, kseq)
                            : epilogue_fp8_small<64>(c, sc, op, ti, tmem, warp, lane, eph, xph, kseq);
