@@ -38,9 +38,9 @@ struct CombineNow {
   __device__ __forceinline__ bool operator()() const { return true; }
 };
 // Inlined, once a kernel (but see combine_tokens_called): called, it took its arguments through local memory and made the persistent kernels
-// spill, round trips to L2 in every tile behind the rows that pass through what L1 the pipelines leave.  us a pass, called / inlined: 12 000 tokens on 8 experts of 0.8 MB
-// 104 / 101, 8000 on 32 of 3 MB 182 / 174, 8192 on 256 of 28 MB 2228 / 2203, one token 55.7 / 54.4; bf16 on 147 CTAs, 4096 tokens on 64 experts
-// 1084 / 1034.
+// spill, round trips to L2 in every tile behind the rows that pass through what L1 the pipelines leave.  us a pass, called / inlined: 12 000
+// tokens on 8 experts of 0.8 MB 104 / 101, 8000 on 32 of 3 MB 182 / 174, 8192 on 256 of 28 MB 2228 / 2203, one token 55.7 / 54.4; bf16 on 147
+// CTAs, 4096 tokens on 64 experts 1084 / 1034.
 template <class Ready>
 __device__ __forceinline__ bool combine_tokens(const OpDev* op, int t0, int t1, int v0, int nv, int k, int H, int tid, int nthr, Ready ready) {
   const unsigned n_rows = (unsigned)op->space_rows;    // rows of the packed space D lives in
@@ -157,9 +157,9 @@ __device__ __forceinline__ bool combine_tokens(const OpDev* op, int t0, int t1, 
   }
   return true;
 }
-// ... called: the e4m3 kernel of tiles of up to 64 rows.  A launch of microseconds pays for more cold code: 1, 2 and 8 tokens on 16 experts of 0.9 MB
-// 25.6, 25.5 and 27.2 us a pass inlined, 25.3, 25.1 and 26.7 called; 64 of them, and 16 on 32 experts
-// of 38 MB, one on 64, 48 on 256, the same either way.
+// ... called: the e4m3 kernel of tiles of up to 64 rows.  A launch of microseconds pays for more cold code: 1, 2 and 8 tokens on 16 experts of
+// 0.9 MB 25.6, 25.5 and 27.2 us a pass inlined, 25.3, 25.1 and 26.7 called; 64 of them, and 16 on 32 experts of 38 MB, one on 64, 48 on 256,
+// the same either way.
 static __device__ __noinline__ void combine_tokens_called(const OpDev* op, int t0, int t1, int k, int H, int tid, int nthr) {
   combine_tokens(op, t0, t1, 0, H / 8, k, H, tid, nthr, CombineNow{});
 }

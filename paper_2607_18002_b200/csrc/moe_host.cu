@@ -538,7 +538,8 @@ int moe_run(moe_ctx_t* ctx, const int32_t* slots, int n_ops, int fuse_combine, v
   //   16 and 8, 32 experts: 2400 83 / 88 (4.0), 4000 112 / 117 (6.7), 6000 144 / 142 (10), 12 000 256 / 249 (20).
   // Where experts get few rows most tiles are short ones that the bound does not count, and two at a time pay earlier:
   //   48 and 24: 777 tokens on 256 experts 1181 / 1159 (7.8), 600 on 128 632 / 626 (5.8); 16 and 8: 1500 on 128 142 / 141 (5.0); but 32 and 16: 700
-  //   on 128 315 / 320 (4.5).  8 or more k-blocks: 5000 tokens on 8 experts with 4 and 8 of them take 61 / 65.
+  //   on 128 315 / 320 (4.5).  Between three and five rounds it depends on how many experts the tokens choose, which is not known here: 400 tokens, 16
+  //   of 256 experts 134 / 144, 32 of them 203 / 206, 96 472 / 473, 192 883 / 876, all 1112 / 1105.  8 or more k-blocks: 5000 tokens on 8 experts with 4 and 8 of them take 61 / 65.
   const long long rounds = routed <= (long long)kDualFewRows * c.n_experts ? kDualRoundsFew : kDualRounds;
   const bool dual = may_run_twos(ctx) && routed / kWorkRowsBf16 * (ctx->L.NT1 + ctx->L.NT2) >= rounds * (ctx->n_ctas / 2) &&
                     a.kb_gate_up >= kDualBlocks && a.kb_down >= kDualBlocks;
